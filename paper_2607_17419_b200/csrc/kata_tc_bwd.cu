@@ -184,7 +184,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
     }
   } else if (warp == 1) {
     // =========================== score MMA issuer: [S | C] ===========================
-    if (lane == 0) {
+    if (elect_one()) {
       const uint32_t idesc = instr_desc(kFmtBF16, kFmtBF16, 0, 0, 128, 64);
       const uint64_t dk = smem_desc(0, 16, 1024, kSwizzle128B);
       const uint32_t x1 = smem_u32(base + OFF_X1), x2 = smem_u32(base + OFF_X2);
@@ -209,7 +209,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
     }
   } else if (warp == 2) {
     // =========================== output MMA issuer ===========================
-    if (lane == 0) {
+    if (elect_one()) {
       const uint32_t idesc = instr_desc(kFmtBF16, kFmtBF16, 0, 1, 128, 64);     // A tmem, B MN-major
       // MN-major, 128B swizzle: 8 streamed rows x 64 columns per 1 KB atom (SBO); 16 rows per MMA
       const uint64_t dmn = smem_desc(0, 8192, 1024, kSwizzle128B);
@@ -526,7 +526,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if ((warp == 1 || warp == 2) && lane == 0) {
+  if ((warp == 1 || warp == 2) && elect_one()) {
     mma_commit(bar(BAR_DRAIN));
     mbar_wait(bar(BAR_DRAIN), 0);
   }

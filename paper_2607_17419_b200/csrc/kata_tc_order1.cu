@@ -287,8 +287,8 @@ tc_order1_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     }
   } else if (warp == W_MMA_A) {
     // =========================== scores P = Q K^T ===========================
-    // Four issuer warps, one per MMA group of a tile: a thread gets an MMA out about every hundred cycles whatever
-    // its size, and the groups of a tile do not depend on one another.  Every lane waits, lane 0 issues (a warp of
+    // Four issuer warps, one per MMA group of a tile: the groups of a tile do not depend on one another, and a
+    // thread that waits for one group's operands should not hold up the next group's MMAs.  Every lane waits, one issues (a warp of
     // waiters is woken sooner than a single waiting lane).
     if (wo) {
       const uint32_t idQK = instr_desc(kFmtBF16, kFmtBF16, 0, 0, 128, 128);
@@ -298,7 +298,7 @@ tc_order1_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         ok = wait_or_abort_counted(bar(BAR_FULL + s), (j / NSTAGE) & 1, abort_flag) &&
              wait_or_abort_counted(bar(BAR_P_EMPTY + b), ((j >> 1) & 1) ^ 1, abort_flag);
         if (!ok) break;
-        if (lane == 0) {
+        if (elect_one()) {
           const uint32_t qa = smem_u32(qtile(s)), ka = smem_u32(ktile(s));
           tc_fence_after();
 #pragma unroll
@@ -324,7 +324,7 @@ tc_order1_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       // the accumulators are free once the snapshot of the previous state has left TMEM
       if (ok && upd && wo && j > 0) ok = wait_or_abort_counted(bar(BAR_SNAP_LD), (j - 1) & 1, abort_flag);
       if (!ok) break;
-      if (lane == 0) {
+      if (elect_one()) {
         const uint32_t ka = smem_u32(ktile(s)), va = smem_u32(vtile(s));
         if (upd) {
           tc_fence_after();
@@ -354,7 +354,7 @@ tc_order1_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         // the snapshot after tile j - 1 went to buffer j & 1; it is that buffer's ((j - 1) / 2)-th
         if (ok && j > 0) ok = wait_or_abort_counted(bar(BAR_SNAP_ST + (j & 1)), ((j - 1) >> 1) & 1, abort_flag);
         if (!ok) break;
-        if (lane == 0) {
+        if (elect_one()) {
           if (resume || j > 0) {
             const uint32_t qa = smem_u32(qtile(s));
             tc_fence_after();
@@ -379,7 +379,7 @@ tc_order1_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
              wait_or_abort_counted(bar(BAR_P_FULL + b), (j >> 1) & 1, abort_flag) &&
              wait_or_abort_counted(bar(BAR_R_DONE + b), (j >> 1) & 1, abort_flag);
         if (!ok) break;
-        if (lane == 0) {
+        if (elect_one()) {
           const uint32_t va = smem_u32(vtile(s));
           tc_fence_after();
 #pragma unroll
@@ -507,7 +507,7 @@ tc_order1_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if ((warp == W_MMA_A || warp == W_MMA_B || warp == W_MMA_U || warp == W_MMA_R) && lane == 0) {
+  if ((warp == W_MMA_A || warp == W_MMA_B || warp == W_MMA_U || warp == W_MMA_R) && elect_one()) {
     mma_commit(bar(BAR_DRAIN));
     mbar_wait(bar(BAR_DRAIN), 0);
   }

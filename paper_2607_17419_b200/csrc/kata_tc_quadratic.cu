@@ -203,7 +203,7 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     }
   } else if (warp == 1) {
     // =========================== score MMA issuer: S = Q K^T ===========================
-    if (lane == 0) {
+    if (elect_one()) {
       const uint32_t idesc = instr_desc(kFmtBF16, kFmtBF16, 0, 0, 128, KT);
       const uint64_t dk = smem_desc(0, 16, 1024, kSwizzle128B);
       uint32_t it = 0;
@@ -231,7 +231,7 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     }
   } else if (warp == 2) {
     // =========================== apply MMA issuer: [O | D] += P [V' | r] ===========================
-    if (lane == 0) {
+    if (elect_one()) {
       const uint32_t idesc = instr_desc(kFmtBF16, kFmtBF16, 0, 1, 128, 80);     // A tmem, B MN-major, N = 64 + 16
       // MN-major, 128B swizzle: 8 key rows per 1024-byte atom (SBO), second group of 64 columns 16 KB on (LBO)
       const uint64_t dmn = smem_desc(0, 16384, 1024, kSwizzle128B);
@@ -439,7 +439,7 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if ((warp == 1 || warp == 2) && lane == 0) {
+  if ((warp == 1 || warp == 2) && elect_one()) {
     mma_commit(bar(BAR_DRAIN));
     mbar_wait(bar(BAR_DRAIN), 0);
   }

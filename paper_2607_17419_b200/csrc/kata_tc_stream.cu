@@ -475,7 +475,7 @@ tc_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     // =========================== update issuers: S += W^T K ===========================
     // Two threads share the MMAs of one 16-token step (their accumulators are disjoint): warp 1 the b-blocks
     // 0..2, warp 0 b-block 3 and Z.  Warp 0 is also the TMA producer of the query and key tiles.
-    if (lane == 0) {
+    if (elect_one()) {
       // A: MN-major, 128B swizzle: 64 rows x 8 tokens per 1 KB atom; next 8 tokens +1 KB (SBO), next 64 rows +2 KB (LBO)
       const uint64_t dA = smem_desc(0, 2048, 1024, kSwizzle128B);
       // B: the key tile read MN-major (N = feature a, K = token): one atom of 64 features x 8 tokens per 1 KB
@@ -543,7 +543,7 @@ tc_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     }
   } else if (warp == WARP_R) {
     // =========================== read issuer: Y = Q S'^T, 8 pieces ===========================
-    if (lane == 0 && wo) {
+    if (wo && elect_one()) {
       const uint32_t idR = instr_desc(kFmtBF16, kFmtBF16, 0, 0, 128, 80);
       const uint64_t dS = smem_desc(0, 16, 1024, kSwizzle128B);
       const uint32_t spa = smem_u32(base + OFF_SP);
@@ -570,7 +570,7 @@ tc_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     }
   } else if (warp == WARP_I) {
     // =========================== intra-tile issuer: scores and [O | D] ===========================
-    if (lane == 0 && wo) {
+    if (wo && elect_one()) {
       constexpr int NP = geo::NP, KH = geo::KH;
       const uint32_t idQK = instr_desc(kFmtBF16, kFmtBF16, 0, 0, 128, KH);
       const uint32_t idPV = instr_desc(kFmtBF16, kFmtBF16, 0, 1, 128, 16);
@@ -1093,7 +1093,7 @@ tc_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (warp <= WARP_I && lane == 0) {
+  if (warp <= WARP_I && elect_one()) {
     mma_commit(bar(BAR_DRAIN));
     mbar_wait(bar(BAR_DRAIN), 0);
   }

@@ -202,6 +202,15 @@ __host__ __device__ constexpr uint32_t instr_desc(uint32_t a_fmt, uint32_t b_fmt
 // ---------------------------------------------------------------------------------------------
 // MMA issue (one thread) and commit
 // ---------------------------------------------------------------------------------------------
+// One lane of a converged warp (the same one every time).  An MMA issuer must be chosen this way and not by `lane == 0`:
+// behind elect.sync the compiler knows that one thread runs and keeps descriptors and TMEM addresses in uniform
+// registers, behind a lane test it moves them there before every tcgen05.mma.  Cycles per MMA back to back, one issuer,
+// M = 128, K = 16 (lane test -> elected): A in TMEM and N = 64 47 -> 32, N = 80 55 -> 40; the pipe's own rate is N / 2.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.u32 %0, 1, 0, P;\n\t}" : "=r"(p));
+  return p != 0;
+}
 // D[tmem] (+)= A[smem] * B[smem]
 __device__ __forceinline__ void mma_f16_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
                                            uint32_t accumulate) {
