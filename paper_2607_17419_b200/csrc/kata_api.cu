@@ -138,18 +138,15 @@ int tensor_scan_group(int BH, int slices, int NC, double* model_us = nullptr) {
   return G < NC ? G : NC;
 }
 
-// inter_chunk = AUTO on the tensor-core kernels: the scan form where its modelled time is below nine tenths of the
-// sequential walk's.  The sequential walk is the feature-split kernel where it applies (nine CTAs per head in whole
-// waves of 148, about 3.3 us a tile of 128 tokens with the GPU full and 2.6 us with a few heads), else the streaming
-// kernel (one CTA per head and value slice, 4.4 us a tile).
-bool tensor_scan_pays(int BH, int NC, int split_ctas) {   // split_ctas: CTAs per head of the feature-split kernel, 0 = not used
+// inter_chunk = AUTO on the streaming kernels: the scan form where its modelled time is below nine tenths of the
+// sequential walk's (one CTA per head and value slice, 4.4 us a tile).
+bool tensor_scan_pays(int BH, int NC) {
   const int cpt = tc_stream_tile() / kChunk;
   const int tiles = (NC + cpt - 1) / cpt;
   const int slices = tc_chunked_slices();
   double scan_us;
   tensor_scan_group(BH, slices, NC, &scan_us);
-  const double seq_us = split_ctas > 0 ? ceil((double)split_ctas * BH / 148.0) * tiles * (split_ctas * BH >= 74 ? 3.3 : 2.6) + 10.0
-                              : scan_pass_us((double)slices * BH, tiles, kFullTileUs);
+  const double seq_us = scan_pass_us((double)slices * BH, tiles, kFullTileUs);
   return scan_us < 0.9 * seq_us;
 }
 
@@ -269,6 +266,19 @@ Staging staging_layout(const Problem& p, size_t inner_bytes) {
   return s;
 }
 
+// Scratch of the sequential chunked form (full lift, no state pointers) as published: callers that sized a buffer once
+// keep it.  The chunk states take less at every size where one segment walks a head; the larger of the two is asked for.
+size_t published_chunked_bytes(int BH, int T) {
+  const size_t nt = (T + 127) / 128, rows = (size_t)BH * T;
+  return align_up((BH * nt + 1) * 4) + align_up(rows * 128) + align_up(rows * 2) + align_up(BH * 9 * nt * (128 * 128 + 128 * 8));
+}
+
+// A state handed in or out on a short call: the streaming kernel while its CTAs (eight per head) are one wave.  Measured,
+// us, chunk states / streaming kernel: 16 heads, T = 256: 34 / 24, 512: 33 / 31, 1024: 35 / 45; 128 heads, T = 256: 98 / 128.
+bool short_state_call(int BH, int T) { return T <= 512 && BH * 8 <= 148; }
+// inter_chunk = AUTO where the model above prefers the scan form: fewer tokens x heads than this stay on its group passes.
+constexpr long long kStreamScanTokens = 16384;
+
 // Diagnostic override: KATA_CHUNKED_KERNEL=stream in the environment keeps the sequential chunked form on the
 // value-sliced streaming kernel (for A/B timing); read once.
 bool stream_kernel_forced() {
@@ -302,7 +312,8 @@ struct Prepared {
   size_t inner_bytes;
   bool tensor;
   int C;
-  bool split;           // sequential chunked form on the feature-split kernel (needs scratch for the links of a head)
+  bool states;          // chunked form on the chunk-state and attend kernels
+  StatePlan sp;         // its chunks
   bool pad;             // bf16 rows narrower than 64 are zero-padded to 64 so that the tensor-core kernels apply
   size_t pad_bytes;     // one padded tensor [B*H*T][64] bf16 (q, k, v, out: four of them at the start of the scratch)
 };
@@ -368,19 +379,23 @@ int prepare(int fn, const void* q, const void* k, const void* v, void* out, int 
     if (r.pad) r.pad_bytes = align_up((size_t)B * H * T * 64 * 2);
   }
   const Problem kp = kernel_problem(r);
+  bool auto_scan = false;
   if (r.o.inter_chunk == KATA_INTER_AUTO) {
     Opts scan = r.o;
     scan.inter_chunk = KATA_SCAN;
     r.o.inter_chunk = KATA_SEQUENTIAL;
-    if (C == kChunk && want_tensor(fn, kp, r.o) && want_tensor(fn, kp, scan) && tensor_scan_pays(B * H, (T + C - 1) / C, (r.o.s_init == nullptr && tc_split_supported(kp) && !stream_kernel_forced()) ? tc_split_ctas_per_head(kp) : 0))
+    if (C == kChunk && want_tensor(fn, kp, r.o) && want_tensor(fn, kp, scan) && tensor_scan_pays(B * H, (T + C - 1) / C)) {
       r.o.inter_chunk = KATA_SCAN;
+      auto_scan = true;
+    }
   }
   r.tensor = want_tensor(fn, kp, r.o);
   if (r.o.impl == KATA_IMPL_TENSOR && !r.tensor) return KATA_ERR_UNSUPPORTED_SHAPE;
   r.C = fn == KATA_FN_QUADRATIC ? kChunk : C;
   r.plan = ScanPlan{(T + r.C - 1) / r.C, 0, 1, 0};
   r.state_elems = 0;
-  r.split = false;
+  r.states = false;
+  if (fn == KATA_FN_QUADRATIC && r.tensor) r.pad = false;      // the attend kernel reads narrow rows as they are
   r.inner_bytes = (fn == KATA_FN_QUADRATIC && r.tensor) ? tc_quadratic_workspace_bytes(kp) : 0;
   if (fn != KATA_FN_QUADRATIC) {
     if (r.tensor && r.o.s_pre != nullptr && fn == KATA_FN_CHUNK_STATE_SCAN) r.tensor = false;   // per-chunk export: SIMT pipeline
@@ -389,10 +404,21 @@ int prepare(int fn, const void* q, const void* k, const void* v, void* out, int 
     st = make_plan(fn, kp, r.o, r.tensor, r.C, r.plan, r.state_elems);
     if (st != KATA_OK) return st;
     r.inner_bytes = inner_workspace(fn, r.plan, kp, r.state_elems);
-    // one pass over the whole sequence, no state handed in or out: the feature-split kernel
-    r.split = fn == KATA_FN_CHUNKED && r.tensor && r.plan.n_groups == 1 && r.o.s_pre == nullptr && r.o.s_init == nullptr &&
-              tc_split_supported(kp) && !stream_kernel_forced();
-    if (r.split) r.inner_bytes = align_up(tc_split_workspace_bytes(kp));
+    const bool state_in = r.o.s_init != nullptr, state_out = r.o.s_pre != nullptr;
+    r.states = fn == KATA_FN_CHUNKED && r.tensor && r.p.feature_order == 2 && !stream_kernel_forced() &&
+               ((r.o.inter_chunk == KATA_SEQUENTIAL && (!(state_in || state_out) || !short_state_call(B * H, T))) ||
+                (auto_scan && (long long)B * H * T >= kStreamScanTokens));
+    if (r.states) {
+      r.pad = false;
+      Problem sp = r.p;
+      r.sp = tc_chunk_plan(sp, state_in, state_out);
+      r.inner_bytes = align_up(tc_chunk_workspace_bytes(sp, r.sp, state_in, state_out));
+      if (r.p.groups == 1 && !state_in && !state_out) {
+        const size_t least = published_chunked_bytes(B * H, T);
+        if (r.inner_bytes < least) r.inner_bytes = least;
+      }
+      return KATA_OK;
+    }
     // state import and final-state export of the fp32 path go through one internal state per head
     if (fn == KATA_FN_CHUNKED && (r.o.s_pre != nullptr || r.o.s_init != nullptr) && !r.tensor)
       r.inner_bytes = align_up((size_t)B * H * r.state_elems * sizeof(float));
@@ -401,7 +427,7 @@ int prepare(int fn, const void* q, const void* k, const void* v, void* out, int 
     if (fn == KATA_FN_CHUNKED && r.tensor && r.o.z_init != nullptr && r.o.z_init == r.o.z_pre)
       r.inner_bytes = align_up((size_t)B * H * decode_n_psi(d_k, r.o.state_layout, 2, r.o.groups) * sizeof(float));
   }
-  r.inner_bytes += 4 * r.pad_bytes;
+  if (r.pad) r.inner_bytes += 4 * r.pad_bytes;
   return KATA_OK;
 }
 
@@ -436,8 +462,8 @@ int run_device(int fn, Prepared& r, void* ws) {
     const bool use_scan = (fn == KATA_FN_CHUNK_STATE_SCAN) || r.plan.n_groups > 1;
     if (r.tensor && P.feature_order == 1) {
       tc_order1(P, r.plan, use_scan, r.C, wsf, r.o.device_status, ctx);
-    } else if (r.split) {
-      tc_chunked_split(P, ws, r.o.device_status, ctx);
+    } else if (r.states) {
+      tc_chunked_states(P, r.sp, ws, r.o.device_status, r.o.s_init, r.o.z_init, r.o.s_pre, r.o.z_pre, r.o.state_layout, ctx);
     } else if (r.tensor) {
       const float* z_init = r.o.z_init;
       if (fn == KATA_FN_CHUNKED && z_init != nullptr && z_init == r.o.z_pre) {
@@ -569,11 +595,18 @@ bool host_pipe_plan(int fn, const Prepared& r, const kata_opts* opts, int C, Pip
   const size_t n_psi = (size_t)decode_n_psi(p.d_k, KATA_LAYOUT_DIRECT, 2, p.groups);
   pp.s_bytes = align_up((size_t)p.B * p.H * n_psi * p.d_v * sizeof(float));
   pp.z_bytes = align_up((size_t)p.B * p.H * n_psi * sizeof(float));
-  kata_opts po = *opts;
-  po.state_layout = KATA_LAYOUT_DIRECT;
-  po.s_init = po.s_pre = reinterpret_cast<float*>(kAlign);       // any non-null, aligned value: sizes only
-  po.z_init = po.z_pre = reinterpret_cast<float*>(kAlign);
-  pp.inner_bytes = align_up(kata_workspace_bytes(KATA_FN_CHUNKED, p.B, p.H, pp.piece_T, p.d_k, p.d_v, C, &po));
+  // the largest need of the first piece (state out), the middle ones (in place) and the last (state in, its own length)
+  const int last_T = p.T - (pp.pieces - 1) * pp.piece_T;
+  pp.inner_bytes = 0;
+  for (int i = 0; i < 3; ++i) {
+    float* const some = reinterpret_cast<float*>(kAlign);        // any non-null, aligned value: sizes only
+    kata_opts po = *opts;
+    po.state_layout = KATA_LAYOUT_DIRECT;
+    po.s_init = po.z_init = i > 0 ? some : nullptr;
+    po.s_pre = po.z_pre = i < 2 ? some : nullptr;
+    const size_t b = align_up(kata_workspace_bytes(KATA_FN_CHUNKED, p.B, p.H, i < 2 ? pp.piece_T : last_T, p.d_k, p.d_v, C, &po));
+    if (b > pp.inner_bytes) pp.inner_bytes = b;
+  }
   pp.total = 8 * pp.tensor_bytes + pp.s_bytes + pp.z_bytes + pp.inner_bytes;
   return pp.total <= r.o.workspace_bytes;
 }

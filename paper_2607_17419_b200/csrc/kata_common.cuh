@@ -97,12 +97,44 @@ void decode_step(const void* q, const void* k, const void* v, void* out, float* 
 bool tc_supported(const Problem& p, int fn);
 size_t tc_quadratic_workspace_bytes(const Problem& p);
 void tc_quadratic(const Problem& p, void* workspace, int* device_status, LaunchCtx& ctx);
+// r = 1 / ||k||^2 [BH][T] (bf16), which the kernels below take
+void tc_rscale(const Problem& p, __nv_bfloat16* rscale, LaunchCtx& ctx);
+// States before the chunks (kata_tc_state.cu), for tc_attend.
+struct StatePlan {
+  int chunk_tokens;            // a multiple of 256
+  int n_chunks;
+  int segments, seg_chunks;    // segments of the chunk axis walked side by side
+};
+struct StateBuffers {
+  __nv_bfloat16* s;            // as in AttendStates
+  __nv_bfloat16* z;
+  float* s_loc;                // [BH][n_chunks][rows][64] and [BH][n_chunks][rows], used with several segments
+  float* z_loc;
+  const float* s_init;         // public layouts (null: zero / not wanted)
+  const float* z_init;
+  float* s_final;
+  float* z_final;
+  int layout;
+};
+int tc_state_rows(int groups);
+void tc_states(const Problem& p, const __nv_bfloat16* rscale, const StatePlan& plan, const StateBuffers& buf, int* device_status,
+               LaunchCtx& ctx);
+// Outputs of blocks of 256 queries: over the keys of their chunk and the state before it (zero-initialise for the
+// quadratic form: one chunk, no state).
+struct AttendStates {
+  const __nv_bfloat16* s;      // [BH][n_chunks][rows of PairTable<G>][64]: the state before each chunk, weights of the pairs included
+  const __nv_bfloat16* z;      // [BH][n_chunks][64][64]: its normaliser as a symmetric matrix
+  int n_chunks, chunk_tokens;  // chunk_tokens: a multiple of 256
+  int first_state;             // first chunk that has a state before it (0 or 1)
+};
+void tc_attend(const Problem& p, const __nv_bfloat16* rscale, const AttendStates& st, int* device_status, LaunchCtx& ctx);
 void tc_chunked_stream(const Problem& p, int* device_status, LaunchCtx& ctx);
-// Sequential chunked form with the feature axis of the state split over the CTAs of a head (kata_tc_split.cu)
-bool tc_split_supported(const Problem& p);
-size_t tc_split_workspace_bytes(const Problem& p);
-int tc_split_ctas_per_head(const Problem& p);
-void tc_chunked_split(const Problem& p, void* workspace, int* device_status, LaunchCtx& ctx);
+// Chunked form on the chunk-state and attend kernels (kata_tc_chunked.cu).  n_chunks = 1 without state pointers: the
+// quadratic form alone.
+StatePlan tc_chunk_plan(const Problem& p, bool state_in, bool state_out);
+size_t tc_chunk_workspace_bytes(const Problem& p, const StatePlan& plan, bool state_in, bool state_out);
+void tc_chunked_states(const Problem& p, const StatePlan& plan, void* workspace, int* device_status, const float* s_init,
+                       const float* z_init, float* s_final, float* z_final, int state_layout, LaunchCtx& ctx);
 // State hand-off and groups of tiles for the second build of the streaming kernel (zero-initialise, then set).
 struct StreamIO {
   const float* s_init;         // state before the first token in the public layout (null: zero)

@@ -1,0 +1,715 @@
+// KATA forward of blocks of 256 queries on the Blackwell tensor cores (tcgen05 + TMEM), bf16: the quadratic
+// ("flash-style") form, and the output stage of the chunked form.
+//
+// Pre-pass (one light kernel per call): r[i] = 1 / ||k_i||^2 (bf16) into the workspace.
+//
+// Main kernel: persistent, one CTA per SM.  A work item = one head x 256 queries (two tiles of 128: the halves A and B);
+// the items are ordered heaviest first and dealt to the CTAs in rounds, forwards and backwards in turn.  An item is a
+// list of tiles that both halves walk:
+//   state tiles (chunked form, chunks after the first): the state S, Z before the chunk, in bf16
+//     Y = Q Z              one tile: Z as a symmetric 64 x 64 matrix; the normaliser of the state is q . Y per row
+//     O += Psi(Q) S        256 rows of the state per tile; the builders write the 256 feature products of their query
+//                          row as the A operand (TMEM)
+//   key tiles of 128 keys, from the start of the chunk (quadratic form: of the sequence) up to the diagonal:
+//     scores   S = Q K_j^T            A = the query tile in TMEM, B = the key tile (TMA, 128B swizzle)
+//     weights  P = r S^2 (causal mask on the diagonal tiles)  packed fp32x2 multiplies on the TMEM read-back, rounded
+//                                     to bf16, times r, stored back over the scores
+//     apply    [O | D] += P [V | 1]   A = P from TMEM, B = the value tile and a constant column of ones (MN-major,
+//                                     N = 80): the normaliser is column 64 of the same accumulator
+//   epilogue out = O / (D + q.Y)  (0 where that is 0)      the gate/normalise step of the readout
+// There is no running maximum and no rescaling: the weights are polynomial.  The query norm cancels between
+// numerator and denominator and is never applied.  In the quadratic form the d^2-wide feature state is never formed.
+// Rows narrower than 64 entries are read by TMA boxes of 64 columns, whose columns beyond the row are zero.
+//
+// What bounds it and why this split.  A key tile is 576 cycles of MMA per half (4 x N=128, 8 x N=80) and a chain
+// scores -> builders -> apply of about 1700, most of it hand-offs.  Four chains run side by side: two halves times two
+// sub-buffers of 64 score columns each.  Both halves share every key, value and state tile, which halves the tile
+// traffic into shared memory: with one query tile per CTA and Q as a shared-memory operand the port (A and B operands,
+// TMA writes, r) was asked for about 800 cycles per key tile, more than the MMAs take; here it is about 480.
+//
+// Nothing is set up per item: TMEM and the barriers are the CTA's, the stage ring runs on across items (every role
+// counts tiles cumulatively), the query tiles are double-buffered in shared memory and copied to TMEM before the
+// epilogue of the item before.
+//
+// Warps (640 threads): 0 TMA producer, 1 and 2 the MMA issuers of the halves, 3 key scales, 4-11 builders of half A,
+// 12-19 builders of half B (TMEM lane quadrant = warp % 4; the two warps of a quadrant have a sub-buffer each).  All
+// waits are bounded.
+#include <cuda.h>
+#include <type_traits>
+
+#include "kata_common.cuh"
+#include "kata_pairs.cuh"
+#include "kata_tmap.cuh"
+#include "kata_umma.cuh"
+
+namespace kata {
+namespace {
+
+using namespace umma;
+
+constexpr int D = 64;
+constexpr int QT = 128;          // queries per half
+constexpr int KTILE = 128;       // score columns per tile
+constexpr int NSTAGE = 4;        // shared-memory stages: a key and a value tile, or 256 rows of a state
+constexpr int NTHREADS = 640;
+constexpr int WARP_BLD0 = 4;
+
+constexpr uint32_t COL_S = 0;    // 2 x 128 fp32 score columns, one buffer per half; the operand of the apply MMA overwrites it
+constexpr uint32_t COL_O = 256;  // 2 x 80 fp32 accumulators: 64 outputs, column 64 = normaliser
+constexpr uint32_t COL_Q = 416;  // 2 x 32: the query tiles (bf16 A operands)
+constexpr uint32_t TMEM_COLS = 512;
+
+constexpr uint32_t OFF_Q = 0;                       // 2 x 2 x (128 x 64 bf16, 128B swizzle): the query tiles of this and the next item
+constexpr uint32_t STAGE_BYTES = 32768;             // K tile 16 KB, V tile 16 KB
+constexpr uint32_t OFF_ST = 65536;
+constexpr uint32_t OFF_ONES = OFF_ST + NSTAGE * STAGE_BYTES;   // 16 rows of [1, 0 ...]: columns 64.. of the values
+constexpr uint32_t OFF_ZEROS = OFF_ONES + 2048;                // 16 rows of zeros: columns 64.. of a state
+constexpr uint32_t OFF_RV = OFF_ZEROS + 2048;                  // NSTAGE x 128 bf16: 1 / ||k||^2 of the keys of a tile
+constexpr uint32_t OFF_DEN = OFF_RV + NSTAGE * 256;            // [half][sub][128] floats: the two shares of q . Y of a row meet here
+constexpr uint32_t OFF_BAR = OFF_DEN + 2048;
+constexpr uint32_t SMEM_BYTES = OFF_BAR + 512;
+constexpr uint32_t SMEM_ALLOC = SMEM_BYTES + 1024;
+static_assert(SMEM_ALLOC > 116 * 1024, "one CTA per SM is assumed (the CTA allocates all of TMEM)");
+
+// No barrier can complete two phases ahead of a waiter; a waiter that skips a phase (the builders the last one of an item
+// at BAR_SFREE) knows from a barrier that it waited for since that it is complete.
+enum {
+  BAR_QFULL = 0,     // [2] the query tiles of an item landed in shared memory
+  BAR_QEMPTY = 2,    // [2] ... and have been read (512 builders)
+  BAR_FULL = 4,      // [NSTAGE] tile (TMA bytes) and its key scales (scale warp) landed
+  BAR_EMPTY = 8,     // [NSTAGE] stage free: both issuers
+  BAR_SFULL = 12,    // [half][sub] scores in TMEM
+  BAR_PFULL = 16,    // [half][sub] the builders are done with the sub-buffer (128)
+  BAR_FFULL = 20,    // [half][sub][piece] features of a state tile in TMEM (128)
+  BAR_SFREE = 28,    // [half][sub][piece] ... and consumed
+  BAR_QT = 36,       // [2] query tile in TMEM (256)
+  BAR_ODONE = 38,    // [2] the MMAs of an item are complete: [O | D] is final
+  BAR_OFREE = 40,    // [2] [O | D] has been read (256): the next item may overwrite it
+  BAR_DRAIN = 42,
+  BAR_COUNT = 43
+};
+
+// Pre-pass: r = 1 / ||k||^2 per key row (0 for a zero row), one warp per 4 rows (8 lanes x 16 bytes per row).
+__global__ void __launch_bounds__(256) rscale_kernel(const __nv_bfloat16* __restrict__ k, __nv_bfloat16* __restrict__ rscale,
+                                                     size_t n_rows, int d) {
+  const size_t row = (size_t)blockIdx.x * 32 + (threadIdx.x >> 3);
+  const int part = threadIdx.x & 7;
+  if (row >= n_rows) return;
+  uint4 kraw = make_uint4(0u, 0u, 0u, 0u);
+  if (part * 8 < d) kraw = *reinterpret_cast<const uint4*>(k + row * d + part * 8);
+  const uint32_t kw[4] = {kraw.x, kraw.y, kraw.z, kraw.w};
+  float ss = 0.f;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const float lo = __uint_as_float(kw[e] << 16), hi = __uint_as_float(kw[e] & 0xFFFF0000u);
+    ss = fmaf(lo, lo, ss);
+    ss = fmaf(hi, hi, ss);
+  }
+  ss += __shfl_xor_sync(0xffffffffu, ss, 1);
+  ss += __shfl_xor_sync(0xffffffffu, ss, 2);
+  ss += __shfl_xor_sync(0xffffffffu, ss, 4);
+  if (part == 0) rscale[row] = __float2bfloat16_rn(inv_or_zero(ss));
+}
+
+__device__ __forceinline__ uint32_t mul_bf16x2(uint32_t a, uint32_t b) {
+  const __nv_bfloat162 p = __hmul2(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));
+  return *reinterpret_cast<const uint32_t*>(&p);
+}
+__device__ __forceinline__ uint4 lds128(uint32_t addr) {
+  uint4 v;
+  asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+  return v;
+}
+
+// Registers: 640 threads x 96 at launch; the four warps that issue and copy give theirs to the builders
+// (128 x 64 + 512 x 104 = 640 x 96).
+template <int N> __device__ __forceinline__ void regs_release() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
+template <int N> __device__ __forceinline__ void regs_take() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
+
+struct AArgs {
+  __nv_bfloat16* out;
+  const __nv_bfloat16* rscale;   // [BH][T] bf16: 1 / ||k||^2 (pre-pass)
+  int* device_status;
+  int Tlen;
+  int d_v;
+  int BH;
+  int n_pairs;                   // blocks of 256 queries of a head
+  int chunk_pairs;               // ... of a chunk (the quadratic form: n_pairs)
+  int n_chunks;
+  int first_state;               // first chunk that has a state before it
+};
+
+// G = feature groups of the blockwise map: a key tile holds KT = 128 / G keys, and the 128 score columns of a buffer
+// hold, for each half of those keys, the G per-group score blocks Q_a K_a^T side by side (group a in columns [a KT/2,
+// a KT/2 + KT/2) of the sub-buffer); the weight of a key is the sum over the groups of the squared scores.
+template <int G>
+__global__ void __launch_bounds__(NTHREADS, 1)
+tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
+                 const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmS,
+                 const __grid_constant__ CUtensorMap tmZ, const AArgs args) {
+  extern __shared__ unsigned char smem_raw[];
+  unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  auto bar = [&](int i) { return reinterpret_cast<uint64_t*>(base + OFF_BAR) + i; };
+  auto stage = [&](int s) { return base + OFF_ST + s * STAGE_BYTES; };
+  __shared__ uint32_t tmem_base_s;
+  __shared__ int abort_s;
+  volatile int* abort_flag = &abort_s;
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  constexpr int KT = KTILE / G;                   // keys per tile
+  constexpr int KH = KT / 2;                      // keys of a sub-tile
+  constexpr int KPL = KT / 32;                    // keys per lane of the scale warp
+  constexpr int NST = PairTable<G>::kSlices;      // state tiles
+
+  // Work items.  Rank -> (block of its chunk, chunk, head): the last blocks of the chunks (the most key tiles) first,
+  // among them the chunks in descending order, so that chunk 0, which reads no state, comes last.  The n-th item of a CTA:
+  // rounds of gridDim.x items, dealt forwards and backwards in turn, so that the CTA that got the heaviest item of one
+  // round gets the lightest of the next.
+  struct Item {
+    int bh, chunk, q0;            // head, chunk, first query
+    int k0;                       // first key tile (in tiles of KT keys)
+    int nk_a, nk_b;               // key tiles of the halves (0: half B lies beyond the sequence)
+    int ns;                       // state tiles (0: no state)
+    int n_tiles;
+  };
+  const int per_block = args.n_chunks * args.BH;
+  const int n_ranks = args.chunk_pairs * per_block;
+  auto next_item = [&](int& n, Item& it) -> bool {   // the item at or after the n-th; n is left at it
+    for (;; ++n) {
+      const long long id = (long long)n * gridDim.x + ((n & 1) ? (int)gridDim.x - 1 - (int)blockIdx.x : (int)blockIdx.x);
+      if ((long long)n * gridDim.x >= n_ranks) return false;
+      if (id >= n_ranks) continue;
+      const int p = args.chunk_pairs - 1 - (int)id / per_block;
+      const int rem = (int)id % per_block;
+      it.chunk = args.n_chunks - 1 - rem / args.BH;
+      it.bh = rem % args.BH;
+      const int pair = it.chunk * args.chunk_pairs + p;
+      if (pair >= args.n_pairs) continue;
+      it.q0 = pair * 2 * QT;
+      it.k0 = it.chunk * args.chunk_pairs * 2 * G;
+      it.nk_a = (2 * p + 1) * G;
+      it.nk_b = it.q0 + QT < args.Tlen ? (2 * p + 2) * G : 0;
+      it.ns = it.chunk >= args.first_state ? NST + 1 : 0;
+      it.n_tiles = it.ns + (it.nk_b > 0 ? it.nk_b : it.nk_a);
+      return true;
+    }
+  };
+
+  if (tid == 0) {
+    abort_s = 0;
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(bar(BAR_QFULL + i), 1);
+      mbar_init(bar(BAR_QEMPTY + i), 512);
+      mbar_init(bar(BAR_QT + i), 256);
+      mbar_init(bar(BAR_ODONE + i), 1);
+      mbar_init(bar(BAR_OFREE + i), 256);
+    }
+    for (int i = 0; i < 4; ++i) {
+      mbar_init(bar(BAR_SFULL + i), 1);
+      mbar_init(bar(BAR_PFULL + i), 128);
+    }
+    for (int i = 0; i < NSTAGE; ++i) {
+      mbar_init(bar(BAR_FULL + i), 2);
+      mbar_init(bar(BAR_EMPTY + i), 2);
+    }
+    for (int i = 0; i < 8; ++i) {
+      mbar_init(bar(BAR_FFULL + i), 128);
+      mbar_init(bar(BAR_SFREE + i), 1);
+    }
+    mbar_init(bar(BAR_DRAIN), 2);
+    fence_mbar_init();
+    tma_prefetch_desc(&tmQ);
+    tma_prefetch_desc(&tmK);
+    tma_prefetch_desc(&tmV);
+    if (args.first_state < args.n_chunks) {
+      tma_prefetch_desc(&tmS);
+      tma_prefetch_desc(&tmZ);
+    }
+  }
+  // columns 64..127 of 16 rows of the B operands: [1, 0, ...] for the values, zeros for the state (every step of 16 rows
+  // reads the same block: the descriptor's leading offset is the distance to it)
+  for (int i = tid; i < 256; i += NTHREADS) {
+    const int row = (i & 127) >> 3, c = i & 7;
+    *reinterpret_cast<uint4*>(base + OFF_ONES + (i >> 7) * 2048 + sw128_offset(row, c)) =
+        make_uint4(i < 128 && c == 0 ? 0x3F80u : 0u, 0u, 0u, 0u);
+  }
+  fence_async_smem();
+  if (warp == 0) {
+    tmem_alloc(&tmem_base_s, TMEM_COLS);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tb = tmem_base_s;
+  bool ok = true;
+
+  if (warp == 0) {
+    regs_release<64>();
+    // =========================== TMA producer ===========================
+    if (elect_one()) {
+      uint32_t it = 0;                                   // tiles loaded so far, over all items
+      int ni = 0;
+      Item w;
+      // the kernel is a programmatic dependent launch: the states are the work of the kernel before it
+      if (args.first_state < args.n_chunks) cudaGridDependencySynchronize();
+      for (int n = 0; ok && next_item(n, w); ++n, ++ni) {
+        const int qb = ni & 1;
+        ok = wait_or_abort(bar(BAR_QEMPTY + qb), ((ni >> 1) & 1) ^ 1, abort_flag);
+        if (!ok) break;
+        mbar_arrive_expect_tx(bar(BAR_QFULL + qb), w.nk_b > 0 ? 32768 : 16384);
+        tma_load_3d(base + OFF_Q + qb * 32768, &tmQ, bar(BAR_QFULL + qb), 0, w.q0, w.bh);
+        if (w.nk_b > 0) tma_load_3d(base + OFF_Q + qb * 32768 + 16384, &tmQ, bar(BAR_QFULL + qb), 0, w.q0 + QT, w.bh);
+        for (int j = 0; j < w.n_tiles && ok; ++j, ++it) {
+          const int s = it % NSTAGE;
+          ok = wait_or_abort(bar(BAR_EMPTY + s), ((it / NSTAGE) & 1) ^ 1, abort_flag);
+          if (!ok) break;
+          if (j >= w.ns) {
+            const int key = (w.k0 + j - w.ns) * KT;
+            mbar_arrive_expect_tx(bar(BAR_FULL + s), 2 * KT * 128);   // K and V tiles
+            tma_load_3d(stage(s), &tmK, bar(BAR_FULL + s), 0, key, w.bh);
+            tma_load_3d(stage(s) + 16384, &tmV, bar(BAR_FULL + s), 0, key, w.bh);
+          } else {
+            const int slot = w.bh * args.n_chunks + w.chunk;
+            mbar_arrive_expect_tx(bar(BAR_FULL + s), j == 0 ? 8192 : 32768);
+            if (j == 0) tma_load_3d(stage(s), &tmZ, bar(BAR_FULL + s), 0, 0, slot);
+            else tma_load_3d(stage(s), &tmS, bar(BAR_FULL + s), 0, (j - 1) * 256, slot);
+          }
+        }
+      }
+    }
+  } else if (warp == 1 || warp == 2) {
+    regs_release<64>();
+    // =========================== MMA issuer of half A or B ===========================
+    // The 128 columns of a half's buffer are two sub-buffers of 64, each a chain of its own.  Key tiles: open (score MMAs)
+    // -> builders -> close (apply MMAs) -> open of the next tile; the thread goes round close 0, open 0, close 1, open 1,
+    // so the chains run half a period apart.  State tiles: a sub-buffer is two pieces of 32 columns (64 features), which the
+    // builders fill as they become free.  MMAs that overwrite columns follow the MMAs that read them in the same thread.
+    if (elect_one()) {
+      const int h = warp - 1;
+      const uint32_t id_s = instr_desc(kFmtBF16, kFmtBF16, 0, 0, 128, KH);      // scores: B K-major
+      const uint32_t id_y = instr_desc(kFmtBF16, kFmtBF16, 0, 0, 128, 32);      // Q Z, 32 columns
+      const uint32_t id_p = instr_desc(kFmtBF16, kFmtBF16, 0, 1, 128, 80);      // apply: B MN-major, N = 64 + 16
+      const uint32_t id_f = instr_desc(kFmtBF16, kFmtBF16, 0, 1, 128, 64);      // Psi(Q) S
+      const uint64_t dk = smem_desc(0, 16, 1024, kSwizzle128B);
+      const uint32_t tS = tb + COL_S + h * 128, tO = tb + COL_O + h * 80, tQ = tb + COL_Q + h * 32;
+      const uint32_t ones = smem_u32(base + OFF_ONES), zeros = smem_u32(base + OFF_ZEROS);
+      // MN-major, 128B swizzle: 8 rows per 1024-byte atom (SBO), columns 64.. in the constant block (LBO)
+      auto bdesc = [&](uint32_t addr, uint32_t extra) { return smem_desc(addr, extra - addr, 1024, kSwizzle128B); };
+      uint32_t it = 0, cnt = 0, n_st = 0;   // tiles, key tiles of this half, its state tiles
+      int n_done = 0;                       // items of this half so far
+      Item w;
+      for (int n = 0; ok && next_item(n, w); ++n) {
+        const int nk = h == 0 ? w.nk_a : w.nk_b;
+        const int nt = nk > 0 ? w.ns + nk : 0;      // tiles of this half
+        uint32_t acc = 0;
+        auto landed = [&](uint32_t g_it) { return wait_or_abort(bar(BAR_FULL + g_it % NSTAGE), (g_it / NSTAGE) & 1, abort_flag); };
+        auto o_free = [&]() { return acc != 0 || n_done == 0 || wait_or_abort(bar(BAR_OFREE + h), (n_done - 1) & 1, abort_flag); };
+        auto open = [&](uint32_t g_it, int c) {
+          const uint32_t st = smem_u32(stage(g_it % NSTAGE));
+#pragma unroll
+          for (int ks = 0; ks < 4; ++ks)   // 16 features per step; group ks / (4 / G) accumulates over its own steps
+            mma_f16_ts(tS + c * 64 + (ks / (4 / G)) * KH, tQ + ks * 8, at(dk, st + c * KH * 128 + ks * 32), id_s, (ks % (4 / G)) > 0);
+          mma_commit(bar(BAR_SFULL + 2 * h + c));
+        };
+        auto close = [&](uint32_t g_it, int c) -> bool {
+          if (!wait_or_abort(bar(BAR_PFULL + 2 * h + c), cnt & 1, abort_flag) || !o_free()) return false;
+          tc_fence_after();
+          const uint32_t va = smem_u32(stage(g_it % NSTAGE)) + 16384 + c * KH * 128;
+#pragma unroll
+          for (int ks = 0; ks < KH / 16; ++ks) {
+            mma_f16_ts(tO, tS + c * 64 + ks * 8, bdesc(va + ks * 2048, ones), id_p, acc);
+            acc = 1;
+          }
+          return true;
+        };
+        if (nt > 0) ok = wait_or_abort(bar(BAR_QT + h), n_done & 1, abort_flag) && landed(it);
+        if (nt > 0 && ok) {
+          tc_fence_after();
+          if (w.ns > 0) {
+            // Y = Q Z, 32 columns per sub-buffer
+            const uint32_t st = smem_u32(stage(it % NSTAGE));
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+#pragma unroll
+              for (int ks = 0; ks < 4; ++ks) mma_f16_ts(tS + c * 64, tQ + ks * 8, at(dk, st + c * 32 * 128 + ks * 32), id_y, ks > 0);
+              mma_commit(bar(BAR_SFULL + 2 * h + c));
+            }
+            mma_commit(bar(BAR_EMPTY + it % NSTAGE));
+            ++it;        // (the builders' features follow their reading of Y: no close)
+#pragma unroll 1
+            for (int t = 0; t < NST && ok; ++t, ++it, ++n_st) {
+              ok = landed(it) && o_free() && (t + 1 < NST || landed(it + 1));
+              const uint32_t sa = smem_u32(stage(it % NSTAGE));
+#pragma unroll
+              for (int c = 0; c < 2; ++c) {
+#pragma unroll
+                for (int pp = 0; pp < 2; ++pp) {
+                  ok = ok && wait_or_abort(bar(BAR_FFULL + 4 * h + 2 * c + pp), n_st & 1, abort_flag);
+                  if (!ok) break;
+                  tc_fence_after();
+#pragma unroll
+                  for (int ks = 0; ks < 4; ++ks) {
+                    // the very first step also clears the normaliser column (N = 80, zeros beyond column 64)
+                    mma_f16_ts(tO, tS + c * 64 + pp * 32 + ks * 8, bdesc(sa + c * 16384 + pp * 8192 + ks * 2048, zeros), acc == 0 ? id_p : id_f, acc);
+                    acc = 1;
+                  }
+                  mma_commit(bar(BAR_SFREE + 4 * h + 2 * c + pp));
+                }
+                if (!ok) break;
+                if (c == 1) mma_commit(bar(BAR_EMPTY + it % NSTAGE));
+                if (t + 1 == NST) open(it + 1, c);       // the first key tile
+              }
+            }
+          } else {
+            open(it, 0);
+            open(it, 1);
+          }
+        }
+        for (int j = 0; j < nk && ok; ++j, ++it, ++cnt) {
+          const bool next = j + 1 < nk;
+          ok = (!next || landed(it + 1)) && close(it, 0);
+          if (ok && next) open(it + 1, 0);
+          ok = ok && close(it, 1);
+          if (!ok) break;
+          mma_commit(bar(BAR_EMPTY + it % NSTAGE));
+          if (next) open(it + 1, 1);
+        }
+        for (int j = nt; j < w.n_tiles && ok; ++j, ++it) {      // the other half's tiles
+          ok = landed(it);
+          if (ok) mbar_arrive(bar(BAR_EMPTY + it % NSTAGE));
+        }
+        if (nt > 0) {
+          if (ok) mma_commit(bar(BAR_ODONE + h));
+          ++n_done;
+        }
+      }
+    }
+  } else if (warp == 3) {
+    regs_release<64>();
+    // =========================== scale warp: r = 1 / ||k||^2 of the keys of every tile, from the pre-pass to shared memory ===========================
+    // (the key scale multiplies the weights, so the values are used as they are; a zero key row has r = 0: zero
+    // feature).  A programmatic dependent launch: this warp waits for the pre-pass.
+    cudaGridDependencySynchronize();
+    uint32_t it = 0;
+    Item w;
+    for (int n = 0; ok && next_item(n, w); ++n) {
+      const unsigned short* rs = reinterpret_cast<const unsigned short*>(args.rscale) + (size_t)w.bh * args.Tlen;
+      auto load_r = [&](int j, unsigned short (&rv)[KPL]) {       // r of this lane's keys of tile j
+#pragma unroll
+        for (int e = 0; e < KPL; ++e) {
+          const int key = (w.k0 + j - w.ns) * KT + lane * KPL + e;
+          rv[e] = (j >= w.ns && j < w.n_tiles && key < args.Tlen) ? rs[key] : (unsigned short)0;
+        }
+      };
+      unsigned short rv[KPL];
+      load_r(0, rv);
+      for (int j = 0; j < w.n_tiles && ok; ++j, ++it) {
+        const int s = it % NSTAGE;
+        unsigned short rn[KPL];
+        load_r(j + 1, rn);              // one tile ahead: the global-load latency stays off the ring
+        ok = wait_or_abort(bar(BAR_EMPTY + s), ((it / NSTAGE) & 1) ^ 1, abort_flag);
+        if (!ok) break;
+#pragma unroll
+        for (int e = 0; e < KPL; ++e) {
+          reinterpret_cast<unsigned short*>(base + OFF_RV + s * 256)[lane * KPL + e] = rv[e];
+          rv[e] = rn[e];
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(BAR_FULL + s));      // (the builders of the tile come after its score MMAs)
+      }
+    }
+  } else {
+    regs_take<104>();
+    // =========================== builders (256 threads per half) ===========================
+    const uint32_t q4 = warp & 3;
+    const int bw = warp - WARP_BLD0;
+    const int h = bw >> 3;                       // half
+    const int ch = (bw >> 2) & 1;                // sub-buffer: the first or second half of the keys (features) of a tile
+    const int rowl = q4 * 32 + lane;             // query row inside the tile (= TMEM lane)
+    const uint32_t tS = tmem_addr(tb, q4 * 32, COL_S + h * 128 + ch * 64), tO = tmem_addr(tb, q4 * 32, COL_O + h * 80);
+    const uint32_t qrow_s = smem_u32(base + OFF_Q) + h * 16384;
+    // 16 bytes (eight features) of this thread's query row, from the item's tile in shared memory
+    auto qrun = [&](int qb, int c) { return lds128(qrow_s + qb * 32768 + sw128_offset(rowl, c)); };
+    // the query tile of an item into TMEM: this thread's row, 32 of its features
+    auto copy_q = [&](int ni, const Item& w) {
+      const int qb = ni & 1;
+      ok = ok && wait_or_abort(bar(BAR_QFULL + qb), (ni >> 1) & 1, abort_flag);
+      if (!ok) return;
+      if (h == 0 || w.nk_b > 0) {
+        uint32_t r[16];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const uint4 x = qrun(qb, ch * 4 + c);
+          r[4 * c] = x.x; r[4 * c + 1] = x.y; r[4 * c + 2] = x.z; r[4 * c + 3] = x.w;
+        }
+        tmem_st16(tmem_addr(tb, q4 * 32, COL_Q + h * 32 + ch * 16), r);
+        tmem_wait_st();
+        tc_fence_before();
+        mbar_arrive(bar(BAR_QT + h));
+      }
+      if (w.ns == 0) mbar_arrive(bar(BAR_QEMPTY + qb));
+    };
+    uint32_t it = 0, cnt = 0, n_st = 0;
+    int n_done = 0, ni = 0, n = 0;
+    Item w;
+    bool more = next_item(n, w);
+    if (more) copy_q(0, w);
+    for (; more && ok; ++ni) {
+      const int nk = h == 0 ? w.nk_a : w.nk_b;
+      const int qrow = w.q0 + h * QT + rowl;
+      float den0 = 0.f;                          // the state's part of the normaliser
+      const uint32_t it0 = it;
+      it += w.n_tiles;
+      if (nk > 0 && w.ns > 0) {
+        const int qb = ni & 1;
+        // ---- Y = Q Z: den0 = q . Y, this warp's 32 of the 64 columns ----
+        ok = wait_or_abort(bar(BAR_SFULL + 2 * h + ch), cnt & 1, abort_flag);
+        if (!ok) break;
+        tc_fence_after();
+        uint32_t y[32];
+        tmem_ld32(tS, y);
+        tmem_wait_ld(y);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const uint4 x = qrun(qb, ch * 4 + c);
+          const uint32_t xs[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            den0 = fmaf(__uint_as_float(xs[e] << 16), __uint_as_float(y[8 * c + 2 * e]), den0);
+            den0 = fmaf(__uint_as_float(xs[e] & 0xFFFF0000u), __uint_as_float(y[8 * c + 2 * e + 1]), den0);
+          }
+        }
+        ++cnt;
+        // ---- the features of this query row, 256 per tile, this warp's two pairs of runs ----
+        static constexpr PairTable<G> kPairs{};
+#pragma unroll 1
+        for (int t = 0; t < NST && ok; ++t, ++n_st) {
+#pragma unroll 1
+          for (int pp = 0; pp < 2; ++pp) {
+            const int p = 4 * t + 2 * ch + pp;
+            const uint4 xg = qrun(qb, kPairs.g[p]), xh = qrun(qb, kPairs.h[p]);
+            const uint32_t gs[4] = {xg.x, xg.y, xg.z, xg.w}, hs[4] = {xh.x, xh.y, xh.z, xh.w};
+            uint32_t f[32];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              const uint32_t b2 = (j & 1) ? __byte_perm(hs[j >> 1], 0, 0x3232) : __byte_perm(hs[j >> 1], 0, 0x1010);
+#pragma unroll
+              for (int e = 0; e < 4; ++e) f[4 * j + e] = mul_bf16x2(gs[e], b2);
+            }
+            // the piece is free: Y has been read by this warp, or the MMAs of the tile before have read its features
+            if (t > 0) ok = ok && wait_or_abort(bar(BAR_SFREE + 4 * h + 2 * ch + pp), (n_st - 1) & 1, abort_flag);
+            if (!ok) break;
+            tc_fence_after();
+            tmem_st32(tS + pp * 32, f);
+            tmem_wait_st();
+            tc_fence_before();
+            mbar_arrive(bar(BAR_FFULL + 4 * h + 2 * ch + pp));
+          }
+        }
+        if (!ok) break;
+      }
+      if (w.ns > 0) mbar_arrive(bar(BAR_QEMPTY + (ni & 1)));
+      for (int j = 0; j < nk && ok; ++j, ++cnt) {
+        const uint32_t g_it = it0 + w.ns + j;
+        const int s = g_it % NSTAGE;
+        ok = wait_or_abort(bar(BAR_SFULL + 2 * h + ch), cnt & 1, abort_flag);
+        if (!ok) break;
+        tc_fence_after();
+        const bool diag = j >= nk - G;
+        if constexpr (G > 1) {
+          // this warp weighs keys [ch KT/2, ch KT/2 + KT/2) of the tile: one column run per group
+          const int key0 = (w.k0 + j) * KT + ch * KH;
+          uint32_t y[G][KH], pk[KH / 2];
+          const uint32_t* rw = reinterpret_cast<const uint32_t*>(base + OFF_RV + s * 256) + ch * (KH / 2);   // r of this warp's keys, in pairs
+#pragma unroll
+          for (int g = 0; g < G; ++g) {
+            if constexpr (KH == 32) tmem_ld32(tS + g * KH, y[g]); else tmem_ld16(tS + g * KH, y[g]);
+          }
+#pragma unroll
+          for (int g = 0; g < G; ++g) tmem_wait_ld(y[g]);
+          // two copies of the loop, chosen once per tile: the causal test exists on the diagonal tiles only
+          auto weigh_g = [&](auto masked) {
+#pragma unroll
+            for (int c = 0; c < KH; c += 2) {
+              float2 x = make_float2(0.f, 0.f);
+#pragma unroll
+              for (int g = 0; g < G; ++g) {
+                const float2 sv = make_float2(__uint_as_float(y[g][c]), __uint_as_float(y[g][c + 1]));
+                x = __ffma2_rn(sv, sv, x);
+              }
+              if constexpr (decltype(masked)::value) {
+                if (key0 + c > qrow) x.x = 0.f;
+                if (key0 + c + 1 > qrow) x.y = 0.f;
+              }
+              pk[c / 2] = mul_bf16x2(pack_bf16(x.x, x.y), rw[c / 2]);
+            }
+          };
+          if (diag) weigh_g(std::true_type{}); else weigh_g(std::false_type{});
+          // the weights overwrite this warp's own score columns of group 0
+          if constexpr (KH == 32) tmem_st16(tS, pk); else tmem_st8(tS, pk);
+        } else {
+          const uint32_t rbase = smem_u32(base + OFF_RV) + s * 256 + ch * 128;   // r of this warp's 64 keys, 8 per load
+          const int key0 = (w.k0 + j) * KT + ch * 64;
+          uint32_t ya[32], yb[32], pk[16];
+          auto weigh = [&](const uint32_t (&y)[32], int col0, auto masked) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const uint4 t4 = lds128(rbase + (col0 / 8 + i) * 16);
+              const uint32_t rr[4] = {t4.x, t4.y, t4.z, t4.w};
+#pragma unroll
+              for (int e = 0; e < 8; e += 2) {
+                const int jj = 8 * i + e;
+                const float2 sv = make_float2(__uint_as_float(y[jj]), __uint_as_float(y[jj + 1]));
+                float2 x = __fmul2_rn(sv, sv);
+                if constexpr (decltype(masked)::value) {
+                  if (key0 + col0 + jj > qrow) x.x = 0.f;
+                  if (key0 + col0 + jj + 1 > qrow) x.y = 0.f;
+                }
+                pk[jj / 2] = mul_bf16x2(pack_bf16(x.x, x.y), rr[e / 2]);
+              }
+            }
+          };
+          auto weigh_tile = [&](auto masked) {
+            tmem_ld32(tS, ya);
+            tmem_ld32(tS + 32, yb);
+            tmem_wait_ld(ya);
+            tmem_wait_ld(yb);
+            weigh(ya, 0, masked);
+            tmem_st16(tS, pk);          // over this warp's own scores, which are in registers
+            weigh(yb, 32, masked);
+            tmem_st16(tS + 16, pk);
+          };
+          if (diag) weigh_tile(std::true_type{}); else weigh_tile(std::false_type{});
+        }
+        tmem_wait_st();
+        tc_fence_before();
+        mbar_arrive(bar(BAR_PFULL + 2 * h + ch));
+      }
+      if (!ok) break;
+      // the next item's queries go to TMEM before the wait for this item's last MMAs (its score MMAs are all through)
+      const int bh = w.bh, ns = w.ns;
+      ++n;
+      more = next_item(n, w);
+      if (more) copy_q(ni + 1, w);
+      if (nk == 0) continue;
+      // ---- epilogue: out = O / D ----
+      ok = ok && wait_or_abort(bar(BAR_ODONE + h), n_done & 1, abort_flag);
+      if (!ok) break;
+      ++n_done;
+      tc_fence_after();
+      uint32_t o[32], dn[4];
+      tmem_ld32(tO + ch * 32, o);
+      tmem_ld4(tO + 64, dn);
+      tmem_wait_ld(o);
+      tmem_wait_ld(dn);
+      tc_fence_before();
+      mbar_arrive(bar(BAR_OFREE + h));           // the MMAs of the next item may overwrite [O | D]
+      if (ns > 0) {                              // the two warps of a row hold the two halves of q . Y
+        float* part = reinterpret_cast<float*>(base + OFF_DEN) + h * 256 + rowl;
+        part[ch * 128] = den0;
+        asm volatile("bar.sync %0, 64;" ::"r"(1 + h * 4 + (int)q4) : "memory");
+        den0 = part[0] + part[128];
+        asm volatile("bar.sync %0, 64;" ::"r"(1 + h * 4 + (int)q4) : "memory");   // before the next item overwrites the shares
+      }
+      const float den = __uint_as_float(dn[0]) + den0;
+      const float inv = den > 0.f ? 1.f / den : 0.f;
+      if (qrow < args.Tlen) {
+        __nv_bfloat16* dst = args.out + ((size_t)bh * args.Tlen + qrow) * args.d_v + ch * 32;
+#pragma unroll
+        for (int jj = 0; jj < 32; jj += 8) {
+          if (ch * 32 + jj >= args.d_v) break;
+          uint4 pkt;
+          pkt.x = pack_bf16(__uint_as_float(o[jj]) * inv, __uint_as_float(o[jj + 1]) * inv);
+          pkt.y = pack_bf16(__uint_as_float(o[jj + 2]) * inv, __uint_as_float(o[jj + 3]) * inv);
+          pkt.z = pack_bf16(__uint_as_float(o[jj + 4]) * inv, __uint_as_float(o[jj + 5]) * inv);
+          pkt.w = pack_bf16(__uint_as_float(o[jj + 6]) * inv, __uint_as_float(o[jj + 7]) * inv);
+          *reinterpret_cast<uint4*>(dst + jj) = pkt;
+        }
+      }
+    }
+  }
+
+  // ---------------- teardown ----------------
+  if (!ok && args.device_status != nullptr) atomicExch(args.device_status, (int)KATA_ERR_DEVICE_TIMEOUT);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if ((warp == 1 || warp == 2) && elect_one()) {
+    mma_commit(bar(BAR_DRAIN));
+    mbar_wait(bar(BAR_DRAIN), 0);
+  }
+  __syncthreads();
+  if (warp == 0) tmem_dealloc(tb, TMEM_COLS);
+}
+
+}  // namespace
+
+// workspace: r [BH][T] bf16
+size_t tc_quadratic_workspace_bytes(const Problem& p) { return ((size_t)p.B * p.H * p.T * 2 + 255) / 256 * 256; }
+
+void tc_rscale(const Problem& p, __nv_bfloat16* rscale, LaunchCtx& ctx) {
+  const size_t n_rows = (size_t)p.B * p.H * p.T;
+  rscale_kernel<<<(unsigned)((n_rows + 31) / 32), 256, 0, ctx.stream>>>(static_cast<const __nv_bfloat16*>(p.k), rscale, n_rows, p.d_k);
+  note_launch(ctx);
+}
+
+void tc_attend(const Problem& p, const __nv_bfloat16* rscale, const AttendStates& st, int* device_status, LaunchCtx& ctx) {
+  const int BH = p.B * p.H;
+  CUtensorMap tmQ, tmK, tmV, tmS, tmZ;
+  const int kt = KTILE / p.groups;
+  const int n_pairs = (p.T + 2 * QT - 1) / (2 * QT);
+  AArgs a{static_cast<__nv_bfloat16*>(p.out), rscale, device_status, p.T, p.d_v, BH, n_pairs, n_pairs, 1, 1};
+  bool maps = make_tile_map(&tmQ, p.q, BH, p.T, QT, p.d_k) && make_tile_map(&tmK, p.k, BH, p.T, kt, p.d_k) &&
+              make_tile_map(&tmV, p.v, BH, p.T, kt, p.d_v);
+  if (st.n_chunks > 0) {
+    a.chunk_pairs = st.chunk_tokens / (2 * QT);
+    a.n_chunks = st.n_chunks;
+    a.first_state = st.first_state;
+    maps = maps && make_tile_map(&tmS, st.s, BH * st.n_chunks, tc_state_rows(p.groups), 256) &&
+           make_tile_map(&tmZ, st.z, BH * st.n_chunks, 64, 64);
+  } else {
+    tmS = tmK;
+    tmZ = tmK;
+  }
+  if (!maps) {
+    ctx.status = KATA_ERR_CUDA;
+    return;
+  }
+  auto kern = p.groups == 1 ? tc_attend_kernel<1> : p.groups == 2 ? tc_attend_kernel<2> : tc_attend_kernel<4>;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_ALLOC) != cudaSuccess) {
+    cudaGetLastError();
+    ctx.status = KATA_ERR_CUDA;
+    return;
+  }
+  int dev = 0, sms = 148;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    cudaGetLastError();
+    sms = 148;
+  }
+  const long long n_items = (long long)BH * n_pairs;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(n_items < sms ? n_items : sms));   // persistent: one CTA per SM
+  cfg.blockDim = dim3(NTHREADS);
+  cfg.dynamicSmemBytes = SMEM_ALLOC;
+  cfg.stream = ctx.stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (cudaLaunchKernelEx(&cfg, kern, tmQ, tmK, tmV, tmS, tmZ, a) != cudaSuccess) {
+    cudaGetLastError();
+    ctx.status = KATA_ERR_CUDA;
+    return;
+  }
+  ++ctx.launches;
+}
+
+void tc_quadratic(const Problem& p, void* workspace, int* device_status, LaunchCtx& ctx) {
+  __nv_bfloat16* rscale = static_cast<__nv_bfloat16*>(workspace);
+  tc_rscale(p, rscale, ctx);
+  if (ctx.status == KATA_OK) tc_attend(p, rscale, AttendStates{}, device_status, ctx);
+}
+
+}  // namespace kata

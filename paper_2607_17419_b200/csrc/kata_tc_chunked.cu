@@ -1,12 +1,95 @@
-// Chunked (linear-state) KATA forward on the tensor cores, bf16, d_k = d_v = 64: which launches make up each form.
-// The kernel is the token-major streaming kernel (kata_tc_stream.cu); the scan forms run it over groups of
-// 128-token tiles as reduce -> scan -> restart:
+// Chunked (linear-state) KATA forward on the tensor cores, bf16: which launches make up each form.
+// Sequential form (tc_chunked_states): the key scales, the states before the chunks (kata_tc_state.cu), the outputs
+// (kata_tc_attend.cu); a short sequence is one chunk, the quadratic form alone.
+// Scan forms and short calls with a state handed in or out (tc_chunked): the token-major streaming kernel
+// (kata_tc_stream.cu); the scan forms run it over groups of 128-token tiles as reduce -> scan -> restart:
 //   pass 1  every group but the last computes the state it adds (state-only mode: keys and values only)
 //   pass 2  inclusive scan over the group states (scan_round_kernel, fp32 adds)
 //   pass 3  every group starts from the prefix before it and writes its outputs
 #include "kata_common.cuh"
 
 namespace kata {
+
+namespace {
+size_t align256(size_t n) { return (n + 255) / 256 * 256; }
+
+// Workspace of the chunk-state route: key scales, the states before the chunks, and with several segments their fp32 sums.
+struct ChunkBuffers {
+  size_t r, s, z, s_loc, z_loc, total;
+};
+ChunkBuffers chunk_buffers(const Problem& p, const StatePlan& plan, bool states) {
+  const size_t BH = (size_t)p.B * p.H, slots = BH * plan.n_chunks, rows = (size_t)tc_state_rows(p.groups);
+  ChunkBuffers b{};
+  b.r = 0;
+  b.s = align256(BH * p.T * 2);
+  b.z = b.s + (states ? align256(slots * rows * 64 * 2) : 0);
+  b.s_loc = b.z + (states ? align256(slots * 64 * 64 * 2) : 0);
+  b.z_loc = b.s_loc + (states && plan.segments > 1 ? align256(slots * rows * 64 * 4) : 0);
+  b.total = b.z_loc + (states && plan.segments > 1 ? align256(slots * rows * 4) : 0);
+  return b;
+}
+}  // namespace
+
+// Chunk length and segments.
+// No state pointers and a short sequence: one chunk, the quadratic form alone.  Per tile of 128 tokens and head the chunk
+// states cost about 9 us of one SM to build and 7 to read (full lift), a key tile 0.55: the quadratic form wins until the
+// average query sees about 29 key tiles.  Measured, us, quadratic / chunks of 1024, for 16, 128 and 3 heads:
+//   full lift   T = 6000: 75 / 99, 587 / 645, 49 / 44     T = 8192: 119 / 130, 1148 / 900, 65 / 54
+//   two groups  T = 2000: 31 / 38, 147 / 152, 30 / 37     T = 4096: 53 / 60, 450 / 315, 51 / 39
+//   four groups T = 2000: 45 / 42, 193 / 161, 43 / 41
+// Chunks of 1024: 16 heads x 131072 tokens 2.26 ms; 512: 2.30, 2048: 2.44 (shorter chunks write and read more state, longer
+// ones have more key tiles).  Halved where even one chunk per CTA leaves SMs idle (3 heads x 2048 tokens with the state
+// handed out: 43 -> 38 us).
+StatePlan tc_chunk_plan(const Problem& p, bool state_in, bool state_out) {
+  const int BH = p.B * p.H, slices = tc_state_rows(p.groups) / 256;
+  const int quad_tokens = p.groups == 1 ? 7168 : p.groups == 2 ? 3072 : 1536;
+  StatePlan plan{};
+  int L = 1024;
+  if (!state_in && !state_out && p.T <= quad_tokens) L = (p.T + 255) / 256 * 256;
+  else if ((long long)BH * slices * ((p.T + L - 1) / L) < 148) L = 512;
+  plan.chunk_tokens = L;
+  plan.n_chunks = (p.T + L - 1) / L;
+  const int walk = state_out ? plan.n_chunks : plan.n_chunks - 1;
+  plan.segments = 148 / (BH * slices);        // one CTA per SM
+  if (plan.segments > walk) plan.segments = walk;
+  if (plan.segments < 1) plan.segments = 1;
+  plan.seg_chunks = walk > 0 ? (walk + plan.segments - 1) / plan.segments : 1;
+  plan.segments = walk > 0 ? (walk + plan.seg_chunks - 1) / plan.seg_chunks : 1;
+  return plan;
+}
+
+size_t tc_chunk_workspace_bytes(const Problem& p, const StatePlan& plan, bool state_in, bool state_out) {
+  return chunk_buffers(p, plan, plan.n_chunks > 1 || state_in || state_out).total;
+}
+
+void tc_chunked_states(const Problem& p, const StatePlan& plan, void* workspace, int* device_status, const float* s_init,
+                       const float* z_init, float* s_final, float* z_final, int state_layout, LaunchCtx& ctx) {
+  const bool states = plan.n_chunks > 1 || s_init != nullptr || s_final != nullptr;
+  const ChunkBuffers b = chunk_buffers(p, plan, states);
+  unsigned char* w = static_cast<unsigned char*>(workspace);
+  __nv_bfloat16* r = reinterpret_cast<__nv_bfloat16*>(w + b.r);
+  tc_rscale(p, r, ctx);
+  AttendStates at{};
+  if (states) {
+    StateBuffers buf{};
+    buf.s = reinterpret_cast<__nv_bfloat16*>(w + b.s);
+    buf.z = reinterpret_cast<__nv_bfloat16*>(w + b.z);
+    buf.s_loc = reinterpret_cast<float*>(w + b.s_loc);
+    buf.z_loc = reinterpret_cast<float*>(w + b.z_loc);
+    buf.s_init = s_init;
+    buf.z_init = z_init;
+    buf.s_final = s_final;
+    buf.z_final = z_final;
+    buf.layout = state_layout;
+    if (ctx.status == KATA_OK) tc_states(p, r, plan, buf, device_status, ctx);
+    at.s = buf.s;
+    at.z = buf.z;
+    at.n_chunks = plan.n_chunks;
+    at.chunk_tokens = plan.chunk_tokens;
+    at.first_state = s_init != nullptr ? 0 : 1;
+  }
+  if (ctx.status == KATA_OK) tc_attend(p, r, at, device_status, ctx);
+}
 
 size_t tc_chunked_state_elems() { return tc_stream_state_elems(); }
 int tc_chunked_slices() { return tc_stream_slices(); }

@@ -23,12 +23,13 @@ inline EncodeTiledFn tensor_map_encoder() {
   return fn;
 }
 
-// [BH][T][64] bf16 tensor, box = 64 columns x rows x 1 head, 128B swizzle; rows beyond T read as zero.
-inline bool make_tile_map(CUtensorMap* tm, const void* ptr, int BH, int T, int rows) {
+// [BH][T][d] bf16 tensor (d = 64, or 16 or 32: columns d..63 of the box read as zero), box = 64 columns x rows x 1 head,
+// 128B swizzle; rows beyond T read as zero.
+inline bool make_tile_map(CUtensorMap* tm, const void* ptr, int BH, int T, int rows, int d = 64) {
   EncodeTiledFn fn = tensor_map_encoder();
   if (fn == nullptr) return false;
-  cuuint64_t dims[3] = {64, (cuuint64_t)T, (cuuint64_t)BH};
-  cuuint64_t strides[2] = {64 * 2, (cuuint64_t)T * 64 * 2};
+  cuuint64_t dims[3] = {(cuuint64_t)d, (cuuint64_t)T, (cuuint64_t)BH};
+  cuuint64_t strides[2] = {(cuuint64_t)d * 2, (cuuint64_t)T * d * 2};
   cuuint32_t box[3] = {64, (cuuint32_t)rows, 1};
   cuuint32_t es[3] = {1, 1, 1};
   return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, es,

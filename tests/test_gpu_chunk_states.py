@@ -1,0 +1,71 @@
+"""GPU parity of the chunk-state and attend kernels (bf16): edges of chunks (512 or 1024 tokens), of blocks of 256 queries
+and of the segments of the chunk axis, state in and out, one and several segments, narrow rows.
+
+Tolerances: outputs as everywhere (2e-2).  Final state: operands are products of bf16 entries rounded twice (2^-8 each,
+signs at random over the sum), so max |s - ref| <= 2e-2 of the largest entry."""
+import numpy as np
+import pytest
+
+from oracle import kata_oracle as ko
+from paper_2607_17419_b200 import binding as kb
+from paper_2607_17419_b200 import inputs
+
+from helpers import check, dev_tensors, oracle_rows, sample_picks, to_numpy64
+
+pytestmark = pytest.mark.gpu
+
+
+def feature_of(g, layout="psd_direct"):
+    return layout if g == 1 else f"{layout}:g{g}"
+
+
+# the smallest lengths that run as chunks without a state, and a few edges above them
+@pytest.mark.parametrize("g,H,T,d", [(1, 1, 7169, 64), (1, 17, 7425, 64), (1, 2, 8192, 32), (2, 1, 3073, 64), (2, 30, 4097, 64),
+                                     (4, 1, 1537, 64), (4, 2, 2048, 64), (4, 50, 2049, 64)])
+def test_chunked_without_state(g, H, T, d):
+    import torch
+    w = inputs.gaussian_workload(f"chunks_{g}_{H}_{T}_{d}", "bf16", 1, H, T, d, d, 64, 5100 + T + g)
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    q, k, v = dev_tensors(w)
+    o = kb.kata_fwd_chunked(q, k, v, feature_groups=g, device_status=st)
+    torch.cuda.synchronize()
+    assert kb.kata_last_impl() == kb.KATA_IMPL_TENSOR and int(st.item()) == 0
+    assert kb.kata_last_launch_count() in (3, 4), "key scales, chunk states (and their segments' sums), outputs"
+    o2 = kb.kata_fwd_chunked(q, k, v, feature_groups=g)
+    torch.cuda.synchronize()
+    assert torch.equal(o, o2), "fixed summation order"
+    picks = sample_picks(w, 64, T) + [(0, H - 1, t) for c in (512, 1024, 1536, 2048, T // 256 * 256) for t in (c - 1, c, c + 127, c + 128)
+                                      if t < T]
+    gpu = to_numpy64(o)
+    check(np.stack([gpu[b, h, t] for b, h, t in picks]), oracle_rows(w, picks, feature_of(g)), "bf16", f"M{g} T={T} H={H} d={d}")
+
+
+@pytest.mark.parametrize("layout", ["psd_direct", "psd_packed"])
+@pytest.mark.parametrize("g,H,cuts", [(1, 2, (513, 1537)), (1, 20, (100, 612)), (2, 3, (1024, 1025)), (4, 2, (700, 2300))])
+def test_state_in_and_out(layout, g, H, cuts):
+    """Two pieces, the state handed from one to the other in place, outputs and final state against the definition."""
+    import torch
+    T, d = cuts[1], 64
+    w = inputs.gaussian_workload(f"hand_{g}_{H}_{T}", "bf16", 1, H, T, d, d, 64, 5300 + T + g)
+    q, k, v = dev_tensors(w)
+    code = kb.KATA_LAYOUT_PACKED if layout == "psd_packed" else kb.KATA_LAYOUT_DIRECT
+    n = kb.decode_n_psi(d, 2, code, g)
+    S, Z = torch.zeros(1, H, n, d, device="cuda"), torch.zeros(1, H, n, device="cuda")
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    outs, a = [], 0
+    for b in cuts:
+        kw = dict(s_pre=S, z_pre=Z, state_layout=code, feature_groups=g, device_status=st)
+        if a > 0:
+            kw.update(s_init=S, z_init=Z)
+        outs.append(kb.kata_fwd_chunked(*(x[:, :, a:b].contiguous() for x in (q, k, v)), **kw))
+        assert kb.kata_last_impl() == kb.KATA_IMPL_TENSOR
+        a = b
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0
+    gpu = to_numpy64(torch.cat(outs, dim=2))
+    for h in sorted({0, H - 1}):
+        r = ko.kata_quadratic(w.q_ref[0, h], w.k_ref[0, h], w.v_ref[0, h], feature_of(g))[0]
+        check(gpu[0, h], r, "bf16", f"M{g} pieces {cuts} head {h}")
+        f = ko.apply_feature(w.k_ref[0, h], feature_of(g, layout))
+        for got, ref in ((S, f.T @ w.v_ref[0, h]), (Z, f.sum(axis=0))):
+            assert np.max(np.abs(to_numpy64(got[0, h]) - ref)) <= 2e-2 * max(1.0, np.abs(ref).max())
