@@ -80,6 +80,9 @@ void simt_bwd_chunked(const Problem& p, const void* dout, void* dq, void* dk, vo
 size_t tc_bwd_workspace_bytes(const Problem& p);
 void tc_bwd_quadratic(const Problem& p, const void* dout, void* dq, void* dk, void* dv, void* workspace, int* device_status,
                       LaunchCtx& ctx);
+size_t tc_bwd_exact_workspace_bytes(const Problem& p);
+void tc_bwd_exact(const Problem& p, const void* dout, void* dq, void* dk, void* dv, void* workspace, int* device_status,
+                  LaunchCtx& ctx);
 
 // feature_order = 1: rows of q,k are the features (plain normalised linear attention, state d_k x d_v)
 size_t order1_state_elems(int d_k, int d_v);
@@ -123,7 +126,7 @@ void tc_states(const Problem& p, const __nv_bfloat16* rscale, const StatePlan& p
 // quadratic form: one chunk, no state).
 struct AttendStates {
   const __nv_bfloat16* s;      // [BH][n_chunks][rows of PairTable<G>][64]: the state before each chunk, weights of the pairs included
-  const __nv_bfloat16* z;      // [BH][n_chunks][64][64]: its normaliser as a symmetric matrix
+  const __nv_bfloat16* z;      // [BH][n_chunks][rows]: its normaliser, likewise
   int n_chunks, chunk_tokens;  // chunk_tokens: a multiple of 256
   int first_state;             // first chunk that has a state before it (0 or 1)
 };

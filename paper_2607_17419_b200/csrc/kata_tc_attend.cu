@@ -7,16 +7,17 @@
 // the items are ordered heaviest first and dealt to the CTAs in rounds, forwards and backwards in turn.  An item is a
 // list of tiles that both halves walk:
 //   state tiles (chunked form, chunks after the first): the state S, Z before the chunk, in bf16
-//     Y = Q Z              one tile: Z as a symmetric 64 x 64 matrix; the normaliser of the state is q . Y per row
-//     O += Psi(Q) S        256 rows of the state per tile; the builders write the 256 feature products of their query
-//                          row as the A operand (TMEM)
+//     [O | D] += Psi(Q) [S | Z]   256 rows of the state per tile; the builders write the 256 feature products of their
+//                                 query row as the A operand (TMEM); Z is column 64 of B, so numerator and normaliser
+//                                 see the same rounded features (a Z of its own, q . Z q from the fp32 products, left
+//                                 rows with a small normaliser outside the bf16 tolerance)
 //   key tiles of 128 keys, from the start of the chunk (quadratic form: of the sequence) up to the diagonal:
 //     scores   S = Q K_j^T            A = the query tile in TMEM, B = the key tile (TMA, 128B swizzle)
 //     weights  P = r S^2 (causal mask on the diagonal tiles)  packed fp32x2 multiplies on the TMEM read-back, rounded
 //                                     to bf16, times r, stored back over the scores
 //     apply    [O | D] += P [V | 1]   A = P from TMEM, B = the value tile and a constant column of ones (MN-major,
 //                                     N = 80): the normaliser is column 64 of the same accumulator
-//   epilogue out = O / (D + q.Y)  (0 where that is 0)      the gate/normalise step of the readout
+//   epilogue out = O / D  (0 where that is 0)      the gate/normalise step of the readout
 // There is no running maximum and no rescaling: the weights are polynomial.  The query norm cancels between
 // numerator and denominator and is never applied.  In the quadratic form the d^2-wide feature state is never formed.
 // Rows narrower than 64 entries are read by TMA boxes of 64 columns, whose columns beyond the row are zero.
@@ -28,8 +29,8 @@
 // TMA writes, r) was asked for about 800 cycles per key tile, more than the MMAs take; here it is about 480.
 //
 // Nothing is set up per item: TMEM and the barriers are the CTA's, the stage ring runs on across items (every role
-// counts tiles cumulatively), the query tiles are double-buffered in shared memory and copied to TMEM before the
-// epilogue of the item before.
+// counts tiles cumulatively), and the next item's query tiles are loaded once the features of this one are built and
+// copied to TMEM before its epilogue.
 //
 // Warps (640 threads): 0 TMA producer, 1 and 2 the MMA issuers of the halves, 3 key scales, 4-11 builders of half A,
 // 12-19 builders of half B (TMEM lane quadrant = warp % 4; the two warps of a quadrant have a sub-buffer each).  All
@@ -59,14 +60,13 @@ constexpr uint32_t COL_O = 256;  // 2 x 80 fp32 accumulators: 64 outputs, column
 constexpr uint32_t COL_Q = 416;  // 2 x 32: the query tiles (bf16 A operands)
 constexpr uint32_t TMEM_COLS = 512;
 
-constexpr uint32_t OFF_Q = 0;                       // 2 x 2 x (128 x 64 bf16, 128B swizzle): the query tiles of this and the next item
+constexpr uint32_t OFF_Q = 0;                       // 2 x (128 x 64 bf16, 128B swizzle): the query tiles of an item
 constexpr uint32_t STAGE_BYTES = 32768;             // K tile 16 KB, V tile 16 KB
-constexpr uint32_t OFF_ST = 65536;
+constexpr uint32_t OFF_ST = 32768;
 constexpr uint32_t OFF_ONES = OFF_ST + NSTAGE * STAGE_BYTES;   // 16 rows of [1, 0 ...]: columns 64.. of the values
-constexpr uint32_t OFF_ZEROS = OFF_ONES + 2048;                // 16 rows of zeros: columns 64.. of a state
-constexpr uint32_t OFF_RV = OFF_ZEROS + 2048;                  // NSTAGE x 128 bf16: 1 / ||k||^2 of the keys of a tile
-constexpr uint32_t OFF_DEN = OFF_RV + NSTAGE * 256;            // [half][sub][128] floats: the two shares of q . Y of a row meet here
-constexpr uint32_t OFF_BAR = OFF_DEN + 2048;
+constexpr uint32_t OFF_Z = OFF_ONES + 2048;                    // columns 64.. of a state: 256 rows of 128 bytes, stage s in bytes [32 s, 32 s + 32)
+constexpr uint32_t OFF_RV = OFF_Z + 32768;                     // NSTAGE x 128 bf16: 1 / ||k||^2 of the keys of a tile
+constexpr uint32_t OFF_BAR = OFF_RV + NSTAGE * 256;
 constexpr uint32_t SMEM_BYTES = OFF_BAR + 512;
 constexpr uint32_t SMEM_ALLOC = SMEM_BYTES + 1024;
 static_assert(SMEM_ALLOC > 116 * 1024, "one CTA per SM is assumed (the CTA allocates all of TMEM)");
@@ -74,9 +74,9 @@ static_assert(SMEM_ALLOC > 116 * 1024, "one CTA per SM is assumed (the CTA alloc
 // No barrier can complete two phases ahead of a waiter; a waiter that skips a phase (the builders the last one of an item
 // at BAR_SFREE) knows from a barrier that it waited for since that it is complete.
 enum {
-  BAR_QFULL = 0,     // [2] the query tiles of an item landed in shared memory
-  BAR_QEMPTY = 2,    // [2] ... and have been read (512 builders)
-  BAR_FULL = 4,      // [NSTAGE] tile (TMA bytes) and its key scales (scale warp) landed
+  BAR_QFULL = 0,     // the query tiles of an item landed in shared memory
+  BAR_QEMPTY = 1,    // ... and have been read (512 builders)
+  BAR_FULL = 4,      // [NSTAGE] tile (TMA bytes) and its key scales or Z column (warp 3) landed
   BAR_EMPTY = 8,     // [NSTAGE] stage free: both issuers
   BAR_SFULL = 12,    // [half][sub] scores in TMEM
   BAR_PFULL = 16,    // [half][sub] the builders are done with the sub-buffer (128)
@@ -137,6 +137,7 @@ struct AArgs {
   int chunk_pairs;               // ... of a chunk (the quadratic form: n_pairs)
   int n_chunks;
   int first_state;               // first chunk that has a state before it
+  const unsigned short* z;       // [BH][n_chunks][state rows] bf16: Z before each chunk
 };
 
 // G = feature groups of the blockwise map: a key tile holds KT = 128 / G keys, and the 128 score columns of a buffer
@@ -145,8 +146,7 @@ struct AArgs {
 template <int G>
 __global__ void __launch_bounds__(NTHREADS, 1)
 tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
-                 const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmS,
-                 const __grid_constant__ CUtensorMap tmZ, const AArgs args) {
+                 const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmS, const AArgs args) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   auto bar = [&](int i) { return reinterpret_cast<uint64_t*>(base + OFF_BAR) + i; };
@@ -189,7 +189,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       it.k0 = it.chunk * args.chunk_pairs * 2 * G;
       it.nk_a = (2 * p + 1) * G;
       it.nk_b = it.q0 + QT < args.Tlen ? (2 * p + 2) * G : 0;
-      it.ns = it.chunk >= args.first_state ? NST + 1 : 0;
+      it.ns = it.chunk >= args.first_state ? NST : 0;
       it.n_tiles = it.ns + (it.nk_b > 0 ? it.nk_b : it.nk_a);
       return true;
     }
@@ -197,9 +197,9 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
 
   if (tid == 0) {
     abort_s = 0;
+    mbar_init(bar(BAR_QFULL), 1);
+    mbar_init(bar(BAR_QEMPTY), 512);
     for (int i = 0; i < 2; ++i) {
-      mbar_init(bar(BAR_QFULL + i), 1);
-      mbar_init(bar(BAR_QEMPTY + i), 512);
       mbar_init(bar(BAR_QT + i), 256);
       mbar_init(bar(BAR_ODONE + i), 1);
       mbar_init(bar(BAR_OFREE + i), 256);
@@ -221,18 +221,14 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     tma_prefetch_desc(&tmQ);
     tma_prefetch_desc(&tmK);
     tma_prefetch_desc(&tmV);
-    if (args.first_state < args.n_chunks) {
-      tma_prefetch_desc(&tmS);
-      tma_prefetch_desc(&tmZ);
-    }
+    if (args.first_state < args.n_chunks) tma_prefetch_desc(&tmS);
   }
-  // columns 64..127 of 16 rows of the B operands: [1, 0, ...] for the values, zeros for the state (every step of 16 rows
-  // reads the same block: the descriptor's leading offset is the distance to it)
-  for (int i = tid; i < 256; i += NTHREADS) {
-    const int row = (i & 127) >> 3, c = i & 7;
-    *reinterpret_cast<uint4*>(base + OFF_ONES + (i >> 7) * 2048 + sw128_offset(row, c)) =
-        make_uint4(i < 128 && c == 0 ? 0x3F80u : 0u, 0u, 0u, 0u);
-  }
+  // columns 64..127 of 16 rows of the value operand: [1, 0, ...] (every step of 16 rows reads the same block: the
+  // descriptor's leading offset is the distance to it); the Z columns of the state start as zeros
+  if (tid < 128)
+    *reinterpret_cast<uint4*>(base + OFF_ONES + sw128_offset(tid >> 3, tid & 7)) = make_uint4((tid & 7) == 0 ? 0x3F80u : 0u, 0u, 0u, 0u);
+  if (args.first_state < args.n_chunks)
+    for (int i = tid; i < 2048; i += NTHREADS) *reinterpret_cast<uint4*>(base + OFF_Z + i * 16) = make_uint4(0u, 0u, 0u, 0u);
   fence_async_smem();
   if (warp == 0) {
     tmem_alloc(&tmem_base_s, TMEM_COLS);
@@ -254,12 +250,11 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       // the kernel is a programmatic dependent launch: the states are the work of the kernel before it
       if (args.first_state < args.n_chunks) cudaGridDependencySynchronize();
       for (int n = 0; ok && next_item(n, w); ++n, ++ni) {
-        const int qb = ni & 1;
-        ok = wait_or_abort(bar(BAR_QEMPTY + qb), ((ni >> 1) & 1) ^ 1, abort_flag);
+        ok = wait_or_abort(bar(BAR_QEMPTY), (ni & 1) ^ 1, abort_flag);
         if (!ok) break;
-        mbar_arrive_expect_tx(bar(BAR_QFULL + qb), w.nk_b > 0 ? 32768 : 16384);
-        tma_load_3d(base + OFF_Q + qb * 32768, &tmQ, bar(BAR_QFULL + qb), 0, w.q0, w.bh);
-        if (w.nk_b > 0) tma_load_3d(base + OFF_Q + qb * 32768 + 16384, &tmQ, bar(BAR_QFULL + qb), 0, w.q0 + QT, w.bh);
+        mbar_arrive_expect_tx(bar(BAR_QFULL), w.nk_b > 0 ? 32768 : 16384);
+        tma_load_3d(base + OFF_Q, &tmQ, bar(BAR_QFULL), 0, w.q0, w.bh);
+        if (w.nk_b > 0) tma_load_3d(base + OFF_Q + 16384, &tmQ, bar(BAR_QFULL), 0, w.q0 + QT, w.bh);
         for (int j = 0; j < w.n_tiles && ok; ++j, ++it) {
           const int s = it % NSTAGE;
           ok = wait_or_abort(bar(BAR_EMPTY + s), ((it / NSTAGE) & 1) ^ 1, abort_flag);
@@ -271,9 +266,8 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
             tma_load_3d(stage(s) + 16384, &tmV, bar(BAR_FULL + s), 0, key, w.bh);
           } else {
             const int slot = w.bh * args.n_chunks + w.chunk;
-            mbar_arrive_expect_tx(bar(BAR_FULL + s), j == 0 ? 8192 : 32768);
-            if (j == 0) tma_load_3d(stage(s), &tmZ, bar(BAR_FULL + s), 0, 0, slot);
-            else tma_load_3d(stage(s), &tmS, bar(BAR_FULL + s), 0, (j - 1) * 256, slot);
+            mbar_arrive_expect_tx(bar(BAR_FULL + s), 32768);
+            tma_load_3d(stage(s), &tmS, bar(BAR_FULL + s), 0, j * 256, slot);
           }
         }
       }
@@ -288,12 +282,10 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     if (elect_one()) {
       const int h = warp - 1;
       const uint32_t id_s = instr_desc(kFmtBF16, kFmtBF16, 0, 0, 128, KH);      // scores: B K-major
-      const uint32_t id_y = instr_desc(kFmtBF16, kFmtBF16, 0, 0, 128, 32);      // Q Z, 32 columns
-      const uint32_t id_p = instr_desc(kFmtBF16, kFmtBF16, 0, 1, 128, 80);      // apply: B MN-major, N = 64 + 16
-      const uint32_t id_f = instr_desc(kFmtBF16, kFmtBF16, 0, 1, 128, 64);      // Psi(Q) S
+      const uint32_t id_p = instr_desc(kFmtBF16, kFmtBF16, 0, 1, 128, 80);      // apply, Psi(Q) [S | Z]: B MN-major, N = 64 + 16
       const uint64_t dk = smem_desc(0, 16, 1024, kSwizzle128B);
       const uint32_t tS = tb + COL_S + h * 128, tO = tb + COL_O + h * 80, tQ = tb + COL_Q + h * 32;
-      const uint32_t ones = smem_u32(base + OFF_ONES), zeros = smem_u32(base + OFF_ZEROS);
+      const uint32_t ones = smem_u32(base + OFF_ONES), zcol = smem_u32(base + OFF_Z);
       // MN-major, 128B swizzle: 8 rows per 1024-byte atom (SBO), columns 64.. in the constant block (LBO)
       auto bdesc = [&](uint32_t addr, uint32_t extra) { return smem_desc(addr, extra - addr, 1024, kSwizzle128B); };
       uint32_t it = 0, cnt = 0, n_st = 0;   // tiles, key tiles of this half, its state tiles
@@ -323,24 +315,14 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
           }
           return true;
         };
-        if (nt > 0) ok = wait_or_abort(bar(BAR_QT + h), n_done & 1, abort_flag) && landed(it);
+        if (nt > 0) ok = wait_or_abort(bar(BAR_QT + h), n_done & 1, abort_flag) && (w.ns > 0 || landed(it));
         if (nt > 0 && ok) {
           tc_fence_after();
           if (w.ns > 0) {
-            // Y = Q Z, 32 columns per sub-buffer
-            const uint32_t st = smem_u32(stage(it % NSTAGE));
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-#pragma unroll
-              for (int ks = 0; ks < 4; ++ks) mma_f16_ts(tS + c * 64, tQ + ks * 8, at(dk, st + c * 32 * 128 + ks * 32), id_y, ks > 0);
-              mma_commit(bar(BAR_SFULL + 2 * h + c));
-            }
-            mma_commit(bar(BAR_EMPTY + it % NSTAGE));
-            ++it;        // (the builders' features follow their reading of Y: no close)
 #pragma unroll 1
             for (int t = 0; t < NST && ok; ++t, ++it, ++n_st) {
               ok = landed(it) && o_free() && (t + 1 < NST || landed(it + 1));
-              const uint32_t sa = smem_u32(stage(it % NSTAGE));
+              const uint32_t sa = smem_u32(stage(it % NSTAGE)), za = zcol + (it % NSTAGE) * 32;
 #pragma unroll
               for (int c = 0; c < 2; ++c) {
 #pragma unroll
@@ -350,8 +332,8 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                   tc_fence_after();
 #pragma unroll
                   for (int ks = 0; ks < 4; ++ks) {
-                    // the very first step also clears the normaliser column (N = 80, zeros beyond column 64)
-                    mma_f16_ts(tO, tS + c * 64 + pp * 32 + ks * 8, bdesc(sa + c * 16384 + pp * 8192 + ks * 2048, zeros), acc == 0 ? id_p : id_f, acc);
+                    const uint32_t blk = (c * 8 + pp * 4 + ks) * 2048;     // 16 rows
+                    mma_f16_ts(tO, tS + c * 64 + pp * 32 + ks * 8, bdesc(sa + blk, za + blk), id_p, acc);
                     acc = 1;
                   }
                   mma_commit(bar(BAR_SFREE + 4 * h + 2 * c + pp));
@@ -387,36 +369,50 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     }
   } else if (warp == 3) {
     regs_release<64>();
-    // =========================== scale warp: r = 1 / ||k||^2 of the keys of every tile, from the pre-pass to shared memory ===========================
+    // =========================== per tile: r = 1 / ||k||^2 of its keys, or its column of Z, to shared memory ===========================
     // (the key scale multiplies the weights, so the values are used as they are; a zero key row has r = 0: zero
-    // feature).  A programmatic dependent launch: this warp waits for the pre-pass.
+    // feature).  A programmatic dependent launch: this warp and the producer wait for the kernels before.
     cudaGridDependencySynchronize();
     uint32_t it = 0;
     Item w;
     for (int n = 0; ok && next_item(n, w); ++n) {
       const unsigned short* rs = reinterpret_cast<const unsigned short*>(args.rscale) + (size_t)w.bh * args.Tlen;
-      auto load_r = [&](int j, unsigned short (&rv)[KPL]) {       // r of this lane's keys of tile j
+      const unsigned short* zs = args.z + ((size_t)w.bh * args.n_chunks + w.chunk) * (NST * 256);
+      auto load = [&](int j, unsigned short (&x)[8]) {            // tile j: r of KPL keys, or Z of 8 rows, per lane
+        if (j < w.ns) {
 #pragma unroll
-        for (int e = 0; e < KPL; ++e) {
-          const int key = (w.k0 + j - w.ns) * KT + lane * KPL + e;
-          rv[e] = (j >= w.ns && j < w.n_tiles && key < args.Tlen) ? rs[key] : (unsigned short)0;
+          for (int e = 0; e < 8; ++e) x[e] = zs[j * 256 + e * 32 + lane];
+        } else {
+#pragma unroll
+          for (int e = 0; e < KPL; ++e) {
+            const int key = (w.k0 + j - w.ns) * KT + lane * KPL + e;
+            x[e] = (j < w.n_tiles && key < args.Tlen) ? rs[key] : (unsigned short)0;
+          }
         }
       };
-      unsigned short rv[KPL];
-      load_r(0, rv);
+      unsigned short x[8] = {};
+      load(0, x);
       for (int j = 0; j < w.n_tiles && ok; ++j, ++it) {
         const int s = it % NSTAGE;
-        unsigned short rn[KPL];
-        load_r(j + 1, rn);              // one tile ahead: the global-load latency stays off the ring
+        unsigned short nx[8] = {};
+        load(j + 1, nx);                // one tile ahead: the global-load latency stays off the ring
         ok = wait_or_abort(bar(BAR_EMPTY + s), ((it / NSTAGE) & 1) ^ 1, abort_flag);
         if (!ok) break;
+        if (j < w.ns) {
 #pragma unroll
-        for (int e = 0; e < KPL; ++e) {
-          reinterpret_cast<unsigned short*>(base + OFF_RV + s * 256)[lane * KPL + e] = rv[e];
-          rv[e] = rn[e];
+          for (int e = 0; e < 8; ++e) {
+            const int row = e * 32 + lane;
+            *reinterpret_cast<unsigned short*>(base + OFF_Z + (row >> 4) * 2048 + sw128_offset(row & 15, 2 * s)) = x[e];
+          }
+          fence_async_smem();
+        } else {
+#pragma unroll
+          for (int e = 0; e < KPL; ++e) reinterpret_cast<unsigned short*>(base + OFF_RV + s * 256)[lane * KPL + e] = x[e];
         }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) x[e] = nx[e];
         __syncwarp();
-        if (lane == 0) mbar_arrive(bar(BAR_FULL + s));      // (the builders of the tile come after its score MMAs)
+        if (lane == 0) mbar_arrive(bar(BAR_FULL + s));      // (the builders of a key tile come after its score MMAs)
       }
     }
   } else {
@@ -430,17 +426,16 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     const uint32_t tS = tmem_addr(tb, q4 * 32, COL_S + h * 128 + ch * 64), tO = tmem_addr(tb, q4 * 32, COL_O + h * 80);
     const uint32_t qrow_s = smem_u32(base + OFF_Q) + h * 16384;
     // 16 bytes (eight features) of this thread's query row, from the item's tile in shared memory
-    auto qrun = [&](int qb, int c) { return lds128(qrow_s + qb * 32768 + sw128_offset(rowl, c)); };
+    auto qrun = [&](int c) { return lds128(qrow_s + sw128_offset(rowl, c)); };
     // the query tile of an item into TMEM: this thread's row, 32 of its features
     auto copy_q = [&](int ni, const Item& w) {
-      const int qb = ni & 1;
-      ok = ok && wait_or_abort(bar(BAR_QFULL + qb), (ni >> 1) & 1, abort_flag);
+      ok = ok && wait_or_abort(bar(BAR_QFULL), ni & 1, abort_flag);
       if (!ok) return;
       if (h == 0 || w.nk_b > 0) {
         uint32_t r[16];
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-          const uint4 x = qrun(qb, ch * 4 + c);
+          const uint4 x = qrun(ch * 4 + c);
           r[4 * c] = x.x; r[4 * c + 1] = x.y; r[4 * c + 2] = x.z; r[4 * c + 3] = x.w;
         }
         tmem_st16(tmem_addr(tb, q4 * 32, COL_Q + h * 32 + ch * 16), r);
@@ -448,7 +443,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         tc_fence_before();
         mbar_arrive(bar(BAR_QT + h));
       }
-      if (w.ns == 0) mbar_arrive(bar(BAR_QEMPTY + qb));
+      if (w.ns == 0) mbar_arrive(bar(BAR_QEMPTY));
     };
     uint32_t it = 0, cnt = 0, n_st = 0;
     int n_done = 0, ni = 0, n = 0;
@@ -458,29 +453,9 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     for (; more && ok; ++ni) {
       const int nk = h == 0 ? w.nk_a : w.nk_b;
       const int qrow = w.q0 + h * QT + rowl;
-      float den0 = 0.f;                          // the state's part of the normaliser
       const uint32_t it0 = it;
       it += w.n_tiles;
       if (nk > 0 && w.ns > 0) {
-        const int qb = ni & 1;
-        // ---- Y = Q Z: den0 = q . Y, this warp's 32 of the 64 columns ----
-        ok = wait_or_abort(bar(BAR_SFULL + 2 * h + ch), cnt & 1, abort_flag);
-        if (!ok) break;
-        tc_fence_after();
-        uint32_t y[32];
-        tmem_ld32(tS, y);
-        tmem_wait_ld(y);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const uint4 x = qrun(qb, ch * 4 + c);
-          const uint32_t xs[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            den0 = fmaf(__uint_as_float(xs[e] << 16), __uint_as_float(y[8 * c + 2 * e]), den0);
-            den0 = fmaf(__uint_as_float(xs[e] & 0xFFFF0000u), __uint_as_float(y[8 * c + 2 * e + 1]), den0);
-          }
-        }
-        ++cnt;
         // ---- the features of this query row, 256 per tile, this warp's two pairs of runs ----
         static constexpr PairTable<G> kPairs{};
 #pragma unroll 1
@@ -488,7 +463,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
 #pragma unroll 1
           for (int pp = 0; pp < 2; ++pp) {
             const int p = 4 * t + 2 * ch + pp;
-            const uint4 xg = qrun(qb, kPairs.g[p]), xh = qrun(qb, kPairs.h[p]);
+            const uint4 xg = qrun(kPairs.g[p]), xh = qrun(kPairs.h[p]);
             const uint32_t gs[4] = {xg.x, xg.y, xg.z, xg.w}, hs[4] = {xh.x, xh.y, xh.z, xh.w};
             uint32_t f[32];
 #pragma unroll
@@ -497,7 +472,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
 #pragma unroll
               for (int e = 0; e < 4; ++e) f[4 * j + e] = mul_bf16x2(gs[e], b2);
             }
-            // the piece is free: Y has been read by this warp, or the MMAs of the tile before have read its features
+            // the piece is free: the item before is complete, or the MMAs of the tile before have read its features
             if (t > 0) ok = ok && wait_or_abort(bar(BAR_SFREE + 4 * h + 2 * ch + pp), (n_st - 1) & 1, abort_flag);
             if (!ok) break;
             tc_fence_after();
@@ -509,7 +484,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         }
         if (!ok) break;
       }
-      if (w.ns > 0) mbar_arrive(bar(BAR_QEMPTY + (ni & 1)));
+      if (w.ns > 0) mbar_arrive(bar(BAR_QEMPTY));
       for (int j = 0; j < nk && ok; ++j, ++cnt) {
         const uint32_t g_it = it0 + w.ns + j;
         const int s = g_it % NSTAGE;
@@ -588,7 +563,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       }
       if (!ok) break;
       // the next item's queries go to TMEM before the wait for this item's last MMAs (its score MMAs are all through)
-      const int bh = w.bh, ns = w.ns;
+      const int bh = w.bh;
       ++n;
       more = next_item(n, w);
       if (more) copy_q(ni + 1, w);
@@ -605,14 +580,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       tmem_wait_ld(dn);
       tc_fence_before();
       mbar_arrive(bar(BAR_OFREE + h));           // the MMAs of the next item may overwrite [O | D]
-      if (ns > 0) {                              // the two warps of a row hold the two halves of q . Y
-        float* part = reinterpret_cast<float*>(base + OFF_DEN) + h * 256 + rowl;
-        part[ch * 128] = den0;
-        asm volatile("bar.sync %0, 64;" ::"r"(1 + h * 4 + (int)q4) : "memory");
-        den0 = part[0] + part[128];
-        asm volatile("bar.sync %0, 64;" ::"r"(1 + h * 4 + (int)q4) : "memory");   // before the next item overwrites the shares
-      }
-      const float den = __uint_as_float(dn[0]) + den0;
+      const float den = __uint_as_float(dn[0]);
       const float inv = den > 0.f ? 1.f / den : 0.f;
       if (qrow < args.Tlen) {
         __nv_bfloat16* dst = args.out + ((size_t)bh * args.Tlen + qrow) * args.d_v + ch * 32;
@@ -656,21 +624,20 @@ void tc_rscale(const Problem& p, __nv_bfloat16* rscale, LaunchCtx& ctx) {
 
 void tc_attend(const Problem& p, const __nv_bfloat16* rscale, const AttendStates& st, int* device_status, LaunchCtx& ctx) {
   const int BH = p.B * p.H;
-  CUtensorMap tmQ, tmK, tmV, tmS, tmZ;
+  CUtensorMap tmQ, tmK, tmV, tmS;
   const int kt = KTILE / p.groups;
   const int n_pairs = (p.T + 2 * QT - 1) / (2 * QT);
-  AArgs a{static_cast<__nv_bfloat16*>(p.out), rscale, device_status, p.T, p.d_v, BH, n_pairs, n_pairs, 1, 1};
+  AArgs a{static_cast<__nv_bfloat16*>(p.out), rscale, device_status, p.T, p.d_v, BH, n_pairs, n_pairs, 1, 1, nullptr};
   bool maps = make_tile_map(&tmQ, p.q, BH, p.T, QT, p.d_k) && make_tile_map(&tmK, p.k, BH, p.T, kt, p.d_k) &&
               make_tile_map(&tmV, p.v, BH, p.T, kt, p.d_v);
   if (st.n_chunks > 0) {
     a.chunk_pairs = st.chunk_tokens / (2 * QT);
     a.n_chunks = st.n_chunks;
     a.first_state = st.first_state;
-    maps = maps && make_tile_map(&tmS, st.s, BH * st.n_chunks, tc_state_rows(p.groups), 256) &&
-           make_tile_map(&tmZ, st.z, BH * st.n_chunks, 64, 64);
+    a.z = reinterpret_cast<const unsigned short*>(st.z);
+    maps = maps && make_tile_map(&tmS, st.s, BH * st.n_chunks, tc_state_rows(p.groups), 256);
   } else {
     tmS = tmK;
-    tmZ = tmK;
   }
   if (!maps) {
     ctx.status = KATA_ERR_CUDA;
@@ -698,7 +665,7 @@ void tc_attend(const Problem& p, const __nv_bfloat16* rscale, const AttendStates
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, kern, tmQ, tmK, tmV, tmS, tmZ, a) != cudaSuccess) {
+  if (cudaLaunchKernelEx(&cfg, kern, tmQ, tmK, tmV, tmS, a) != cudaSuccess) {
     cudaGetLastError();
     ctx.status = KATA_ERR_CUDA;
     return;

@@ -23,7 +23,7 @@ ChunkBuffers chunk_buffers(const Problem& p, const StatePlan& plan, bool states)
   b.r = 0;
   b.s = align256(BH * p.T * 2);
   b.z = b.s + (states ? align256(slots * rows * 64 * 2) : 0);
-  b.s_loc = b.z + (states ? align256(slots * 64 * 64 * 2) : 0);
+  b.s_loc = b.z + (states ? align256(slots * rows * 2) : 0);
   b.z_loc = b.s_loc + (states && plan.segments > 1 ? align256(slots * rows * 64 * 4) : 0);
   b.total = b.z_loc + (states && plan.segments > 1 ? align256(slots * rows * 4) : 0);
   return b;

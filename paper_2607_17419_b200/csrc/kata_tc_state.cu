@@ -13,8 +13,8 @@
 //   update   [S | Z] += A [V | 1]   A from TMEM, B = the value tile as it is and a constant column of ones, N = 80,
 //            two accumulators of 128 rows
 // The accumulators hold one chunk; between chunks eight warps add them to a running sum in registers (fp32, one state
-// row per thread) and write it out in bf16 (the state before the next chunk, pair weights included, and Z as a
-// symmetric 64 x 64 matrix), while the update goes on in the other pair of accumulators.
+// row per thread) and write it out in bf16 (the state before the next chunk, pair weights included), while the update goes
+// on in the other pair of accumulators.
 //
 // What bounds it: shared memory.  Per tile and CTA: 640 cycles of MMA, and at 128 B per cycle 256 for the TMA writes, 320
 // for the value operand, about 460 for the builders' fragment loads, scales and shuffles.  Built in shared memory and read
@@ -72,7 +72,7 @@ enum {
 struct SArgs {
   const __nv_bfloat16* rscale;   // [BH][T]
   __nv_bfloat16* s;              // [BH][n_chunks][rows][64]: state before each chunk (one segment)
-  __nv_bfloat16* z;              // [BH][n_chunks][64][64]
+  __nv_bfloat16* z;              // [BH][n_chunks][rows]
   float* s_loc;                  // [BH][n_chunks][rows][64]: sum of the segment up to and including the chunk (several segments)
   float* z_loc;                  // [BH][n_chunks][rows]
   const float* s_init;           // state before the first token, public layout (null: zero)
@@ -102,7 +102,7 @@ template <int G> __device__ __forceinline__ size_t public_rows(int packed) {
 
 template <int N> __device__ __forceinline__ void regs_release() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
 template <int N> __device__ __forceinline__ void regs_take() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
-static_assert(384 * 72 + 256 * 128 <= 640 * 96, "register budget");
+static_assert(384 * 80 + 256 * 120 <= 640 * 96, "register budget");
 
 __device__ __forceinline__ uint32_t mul_bf16x2(uint32_t a, uint32_t b) {
   const __nv_bfloat162 p = __hmul2(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));
@@ -179,7 +179,7 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
   bool ok = true;
 
   if (warp == 0) {
-    regs_release<72>();
+    regs_release<80>();
     // =========================== TMA producer ===========================
     if (elect_one()) {
       for (int j = 0; j < n && ok; ++j) {
@@ -192,7 +192,7 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
       }
     }
   } else if (warp == 1) {
-    regs_release<72>();
+    regs_release<80>();
     // =========================== update issuer ===========================
     if (elect_one()) {
       const uint32_t idesc = instr_desc(kFmtBF16, kFmtBF16, 0, 1, 128, 80);
@@ -231,7 +231,7 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
       }
     }
   } else if (warp == 2) {
-    regs_release<72>();
+    regs_release<80>();
     // =========================== key scales, from the pre-pass to shared memory ===========================
     cudaGridDependencySynchronize();
     const unsigned short* rs = reinterpret_cast<const unsigned short*>(args.rscale) + (size_t)bh * args.Tlen;
@@ -262,9 +262,9 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
       if (lane == 0) mbar_arrive(bar(BAR_FULL + s));
     }
   } else if (warp == 3) {
-    regs_release<72>();
+    regs_release<80>();
   } else if (warp < WARP_SUM0) {
-    regs_release<72>();
+    regs_release<80>();
     // =========================== builders ===========================
     const int q4 = warp & 3, th = (warp - WARP_BLD0) >> 2;
     const int pa = 4 * slice + (q4 >> 1), pb = pa + 2;
@@ -334,7 +334,7 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     };
     if (ha != hb) build(std::true_type{}); else build(std::false_type{});
   } else {
-    regs_take<128>();
+    regs_take<120>();
     // =========================== running sums: one state row per thread ===========================
     const int q4 = warp & 3, m = (warp - WARP_SUM0) >> 2;
     const int row = slice * 256 + m * 128 + q4 * 32 + lane;
@@ -373,13 +373,7 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         x.w = pack_bf16(sum[8 * i + 6] * wgt, sum[8 * i + 7] * wgt);
         dst[i] = x;
       }
-      __nv_bfloat16* zm = args.z + slot * D * D;
-      zm[a * D + b] = __float2bfloat16_rn(zsum);
-      if (mirror) zm[b * D + a] = __float2bfloat16_rn(zsum);
-      if (G > 1 && slice == 0) {                             // outside the feature groups
-        for (int i = m * 128 + q4 * 32 + lane; i < D * D; i += 256)
-          if ((i / D) / (D / G) != (i % D) / (D / G)) zm[i] = __float2bfloat16_rn(0.f);
-      }
+      args.z[slot * ROWS + row] = __float2bfloat16_rn(zsum * wgt);
     };
     if (first) write_state(0);
     for (int c = c_beg, i = 0; c < c_end && ok; ++c, ++i) {
@@ -480,12 +474,7 @@ __global__ void __launch_bounds__(256) state_fix_kernel(const float* __restrict_
       if (c + 1 < n_chunks) {
         reinterpret_cast<uint2*>(s)[((slot0 + c + 1) * ROWS + row) * 16 + c4] =
             make_uint2(pack_bf16(y.x * wgt, y.y * wgt), pack_bf16(y.z * wgt, y.w * wgt));
-        __nv_bfloat16* zm = z + (slot0 + c + 1) * D * D;
-        if (c4 == 0) {
-          zm[a * D + b] = __float2bfloat16_rn(zy);
-          if (mirror) zm[b * D + a] = __float2bfloat16_rn(zy);
-        }
-        if (G > 1 && idx < D * D && (idx / D) / (D / G) != (idx % D) / (D / G)) zm[idx] = __float2bfloat16_rn(0.f);
+        if (c4 == 0) z[(slot0 + c + 1) * ROWS + row] = __float2bfloat16_rn(zy * wgt);
       } else {
         const size_t n_pub = public_rows<G>(packed);
         auto put = [&](int r, float f) {
