@@ -78,6 +78,10 @@ int check_shape(int fn, int B, int H, int T, int d_k, int d_v, int C) {
   return KATA_OK;
 }
 
+// Lengths of that route.  Below 512 tokens the entry stays on its plain FMA kernels (their cost there is a millisecond at
+// most); above 16384 it keeps the O(T) walk that it promises.
+constexpr int kBwdExactMin = 512, kBwdExactMax = 16384;
+
 bool want_tensor(int fn, const Problem& p, const Opts& o) {
   return o.impl != KATA_IMPL_SIMT && tc_supported(p, fn);
 }
@@ -88,6 +92,13 @@ bool bwd_tensor(const Problem& p, const Opts& o) {
   if (o.impl == KATA_IMPL_SIMT || p.dtype != KATA_BF16 || p.feature_order != 2) return false;
   // feature blocks depend on the true width: no padding there
   return p.groups == 1 || ((p.groups == 2 || p.groups == 4) && p.d_k == 64 && p.d_v == 64);
+}
+
+// kata_bwd_chunked on the tensor cores: the quadratic form with fp32 weights (kata_tc_bwd.cu) for bf16 rows of 64 entries
+// and lengths at which its O(T^2) work is the smaller.
+bool bwd_exact(const Problem& p, const Opts& o) {
+  return o.impl != KATA_IMPL_SIMT && p.dtype == KATA_BF16 && p.feature_order == 2 && p.groups == 1 && p.d_k == 64 && p.d_v == 64 &&
+         p.T >= kBwdExactMin && p.T <= kBwdExactMax && (long long)p.B * p.H <= 65535;
 }
 
 // Scratch of the backward: the fp32 kernels' row scalars, or the tensor-core kernels' scratch behind seven padded
@@ -849,23 +860,25 @@ int kata_bwd_chunked(const void* q, const void* k, const void* v, const void* do
   if (B < 1 || H < 1 || T < 1 || d_k < 1 || d_v < 1) return KATA_ERR_INVALID_ARG;
   if (o.s_pre != nullptr || o.s_init != nullptr || o.z_init != nullptr) return KATA_ERR_INVALID_ARG;
   const Problem p{q, k, v, nullptr, B, H, T, d_k, d_v, o.dtype, o.feature_order, o.groups};
-  if (C != kChunk || !simt_bwd_chunked_supported(p) || o.impl == KATA_IMPL_TENSOR) return KATA_ERR_UNSUPPORTED_SHAPE;
+  const bool exact = bwd_exact(p, o);
+  if (C != kChunk || !simt_bwd_chunked_supported(p) || (o.impl == KATA_IMPL_TENSOR && !exact)) return KATA_ERR_UNSUPPORTED_SHAPE;
   if ((long long)B * H * (d_v / 8) > 2147483647LL) return KATA_ERR_UNSUPPORTED_SHAPE;
   if (q == nullptr || k == nullptr || v == nullptr || dout == nullptr || dq == nullptr || dk == nullptr || dv == nullptr)
     return KATA_ERR_INVALID_ARG;
   if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(dout) || !aligned16(dq) || !aligned16(dk) ||
       !aligned16(dv))
     return KATA_ERR_ALIGNMENT;
-  const size_t need = align_up(simt_bwd_chunked_workspace_elems(p) * sizeof(float));
+  const size_t need = exact ? align_up(tc_bwd_exact_workspace_bytes(p)) : align_up(simt_bwd_chunked_workspace_elems(p) * sizeof(float));
   if (o.workspace == nullptr || o.workspace_bytes < need) return KATA_ERR_WORKSPACE_TOO_SMALL;
   if ((reinterpret_cast<uintptr_t>(o.workspace) & (kAlign - 1)) != 0) return KATA_ERR_ALIGNMENT;
   st = check_arch();
   if (st != KATA_OK) return st;
   LaunchCtx ctx{o.stream, 0, KATA_OK};
-  simt_bwd_chunked(p, dout, dq, dk, dv, static_cast<float*>(o.workspace), ctx);
+  if (exact) tc_bwd_exact(p, dout, dq, dk, dv, o.workspace, o.device_status, ctx);
+  else simt_bwd_chunked(p, dout, dq, dk, dv, static_cast<float*>(o.workspace), ctx);
   if (ctx.status == KATA_OK) {
     g_last_launches = ctx.launches;
-    g_last_impl = KATA_IMPL_SIMT;
+    g_last_impl = exact ? KATA_IMPL_TENSOR : KATA_IMPL_SIMT;
   }
   return ctx.status;
 }
@@ -878,6 +891,7 @@ size_t kata_workspace_bytes(int fn, int B, int H, int T, int d_k, int d_v, int C
     if (host_io || read_opts(opts, o) != KATA_OK || B < 1 || H < 1 || T < 1 || C != kChunk) return 0;
     const Problem p{nullptr, nullptr, nullptr, nullptr, B, H, T, d_k, d_v, o.dtype, o.feature_order, o.groups};
     if (!simt_bwd_chunked_supported(p)) return 0;
+    if (bwd_exact(p, o)) return align_up(tc_bwd_exact_workspace_bytes(p));
     return align_up(simt_bwd_chunked_workspace_elems(p) * sizeof(float));
   }
   if (fn == KATA_FN_BWD_QUADRATIC) {    // C is ignored

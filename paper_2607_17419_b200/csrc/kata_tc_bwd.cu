@@ -1,23 +1,36 @@
-// Backward of the quadratic form on the Blackwell tensor cores: bf16, d_k = d_v = 64, full rank-one feature.
+// Backward of the quadratic form on the Blackwell tensor cores: bf16, d_k = d_v = 64, full or blockwise rank-one feature.
 //
 // With s_ti = q_t . k_i, r_i = 1/||k_i||^2, a_ti = r_i s_ti^2 (i <= t), D_t = sum_i a_ti, o_t = sum_i a_ti v_i / D_t:
-//   c_ti = dout_t . v_i,   g_ti = (c_ti - dout_t . o_t) / D_t,   e_ti = 2 g_ti s_ti,   p_ti = s_ti^2 / D_t
-//   dq_t = sum_i e_ti k'_i                       (k' = r k, written by the pre-pass)
+//   c_ti = dout_t . v_i,   g_ti = (c_ti - dout_t . o_t) / D_t,   p_ti = s_ti^2 / D_t
+//   dq_t = sum_i 2 g_ti s_ti r_i k_i
 //   dv_i = r_i sum_t p_ti dout_t
-//   dk_i = r_i (u_i - r_i (k_i . u_i) k_i),  u_i = sum_t e_ti q_t      (the second term is the derivative of r_i; it
+//   dk_i = r_i (u_i - r_i (k_i . u_i) k_i),  u_i = sum_t 2 g_ti s_ti q_t     (the second term is the derivative of r_i; it
 //                                                                       makes dk_i orthogonal to k_i: o has degree 0 in k_i)
-// A pre-pass writes k' and r; then one kernel in two modes, both with a fixed tile of 128 rows on the TMEM lanes and
-// tiles of 64 rows streamed past it:
-//   MODE_DQ   fixed = 128 queries (Q, dout), streamed = keys (K, V, K', r), twice:  S = Q K^T, C = dout V^T (SS MMAs,
-//             N = 64); in the first sweep the weight warps sum D_t = sum_i r_i s^2 and sum_i r_i s^2 c in fp32 (the
-//             same weights in both, so dout_t . o_t is consistent with c: their difference is what the gradient is
-//             made of) and leave (1/D_t, dout_t . o_t) in the workspace; in the second sweep they form E, and
-//             dq += E K' (A = E from TMEM)
+// A pre-pass writes r; then one kernel in two modes, both with a fixed tile of 128 rows on the TMEM lanes and tiles of NT
+// rows streamed past it:
+//   MODE_DQ   fixed = 128 queries (Q, dout), streamed = keys (K, V, r), twice:  S = Q K^T, C = dout V^T (SS MMAs); in the
+//             first sweep the weight warps sum D_t = sum_i r_i s^2 and sum_i r_i s^2 c in fp32 (the same weights in both,
+//             so dout_t . o_t is consistent with c: their difference is what the gradient is made of) and leave
+//             (1/D_t, dout_t . o_t) in the workspace; in the second sweep they form E = (c - dout.o) r s, and dq += E K
+//             (A = E from TMEM; the row factor 2/D_t in the epilogue)
 //   MODE_DKV  fixed = 128 keys (K, V), streamed = queries (Q, dout, their scalars):  S^T = K Q^T, C^T = V dout^T,
 //             the weight warps form P^T and E^T with the scalars of the columns, then dv~ += P^T dout, u += E^T Q
 //             (B = the streamed tiles read MN-major), and the epilogue applies r_i and the projection.
-// No atomics, every sum in a fixed order.  Warps (384 threads): 0 TMA producer, 1 score-MMA issuer, 2 output-MMA
-// issuer, 4-11 weights and epilogue.  All waits are bounded.
+// No atomics, every sum in a fixed order.
+//
+// NS = bf16 terms of the weights P and E.  One: kata_bwd_quadratic.  Three (24 bits: fp32 weights; every other operand is
+// a bf16 input, exact, and every sum fp32): kata_bwd_chunked on sequences short enough for the quadratic form, whose
+// contract is fp32 arithmetic.
+//
+// What bounds it: the MMAs of a step (128 x 64 pairs: scores 2 x 192 cycles, one output 128, another 128) and the chain
+// scores -> weights -> outputs, about 1700 cycles of which half is hand-offs.  Each of the NBUF TMEM buffers is a chain of
+// its own with its own group of four weight warps; one thread issues all MMAs, closing the steps in order and opening each
+// buffer again right behind its close, so no wait stands between the outputs of a step and the scores that reuse its
+// columns.  The CTAs are persistent (one per SM, items dealt heaviest first, forwards and backwards in turn) and the next
+// item's scores are opened before the current one's last outputs.
+//
+// Warps: 0 TMA producer, 1 MMA issuer, 2 idle, 3 scalars of the streamed rows, 4.. weights and epilogue (NBUF groups of
+// four, quadrant = warp % 4).  All waits are bounded.
 #include <cuda.h>
 #include <type_traits>
 
@@ -32,27 +45,38 @@ using namespace umma;
 
 constexpr int D = 64;
 constexpr int MT = 128;          // rows of the fixed tile (TMEM lanes)
-constexpr int NT = 64;           // rows of a streamed tile
-constexpr int NSTAGE = 4;
-constexpr int NBUF_MAX = 3;
-constexpr int NTHREADS = 384;
+constexpr int NSTAGE = 6;
 constexpr int WARP_BLD0 = 4;
 enum { MODE_DQ = 0, MODE_DKV = 1 };
 
-constexpr uint32_t COL_B = 0;      // score buffers of (G + 1) x 64 fp32 columns: [S_0 | .. | S_{G-1} | C] of a streamed tile
-                                   // (G feature groups; three buffers for G = 1, two for G = 2, one for G = 4); the
-                                   // bf16 weights overwrite columns [0,32) of each block
 constexpr uint32_t COL_ACC = 384;  // 2 x 64 fp32 accumulators
 constexpr uint32_t TMEM_COLS = 512;
 
-constexpr uint32_t OFF_X1 = 0;                     // fixed tiles: 128 x 64 bf16, 128B swizzle
-constexpr uint32_t OFF_X2 = 16384;
-constexpr uint32_t OFF_ST = 32768;                 // stages: two streamed tiles of 8 KB, then K' (MODE_DQ)
-constexpr uint32_t STAGE_BYTES = 24576;
-constexpr uint32_t OFF_SC = OFF_ST + NSTAGE * STAGE_BYTES;   // per stage 512 bytes of scalars of the 64 streamed rows:
+// G feature groups of the blockwise map: s_g = q_g . k_g per group, a = r sum_g s_g^2, e_g from s_g; dq and u are formed
+// group by group (N = 64 / G columns of the accumulator, the B operand offset into the 128-byte rows).
+template <int MODE, int G, int NS> struct Geo {
+  static constexpr int NT = G == 4 ? 32 : 64;               // rows of a streamed tile
+  static constexpr int NBUF = G == 1 && NS == 1 ? 3 : 2;    // score buffers = groups of weight warps
+  // a buffer: [S_0 | .. | S_{G-1} | C], NT fp32 columns each (and 64 more for the extra terms of the weights)
+  static constexpr uint32_t BW = NS == 3 ? 192u : (uint32_t)(G + 1) * NT;
+  static constexpr uint32_t CB = G * NT;                    // its C block
+  static constexpr int NTHREADS = 128 + NBUF * 128;
+  static_assert(NBUF * BW <= COL_ACC, "TMEM columns");
+  // first column of the bf16 weights inside the buffer (they overwrite scores that are already in registers)
+  __host__ __device__ static constexpr uint32_t p_col(int term) { return NS == 3 ? (term == 0 ? 0u : term == 1 ? 128u : 160u) : G == 1 ? 0u : CB; }
+  __host__ __device__ static constexpr uint32_t e_col(int g, int term) {
+    if (NS == 3) return MODE == MODE_DQ ? 64u * term : term == 0 ? 64u : term == 1 ? 32u : 96u;
+    return MODE == MODE_DKV && G == 1 ? CB : (uint32_t)g * NT;
+  }
+};
+
+constexpr uint32_t OFF_X = 0;                      // 2 x (two fixed tiles of 128 x 64 bf16, 128B swizzle): this and the next item
+constexpr uint32_t OFF_ST = 65536;                 // stages: two streamed tiles of up to 8 KB
+constexpr uint32_t STAGE_BYTES = 16384;
+constexpr uint32_t OFF_SC = OFF_ST + NSTAGE * STAGE_BYTES;   // per stage 512 bytes of scalars of the streamed rows:
                                                              // r_i (MODE_DQ) or (1/D_t, dout_t . o_t) (MODE_DKV)
-constexpr uint32_t OFF_PART = OFF_SC + NSTAGE * 512;         // 2 x 128 float2: the column halves of a row meet here
-constexpr uint32_t OFF_BAR = OFF_PART + 2048;
+constexpr uint32_t OFF_PART = OFF_SC + NSTAGE * 512;         // 2 (item parity) x 3 groups x 128 float2: the sums of a row meet here
+constexpr uint32_t OFF_BAR = OFF_PART + 6144;
 constexpr uint32_t SMEM_BYTES = OFF_BAR + 256;
 constexpr uint32_t SMEM_ALLOC = SMEM_BYTES + 1024;
 static_assert(SMEM_ALLOC > 116 * 1024, "one CTA per SM is assumed (the CTA allocates all of TMEM)");
@@ -60,15 +84,16 @@ static_assert(SMEM_ALLOC > 116 * 1024, "one CTA per SM is assumed (the CTA alloc
 // Every barrier has waiters that consume each of its phases in order; a producer of a phase always depends on the
 // waiter's progress (no barrier can complete two phases ahead of a waiter).
 enum {
-  BAR_XFULL = 0,     // fixed tiles landed
-  BAR_FULL = 1,      // [4] streamed tiles landed (TMA bytes + 32 producer lanes)
-  BAR_EMPTY = 5,     // [4] stage free: both issuers' commits
-  BAR_SFULL = 9,     // [3] scores in TMEM
-  BAR_PFULL = 12,    // [3] weights stored (256 threads)
-  BAR_PEMPTY = 15,   // [3] weights consumed: the buffer may take new scores
-  BAR_ODONE = 18,
-  BAR_DRAIN = 19,
-  BAR_COUNT = 20
+  BAR_XFULL = 0,     // [2] fixed tiles of an item landed
+  BAR_XEMPTY = 2,    // [2] ... and are no longer needed
+  BAR_FULL = 4,      // [NSTAGE] streamed tiles (TMA bytes) and their scalars landed
+  BAR_EMPTY = 10,    // [NSTAGE] stage free
+  BAR_SFULL = 16,    // [3] scores in TMEM
+  BAR_PFULL = 19,    // [3] weights stored (128 threads)
+  BAR_ODONE = 22,    // the accumulators of an item are complete
+  BAR_OFREE = 23,    // ... and have been read (256 threads)
+  BAR_DRAIN = 24,
+  BAR_COUNT = 25
 };
 
 struct BArgs {
@@ -78,63 +103,93 @@ struct BArgs {
   const float* rk;           // [BH][T]: 1 / ||k_i||^2
   int* device_status;
   int Tlen;
+  int BH;
 };
 
-// G feature groups of the blockwise map: s_g = q_g . k_g per group, a = r sum_g s_g^2, e_g = 2 g s_g; dq and u are
-// formed group by group (N = 64 / G columns of the accumulator, the B operand offset into the 128-byte rows).
-template <int MODE, int G>
-__global__ void __launch_bounds__(NTHREADS, 1)
+__device__ __forceinline__ float2 unpack_bf16(uint32_t x) {
+  return make_float2(__uint_as_float(x << 16), __uint_as_float(x & 0xFFFF0000u));
+}
+// v as the sum of NS pairs of bf16 (three: all 24 bits)
+template <int NS> __device__ __forceinline__ void split_pack(float2 v, uint32_t (&t)[NS]) {
+#pragma unroll
+  for (int i = 0; i < NS; ++i) {
+    t[i] = pack_bf16(v.x, v.y);
+    if (i + 1 < NS) {
+      const float2 u = unpack_bf16(t[i]);
+      v = __fadd2_rn(v, make_float2(-u.x, -u.y));
+    }
+  }
+}
+
+template <int MODE, int G, int NS>
+__global__ void __launch_bounds__(Geo<MODE, G, NS>::NTHREADS, 1)
 tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ CUtensorMap tmX2,
-              const __grid_constant__ CUtensorMap tmY1, const __grid_constant__ CUtensorMap tmY2,
-              const __grid_constant__ CUtensorMap tmY3, const BArgs args) {
+              const __grid_constant__ CUtensorMap tmY1, const __grid_constant__ CUtensorMap tmY2, const BArgs args) {
+  using geo = Geo<MODE, G, NS>;
+  constexpr int NT = geo::NT, NBUF = geo::NBUF;
+  constexpr uint32_t BW = geo::BW, CB = geo::CB;
+  constexpr int MG = D / G;                        // features per group
   extern __shared__ unsigned char smem_raw[];
   unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   auto bar = [&](int i) { return reinterpret_cast<uint64_t*>(base + OFF_BAR) + i; };
+  auto x1 = [&](int b) { return base + OFF_X + b * 32768; };
+  auto x2 = [&](int b) { return base + OFF_X + b * 32768 + 16384; };
   auto y1 = [&](int s) { return base + OFF_ST + s * STAGE_BYTES; };
   auto y2 = [&](int s) { return base + OFF_ST + s * STAGE_BYTES + 8192; };
-  auto y3 = [&](int s) { return base + OFF_ST + s * STAGE_BYTES + 16384; };
   auto sc = [&](int s) { return base + OFF_SC + s * 512; };
   __shared__ uint32_t tmem_base_s;
   __shared__ int abort_s;
   volatile int* abort_flag = &abort_s;
 
-  constexpr int NBUF = G == 1 ? 3 : G == 2 ? 2 : 1;
-  constexpr uint32_t BW = (G + 1) * 64;            // columns of a score buffer
-  constexpr uint32_t CB = G * 64;                  // its C block
-  constexpr int MG = D / G;                        // features per group
-  static_assert(NBUF * BW <= COL_ACC, "TMEM columns");
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int bh = blockIdx.y;
+  const int n_m = (args.Tlen + MT - 1) / MT;                      // fixed tiles of a head
   const int n_stream = (args.Tlen + NT - 1) / NT;                 // streamed tiles of the whole sequence
-  // MODE_DQ: heaviest (last) query tiles first, keys 0 .. m0 + 127;  MODE_DKV: key tile blockIdx.x (the first are
-  // the heaviest), queries m0 .. T - 1
-  const int mtile = MODE == MODE_DQ ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x;
-  const int m0 = mtile * MT;
-  const int jbeg = MODE == MODE_DQ ? 0 : 2 * mtile;
-  const int jend = MODE == MODE_DQ ? min(n_stream, 2 * mtile + 2) : n_stream;
-  const int ntiles = jend - jbeg;
-  const int nsteps = MODE == MODE_DQ ? 2 * ntiles : ntiles;       // MODE_DQ streams the keys twice
+  const long long n_items = (long long)args.BH * n_m;
+  struct Item {
+    int bh, m0;
+    int jbeg, ntiles;             // streamed tiles
+    int nsteps;                   // MODE_DQ streams the keys twice
+  };
+  // MODE_DQ: heaviest (last) query tiles first, keys 0 .. m0 + 127;  MODE_DKV: the first key tiles are the heaviest,
+  // queries m0 .. T - 1.  Rounds of gridDim.x items, dealt forwards and backwards in turn.
+  auto next_item = [&](int& n, Item& it) -> bool {   // the item at or after the n-th; n is left at it
+    for (;; ++n) {
+      if ((long long)n * gridDim.x >= n_items) return false;
+      const long long id = (long long)n * gridDim.x + ((n & 1) ? (int)gridDim.x - 1 - (int)blockIdx.x : (int)blockIdx.x);
+      if (id >= n_items) continue;
+      const int rank = (int)(id / args.BH), mtile = MODE == MODE_DQ ? n_m - 1 - rank : rank;
+      it.bh = (int)(id % args.BH);
+      it.m0 = mtile * MT;
+      it.jbeg = MODE == MODE_DQ ? 0 : mtile * (MT / NT);
+      const int jend = MODE == MODE_DQ ? min(n_stream, (mtile + 1) * (MT / NT)) : n_stream;
+      it.ntiles = jend - it.jbeg;
+      it.nsteps = MODE == MODE_DQ ? 2 * it.ntiles : it.ntiles;
+      return true;
+    }
+  };
 
   if (tid == 0) {
     abort_s = 0;
-    mbar_init(bar(BAR_XFULL), 1);
-    for (int i = 0; i < NSTAGE; ++i) {
-      mbar_init(bar(BAR_FULL + i), 1 + 32);
-      mbar_init(bar(BAR_EMPTY + i), 2);
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(bar(BAR_XFULL + i), 1);
+      mbar_init(bar(BAR_XEMPTY + i), MODE == MODE_DQ ? 1 : 1 + 256);
     }
-    for (int i = 0; i < NBUF_MAX; ++i) {
+    for (int i = 0; i < NSTAGE; ++i) {
+      mbar_init(bar(BAR_FULL + i), 2);
+      mbar_init(bar(BAR_EMPTY + i), 1);
+    }
+    for (int i = 0; i < NBUF; ++i) {
       mbar_init(bar(BAR_SFULL + i), 1);
-      mbar_init(bar(BAR_PFULL + i), 256);
-      mbar_init(bar(BAR_PEMPTY + i), 1);
+      mbar_init(bar(BAR_PFULL + i), 128);
     }
     mbar_init(bar(BAR_ODONE), 1);
-    mbar_init(bar(BAR_DRAIN), 2);
+    mbar_init(bar(BAR_OFREE), 256);
+    mbar_init(bar(BAR_DRAIN), 1);
     fence_mbar_init();
     tma_prefetch_desc(&tmX1);
     tma_prefetch_desc(&tmX2);
     tma_prefetch_desc(&tmY1);
     tma_prefetch_desc(&tmY2);
-    if (MODE == MODE_DQ) tma_prefetch_desc(&tmY3);
   }
   if (warp == 0) {
     tmem_alloc(&tmem_base_s, TMEM_COLS);
@@ -147,322 +202,345 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
   bool ok = true;
 
   if (warp == 0) {
-    // =========================== TMA producer (+ the scalars of the streamed queries) ===========================
-    if (lane == 0) {
-      mbar_arrive_expect_tx(bar(BAR_XFULL), 32768);
-      tma_load_3d(base + OFF_X1, &tmX1, bar(BAR_XFULL), 0, m0, bh);
-      tma_load_3d(base + OFF_X2, &tmX2, bar(BAR_XFULL), 0, m0, bh);
-    }
-    for (int j = 0; j < nsteps && ok; ++j) {
-      const int s = j % NSTAGE;
-      const int n0 = (jbeg + j % ntiles) * NT;
-      ok = wait_or_abort(bar(BAR_EMPTY + s), ((j / NSTAGE) & 1) ^ 1, abort_flag);
-      if (!ok) break;
-      if (lane == 0) {
-        mbar_arrive_expect_tx(bar(BAR_FULL + s), MODE == MODE_DQ ? 24576u : 16384u);
-        tma_load_3d(y1(s), &tmY1, bar(BAR_FULL + s), 0, n0, bh);
-        tma_load_3d(y2(s), &tmY2, bar(BAR_FULL + s), 0, n0, bh);
-        if (MODE == MODE_DQ) tma_load_3d(y3(s), &tmY3, bar(BAR_FULL + s), 0, n0, bh);
+    // =========================== TMA producer ===========================
+    if (elect_one()) {
+      uint32_t t = 0;
+      int ni = 0;
+      Item w;
+      for (int n = 0; ok && next_item(n, w); ++n, ++ni) {
+        const int xb = ni & 1;
+        ok = wait_or_abort(bar(BAR_XEMPTY + xb), ((ni >> 1) & 1) ^ 1, abort_flag);
+        if (!ok) break;
+        mbar_arrive_expect_tx(bar(BAR_XFULL + xb), 32768);
+        tma_load_3d(x1(xb), &tmX1, bar(BAR_XFULL + xb), 0, w.m0, w.bh);
+        tma_load_3d(x2(xb), &tmX2, bar(BAR_XFULL + xb), 0, w.m0, w.bh);
+        for (int j = 0, jt = 0; j < w.nsteps && ok; ++j, ++t) {
+          const int s = t % NSTAGE;
+          ok = wait_or_abort(bar(BAR_EMPTY + s), ((t / NSTAGE) & 1) ^ 1, abort_flag);
+          if (!ok) break;
+          mbar_arrive_expect_tx(bar(BAR_FULL + s), 2 * NT * 128);
+          tma_load_3d(y1(s), &tmY1, bar(BAR_FULL + s), 0, (w.jbeg + jt) * NT, w.bh);
+          tma_load_3d(y2(s), &tmY2, bar(BAR_FULL + s), 0, (w.jbeg + jt) * NT, w.bh);
+          if (++jt == w.ntiles) jt = 0;
+        }
       }
-      const int t = n0 + 2 * lane;                       // two streamed rows per lane
-      if (MODE == MODE_DKV) {
-        // (1 / D_t, dout_t . o_t) of the 64 streamed queries
-        float4 st = make_float4(0.f, 0.f, 0.f, 0.f);
-        const float* src = args.stats + ((size_t)bh * args.Tlen + t) * 2;
-        if (t < args.Tlen) { st.x = src[0]; st.y = src[1]; }
-        if (t + 1 < args.Tlen) { st.z = src[2]; st.w = src[3]; }
-        *reinterpret_cast<float4*>(sc(s) + lane * 16) = st;
-      } else {
-        // r_i of the 64 streamed keys
-        float2 r2 = make_float2(0.f, 0.f);
-        const float* src = args.rk + (size_t)bh * args.Tlen + t;
-        if (t < args.Tlen) r2.x = src[0];
-        if (t + 1 < args.Tlen) r2.y = src[1];
-        *reinterpret_cast<float2*>(sc(s) + lane * 8) = r2;
-      }
-      mbar_arrive(bar(BAR_FULL + s));
     }
   } else if (warp == 1) {
-    // =========================== score MMA issuer: [S | C] ===========================
+    // =========================== MMA issuer ===========================
     if (elect_one()) {
-      const uint32_t idesc = instr_desc(kFmtBF16, kFmtBF16, 0, 0, 128, 64);
+      const uint32_t id_s = instr_desc(kFmtBF16, kFmtBF16, 0, 0, 128, NT);      // scores: both K-major
+      const uint32_t id_o = instr_desc(kFmtBF16, kFmtBF16, 0, 1, 128, 64);      // dv~: A tmem, B MN-major
+      const uint32_t id_g = instr_desc(kFmtBF16, kFmtBF16, 0, 1, 128, MG);      // dq, u of a feature group
       const uint64_t dk = smem_desc(0, 16, 1024, kSwizzle128B);
-      const uint32_t x1 = smem_u32(base + OFF_X1), x2 = smem_u32(base + OFF_X2);
-      ok = wait_or_abort(bar(BAR_XFULL), 0, abort_flag);
-      for (int j = 0; j < nsteps && ok; ++j) {
-        const int s = j % NSTAGE, b = j % NBUF;
-        ok = wait_or_abort(bar(BAR_FULL + s), (j / NSTAGE) & 1, abort_flag) &&
-             wait_or_abort(bar(BAR_PEMPTY + b), ((j / NBUF) & 1) ^ 1, abort_flag);
-        if (!ok) break;
+      const uint64_t dmn = smem_desc(0, 8192, 1024, kSwizzle128B);              // 8 streamed rows x 64 columns per 1 KB atom
+      // opening side: scores of the steps, NBUF ahead of the closing side, across items
+      Item wo;
+      int no = 0, jo = 0, io = 0;
+      uint32_t t_open = 0;
+      bool mo = next_item(no, wo);
+      auto open = [&]() -> bool {
+        if (!mo) return true;
+        const int s = t_open % NSTAGE, b = t_open % NBUF, xb = io & 1;
+        if (jo == 0 && !wait_or_abort(bar(BAR_XFULL + xb), (io >> 1) & 1, abort_flag)) return false;
+        if (!wait_or_abort(bar(BAR_FULL + s), (t_open / NSTAGE) & 1, abort_flag)) return false;
         tc_fence_after();
-        const uint32_t a1 = smem_u32(y1(s)), a2 = smem_u32(y2(s));
+        const uint32_t f1 = smem_u32(x1(xb)), f2 = smem_u32(x2(xb)), a1 = smem_u32(y1(s)), a2 = smem_u32(y2(s));
 #pragma unroll
-        for (int ks = 0; ks < 4; ++ks)      // 16 features per step; group ks / (4 / G) has its own 64 score columns
-          mma_f16_ss(tb + COL_B + b * BW + (ks / (4 / G)) * 64, at(dk, x1 + ks * 32), at(dk, a1 + ks * 32), idesc,
-                     (ks % (4 / G)) > 0);
+        for (int ks = 0; ks < 4; ++ks)      // 16 features per step; group ks / (4 / G) has its own NT score columns
+          mma_f16_ss(tb + b * BW + (ks / (4 / G)) * NT, at(dk, f1 + ks * 32), at(dk, a1 + ks * 32), id_s, (ks % (4 / G)) > 0);
 #pragma unroll
         for (int ks = 0; ks < 4; ++ks)
-          mma_f16_ss(tb + COL_B + b * BW + CB, at(dk, x2 + ks * 32), at(dk, a2 + ks * 32), idesc, ks > 0);
+          mma_f16_ss(tb + b * BW + CB, at(dk, f2 + ks * 32), at(dk, a2 + ks * 32), id_s, ks > 0);
         mma_commit(bar(BAR_SFULL + b));
-        mma_commit(bar(BAR_EMPTY + s));
-      }
-    }
-  } else if (warp == 2) {
-    // =========================== output MMA issuer ===========================
-    if (elect_one()) {
-      const uint32_t idesc = instr_desc(kFmtBF16, kFmtBF16, 0, 1, 128, 64);     // A tmem, B MN-major
-      // MN-major, 128B swizzle: 8 streamed rows x 64 columns per 1 KB atom (SBO); 16 rows per MMA
-      const uint64_t dmn = smem_desc(0, 8192, 1024, kSwizzle128B);
-      for (int j = 0; j < nsteps && ok; ++j) {
-        const int s = j % NSTAGE, b = j % NBUF;
-        ok = wait_or_abort(bar(BAR_FULL + s), (j / NSTAGE) & 1, abort_flag) &&
-             wait_or_abort(bar(BAR_PFULL + b), (j / NBUF) & 1, abort_flag);
-        if (!ok) break;
-        tc_fence_after();
-        // group g: N = 64 / G accumulator columns, the B operand starts 2 * 64 / G bytes further into the rows
-        const uint32_t idg = instr_desc(kFmtBF16, kFmtBF16, 0, 1, 128, MG);
-        if (MODE == MODE_DQ) {
-          if (j >= ntiles) {      // the first sweep only sums the row scalars: nothing to multiply
-            const uint32_t kp = smem_u32(y3(s));
+        ++t_open;
+        if (++jo == wo.nsteps) {
+          jo = 0;
+          ++no;
+          ++io;
+          mo = next_item(no, wo);
+        }
+        return true;
+      };
+      for (int i = 0; i < NBUF && ok; ++i) ok = open();
+      uint32_t t = 0;
+      int ni = 0;
+      Item w;
+      for (int n = 0; ok && next_item(n, w); ++n, ++ni) {
+        uint32_t acc = 0;
+        for (int j = 0; j < w.nsteps && ok; ++j, ++t) {
+          const int s = t % NSTAGE, b = t % NBUF;
+          ok = wait_or_abort(bar(BAR_PFULL + b), (t / NBUF) & 1, abort_flag);
+          // the accumulators are free once the epilogue of the item before has read them
+          if (ok && j == (MODE == MODE_DQ ? w.ntiles : 0) && ni > 0) ok = wait_or_abort(bar(BAR_OFREE), (ni - 1) & 1, abort_flag);
+          if (!ok) break;
+          if (MODE == MODE_DKV || j >= w.ntiles) {       // (the first sweep of MODE_DQ only sums the row scalars)
+            tc_fence_after();
+            const uint32_t buf = tb + b * BW, ya = smem_u32(y1(s)), yb = smem_u32(y2(s));
+            if (MODE == MODE_DKV) {
+#pragma unroll
+              for (int term = 0; term < NS; ++term)
+#pragma unroll
+                for (int ks = 0; ks < NT / 16; ++ks)      // dv~ += P^T dout
+                  mma_f16_ts(tb + COL_ACC, buf + geo::p_col(term) + ks * 8, at(dmn, yb + ks * 2048), id_o, (acc || term > 0 || ks > 0) ? 1u : 0u);
+            }
+            constexpr uint32_t col = COL_ACC + (MODE == MODE_DKV ? 64 : 0);
 #pragma unroll
             for (int g = 0; g < G; ++g)
 #pragma unroll
-              for (int ks = 0; ks < 4; ++ks)
-                mma_f16_ts(tb + COL_ACC + g * MG, tb + COL_B + b * BW + g * 64 + ks * 8,
-                           at(dmn, kp + ks * 2048 + g * MG * 2), idg, (j > ntiles || ks > 0) ? 1u : 0u);
+              for (int term = 0; term < NS; ++term)
+#pragma unroll
+                for (int ks = 0; ks < NT / 16; ++ks)      // dq += E K, u += E^T Q
+                  mma_f16_ts(tb + col + g * MG, buf + geo::e_col(g, term) + ks * 8, at(dmn, ya + ks * 2048 + g * MG * 2), id_g,
+                             (acc || term > 0 || ks > 0) ? 1u : 0u);
+            acc = 1;
           }
-        } else {
-          const uint32_t qa = smem_u32(y1(s)), ga = smem_u32(y2(s));
-          // P^T sits over the first score block for G = 1 and over the C block otherwise; E_g^T over the other / its own
-          const uint32_t pcol = G == 1 ? 0u : CB;
-#pragma unroll
-          for (int ks = 0; ks < 4; ++ks)      // dv~ += P^T dout
-            mma_f16_ts(tb + COL_ACC, tb + COL_B + b * BW + pcol + ks * 8, at(dmn, ga + ks * 2048), idesc, (j > 0 || ks > 0) ? 1u : 0u);
-#pragma unroll
-          for (int g = 0; g < G; ++g)
-#pragma unroll
-            for (int ks = 0; ks < 4; ++ks)    // u_g += E_g^T Q_g
-              mma_f16_ts(tb + COL_ACC + 64 + g * MG, tb + COL_B + b * BW + (G == 1 ? 64u : (uint32_t)g * 64u) + ks * 8,
-                         at(dmn, qa + ks * 2048 + g * MG * 2), idg, (j > 0 || ks > 0) ? 1u : 0u);
+          mma_commit(bar(BAR_EMPTY + s));
+          if (j + 1 == w.nsteps) {
+            mma_commit(bar(BAR_ODONE));
+            mma_commit(bar(BAR_XEMPTY + (ni & 1)));
+          }
+          ok = open();
         }
-        mma_commit(bar(BAR_PEMPTY + b));
-        mma_commit(bar(BAR_EMPTY + s));
       }
-      if (ok) mma_commit(bar(BAR_ODONE));
     }
+  } else if (warp == 3) {
+    // =========================== scalars of the streamed rows, two tiles ahead ===========================
+    // A programmatic dependent launch: only this warp reads what the kernel before it wrote.
+    cudaGridDependencySynchronize();
+    constexpr int RPL = NT / 32;                       // rows per lane
+    constexpr int FPR = MODE == MODE_DQ ? 1 : 2;       // floats per row
+    const float* src = MODE == MODE_DQ ? args.rk : args.stats;
+    Item wl, w;
+    int nl = 0, jl = 0;
+    bool ml = next_item(nl, wl);
+    auto fetch = [&](float (&v)[RPL * FPR]) {
+#pragma unroll
+      for (int e = 0; e < RPL; ++e) {
+        const int row = (wl.jbeg + (jl >= wl.ntiles ? jl - wl.ntiles : jl)) * NT + lane * RPL + e;
+        const bool in = ml && row < args.Tlen;
+#pragma unroll
+        for (int f = 0; f < FPR; ++f) v[e * FPR + f] = in ? src[((size_t)wl.bh * args.Tlen + row) * FPR + f] : 0.f;
+      }
+      if (ml && ++jl == wl.nsteps) {
+        jl = 0;
+        ++nl;
+        ml = next_item(nl, wl);
+      }
+    };
+    float v0[RPL * FPR], v1[RPL * FPR], v2[RPL * FPR];
+    fetch(v0);
+    fetch(v1);
+    uint32_t t = 0;
+    for (int n = 0; ok && next_item(n, w); ++n)
+      for (int j = 0; j < w.nsteps && ok; ++j, ++t) {
+        const int s = t % NSTAGE;
+        fetch(v2);
+        ok = wait_or_abort(bar(BAR_EMPTY + s), ((t / NSTAGE) & 1) ^ 1, abort_flag);
+        if (!ok) break;
+#pragma unroll
+        for (int e = 0; e < RPL * FPR; ++e) {
+          reinterpret_cast<float*>(sc(s))[lane * RPL * FPR + e] = v0[e];
+          v0[e] = v1[e];
+          v1[e] = v2[e];
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(BAR_FULL + s));
+      }
   } else if (warp >= WARP_BLD0) {
-    // =========================== weights and epilogue (256 threads) ===========================
+    // =========================== weights and epilogue (NBUF groups of 128 threads) ===========================
     const uint32_t q4 = warp & 3;
-    const int ch = (warp - WARP_BLD0) >> 2;      // column half: streamed rows [32 ch, 32 ch + 32) of the tile
+    const int grp = (warp - WARP_BLD0) >> 2;     // this group's buffer: the steps t with t % NBUF = grp
     const int rowl = q4 * 32 + lane;             // row of the fixed tile (= TMEM lane)
-    const int grow = m0 + rowl;
-    float inv_row = 0.f, del_row = 0.f;          // MODE_DQ: the scalars of this query (1 / D_t, dout_t . o_t)
-    float sum_d = 0.f, sum_m = 0.f;              // MODE_DQ, first sweep: this warp's share of D_t and of sum a c
-    float2* part = reinterpret_cast<float2*>(base + OFF_PART);
-    for (int j = 0; j < nsteps && ok; ++j) {
-      const int s = j % NSTAGE, b = j % NBUF;
-      const int n0 = (jbeg + j % ntiles) * NT + ch * 32;   // first streamed row of this warp's columns
-      if (MODE == MODE_DQ && j == ntiles) {
-        // between the sweeps: the two column halves of a row meet, the scalars go to registers and to the workspace
-        part[ch * MT + rowl] = make_float2(sum_d, sum_m);
-        asm volatile("bar.sync %0, 64;" ::"r"(1 + (int)q4) : "memory");
-        const float2 other = part[(1 - ch) * MT + rowl];
-        const float dt = ch == 0 ? sum_d + other.x : other.x + sum_d;      // fixed order of the halves
-        const float mt = ch == 0 ? sum_m + other.y : other.y + sum_m;
+    const uint32_t buf = tmem_addr(tb, q4 * 32, grp * BW), accu = tmem_addr(tb, q4 * 32, COL_ACC);
+    uint32_t t0 = 0;                             // steps of the items before
+    int ni = 0;
+    Item w;
+    for (int n = 0; ok && next_item(n, w); ++n, ++ni) {
+      const int grow = w.m0 + rowl;
+      float inv_row = 0.f, del_row = 0.f;        // MODE_DQ: the scalars of this query (1 / D_t, dout_t . o_t)
+      int j = (grp + NBUF - (int)(t0 % NBUF)) % NBUF;
+      auto begin = [&](uint32_t t) -> bool {
+        if (!wait_or_abort(bar(BAR_SFULL + grp), (t / NBUF) & 1, abort_flag)) return false;
+        tc_fence_after();
+        return true;
+      };
+      auto end = [&]() {
+        tc_fence_before();
+        mbar_arrive(bar(BAR_PFULL + grp));
+      };
+      if (MODE == MODE_DQ) {
+        // ---- first sweep: a = r_i sum_g s_g^2 for the keys n <= this query; D_t += a, sum += a c ----
+        float sum_d = 0.f, sum_m = 0.f;
+        for (; j < w.ntiles && ok; j += NBUF) {
+          ok = begin(t0 + j);
+          if (!ok) break;
+          const int s = (t0 + j) % NSTAGE;
+#pragma unroll 1
+          for (int ch = 0; ch < NT / 32; ++ch) {
+            const int n0 = (w.jbeg + j) * NT + ch * 32;
+            const float2* cs = reinterpret_cast<const float2*>(sc(s) + ch * 128);
+            uint32_t cv[32], sv[32];
+            float2 ss[16];
+            tmem_ld32(buf + ch * 32, sv);
+            tmem_ld32(buf + CB + ch * 32, cv);
+            tmem_wait_ld(sv);
+            tmem_wait_ld(cv);
+#pragma unroll
+            for (int g = 0; g < G; ++g) {
+              if (g > 0) {
+                tmem_ld32(buf + g * NT + ch * 32, sv);
+                tmem_wait_ld(sv);
+              }
+#pragma unroll
+              for (int c = 0; c < 32; c += 2) {
+                const float2 s2 = make_float2(__uint_as_float(sv[c]), __uint_as_float(sv[c + 1]));
+                ss[c / 2] = g == 0 ? __fmul2_rn(s2, s2) : __ffma2_rn(s2, s2, ss[c / 2]);
+              }
+            }
+            float2 d2 = make_float2(0.f, 0.f), m2 = make_float2(0.f, 0.f);
+            // two copies of the loop, chosen once per tile: the causal test exists on diagonal tiles only
+            auto sums = [&](auto masked) {
+#pragma unroll
+              for (int c = 0; c < 32; c += 2) {
+                float2 a2 = __fmul2_rn(ss[c / 2], cs[c / 2]);
+                if constexpr (decltype(masked)::value) {
+                  if (n0 + c > grow) a2.x = 0.f;
+                  if (n0 + c + 1 > grow) a2.y = 0.f;
+                }
+                d2 = __fadd2_rn(d2, a2);
+                m2 = __ffma2_rn(a2, make_float2(__uint_as_float(cv[c]), __uint_as_float(cv[c + 1])), m2);
+              }
+            };
+            if (n0 + 31 > w.m0) sums(std::true_type{}); else sums(std::false_type{});
+            sum_d += d2.x + d2.y;
+            sum_m += m2.x + m2.y;
+          }
+          end();                                 // nothing is stored; the buffer is handed on as it is
+        }
+        if (!ok) break;
+        // the groups' shares of a row meet, in a fixed order
+        float2* part = reinterpret_cast<float2*>(base + OFF_PART) + (ni & 1) * 384 + rowl;
+        part[grp * MT] = make_float2(sum_d, sum_m);
+        asm volatile("bar.sync 1, %0;" ::"n"(NBUF * 128) : "memory");
+        float dt = 0.f, mt = 0.f;
+#pragma unroll
+        for (int g = 0; g < NBUF; ++g) {
+          dt += part[g * MT].x;
+          mt += part[g * MT].y;
+        }
         inv_row = dt > 0.f ? 1.f / dt : 0.f;
         del_row = mt * inv_row;
-        if (ch == 0 && grow < args.Tlen)
-          *reinterpret_cast<float2*>(args.stats + ((size_t)bh * args.Tlen + grow) * 2) = make_float2(inv_row, del_row);
+        if (grp == 0 && grow < args.Tlen)
+          *reinterpret_cast<float2*>(args.stats + ((size_t)w.bh * args.Tlen + grow) * 2) = make_float2(inv_row, del_row);
       }
-      ok = wait_or_abort(bar(BAR_FULL + s), (j / NSTAGE) & 1, abort_flag) &&     // the column scalars are in the stage
-           wait_or_abort(bar(BAR_SFULL + b), (j / NBUF) & 1, abort_flag);
-      if (!ok) break;
-      tc_fence_after();
-      if constexpr (G > 1) {
-        // one block of 64 score columns per group, then the C block; this warp's 32 columns of each
-        const uint32_t bcol = tmem_addr(tb, q4 * 32, COL_B + b * BW + ch * 32);
-        uint32_t cvg[32], sg[32], pk[16];
-        tmem_ld32(bcol + CB, cvg);
-        tmem_wait_ld(cvg);
-        const bool first = MODE == MODE_DQ && j < ntiles;
-        const bool diag = MODE == MODE_DQ ? (n0 + 31 > m0) : (n0 < m0 + MT - 1);
-        auto dead = [&](int c) { return MODE == MODE_DQ ? (n0 + c > grow) : (n0 + c < grow); };
-        float2 cf[16], ss[16];
-        // two copies of each loop with a causal test, chosen once per tile: the test exists on diagonal tiles only
-        auto factors = [&](auto masked) {
+      // ---- weights ----
+      for (; j < w.nsteps && ok; j += NBUF) {
+        ok = begin(t0 + j);
+        if (!ok) break;
+        const int s = (t0 + j) % NSTAGE;
+        const int jt = MODE == MODE_DQ ? j - w.ntiles : j;
+        uint32_t held[NS == 3 && MODE == MODE_DKV ? 32 : 1];       // the second and third terms of E of the first chunk
 #pragma unroll
-          for (int c = 0; c < 32; c += 2) {
-            const float2 c2 = make_float2(__uint_as_float(cvg[c]), __uint_as_float(cvg[c + 1]));
-            if (MODE == MODE_DQ) {
-              // second sweep: 2 (c - dout.o) / D; first sweep: c as it is
-              cf[c / 2] = first ? c2 : __fmul2_rn(__fadd2_rn(c2, make_float2(-del_row, -del_row)), make_float2(2.f * inv_row, 2.f * inv_row));
-            } else {
-              const float4 st = reinterpret_cast<const float4*>(sc(s) + ch * 256)[c / 2];
-              cf[c / 2] = __fmul2_rn(__fadd2_rn(c2, make_float2(-st.y, -st.w)), make_float2(2.f * st.x, 2.f * st.z));
+        for (int ch = 0; ch < NT / 32; ++ch) {
+          const int n0 = (w.jbeg + jt) * NT + ch * 32;
+          auto dead = [&](int c) { return MODE == MODE_DQ ? n0 + c > grow : n0 + c < grow; };
+          const bool diag = MODE == MODE_DQ ? n0 + 31 > w.m0 : n0 < w.m0 + MT - 1;
+          uint32_t cv[32], sv[32];
+          tmem_ld32(buf + ch * 32, sv);
+          tmem_ld32(buf + CB + ch * 32, cv);
+          tmem_wait_ld(sv);
+          tmem_wait_ld(cv);
+          if constexpr (NS == 3 && MODE == MODE_DKV) {
+            if (ch == 1) {                       // the columns of the second chunk's scores are free now
+              const uint32_t (&e1)[16] = *reinterpret_cast<const uint32_t (*)[16]>(&held[0]);
+              const uint32_t (&e2)[16] = *reinterpret_cast<const uint32_t (*)[16]>(&held[16]);
+              tmem_st16(buf + geo::e_col(0, 1), e1);
+              tmem_st16(buf + geo::e_col(0, 2), e2);
             }
-            if constexpr (decltype(masked)::value) {
-              if (dead(c)) cf[c / 2].x = 0.f;
-              if (dead(c + 1)) cf[c / 2].y = 0.f;
-            }
-            ss[c / 2] = make_float2(0.f, 0.f);
           }
-        };
-        if (diag && !first) factors(std::true_type{}); else factors(std::false_type{});
-#pragma unroll 1
-        for (int g = 0; g < G; ++g) {
-          tmem_ld32(bcol + g * 64, sg);
-          tmem_wait_ld(sg);
-#pragma unroll
-          for (int c = 0; c < 32; c += 2) {
-            const float2 s2 = make_float2(__uint_as_float(sg[c]), __uint_as_float(sg[c + 1]));
-            ss[c / 2] = __ffma2_rn(s2, s2, ss[c / 2]);
-            const float2 e2 = __fmul2_rn(cf[c / 2], s2);
-            pk[c / 2] = pack_bf16(e2.x, e2.y);
-          }
-          if (first) continue;
-          // E_g goes over columns [0,32) of its own block, which the column-half-0 warp reads
-          tc_fence_before();
-          asm volatile("bar.sync %0, 64;" ::"r"(1 + (int)q4) : "memory");
-          tc_fence_after();
-          tmem_st16(tmem_addr(tb, q4 * 32, COL_B + b * BW + g * 64 + ch * 16), pk);
-        }
-        if (first) {
-          // a = r_i sum_g s_g^2 for the keys n <= this query; D_t += a, sum += a c
-          const float2* cs = reinterpret_cast<const float2*>(sc(s) + ch * 128);
-          float2 d2 = make_float2(0.f, 0.f), m2 = make_float2(0.f, 0.f);
-          auto sums = [&](auto masked) {
+          // f: e = f s.  MODE_DQ: (c - dout.o) r;  MODE_DKV: (c - dout_t.o_t) / D_t;  over c in place
+          auto factors = [&](auto masked) {
 #pragma unroll
             for (int c = 0; c < 32; c += 2) {
-              float2 a2 = __fmul2_rn(ss[c / 2], cs[c / 2]);
-              if constexpr (decltype(masked)::value) {
-                if (dead(c)) a2.x = 0.f;
-                if (dead(c + 1)) a2.y = 0.f;
+              const float2 c2 = make_float2(__uint_as_float(cv[c]), __uint_as_float(cv[c + 1]));
+              float2 f;
+              if (MODE == MODE_DQ) {
+                f = __fmul2_rn(__fadd2_rn(c2, make_float2(-del_row, -del_row)), reinterpret_cast<const float2*>(sc(s) + ch * 128)[c / 2]);
+              } else {
+                const float4 st = reinterpret_cast<const float4*>(sc(s) + ch * 256)[c / 2];     // (1/D, dout.o) of two queries
+                f = __fmul2_rn(__fadd2_rn(c2, make_float2(-st.y, -st.w)), make_float2(st.x, st.z));
               }
-              d2 = __fadd2_rn(d2, a2);
-              m2 = __ffma2_rn(a2, cf[c / 2], m2);
+              if constexpr (decltype(masked)::value) {
+                if (dead(c)) f.x = 0.f;
+                if (dead(c + 1)) f.y = 0.f;
+              }
+              cv[c] = __float_as_uint(f.x);
+              cv[c + 1] = __float_as_uint(f.y);
             }
           };
-          if (diag) sums(std::true_type{}); else sums(std::false_type{});
-          sum_d += d2.x + d2.y;
-          sum_m += m2.x + m2.y;
-        } else if (MODE == MODE_DKV) {
-          // P^T = sum_g s_g^2 / D_t over the C block (both warps of the quadrant hold its scores since the first sync)
-          auto weights = [&](auto masked) {
+          if (diag) factors(std::true_type{}); else factors(std::false_type{});
+          float2 ss[MODE == MODE_DKV && G > 1 ? 16 : 1];
+#pragma unroll
+          for (int g = 0; g < G; ++g) {
+            if (g > 0) {
+              tmem_ld32(buf + g * NT + ch * 32, sv);
+              tmem_wait_ld(sv);
+            }
+            uint32_t pk[NS][16];
 #pragma unroll
             for (int c = 0; c < 32; c += 2) {
-              const float4 st = reinterpret_cast<const float4*>(sc(s) + ch * 256)[c / 2];
-              float2 p2 = __fmul2_rn(ss[c / 2], make_float2(st.x, st.z));
-              if constexpr (decltype(masked)::value) {
-                if (dead(c)) p2.x = 0.f;
-                if (dead(c + 1)) p2.y = 0.f;
-              }
-              pk[c / 2] = pack_bf16(p2.x, p2.y);
+              const float2 s2 = make_float2(__uint_as_float(sv[c]), __uint_as_float(sv[c + 1]));
+              if constexpr (MODE == MODE_DKV && G > 1) ss[c / 2] = g == 0 ? __fmul2_rn(s2, s2) : __ffma2_rn(s2, s2, ss[c / 2]);
+              uint32_t term[NS];
+              split_pack<NS>(__fmul2_rn(make_float2(__uint_as_float(cv[c]), __uint_as_float(cv[c + 1])), s2), term);
+#pragma unroll
+              for (int i = 0; i < NS; ++i) pk[i][c / 2] = term[i];
             }
-          };
-          if (diag) weights(std::true_type{}); else weights(std::false_type{});
-          tmem_st16(tmem_addr(tb, q4 * 32, COL_B + b * BW + CB + ch * 16), pk);
+#pragma unroll
+            for (int i = 0; i < NS; ++i) {
+              if (NS == 3 && MODE == MODE_DKV && ch == 0 && i > 0) {
+#pragma unroll
+                for (int e = 0; e < 16; ++e) held[NS == 3 && MODE == MODE_DKV ? (i - 1) * 16 + e : 0] = pk[i][e];
+              } else {
+                tmem_st16(buf + geo::e_col(g, i) + ch * 16, pk[i]);
+              }
+            }
+          }
+          if (MODE == MODE_DKV) {
+            // p = sum_g s_g^2 / D_t
+            uint32_t pk[NS][16];
+            auto weights = [&](auto masked) {
+#pragma unroll
+              for (int c = 0; c < 32; c += 2) {
+                const float4 st = reinterpret_cast<const float4*>(sc(s) + ch * 256)[c / 2];
+                const float2 s2 = make_float2(__uint_as_float(sv[c]), __uint_as_float(sv[c + 1]));
+                float2 p2 = __fmul2_rn(G > 1 ? ss[MODE == MODE_DKV && G > 1 ? c / 2 : 0] : __fmul2_rn(s2, s2), make_float2(st.x, st.z));
+                if constexpr (decltype(masked)::value) {
+                  if (dead(c)) p2.x = 0.f;
+                  if (dead(c + 1)) p2.y = 0.f;
+                }
+                uint32_t term[NS];
+                split_pack<NS>(p2, term);
+#pragma unroll
+                for (int i = 0; i < NS; ++i) pk[i][c / 2] = term[i];
+              }
+            };
+            if (diag) weights(std::true_type{}); else weights(std::false_type{});
+#pragma unroll
+            for (int i = 0; i < NS; ++i) tmem_st16(buf + geo::p_col(i) + ch * 16, pk[i]);
+          }
         }
         tmem_wait_st();
-        tc_fence_before();
-        mbar_arrive(bar(BAR_PFULL + b));
-        continue;
+        end();
       }
-      const uint32_t scol = tmem_addr(tb, q4 * 32, COL_B + b * 128 + ch * 32);
-      uint32_t sv[32], cv[32], pe[16], pp[16];
-      tmem_ld32(scol, sv);
-      tmem_ld32(scol + 64, cv);
-      tmem_wait_ld(sv);
-      tmem_wait_ld(cv);
-      if (MODE == MODE_DQ && j < ntiles) {
-        // first sweep: a = r_i s^2 for the keys n <= this query; D_t += a, sum += a c
-        const float2* cs = reinterpret_cast<const float2*>(sc(s) + ch * 128);
-        const bool diag = n0 + 31 > m0;                 // some key of these columns lies after some query of the tile
-        float2 d2 = make_float2(0.f, 0.f), m2 = make_float2(0.f, 0.f);
-        // two copies of the loop, chosen once per tile: the causal test exists on diagonal tiles only
-        auto sums = [&](auto masked) {
-#pragma unroll
-          for (int c = 0; c < 32; c += 2) {
-            const float2 s2 = make_float2(__uint_as_float(sv[c]), __uint_as_float(sv[c + 1]));
-            float2 a2 = __fmul2_rn(__fmul2_rn(s2, s2), cs[c / 2]);
-            if constexpr (decltype(masked)::value) {
-              if (n0 + c > grow) a2.x = 0.f;
-              if (n0 + c + 1 > grow) a2.y = 0.f;
-            }
-            d2 = __fadd2_rn(d2, a2);
-            m2 = __ffma2_rn(a2, make_float2(__uint_as_float(cv[c]), __uint_as_float(cv[c + 1])), m2);
-          }
-        };
-        if (diag) sums(std::true_type{}); else sums(std::false_type{});
-        sum_d += d2.x + d2.y;
-        sum_m += m2.x + m2.y;
-        // nothing is stored; the buffer is handed on as it is
-        tc_fence_before();
-        mbar_arrive(bar(BAR_PFULL + b));
-        continue;
-      }
-      if (MODE == MODE_DQ) {
-        // e = 2 (c - dout.o) / D * s, keys n <= this query
-        const float2 f2 = make_float2(2.f * inv_row, 2.f * inv_row), nd2 = make_float2(-del_row, -del_row);
-        const bool diag = n0 + 31 > m0;
-        auto weigh = [&](auto masked) {
-#pragma unroll
-          for (int c = 0; c < 32; c += 2) {
-            const float2 s2 = make_float2(__uint_as_float(sv[c]), __uint_as_float(sv[c + 1]));
-            const float2 c2 = make_float2(__uint_as_float(cv[c]), __uint_as_float(cv[c + 1]));
-            float2 e2 = __fmul2_rn(__fmul2_rn(__fadd2_rn(c2, nd2), f2), s2);
-            if constexpr (decltype(masked)::value) {
-              if (n0 + c > grow) e2.x = 0.f;
-              if (n0 + c + 1 > grow) e2.y = 0.f;
-            }
-            pe[c / 2] = pack_bf16(e2.x, e2.y);
-          }
-        };
-        if (diag) weigh(std::true_type{}); else weigh(std::false_type{});
-      } else {
-        // p = s^2 / D_t, e = 2 (c - dout_t.o_t) / D_t * s with the scalars of the columns (queries t >= this key)
-        const float4* cs = reinterpret_cast<const float4*>(sc(s) + ch * 256);
-        const bool diag = n0 < m0 + MT - 1;             // some query of these columns lies before some key of the tile
-        auto weigh = [&](auto masked) {
-#pragma unroll
-          for (int c = 0; c < 32; c += 2) {
-            const float4 st = cs[c / 2];                       // (1/D, dout.o) of queries n0 + c, n0 + c + 1
-            const float2 s2 = make_float2(__uint_as_float(sv[c]), __uint_as_float(sv[c + 1]));
-            const float2 c2 = make_float2(__uint_as_float(cv[c]), __uint_as_float(cv[c + 1]));
-            const float2 t2 = __fmul2_rn(s2, make_float2(st.x, st.z));                    // s / D
-            float2 p2 = __fmul2_rn(t2, s2);                                               // s^2 / D
-            float2 e2 = __fmul2_rn(__fadd2_rn(c2, make_float2(-st.y, -st.w)), __fadd2_rn(t2, t2));
-            if constexpr (decltype(masked)::value) {
-              if (n0 + c < grow) { p2.x = 0.f; e2.x = 0.f; }
-              if (n0 + c + 1 < grow) { p2.y = 0.f; e2.y = 0.f; }
-            }
-            pp[c / 2] = pack_bf16(p2.x, p2.y);
-            pe[c / 2] = pack_bf16(e2.x, e2.y);
-          }
-        };
-        if (diag) weigh(std::true_type{}); else weigh(std::false_type{});
-      }
-      // the weights overwrite score columns [0,32) of each half, which the column-half-0 warp of this quadrant
-      // reads: both warps of the quadrant must have their scores in registers first
-      tc_fence_before();
-      asm volatile("bar.sync %0, 64;" ::"r"(1 + (int)q4) : "memory");
+      t0 += w.nsteps;
+      if (!ok) break;
+      if (grp > 1) continue;
+      // ---- epilogue: groups 0 and 1 ----
+      ok = wait_or_abort(bar(BAR_ODONE), ni & 1, abort_flag) &&
+           (MODE == MODE_DQ || wait_or_abort(bar(BAR_XFULL + (ni & 1)), (ni >> 1) & 1, abort_flag));   // (k is read below)
+      if (!ok) break;
       tc_fence_after();
-      if (MODE == MODE_DQ) {
-        tmem_st16(tmem_addr(tb, q4 * 32, COL_B + b * 128 + ch * 16), pe);
-      } else {
-        tmem_st16(tmem_addr(tb, q4 * 32, COL_B + b * 128 + ch * 16), pp);
-        tmem_st16(tmem_addr(tb, q4 * 32, COL_B + b * 128 + 64 + ch * 16), pe);
-      }
-      tmem_wait_st();
-      tc_fence_before();
-      mbar_arrive(bar(BAR_PFULL + b));
-    }
-    // ---- epilogue ----
-    if (ok) ok = wait_or_abort(bar(BAR_ODONE), 0, abort_flag);
-    if (ok) {
-      tc_fence_after();
-      uint32_t a0[32];
-      tmem_ld32(tmem_addr(tb, q4 * 32, COL_ACC + ch * 32), a0);
-      tmem_wait_ld(a0);
       auto store32 = [&](__nv_bfloat16* dst, const float (&x)[32]) {
 #pragma unroll
         for (int c = 0; c < 32; c += 8) {
@@ -474,49 +552,65 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
           *reinterpret_cast<uint4*>(dst + c) = pkt;
         }
       };
-      float x[32];
+      const size_t row_off = ((size_t)w.bh * args.Tlen + grow) * D;
       if (MODE == MODE_DQ) {
+        // dq = 2 / D_t x the sum, 32 columns per group
+        uint32_t a0[32];
+        float x[32];
+        tmem_ld32(accu + grp * 32, a0);
+        tmem_wait_ld(a0);
+        tc_fence_before();
+        mbar_arrive(bar(BAR_OFREE));
+        const float f = 2.f * inv_row;
 #pragma unroll
-        for (int c = 0; c < 32; ++c) x[c] = __uint_as_float(a0[c]);
-        if (grow < args.Tlen) store32(args.out0 + ((size_t)bh * args.Tlen + grow) * D + ch * 32, x);
+        for (int c = 0; c < 32; ++c) x[c] = f * __uint_as_float(a0[c]);
+        if (grow < args.Tlen) store32(args.out0 + row_off + grp * 32, x);
       } else {
-        uint32_t u[32];
-        tmem_ld32(tmem_addr(tb, q4 * 32, COL_ACC + 64 + ch * 32), u);
-        tmem_wait_ld(u);
-        // this key's row (32 of its 64 entries), its share of ||k||^2 and of k . u; the halves meet in shared memory
-        float kf[32];
+        // group 0: dk = r (2 u - r (k . 2 u) k);  group 1: dv = r dv~
+        const unsigned char* kt = x1(ni & 1);
+        auto krow = [&](int half, float (&kf)[32]) {
+#pragma unroll
+          for (int cix = 0; cix < 4; ++cix) {
+            const uint4 raw = *reinterpret_cast<const uint4*>(kt + sw128_offset(rowl, half * 4 + cix));
+            const uint32_t kw[4] = {raw.x, raw.y, raw.z, raw.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const float2 f2 = unpack_bf16(kw[e]);
+              kf[8 * cix + 2 * e] = f2.x;
+              kf[8 * cix + 2 * e + 1] = f2.y;
+            }
+          }
+        };
         float n2 = 0.f, dot = 0.f;
+        uint32_t a0[32];
+        float kf[32];
+#pragma unroll 1
+        for (int half = 0; half < 2; ++half) {
+          krow(half, kf);
+          tmem_ld32(accu + 64 + half * 32, a0);
+          tmem_wait_ld(a0);
 #pragma unroll
-        for (int cix = 0; cix < 4; ++cix) {
-          const uint4 raw = *reinterpret_cast<const uint4*>(base + OFF_X1 + sw128_offset(rowl, ch * 4 + cix));
-          const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            kf[8 * cix + 2 * e] = __uint_as_float(w[e] << 16);
-            kf[8 * cix + 2 * e + 1] = __uint_as_float(w[e] & 0xFFFF0000u);
+          for (int c = 0; c < 32; ++c) {
+            n2 = fmaf(kf[c], kf[c], n2);
+            dot = fmaf(kf[c], __uint_as_float(a0[c]), dot);
           }
         }
+        const float r = inv_or_zero(n2);
+        const float proj = r * dot;
+#pragma unroll 1
+        for (int half = 0; half < 2; ++half) {
+          float x[32];
+          if (grp == 0) krow(half, kf);
+          tmem_ld32(accu + (grp == 0 ? 64 : 0) + half * 32, a0);
+          tmem_wait_ld(a0);
 #pragma unroll
-        for (int c = 0; c < 32; ++c) {
-          n2 = fmaf(kf[c], kf[c], n2);
-          dot = fmaf(kf[c], __uint_as_float(u[c]), dot);
+          for (int c = 0; c < 32; ++c)
+            x[c] = grp == 0 ? 2.f * r * (__uint_as_float(a0[c]) - proj * kf[c]) : r * __uint_as_float(a0[c]);
+          if (grow < args.Tlen) store32((grp == 0 ? args.out0 : args.out1) + row_off + half * 32, x);
         }
-        part[ch * MT + rowl] = make_float2(n2, dot);
-        asm volatile("bar.sync %0, 64;" ::"r"(1 + (int)q4) : "memory");
-        const float2 other = part[(1 - ch) * MT + rowl];
-        // fixed order of the two halves
-        const float n2t = ch == 0 ? n2 + other.x : other.x + n2;
-        const float dott = ch == 0 ? dot + other.y : other.y + dot;
-        const float r = inv_or_zero(n2t);
-        const float proj = r * dott;
-        if (grow < args.Tlen) {
-#pragma unroll
-          for (int c = 0; c < 32; ++c) x[c] = r * (__uint_as_float(u[c]) - proj * kf[c]);
-          store32(args.out0 + ((size_t)bh * args.Tlen + grow) * D + ch * 32, x);
-#pragma unroll
-          for (int c = 0; c < 32; ++c) x[c] = r * __uint_as_float(a0[c]);
-          store32(args.out1 + ((size_t)bh * args.Tlen + grow) * D + ch * 32, x);
-        }
+        tc_fence_before();
+        mbar_arrive(bar(BAR_OFREE));
+        mbar_arrive(bar(BAR_XEMPTY + (ni & 1)));
       }
     }
   }
@@ -526,7 +620,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if ((warp == 1 || warp == 2) && elect_one()) {
+  if (warp == 1 && elect_one()) {
     mma_commit(bar(BAR_DRAIN));
     mbar_wait(bar(BAR_DRAIN), 0);
   }
@@ -536,9 +630,8 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
 
 size_t align256(size_t n) { return (n + 255) / 256 * 256; }
 
-// Pre-pass: one warp per 4 key rows (8 lanes x 16 bytes per row).  k' = k / ||k||^2 (bf16), r = 1 / ||k||^2 (fp32).
-__global__ void __launch_bounds__(256) bwd_prescale_kernel(const __nv_bfloat16* __restrict__ k, __nv_bfloat16* __restrict__ ks,
-                                                           float* __restrict__ rk, size_t n_rows) {
+// Pre-pass: one warp per 4 key rows (8 lanes x 16 bytes per row).  r = 1 / ||k||^2 (fp32).
+__global__ void __launch_bounds__(256) bwd_rscale_kernel(const __nv_bfloat16* __restrict__ k, float* __restrict__ rk, size_t n_rows) {
   const size_t row = (size_t)blockIdx.x * 32 + (threadIdx.x >> 3);
   const int part = threadIdx.x & 7;
   if (row >= n_rows) return;
@@ -547,26 +640,70 @@ __global__ void __launch_bounds__(256) bwd_prescale_kernel(const __nv_bfloat16* 
   float ss = 0.f;
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
-    const float lo = __uint_as_float(kw[e] << 16), hi = __uint_as_float(kw[e] & 0xFFFF0000u);
-    ss = fmaf(lo, lo, ss);
-    ss = fmaf(hi, hi, ss);
+    const float2 f = unpack_bf16(kw[e]);
+    ss = fmaf(f.x, f.x, ss);
+    ss = fmaf(f.y, f.y, ss);
   }
   ss += __shfl_xor_sync(0xffffffffu, ss, 1);
   ss += __shfl_xor_sync(0xffffffffu, ss, 2);
   ss += __shfl_xor_sync(0xffffffffu, ss, 4);
-  const float r = inv_or_zero(ss);
-  uint4 kc;
-  kc.x = pack_bf16(__uint_as_float(kw[0] << 16) * r, __uint_as_float(kw[0] & 0xFFFF0000u) * r);
-  kc.y = pack_bf16(__uint_as_float(kw[1] << 16) * r, __uint_as_float(kw[1] & 0xFFFF0000u) * r);
-  kc.z = pack_bf16(__uint_as_float(kw[2] << 16) * r, __uint_as_float(kw[2] & 0xFFFF0000u) * r);
-  kc.w = pack_bf16(__uint_as_float(kw[3] << 16) * r, __uint_as_float(kw[3] & 0xFFFF0000u) * r);
-  *reinterpret_cast<uint4*>(ks + row * D + part * 8) = kc;
-  if (part == 0) rk[row] = r;
+  if (part == 0) rk[row] = inv_or_zero(ss);
+}
+
+template <int MODE, int G, int NS>
+bool launch_bwd(const CUtensorMap& x1, const CUtensorMap& x2, const CUtensorMap& y1, const CUtensorMap& y2, const BArgs& a, LaunchCtx& ctx) {
+  auto kern = tc_bwd_kernel<MODE, G, NS>;
+  int dev = 0, sms = 148;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    cudaGetLastError();
+    sms = 148;
+  }
+  const long long n_items = (long long)a.BH * ((a.Tlen + MT - 1) / MT);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(n_items < sms ? n_items : sms));   // persistent: one CTA per SM
+  cfg.blockDim = dim3(Geo<MODE, G, NS>::NTHREADS);
+  cfg.dynamicSmemBytes = SMEM_ALLOC;
+  cfg.stream = ctx.stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_ALLOC) != cudaSuccess ||
+      cudaLaunchKernelEx(&cfg, kern, x1, x2, y1, y2, a) != cudaSuccess) {
+    cudaGetLastError();
+    ctx.status = KATA_ERR_CUDA;
+    return false;
+  }
+  ++ctx.launches;
+  return true;
+}
+
+// r, then dq and the row scalars, then dk and dv (which read the scalars)
+template <int G, int NS>
+void run_bwd(const Problem& p, const void* dout, void* dq, void* dk, void* dv, float* rk, float* stats, int* device_status, LaunchCtx& ctx) {
+  const int BH = p.B * p.H;
+  const size_t rows = (size_t)BH * p.T;
+  constexpr int NT = Geo<MODE_DQ, G, NS>::NT;
+  bwd_rscale_kernel<<<(unsigned)((rows + 31) / 32), 256, 0, ctx.stream>>>(static_cast<const __nv_bfloat16*>(p.k), rk, rows);
+  note_launch(ctx);
+  CUtensorMap qf, gf, kf, vf, qs, gs, ks, vs;     // fixed tiles of 128 rows, streamed tiles of NT
+  if (!make_tile_map(&qf, p.q, BH, p.T, MT) || !make_tile_map(&gf, dout, BH, p.T, MT) || !make_tile_map(&kf, p.k, BH, p.T, MT) ||
+      !make_tile_map(&vf, p.v, BH, p.T, MT) || !make_tile_map(&qs, p.q, BH, p.T, NT) || !make_tile_map(&gs, dout, BH, p.T, NT) ||
+      !make_tile_map(&ks, p.k, BH, p.T, NT) || !make_tile_map(&vs, p.v, BH, p.T, NT)) {
+    ctx.status = KATA_ERR_CUDA;
+    return;
+  }
+  BArgs a{static_cast<__nv_bfloat16*>(dq), nullptr, stats, rk, device_status, p.T, BH};
+  if (!launch_bwd<MODE_DQ, G, NS>(qf, gf, ks, vs, a, ctx)) return;
+  BArgs b{static_cast<__nv_bfloat16*>(dk), static_cast<__nv_bfloat16*>(dv), stats, rk, device_status, p.T, BH};
+  launch_bwd<MODE_DKV, G, NS>(kf, vf, qs, gs, b, ctx);
 }
 
 }  // namespace
 
-// workspace: K' [BH][T][64] bf16, r [BH][T] fp32, the row scalars [BH][T][2] fp32
+// workspace: 128 bytes per row as published (not used any more: k is read as it is), r [BH][T] fp32, the row scalars
+// [BH][T][2] fp32
 size_t tc_bwd_workspace_bytes(const Problem& p) {
   const size_t rows = (size_t)p.B * p.H * p.T;
   return align256(rows * D * 2) + align256(rows * sizeof(float)) + align256(rows * 2 * sizeof(float));
@@ -574,37 +711,25 @@ size_t tc_bwd_workspace_bytes(const Problem& p) {
 
 void tc_bwd_quadratic(const Problem& p, const void* dout, void* dq, void* dk, void* dv, void* workspace, int* device_status,
                       LaunchCtx& ctx) {
-  const int BH = p.B * p.H;
-  const size_t rows = (size_t)BH * p.T;
-  unsigned char* ws = static_cast<unsigned char*>(workspace);
-  __nv_bfloat16* ks = reinterpret_cast<__nv_bfloat16*>(ws);
-  float* rk = reinterpret_cast<float*>(ws + align256(rows * D * 2));
-  float* stats = reinterpret_cast<float*>(ws + align256(rows * D * 2) + align256(rows * sizeof(float)));
-  bwd_prescale_kernel<<<(unsigned)((rows + 31) / 32), 256, 0, ctx.stream>>>(static_cast<const __nv_bfloat16*>(p.k), ks, rk, rows);
-  note_launch(ctx);
-  CUtensorMap q128, g128, k128, v128, q64, g64, k64, v64, ks64;
-  if (!make_tile_map(&q128, p.q, BH, p.T, MT) || !make_tile_map(&g128, dout, BH, p.T, MT) || !make_tile_map(&k128, p.k, BH, p.T, MT) ||
-      !make_tile_map(&v128, p.v, BH, p.T, MT) || !make_tile_map(&q64, p.q, BH, p.T, NT) || !make_tile_map(&g64, dout, BH, p.T, NT) ||
-      !make_tile_map(&k64, p.k, BH, p.T, NT) || !make_tile_map(&v64, p.v, BH, p.T, NT) || !make_tile_map(&ks64, ks, BH, p.T, NT)) {
-    ctx.status = KATA_ERR_CUDA;
-    return;
-  }
-  auto kq = p.groups == 1 ? tc_bwd_kernel<MODE_DQ, 1> : p.groups == 2 ? tc_bwd_kernel<MODE_DQ, 2> : tc_bwd_kernel<MODE_DQ, 4>;
-  auto kkv = p.groups == 1 ? tc_bwd_kernel<MODE_DKV, 1> : p.groups == 2 ? tc_bwd_kernel<MODE_DKV, 2> : tc_bwd_kernel<MODE_DKV, 4>;
-  if (cudaFuncSetAttribute(kq, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_ALLOC) != cudaSuccess ||
-      cudaFuncSetAttribute(kkv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_ALLOC) != cudaSuccess) {
-    cudaGetLastError();
-    ctx.status = KATA_ERR_CUDA;
-    return;
-  }
-  const dim3 grid((p.T + MT - 1) / MT, BH);
-  // dq and the row scalars, then dk and dv (which read the scalars)
-  BArgs a{static_cast<__nv_bfloat16*>(dq), nullptr, stats, rk, device_status, p.T};
-  kq<<<grid, NTHREADS, SMEM_ALLOC, ctx.stream>>>(q128, g128, k64, v64, ks64, a);
-  note_launch(ctx);
-  BArgs b{static_cast<__nv_bfloat16*>(dk), static_cast<__nv_bfloat16*>(dv), stats, rk, device_status, p.T};
-  kkv<<<grid, NTHREADS, SMEM_ALLOC, ctx.stream>>>(k128, v128, q64, g64, q64, b);
-  note_launch(ctx);
+  const size_t rows = (size_t)p.B * p.H * p.T;
+  float* rk = static_cast<float*>(workspace);
+  float* stats = reinterpret_cast<float*>(static_cast<unsigned char*>(workspace) + align256(rows * sizeof(float)));
+  if (p.groups == 1) run_bwd<1, 1>(p, dout, dq, dk, dv, rk, stats, device_status, ctx);
+  else if (p.groups == 2) run_bwd<2, 1>(p, dout, dq, dk, dv, rk, stats, device_status, ctx);
+  else run_bwd<4, 1>(p, dout, dq, dk, dv, rk, stats, device_status, ctx);
+}
+
+// The gradients with fp32 weights (three bf16 terms): kata_bwd_chunked on sequences short enough for the quadratic form.
+size_t tc_bwd_exact_workspace_bytes(const Problem& p) {
+  const size_t rows = (size_t)p.B * p.H * p.T;
+  return align256(rows * sizeof(float)) + align256(rows * 2 * sizeof(float));
+}
+
+void tc_bwd_exact(const Problem& p, const void* dout, void* dq, void* dk, void* dv, void* workspace, int* device_status, LaunchCtx& ctx) {
+  const size_t rows = (size_t)p.B * p.H * p.T;
+  float* rk = static_cast<float*>(workspace);
+  float* stats = reinterpret_cast<float*>(static_cast<unsigned char*>(workspace) + align256(rows * sizeof(float)));
+  run_bwd<1, 3>(p, dout, dq, dk, dv, rk, stats, device_status, ctx);
 }
 
 }  // namespace kata

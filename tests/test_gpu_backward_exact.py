@@ -1,0 +1,45 @@
+"""kata_bwd_chunked on the tensor cores (bf16, d = 64, 512 to 16384 tokens: the quadratic form with fp32 weights) at the edges
+of its range and of its tiles (128 fixed rows, 64 streamed rows).
+
+The operands are the bf16 inputs, the weights carry 24 bits and the sums are fp32, so beside the rounding of the stored
+gradient (2^-9 of the entry) the error is that of fp32 sums: 1e-5 of the largest entry covers both sweeps' T terms.  The
+plain FMA kernels of the same entry are held to the same bound."""
+import numpy as np
+import pytest
+
+from oracle import kata_oracle as ko
+from paper_2607_17419_b200 import binding as kb
+from paper_2607_17419_b200 import inputs
+
+from helpers import dev_tensors, to_numpy64
+from test_gpu_backward import dout_for
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("T,zero", [(512, False), (513, True), (575, False), (577, False), (639, True), (641, False), (1100, True)])
+def test_backward_exact(T, zero):
+    import torch
+    w = inputs.gaussian_workload(f"bwdx_{T}", "bf16", 1, 3, T, 64, 64, 64, 6100 + T)
+    if zero:
+        for arr in (w.k_ref, w.k_dev):
+            arr[0, 0, [0, 127, 128, 300]] = 0
+        for arr in (w.q_ref, w.q_dev):
+            arr[0, 0, [5, 256, T - 1]] = 0
+    q, k, v = dev_tensors(w)
+    g, g_ref = dout_for(w, 5)
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    grads = kb.kata_bwd_chunked(q, k, v, g, device_status=st)
+    torch.cuda.synchronize()
+    assert kb.kata_last_impl() == kb.KATA_IMPL_TENSOR and kb.kata_last_launch_count() == 3 and int(st.item()) == 0
+    again = kb.kata_bwd_chunked(q, k, v, g, impl=kb.KATA_IMPL_TENSOR)
+    plain = kb.kata_bwd_chunked(q, k, v, g, impl=kb.KATA_IMPL_SIMT)
+    torch.cuda.synchronize()
+    assert kb.kata_last_impl() == kb.KATA_IMPL_SIMT
+    for h in range(w.H):
+        ref = ko.kata_quadratic_bwd(w.q_ref[0, h], w.k_ref[0, h], w.v_ref[0, h], g_ref[0, h])
+        for name, got, same, other, r in zip(("dq", "dk", "dv"), grads, again, plain, ref):
+            assert torch.equal(got, same)
+            for what, x in (("tensor", got), ("plain", other)):
+                err = np.abs(to_numpy64(x[0, h]) - r)
+                assert np.all(err <= 2.0 ** -8 * np.abs(r) + 1e-5 * np.abs(r).max()), (name, what, T, float(err.max()))
