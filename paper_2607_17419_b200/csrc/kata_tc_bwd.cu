@@ -22,15 +22,17 @@
 // a bf16 input, exact, and every sum fp32): kata_bwd_chunked on sequences short enough for the quadratic form, whose
 // contract is fp32 arithmetic.
 //
-// What bounds it: the MMAs of a step (128 x 64 pairs: scores 2 x 192 cycles, one output 128, another 128) and the chain
-// scores -> weights -> outputs, about 1700 cycles of which half is hand-offs.  Each of the NBUF TMEM buffers is a chain of
-// its own with its own group of four weight warps; one thread issues all MMAs, closing the steps in order and opening each
-// buffer again right behind its close, so no wait stands between the outputs of a step and the scores that reuse its
-// columns.  The CTAs are persistent (one per SM, items dealt heaviest first, forwards and backwards in turn) and the next
-// item's scores are opened before the current one's last outputs.
+// What bounds it.  A step (128 x 64 pairs) is 256 to 384 cycles of score MMAs and 128 (dq) or 256 (dk, dv) of output MMAs;
+// the rest is hand-offs, about 300 cycles each from one thread's arrival through the MMAs to the next thread's first
+// instruction.  Where TMEM has room (one group; three terms: dq only) the weights have columns of their own: a score buffer
+// is free as soon as its weight warps have read it, so scores, weights and outputs of successive steps overlap; with the
+// weights stored over the scores the loop scores -> weights -> outputs -> scores was 2100 cycles for two steps.  Scores and
+// outputs are issued by a thread each (an issuer is busy about as long as its MMAs take).  The fixed tiles of dq are TMEM
+// operands: from shared memory every score MMA read 6 KB for 32 cycles of arithmetic.  The CTAs are persistent (one per SM,
+// items dealt heaviest first, forwards and backwards in turn); the score issuer runs ahead into the next item.
 //
-// Warps: 0 TMA producer, 1 MMA issuer, 2 idle, 3 scalars of the streamed rows, 4.. weights and epilogue (NBUF groups of
-// four, quadrant = warp % 4).  All waits are bounded.
+// Warps: 0 TMA producer, 1 score MMAs, 2 output MMAs, 3 scalars of the streamed rows, 4.. weights and epilogue (sets of
+// four, quadrant = warp % 4; CS sets per buffer, each with its part of the columns).  All waits are bounded.
 #include <cuda.h>
 #include <type_traits>
 
@@ -49,34 +51,47 @@ constexpr int NSTAGE = 6;
 constexpr int WARP_BLD0 = 4;
 enum { MODE_DQ = 0, MODE_DKV = 1 };
 
-constexpr uint32_t COL_ACC = 384;  // 2 x 64 fp32 accumulators
 constexpr uint32_t TMEM_COLS = 512;
 
 // G feature groups of the blockwise map: s_g = q_g . k_g per group, a = r sum_g s_g^2, e_g from s_g; dq and u are formed
 // group by group (N = 64 / G columns of the accumulator, the B operand offset into the 128-byte rows).
 template <int MODE, int G, int NS> struct Geo {
   static constexpr int NT = G == 4 ? 32 : 64;               // rows of a streamed tile
-  static constexpr int NBUF = G == 1 && NS == 1 ? 3 : 2;    // score buffers = groups of weight warps
-  // a buffer: [S_0 | .. | S_{G-1} | C], NT fp32 columns each (and 64 more for the extra terms of the weights)
-  static constexpr uint32_t BW = NS == 3 ? 192u : (uint32_t)(G + 1) * NT;
+  static constexpr int NBUF = 2;                            // score buffers
+  static constexpr int CS = G == 1 ? 2 : 1;                 // sets of weight warps per buffer
+  static constexpr int SETS = NBUF * CS;
+  static constexpr int CPW = NT / 32 / CS;                  // runs of 32 columns per set
+  static constexpr bool SEP = G == 1 && !(NS == 3 && MODE == MODE_DKV);   // weights in columns of their own
+  // a score buffer: [S_0 | .. | S_{G-1} | C], NT fp32 columns each (and 64 more for the extra terms of the weights)
+  static constexpr uint32_t BW = SEP ? 128u : NS == 3 ? 192u : (uint32_t)(G + 1) * NT;
   static constexpr uint32_t CB = G * NT;                    // its C block
-  static constexpr int NTHREADS = 128 + NBUF * 128;
-  static_assert(NBUF * BW <= COL_ACC, "TMEM columns");
-  // first column of the bf16 weights inside the buffer (they overwrite scores that are already in registers)
-  __host__ __device__ static constexpr uint32_t p_col(int term) { return NS == 3 ? (term == 0 ? 0u : term == 1 ? 128u : 160u) : G == 1 ? 0u : CB; }
-  __host__ __device__ static constexpr uint32_t e_col(int g, int term) {
-    if (NS == 3) return MODE == MODE_DQ ? 64u * term : term == 0 ? 64u : term == 1 ? 32u : 96u;
-    return MODE == MODE_DKV && G == 1 ? CB : (uint32_t)g * NT;
+  static constexpr uint32_t EW = MODE == MODE_DQ ? 32 * NS : 64;          // SEP: columns of the weights of a buffer, from 256 on
+  static constexpr bool XT = SEP && MODE == MODE_DQ && NS == 1;           // fixed tiles in TMEM, two buffers of 64 columns
+  static constexpr uint32_t COL_X = 384;
+  static constexpr uint32_t COL_ACC = SEP ? 256 + NBUF * EW : 384;        // accumulators: 64 or 128 columns
+  static constexpr int NTHREADS = 128 + SETS * 128;
+  static_assert(NBUF * BW <= (SEP ? 256u : COL_ACC) && COL_ACC + (MODE == MODE_DQ ? 64 : 128) <= (XT ? COL_X : 512u), "TMEM columns");
+  // first column of the bf16 weights of a buffer: their own, or over scores that are already in registers
+  __host__ __device__ static constexpr uint32_t p_col(int b, int term) {
+    return SEP ? 256 + b * EW : b * BW + (NS == 3 ? (term == 0 ? 0u : term == 1 ? 128u : 160u) : CB);
+  }
+  __host__ __device__ static constexpr uint32_t e_col(int b, int g, int term) {
+    return SEP ? 256 + b * EW + (MODE == MODE_DQ ? 32 * term : 32) : b * BW + (NS == 3 ? (term == 0 ? 64u : term == 1 ? 32u : 96u) : g * NT);
   }
 };
+
+// Registers with 640 threads: 96 each at launch; the four warps that issue and copy give theirs to the weight warps.
+template <int N> __device__ __forceinline__ void regs_release() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
+template <int N> __device__ __forceinline__ void regs_take() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
+static_assert(128 * 64 + 512 * 104 <= 640 * 96, "register budget");
 
 constexpr uint32_t OFF_X = 0;                      // 2 x (two fixed tiles of 128 x 64 bf16, 128B swizzle): this and the next item
 constexpr uint32_t OFF_ST = 65536;                 // stages: two streamed tiles of up to 8 KB
 constexpr uint32_t STAGE_BYTES = 16384;
 constexpr uint32_t OFF_SC = OFF_ST + NSTAGE * STAGE_BYTES;   // per stage 512 bytes of scalars of the streamed rows:
                                                              // r_i (MODE_DQ) or (1/D_t, dout_t . o_t) (MODE_DKV)
-constexpr uint32_t OFF_PART = OFF_SC + NSTAGE * 512;         // 2 (item parity) x 3 groups x 128 float2: the sums of a row meet here
-constexpr uint32_t OFF_BAR = OFF_PART + 6144;
+constexpr uint32_t OFF_PART = OFF_SC + NSTAGE * 512;         // 2 (item parity) x 4 sets x 128 float2: the sums of a row meet here
+constexpr uint32_t OFF_BAR = OFF_PART + 8192;
 constexpr uint32_t SMEM_BYTES = OFF_BAR + 256;
 constexpr uint32_t SMEM_ALLOC = SMEM_BYTES + 1024;
 static_assert(SMEM_ALLOC > 116 * 1024, "one CTA per SM is assumed (the CTA allocates all of TMEM)");
@@ -88,12 +103,15 @@ enum {
   BAR_XEMPTY = 2,    // [2] ... and are no longer needed
   BAR_FULL = 4,      // [NSTAGE] streamed tiles (TMA bytes) and their scalars landed
   BAR_EMPTY = 10,    // [NSTAGE] stage free
-  BAR_SFULL = 16,    // [3] scores in TMEM
-  BAR_PFULL = 19,    // [3] weights stored (128 threads)
-  BAR_ODONE = 22,    // the accumulators of an item are complete
-  BAR_OFREE = 23,    // ... and have been read (256 threads)
-  BAR_DRAIN = 24,
-  BAR_COUNT = 25
+  BAR_SFULL = 16,    // [2] scores in TMEM
+  BAR_SFREE = 18,    // [2] the score buffer may take new scores (its weight warps; where weights lie over scores, the output MMAs)
+  BAR_PFULL = 20,    // [2] weights stored, scalars read (CS x 128 threads)
+  BAR_PFREE = 22,    // [2] weights consumed
+  BAR_ODONE = 24,    // the accumulators of an item are complete
+  BAR_OFREE = 25,    // ... and have been read (256 threads)
+  BAR_XT = 26,       // [2] fixed tiles of an item in TMEM (256 threads)
+  BAR_DRAIN = 28,
+  BAR_COUNT = 29
 };
 
 struct BArgs {
@@ -126,8 +144,9 @@ __global__ void __launch_bounds__(Geo<MODE, G, NS>::NTHREADS, 1)
 tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ CUtensorMap tmX2,
               const __grid_constant__ CUtensorMap tmY1, const __grid_constant__ CUtensorMap tmY2, const BArgs args) {
   using geo = Geo<MODE, G, NS>;
-  constexpr int NT = geo::NT, NBUF = geo::NBUF;
-  constexpr uint32_t BW = geo::BW, CB = geo::CB;
+  constexpr int NT = geo::NT, NBUF = geo::NBUF, CS = geo::CS, CPW = geo::CPW, SETS = geo::SETS;
+  constexpr uint32_t BW = geo::BW, CB = geo::CB, COL_ACC = geo::COL_ACC, COL_X = geo::COL_X;
+  constexpr bool XT = geo::XT, SEP = geo::SEP;
   constexpr int MG = D / G;                        // features per group
   extern __shared__ unsigned char smem_raw[];
   unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -172,7 +191,8 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
     abort_s = 0;
     for (int i = 0; i < 2; ++i) {
       mbar_init(bar(BAR_XFULL + i), 1);
-      mbar_init(bar(BAR_XEMPTY + i), MODE == MODE_DQ ? 1 : 1 + 256);
+      mbar_init(bar(BAR_XEMPTY + i), (MODE == MODE_DQ && !XT ? 0 : 256) + (XT ? 0 : 1));   // readers: sets 0 and 1, MMAs
+      mbar_init(bar(BAR_XT + i), 256);
     }
     for (int i = 0; i < NSTAGE; ++i) {
       mbar_init(bar(BAR_FULL + i), 2);
@@ -180,11 +200,13 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
     }
     for (int i = 0; i < NBUF; ++i) {
       mbar_init(bar(BAR_SFULL + i), 1);
-      mbar_init(bar(BAR_PFULL + i), 128);
+      mbar_init(bar(BAR_SFREE + i), SEP ? CS * 128 : 1);
+      mbar_init(bar(BAR_PFULL + i), CS * 128);
+      mbar_init(bar(BAR_PFREE + i), 1);
     }
     mbar_init(bar(BAR_ODONE), 1);
     mbar_init(bar(BAR_OFREE), 256);
-    mbar_init(bar(BAR_DRAIN), 1);
+    mbar_init(bar(BAR_DRAIN), 2);
     fence_mbar_init();
     tma_prefetch_desc(&tmX1);
     tma_prefetch_desc(&tmX2);
@@ -202,18 +224,27 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
   bool ok = true;
 
   if (warp == 0) {
+    if (SETS == 4) regs_release<64>();
     // =========================== TMA producer ===========================
     if (elect_one()) {
+      // the fixed tiles of an item are asked for behind the third step of the item before
       uint32_t t = 0;
       int ni = 0;
-      Item w;
-      for (int n = 0; ok && next_item(n, w); ++n, ++ni) {
-        const int xb = ni & 1;
-        ok = wait_or_abort(bar(BAR_XEMPTY + xb), ((ni >> 1) & 1) ^ 1, abort_flag);
-        if (!ok) break;
+      Item w, wn;
+      int n = 0;
+      auto load_x = [&](const Item& x, int i) {
+        const int xb = i & 1;
+        ok = wait_or_abort(bar(BAR_XEMPTY + xb), ((i >> 1) & 1) ^ 1, abort_flag);
+        if (!ok) return;
         mbar_arrive_expect_tx(bar(BAR_XFULL + xb), 32768);
-        tma_load_3d(x1(xb), &tmX1, bar(BAR_XFULL + xb), 0, w.m0, w.bh);
-        tma_load_3d(x2(xb), &tmX2, bar(BAR_XFULL + xb), 0, w.m0, w.bh);
+        tma_load_3d(x1(xb), &tmX1, bar(BAR_XFULL + xb), 0, x.m0, x.bh);
+        tma_load_3d(x2(xb), &tmX2, bar(BAR_XFULL + xb), 0, x.m0, x.bh);
+      };
+      bool more = next_item(n, w);
+      if (more) load_x(w, 0);
+      for (; more && ok; ++ni) {
+        ++n;
+        const bool more_n = next_item(n, wn);
         for (int j = 0, jt = 0; j < w.nsteps && ok; ++j, ++t) {
           const int s = t % NSTAGE;
           ok = wait_or_abort(bar(BAR_EMPTY + s), ((t / NSTAGE) & 1) ^ 1, abort_flag);
@@ -222,46 +253,56 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
           tma_load_3d(y1(s), &tmY1, bar(BAR_FULL + s), 0, (w.jbeg + jt) * NT, w.bh);
           tma_load_3d(y2(s), &tmY2, bar(BAR_FULL + s), 0, (w.jbeg + jt) * NT, w.bh);
           if (++jt == w.ntiles) jt = 0;
+          if (more_n && j == (w.nsteps > 2 ? 2 : w.nsteps - 1)) load_x(wn, ni + 1);
         }
+        w = wn;
+        more = more_n;
       }
     }
   } else if (warp == 1) {
-    // =========================== MMA issuer ===========================
+    if (SETS == 4) regs_release<64>();
+    // =========================== score MMA issuer ===========================
     if (elect_one()) {
-      const uint32_t id_s = instr_desc(kFmtBF16, kFmtBF16, 0, 0, 128, NT);      // scores: both K-major
+      const uint32_t id_s = instr_desc(kFmtBF16, kFmtBF16, 0, 0, 128, NT);      // both K-major
+      const uint64_t dk = smem_desc(0, 16, 1024, kSwizzle128B);
+      uint32_t t = 0;
+      int ni = 0;
+      Item w;
+      for (int n = 0; ok && next_item(n, w); ++n, ++ni) {
+        const int xb = ni & 1;
+        ok = wait_or_abort(bar((XT ? BAR_XT : BAR_XFULL) + xb), (ni >> 1) & 1, abort_flag);
+        const uint32_t f1 = smem_u32(x1(xb)), f2 = smem_u32(x2(xb)), xt = tb + COL_X + xb * 64;
+        for (int j = 0; j < w.nsteps && ok; ++j, ++t) {
+          const int s = t % NSTAGE, b = t % NBUF;
+          ok = wait_or_abort(bar(BAR_FULL + s), (t / NSTAGE) & 1, abort_flag) &&
+               wait_or_abort(bar(BAR_SFREE + b), ((t / NBUF) & 1) ^ 1, abort_flag);
+          if (!ok) break;
+          tc_fence_after();
+          const uint32_t a1 = smem_u32(y1(s)), a2 = smem_u32(y2(s));
+#pragma unroll
+          for (int ks = 0; ks < 4; ++ks) {    // 16 features per step; group ks / (4 / G) has its own NT score columns
+            const uint32_t d = tb + b * BW + (ks / (4 / G)) * NT;
+            if (XT) mma_f16_ts(d, xt + ks * 8, at(dk, a1 + ks * 32), id_s, (ks % (4 / G)) > 0);
+            else mma_f16_ss(d, at(dk, f1 + ks * 32), at(dk, a1 + ks * 32), id_s, (ks % (4 / G)) > 0);
+          }
+#pragma unroll
+          for (int ks = 0; ks < 4; ++ks) {
+            const uint32_t d = tb + b * BW + CB;
+            if (XT) mma_f16_ts(d, xt + 32 + ks * 8, at(dk, a2 + ks * 32), id_s, ks > 0);
+            else mma_f16_ss(d, at(dk, f2 + ks * 32), at(dk, a2 + ks * 32), id_s, ks > 0);
+          }
+          mma_commit(bar(BAR_SFULL + b));
+        }
+        if (!XT && ok) mma_commit(bar(BAR_XEMPTY + xb));
+      }
+    }
+  } else if (warp == 2) {
+    if (SETS == 4) regs_release<64>();
+    // =========================== output MMA issuer ===========================
+    if (elect_one()) {
       const uint32_t id_o = instr_desc(kFmtBF16, kFmtBF16, 0, 1, 128, 64);      // dv~: A tmem, B MN-major
       const uint32_t id_g = instr_desc(kFmtBF16, kFmtBF16, 0, 1, 128, MG);      // dq, u of a feature group
-      const uint64_t dk = smem_desc(0, 16, 1024, kSwizzle128B);
       const uint64_t dmn = smem_desc(0, 8192, 1024, kSwizzle128B);              // 8 streamed rows x 64 columns per 1 KB atom
-      // opening side: scores of the steps, NBUF ahead of the closing side, across items
-      Item wo;
-      int no = 0, jo = 0, io = 0;
-      uint32_t t_open = 0;
-      bool mo = next_item(no, wo);
-      auto open = [&]() -> bool {
-        if (!mo) return true;
-        const int s = t_open % NSTAGE, b = t_open % NBUF, xb = io & 1;
-        if (jo == 0 && !wait_or_abort(bar(BAR_XFULL + xb), (io >> 1) & 1, abort_flag)) return false;
-        if (!wait_or_abort(bar(BAR_FULL + s), (t_open / NSTAGE) & 1, abort_flag)) return false;
-        tc_fence_after();
-        const uint32_t f1 = smem_u32(x1(xb)), f2 = smem_u32(x2(xb)), a1 = smem_u32(y1(s)), a2 = smem_u32(y2(s));
-#pragma unroll
-        for (int ks = 0; ks < 4; ++ks)      // 16 features per step; group ks / (4 / G) has its own NT score columns
-          mma_f16_ss(tb + b * BW + (ks / (4 / G)) * NT, at(dk, f1 + ks * 32), at(dk, a1 + ks * 32), id_s, (ks % (4 / G)) > 0);
-#pragma unroll
-        for (int ks = 0; ks < 4; ++ks)
-          mma_f16_ss(tb + b * BW + CB, at(dk, f2 + ks * 32), at(dk, a2 + ks * 32), id_s, ks > 0);
-        mma_commit(bar(BAR_SFULL + b));
-        ++t_open;
-        if (++jo == wo.nsteps) {
-          jo = 0;
-          ++no;
-          ++io;
-          mo = next_item(no, wo);
-        }
-        return true;
-      };
-      for (int i = 0; i < NBUF && ok; ++i) ok = open();
       uint32_t t = 0;
       int ni = 0;
       Item w;
@@ -270,40 +311,42 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
         for (int j = 0; j < w.nsteps && ok; ++j, ++t) {
           const int s = t % NSTAGE, b = t % NBUF;
           ok = wait_or_abort(bar(BAR_PFULL + b), (t / NBUF) & 1, abort_flag);
-          // the accumulators are free once the epilogue of the item before has read them
-          if (ok && j == (MODE == MODE_DQ ? w.ntiles : 0) && ni > 0) ok = wait_or_abort(bar(BAR_OFREE), (ni - 1) & 1, abort_flag);
           if (!ok) break;
-          if (MODE == MODE_DKV || j >= w.ntiles) {       // (the first sweep of MODE_DQ only sums the row scalars)
-            tc_fence_after();
-            const uint32_t buf = tb + b * BW, ya = smem_u32(y1(s)), yb = smem_u32(y2(s));
-            if (MODE == MODE_DKV) {
-#pragma unroll
-              for (int term = 0; term < NS; ++term)
-#pragma unroll
-                for (int ks = 0; ks < NT / 16; ++ks)      // dv~ += P^T dout
-                  mma_f16_ts(tb + COL_ACC, buf + geo::p_col(term) + ks * 8, at(dmn, yb + ks * 2048), id_o, (acc || term > 0 || ks > 0) ? 1u : 0u);
-            }
-            constexpr uint32_t col = COL_ACC + (MODE == MODE_DKV ? 64 : 0);
-#pragma unroll
-            for (int g = 0; g < G; ++g)
-#pragma unroll
-              for (int term = 0; term < NS; ++term)
-#pragma unroll
-                for (int ks = 0; ks < NT / 16; ++ks)      // dq += E K, u += E^T Q
-                  mma_f16_ts(tb + col + g * MG, buf + geo::e_col(g, term) + ks * 8, at(dmn, ya + ks * 2048 + g * MG * 2), id_g,
-                             (acc || term > 0 || ks > 0) ? 1u : 0u);
-            acc = 1;
+          if (MODE == MODE_DQ && j < w.ntiles) {         // (the first sweep only sums the row scalars)
+            if (!SEP) mbar_arrive(bar(BAR_SFREE + b));
+            mbar_arrive(bar(BAR_EMPTY + s));
+            continue;
           }
+          // the accumulators are free once the epilogue of the item before has read them
+          if (acc == 0 && ni > 0) ok = wait_or_abort(bar(BAR_OFREE), (ni - 1) & 1, abort_flag);
+          if (!ok) break;
+          tc_fence_after();
+          const uint32_t ya = smem_u32(y1(s)), yb = smem_u32(y2(s));
+          if (MODE == MODE_DKV) {
+#pragma unroll
+            for (int term = 0; term < NS; ++term)
+#pragma unroll
+              for (int ks = 0; ks < NT / 16; ++ks)      // dv~ += P^T dout
+                mma_f16_ts(tb + COL_ACC, tb + geo::p_col(b, term) + ks * 8, at(dmn, yb + ks * 2048), id_o, (acc || term > 0 || ks > 0) ? 1u : 0u);
+          }
+          constexpr uint32_t col = COL_ACC + (MODE == MODE_DKV ? 64 : 0);
+#pragma unroll
+          for (int g = 0; g < G; ++g)
+#pragma unroll
+            for (int term = 0; term < NS; ++term)
+#pragma unroll
+              for (int ks = 0; ks < NT / 16; ++ks)      // dq += E K, u += E^T Q
+                mma_f16_ts(tb + col + g * MG, tb + geo::e_col(b, g, term) + ks * 8, at(dmn, ya + ks * 2048 + g * MG * 2), id_g,
+                           (acc || term > 0 || ks > 0) ? 1u : 0u);
+          acc = 1;
+          mma_commit(bar((SEP ? BAR_PFREE : BAR_SFREE) + b));
           mma_commit(bar(BAR_EMPTY + s));
-          if (j + 1 == w.nsteps) {
-            mma_commit(bar(BAR_ODONE));
-            mma_commit(bar(BAR_XEMPTY + (ni & 1)));
-          }
-          ok = open();
         }
+        if (ok) mma_commit(bar(BAR_ODONE));
       }
     }
   } else if (warp == 3) {
+    if (SETS == 4) regs_release<64>();
     // =========================== scalars of the streamed rows, two tiles ahead ===========================
     // A programmatic dependent launch: only this warp reads what the kernel before it wrote.
     cudaGridDependencySynchronize();
@@ -347,15 +390,51 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
         if (lane == 0) mbar_arrive(bar(BAR_FULL + s));
       }
   } else if (warp >= WARP_BLD0) {
-    // =========================== weights and epilogue (NBUF groups of 128 threads) ===========================
+    if (SETS == 4) regs_take<104>();
+    // =========================== weights and epilogue (SETS sets of 128 threads) ===========================
     const uint32_t q4 = warp & 3;
-    const int grp = (warp - WARP_BLD0) >> 2;     // this group's buffer: the steps t with t % NBUF = grp
+    const int set = (warp - WARP_BLD0) >> 2;
+    const int grp = set / CS;                    // this set's buffer: the steps t with t % NBUF = grp
+    const int ch0 = set % CS;                    // ... and its columns of every block (CPW runs of 32)
     const int rowl = q4 * 32 + lane;             // row of the fixed tile (= TMEM lane)
-    const uint32_t buf = tmem_addr(tb, q4 * 32, grp * BW), accu = tmem_addr(tb, q4 * 32, COL_ACC);
-    uint32_t t0 = 0;                             // steps of the items before
+    const uint32_t lanes = tmem_addr(tb, q4 * 32, 0), buf = lanes + grp * BW, accu = lanes + COL_ACC;
+    // the sets of a buffer have read what the weights of the other are about to overwrite
+    auto both_read = [&]() {
+      if (SEP || CS == 1) return;
+      tc_fence_before();
+      asm volatile("bar.sync %0, 64;" ::"r"(2 + grp * 4 + (int)q4) : "memory");
+      tc_fence_after();
+    };
+    // fixed tiles of item i from shared memory to TMEM: set 0 the first, set 1 the second
+    auto copy_x = [&](int i) {
+      const int xb = i & 1;
+      ok = ok && wait_or_abort(bar(BAR_XFULL + xb), (i >> 1) & 1, abort_flag);
+      if (!ok) return;
+      const unsigned char* src = set == 0 ? x1(xb) : x2(xb);
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf) {
+        uint32_t r[16];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const uint4 v = *reinterpret_cast<const uint4*>(src + sw128_offset(rowl, hf * 4 + c));
+          r[4 * c] = v.x; r[4 * c + 1] = v.y; r[4 * c + 2] = v.z; r[4 * c + 3] = v.w;
+        }
+        tmem_st16(tmem_addr(tb, q4 * 32, COL_X + xb * 64 + set * 32 + hf * 16), r);
+      }
+      tmem_wait_st();
+      tc_fence_before();
+      mbar_arrive(bar(BAR_XT + xb));
+      if (MODE == MODE_DQ) mbar_arrive(bar(BAR_XEMPTY + xb));
+    };
+    uint32_t t0 = 0, n_out = 0;                  // steps of the items before; steps with outputs of this set's buffer
     int ni = 0;
-    Item w;
-    for (int n = 0; ok && next_item(n, w); ++n, ++ni) {
+    Item w, wn;
+    int n = 0, nn = 0;
+    bool more = next_item(n, w);
+    if (XT && more && set < 2) copy_x(0);
+    for (; more && ok; ++ni) {
+      nn = n + 1;
+      const bool more_n = next_item(nn, wn);
       const int grow = w.m0 + rowl;
       float inv_row = 0.f, del_row = 0.f;        // MODE_DQ: the scalars of this query (1 / D_t, dout_t . o_t)
       int j = (grp + NBUF - (int)(t0 % NBUF)) % NBUF;
@@ -364,10 +443,16 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
         tc_fence_after();
         return true;
       };
+      auto read_done = [&]() {                   // the scores are in registers
+        if (!SEP) return;
+        tc_fence_before();
+        mbar_arrive(bar(BAR_SFREE + grp));
+      };
       auto end = [&]() {
         tc_fence_before();
         mbar_arrive(bar(BAR_PFULL + grp));
       };
+      uint32_t cv[32], sv[32];
       if (MODE == MODE_DQ) {
         // ---- first sweep: a = r_i sum_g s_g^2 for the keys n <= this query; D_t += a, sum += a c ----
         float sum_d = 0.f, sum_m = 0.f;
@@ -376,15 +461,16 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
           if (!ok) break;
           const int s = (t0 + j) % NSTAGE;
 #pragma unroll 1
-          for (int ch = 0; ch < NT / 32; ++ch) {
-            const int n0 = (w.jbeg + j) * NT + ch * 32;
-            const float2* cs = reinterpret_cast<const float2*>(sc(s) + ch * 128);
-            uint32_t cv[32], sv[32];
-            float2 ss[16];
-            tmem_ld32(buf + ch * 32, sv);
-            tmem_ld32(buf + CB + ch * 32, cv);
-            tmem_wait_ld(sv);
-            tmem_wait_ld(cv);
+          for (int ch = ch0; ch < ch0 + CPW; ++ch) {
+          const int n0 = (w.jbeg + j) * NT + ch * 32;
+          const float4* cs = reinterpret_cast<const float4*>(sc(s) + ch * 128);       // r of four keys
+          float2 ss[G > 1 ? 16 : 1];
+          tmem_ld32(buf + ch * 32, sv);
+          tmem_ld32(buf + CB + ch * 32, cv);
+          tmem_wait_ld(sv);
+          tmem_wait_ld(cv);
+          read_done();
+          if constexpr (G > 1) {
 #pragma unroll
             for (int g = 0; g < G; ++g) {
               if (g > 0) {
@@ -397,40 +483,46 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
                 ss[c / 2] = g == 0 ? __fmul2_rn(s2, s2) : __ffma2_rn(s2, s2, ss[c / 2]);
               }
             }
-            float2 d2 = make_float2(0.f, 0.f), m2 = make_float2(0.f, 0.f);
-            // two copies of the loop, chosen once per tile: the causal test exists on diagonal tiles only
-            auto sums = [&](auto masked) {
+          }
+          float2 d2 = make_float2(0.f, 0.f), m2 = make_float2(0.f, 0.f);
+          // two copies of the loop, chosen once per tile: the causal test exists on diagonal tiles only
+          auto sums = [&](auto masked) {
 #pragma unroll
-              for (int c = 0; c < 32; c += 2) {
-                float2 a2 = __fmul2_rn(ss[c / 2], cs[c / 2]);
+            for (int c = 0; c < 32; c += 4) {
+              const float4 r4 = cs[c / 4];
+#pragma unroll
+              for (int e = 0; e < 4; e += 2) {
+                const float2 s2 = make_float2(__uint_as_float(sv[c + e]), __uint_as_float(sv[c + e + 1]));
+                float2 a2 = __fmul2_rn(G > 1 ? ss[G > 1 ? (c + e) / 2 : 0] : __fmul2_rn(s2, s2), e == 0 ? make_float2(r4.x, r4.y) : make_float2(r4.z, r4.w));
                 if constexpr (decltype(masked)::value) {
-                  if (n0 + c > grow) a2.x = 0.f;
-                  if (n0 + c + 1 > grow) a2.y = 0.f;
+                  if (n0 + c + e > grow) a2.x = 0.f;
+                  if (n0 + c + e + 1 > grow) a2.y = 0.f;
                 }
                 d2 = __fadd2_rn(d2, a2);
-                m2 = __ffma2_rn(a2, make_float2(__uint_as_float(cv[c]), __uint_as_float(cv[c + 1])), m2);
+                m2 = __ffma2_rn(a2, make_float2(__uint_as_float(cv[c + e]), __uint_as_float(cv[c + e + 1])), m2);
               }
-            };
-            if (n0 + 31 > w.m0) sums(std::true_type{}); else sums(std::false_type{});
-            sum_d += d2.x + d2.y;
-            sum_m += m2.x + m2.y;
+            }
+          };
+          if (n0 + 31 > w.m0) sums(std::true_type{}); else sums(std::false_type{});
+          sum_d += d2.x + d2.y;
+          sum_m += m2.x + m2.y;
           }
-          end();                                 // nothing is stored; the buffer is handed on as it is
+          end();                                 // nothing is stored
         }
         if (!ok) break;
-        // the groups' shares of a row meet, in a fixed order
-        float2* part = reinterpret_cast<float2*>(base + OFF_PART) + (ni & 1) * 384 + rowl;
-        part[grp * MT] = make_float2(sum_d, sum_m);
-        asm volatile("bar.sync 1, %0;" ::"n"(NBUF * 128) : "memory");
+        // the sets' shares of a row meet, in a fixed order
+        float2* part = reinterpret_cast<float2*>(base + OFF_PART) + (ni & 1) * 512 + rowl;
+        part[set * MT] = make_float2(sum_d, sum_m);
+        asm volatile("bar.sync 1, %0;" ::"n"(SETS * 128) : "memory");
         float dt = 0.f, mt = 0.f;
 #pragma unroll
-        for (int g = 0; g < NBUF; ++g) {
+        for (int g = 0; g < SETS; ++g) {
           dt += part[g * MT].x;
           mt += part[g * MT].y;
         }
         inv_row = dt > 0.f ? 1.f / dt : 0.f;
         del_row = mt * inv_row;
-        if (grp == 0 && grow < args.Tlen)
+        if (set == 0 && grow < args.Tlen)
           *reinterpret_cast<float2*>(args.stats + ((size_t)w.bh * args.Tlen + grow) * 2) = make_float2(inv_row, del_row);
       }
       // ---- weights ----
@@ -438,36 +530,76 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
         ok = begin(t0 + j);
         if (!ok) break;
         const int s = (t0 + j) % NSTAGE;
-        const int jt = MODE == MODE_DQ ? j - w.ntiles : j;
-        uint32_t held[NS == 3 && MODE == MODE_DKV ? 32 : 1];       // the second and third terms of E of the first chunk
 #pragma unroll
-        for (int ch = 0; ch < NT / 32; ++ch) {
-          const int n0 = (w.jbeg + jt) * NT + ch * 32;
-          auto dead = [&](int c) { return MODE == MODE_DQ ? n0 + c > grow : n0 + c < grow; };
-          const bool diag = MODE == MODE_DQ ? n0 + 31 > w.m0 : n0 < w.m0 + MT - 1;
-          uint32_t cv[32], sv[32];
-          tmem_ld32(buf + ch * 32, sv);
-          tmem_ld32(buf + CB + ch * 32, cv);
-          tmem_wait_ld(sv);
-          tmem_wait_ld(cv);
-          if constexpr (NS == 3 && MODE == MODE_DKV) {
-            if (ch == 1) {                       // the columns of the second chunk's scores are free now
-              const uint32_t (&e1)[16] = *reinterpret_cast<const uint32_t (*)[16]>(&held[0]);
-              const uint32_t (&e2)[16] = *reinterpret_cast<const uint32_t (*)[16]>(&held[16]);
-              tmem_st16(buf + geo::e_col(0, 1), e1);
-              tmem_st16(buf + geo::e_col(0, 2), e2);
+        for (int cc = 0; cc < CPW; ++cc) {
+        const int ch = ch0 + cc;
+        const int n0 = (w.jbeg + (MODE == MODE_DQ ? j - w.ntiles : j)) * NT + ch * 32;
+        auto dead = [&](int c) { return MODE == MODE_DQ ? n0 + c > grow : n0 + c < grow; };
+        const bool diag = MODE == MODE_DQ ? n0 + 31 > w.m0 : n0 < w.m0 + MT - 1;
+        const float4* cs = reinterpret_cast<const float4*>(sc(s) + ch * (MODE == MODE_DQ ? 128 : 256));
+        tmem_ld32(buf + ch * 32, sv);
+        tmem_ld32(buf + CB + ch * 32, cv);
+        tmem_wait_ld(sv);
+        tmem_wait_ld(cv);
+        read_done();
+        if constexpr (G == 1) {
+          both_read();
+          // the outputs of two steps back have read this buffer's weights
+          if (SEP && n_out > 0) ok = wait_or_abort(bar(BAR_PFREE + grp), (n_out - 1) & 1, abort_flag);
+          if (!ok) break;
+          // e = (c - dout.o) r s, or (c - dout_t.o_t) s / D_t with p = s^2 / D_t; sixteen columns at a time
+          auto weigh = [&](auto masked) {
+#pragma unroll
+            for (int c0 = 0; c0 < 32; c0 += 16) {
+              uint32_t pe[NS][8], pp[MODE == MODE_DKV ? NS : 1][8];
+#pragma unroll
+              for (int c = c0; c < c0 + 16; c += 2) {
+                const float2 s2 = make_float2(__uint_as_float(sv[c]), __uint_as_float(sv[c + 1]));
+                const float2 c2 = make_float2(__uint_as_float(cv[c]), __uint_as_float(cv[c + 1]));
+                float2 e2, p2 = make_float2(0.f, 0.f);
+                if (MODE == MODE_DQ) {
+                  const float4 r4 = cs[c / 4];
+                  e2 = __fmul2_rn(__fmul2_rn(__fadd2_rn(c2, make_float2(-del_row, -del_row)), (c & 2) ? make_float2(r4.z, r4.w) : make_float2(r4.x, r4.y)), s2);
+                } else {
+                  const float4 st = cs[c / 2];                                  // (1/D, dout.o) of two queries
+                  const float2 t2 = __fmul2_rn(s2, make_float2(st.x, st.z));    // s / D
+                  p2 = __fmul2_rn(t2, s2);
+                  e2 = __fmul2_rn(__fadd2_rn(c2, make_float2(-st.y, -st.w)), t2);
+                }
+                if constexpr (decltype(masked)::value) {
+                  if (dead(c)) { e2.x = 0.f; p2.x = 0.f; }
+                  if (dead(c + 1)) { e2.y = 0.f; p2.y = 0.f; }
+                }
+                uint32_t term[NS];
+                split_pack<NS>(e2, term);
+#pragma unroll
+                for (int i = 0; i < NS; ++i) pe[i][(c - c0) / 2] = term[i];
+                if constexpr (MODE == MODE_DKV) {
+                  split_pack<NS>(p2, term);
+#pragma unroll
+                  for (int i = 0; i < NS; ++i) pp[i][(c - c0) / 2] = term[i];
+                }
+              }
+#pragma unroll
+              for (int i = 0; i < NS; ++i) {
+                tmem_st8(lanes + geo::e_col(grp, 0, i) + ch * 16 + c0 / 2, pe[i]);
+                if constexpr (MODE == MODE_DKV) tmem_st8(lanes + geo::p_col(grp, i) + ch * 16 + c0 / 2, pp[i]);
+              }
             }
-          }
-          // f: e = f s.  MODE_DQ: (c - dout.o) r;  MODE_DKV: (c - dout_t.o_t) / D_t;  over c in place
+          };
+          if (diag) weigh(std::true_type{}); else weigh(std::false_type{});
+        } else {
+          // f: e = f s, over c in place
           auto factors = [&](auto masked) {
 #pragma unroll
             for (int c = 0; c < 32; c += 2) {
               const float2 c2 = make_float2(__uint_as_float(cv[c]), __uint_as_float(cv[c + 1]));
               float2 f;
               if (MODE == MODE_DQ) {
-                f = __fmul2_rn(__fadd2_rn(c2, make_float2(-del_row, -del_row)), reinterpret_cast<const float2*>(sc(s) + ch * 128)[c / 2]);
+                const float4 r4 = cs[c / 4];
+                f = __fmul2_rn(__fadd2_rn(c2, make_float2(-del_row, -del_row)), (c & 2) ? make_float2(r4.z, r4.w) : make_float2(r4.x, r4.y));
               } else {
-                const float4 st = reinterpret_cast<const float4*>(sc(s) + ch * 256)[c / 2];     // (1/D, dout.o) of two queries
+                const float4 st = cs[c / 2];
                 f = __fmul2_rn(__fadd2_rn(c2, make_float2(-st.y, -st.w)), make_float2(st.x, st.z));
               }
               if constexpr (decltype(masked)::value) {
@@ -479,64 +611,59 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
             }
           };
           if (diag) factors(std::true_type{}); else factors(std::false_type{});
-          float2 ss[MODE == MODE_DKV && G > 1 ? 16 : 1];
+          float2 ss[MODE == MODE_DKV ? 16 : 1];
+          uint32_t pk[16];
 #pragma unroll
           for (int g = 0; g < G; ++g) {
             if (g > 0) {
               tmem_ld32(buf + g * NT + ch * 32, sv);
               tmem_wait_ld(sv);
             }
-            uint32_t pk[NS][16];
 #pragma unroll
             for (int c = 0; c < 32; c += 2) {
               const float2 s2 = make_float2(__uint_as_float(sv[c]), __uint_as_float(sv[c + 1]));
-              if constexpr (MODE == MODE_DKV && G > 1) ss[c / 2] = g == 0 ? __fmul2_rn(s2, s2) : __ffma2_rn(s2, s2, ss[c / 2]);
-              uint32_t term[NS];
-              split_pack<NS>(__fmul2_rn(make_float2(__uint_as_float(cv[c]), __uint_as_float(cv[c + 1])), s2), term);
-#pragma unroll
-              for (int i = 0; i < NS; ++i) pk[i][c / 2] = term[i];
+              if constexpr (MODE == MODE_DKV) ss[c / 2] = g == 0 ? __fmul2_rn(s2, s2) : __ffma2_rn(s2, s2, ss[c / 2]);
+              const float2 e2 = __fmul2_rn(make_float2(__uint_as_float(cv[c]), __uint_as_float(cv[c + 1])), s2);
+              pk[c / 2] = pack_bf16(e2.x, e2.y);
             }
-#pragma unroll
-            for (int i = 0; i < NS; ++i) {
-              if (NS == 3 && MODE == MODE_DKV && ch == 0 && i > 0) {
-#pragma unroll
-                for (int e = 0; e < 16; ++e) held[NS == 3 && MODE == MODE_DKV ? (i - 1) * 16 + e : 0] = pk[i][e];
-              } else {
-                tmem_st16(buf + geo::e_col(g, i) + ch * 16, pk[i]);
-              }
-            }
+            both_read();
+            tmem_st16(lanes + geo::e_col(grp, g, 0) + ch * 16, pk);
           }
-          if (MODE == MODE_DKV) {
+          if constexpr (MODE == MODE_DKV) {
             // p = sum_g s_g^2 / D_t
-            uint32_t pk[NS][16];
             auto weights = [&](auto masked) {
 #pragma unroll
               for (int c = 0; c < 32; c += 2) {
-                const float4 st = reinterpret_cast<const float4*>(sc(s) + ch * 256)[c / 2];
-                const float2 s2 = make_float2(__uint_as_float(sv[c]), __uint_as_float(sv[c + 1]));
-                float2 p2 = __fmul2_rn(G > 1 ? ss[MODE == MODE_DKV && G > 1 ? c / 2 : 0] : __fmul2_rn(s2, s2), make_float2(st.x, st.z));
+                const float4 st = cs[c / 2];
+                float2 p2 = __fmul2_rn(ss[c / 2], make_float2(st.x, st.z));
                 if constexpr (decltype(masked)::value) {
                   if (dead(c)) p2.x = 0.f;
                   if (dead(c + 1)) p2.y = 0.f;
                 }
-                uint32_t term[NS];
-                split_pack<NS>(p2, term);
-#pragma unroll
-                for (int i = 0; i < NS; ++i) pk[i][c / 2] = term[i];
+                pk[c / 2] = pack_bf16(p2.x, p2.y);
               }
             };
             if (diag) weights(std::true_type{}); else weights(std::false_type{});
-#pragma unroll
-            for (int i = 0; i < NS; ++i) tmem_st16(buf + geo::p_col(i) + ch * 16, pk[i]);
+            tmem_st16(lanes + geo::p_col(grp, 0) + ch * 16, pk);
           }
         }
+        }
+        if (!ok) break;
         tmem_wait_st();
+        ++n_out;
         end();
       }
       t0 += w.nsteps;
+      // the next item's fixed tiles go to TMEM (the item before, in the same buffer, is complete) before the wait for this
+      // item's last MMAs
+      if (XT && set < 2 && more_n && ok) copy_x(ni + 1);
+      const Item cur = w;
+      n = nn;
+      w = wn;
+      more = more_n;
       if (!ok) break;
-      if (grp > 1) continue;
-      // ---- epilogue: groups 0 and 1 ----
+      if (set > 1) continue;
+      // ---- epilogue: sets 0 and 1 ----
       ok = wait_or_abort(bar(BAR_ODONE), ni & 1, abort_flag) &&
            (MODE == MODE_DQ || wait_or_abort(bar(BAR_XFULL + (ni & 1)), (ni >> 1) & 1, abort_flag));   // (k is read below)
       if (!ok) break;
@@ -552,21 +679,21 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
           *reinterpret_cast<uint4*>(dst + c) = pkt;
         }
       };
-      const size_t row_off = ((size_t)w.bh * args.Tlen + grow) * D;
+      const size_t row_off = ((size_t)cur.bh * args.Tlen + grow) * D;
       if (MODE == MODE_DQ) {
-        // dq = 2 / D_t x the sum, 32 columns per group
+        // dq = 2 / D_t x the sum, 32 columns per set
         uint32_t a0[32];
         float x[32];
-        tmem_ld32(accu + grp * 32, a0);
+        tmem_ld32(accu + set * 32, a0);
         tmem_wait_ld(a0);
         tc_fence_before();
         mbar_arrive(bar(BAR_OFREE));
         const float f = 2.f * inv_row;
 #pragma unroll
         for (int c = 0; c < 32; ++c) x[c] = f * __uint_as_float(a0[c]);
-        if (grow < args.Tlen) store32(args.out0 + row_off + grp * 32, x);
+        if (grow < args.Tlen) store32(args.out0 + row_off + set * 32, x);
       } else {
-        // group 0: dk = r (2 u - r (k . 2 u) k);  group 1: dv = r dv~
+        // set 0: dk = r (2 u - r (k . 2 u) k);  set 1: dv = r dv~
         const unsigned char* kt = x1(ni & 1);
         auto krow = [&](int half, float (&kf)[32]) {
 #pragma unroll
@@ -600,13 +727,13 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
 #pragma unroll 1
         for (int half = 0; half < 2; ++half) {
           float x[32];
-          if (grp == 0) krow(half, kf);
-          tmem_ld32(accu + (grp == 0 ? 64 : 0) + half * 32, a0);
+          if (set == 0) krow(half, kf);
+          tmem_ld32(accu + (set == 0 ? 64 : 0) + half * 32, a0);
           tmem_wait_ld(a0);
 #pragma unroll
           for (int c = 0; c < 32; ++c)
-            x[c] = grp == 0 ? 2.f * r * (__uint_as_float(a0[c]) - proj * kf[c]) : r * __uint_as_float(a0[c]);
-          if (grow < args.Tlen) store32((grp == 0 ? args.out0 : args.out1) + row_off + half * 32, x);
+            x[c] = set == 0 ? 2.f * r * (__uint_as_float(a0[c]) - proj * kf[c]) : r * __uint_as_float(a0[c]);
+          if (grow < args.Tlen) store32((set == 0 ? args.out0 : args.out1) + row_off + half * 32, x);
         }
         tc_fence_before();
         mbar_arrive(bar(BAR_OFREE));
@@ -620,7 +747,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (warp == 1 && elect_one()) {
+  if ((warp == 1 || warp == 2) && elect_one()) {
     mma_commit(bar(BAR_DRAIN));
     mbar_wait(bar(BAR_DRAIN), 0);
   }
