@@ -325,6 +325,7 @@ struct Prepared {
   int C;
   bool states;          // chunked form on the chunk-state and attend kernels
   StatePlan sp;         // its chunks
+  bool simt_att;        // sequential chunked form in fp32 on narrow rows: kata_simt_attend.cu
   bool pad;             // bf16 rows narrower than 64 are zero-padded to 64 so that the tensor-core kernels apply
   size_t pad_bytes;     // one padded tensor [B*H*T][64] bf16 (q, k, v, out: four of them at the start of the scratch)
 };
@@ -405,7 +406,7 @@ int prepare(int fn, const void* q, const void* k, const void* v, void* out, int 
   r.C = fn == KATA_FN_QUADRATIC ? kChunk : C;
   r.plan = ScanPlan{(T + r.C - 1) / r.C, 0, 1, 0};
   r.state_elems = 0;
-  r.states = false;
+  r.states = r.simt_att = false;
   if (fn == KATA_FN_QUADRATIC && r.tensor) r.pad = false;      // the attend kernel reads narrow rows as they are
   r.inner_bytes = (fn == KATA_FN_QUADRATIC && r.tensor) ? tc_quadratic_workspace_bytes(kp) : 0;
   if (fn != KATA_FN_QUADRATIC) {
@@ -416,6 +417,12 @@ int prepare(int fn, const void* q, const void* k, const void* v, void* out, int 
     if (st != KATA_OK) return st;
     r.inner_bytes = inner_workspace(fn, r.plan, kp, r.state_elems);
     const bool state_in = r.o.s_init != nullptr, state_out = r.o.s_pre != nullptr;
+    r.simt_att = fn == KATA_FN_CHUNKED && !r.tensor && r.o.inter_chunk == KATA_SEQUENTIAL && !state_in && !state_out &&
+                 simt_attend_supported(r.p);
+    if (r.simt_att) {
+      r.inner_bytes = align_up(simt_attend_workspace_bytes(r.p));
+      return KATA_OK;
+    }
     r.states = fn == KATA_FN_CHUNKED && r.tensor && r.p.feature_order == 2 && !stream_kernel_forced() &&
                ((r.o.inter_chunk == KATA_SEQUENTIAL && (!(state_in || state_out) || !short_state_call(B * H, T))) ||
                 (auto_scan && (long long)B * H * T >= kStreamScanTokens));
@@ -473,6 +480,8 @@ int run_device(int fn, Prepared& r, void* ws) {
     const bool use_scan = (fn == KATA_FN_CHUNK_STATE_SCAN) || r.plan.n_groups > 1;
     if (r.tensor && P.feature_order == 1) {
       tc_order1(P, r.plan, use_scan, r.C, wsf, r.o.device_status, ctx);
+    } else if (r.simt_att) {
+      simt_attend(P, wsf, ctx);
     } else if (r.states) {
       tc_chunked_states(P, r.sp, ws, r.o.device_status, r.o.s_init, r.o.z_init, r.o.s_pre, r.o.z_pre, r.o.state_layout, ctx);
     } else if (r.tensor) {

@@ -60,6 +60,10 @@ struct ScanPlan {
 
 // SIMT kernels (fp32 arithmetic; any supported shape and element type)
 void simt_quadratic(const Problem& p, LaunchCtx& ctx);
+// fp32 rows of 16 or 32 entries: chunk states in parallel, then blocks of queries (kata_simt_attend.cu)
+bool simt_attend_supported(const Problem& p);
+size_t simt_attend_workspace_bytes(const Problem& p);
+void simt_attend(const Problem& p, float* ws, LaunchCtx& ctx);
 size_t simt_chunked_state_elems(int d_k, int d_v);  // floats of internal state per (b,h,group)
 int simt_chunked_slices(int d_k, int d_v);          // CTAs per (b,h,group)
 // Inclusive Hillis-Steele scan over the first g_used of n_groups group states x[BH][n_groups][E]

@@ -1,0 +1,329 @@
+// Chunked KATA forward in fp32 on plain FMAs for rows of 16 or 32 entries (full lift, no state handed over): the states
+// before chunks of 256 tokens, all chunks in parallel, then blocks of 64 queries over the state and the keys of their
+// chunk.  Short sequences are one chunk: one launch, the quadratic form.
+//   state_loc_kernel     S_loc = sum_t w psi(k_hat_t) [v_t, 1] over a chunk: thread = feature pair a <= b (w = 2 off the
+//                        diagonal: the lift is symmetric), its DV + 1 sums in registers, rows broadcast from shared memory
+//   state_prefix_kernel  running sum over the chunks, in order
+//   attend_kernel        lane = two queries; the eight warps of a CTA share out the feature rows of the state and the tiles
+//                        of 32 keys, rows broadcast from shared memory (16 bytes per load feed 8 FMAs), and add their
+//                        numerators and normalisers in a fixed order at the end
+// What bounds it: FMAs.  The walk over the chunks of a head by one CTA (kata_simt_chunked.cu) was a chain of 21 us per 64
+// tokens; 2 heads x 512 tokens of 16 entries took 171 us.
+// Chunk length: at 16 entries a query costs 34 FMAs per key of its chunk and 2.3 k for the state, at 32 66 and 17 k: the
+// lengths up to which one chunk is the cheaper are about 1000 and 1500.
+#include "kata_common.cuh"
+
+namespace kata {
+namespace {
+
+constexpr int QB = 64;           // queries per CTA
+constexpr int NW = 8;            // warps per CTA
+constexpr int CHUNK = 256;       // tokens per chunk
+
+__host__ __device__ constexpr int n_features(int d) { return d * (d + 1) / 2; }
+__host__ __device__ constexpr int state_stride(int dv) { return dv + 4; }       // [values | normaliser | 3 x padding]
+
+__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+
+// rows [t0, t0 + n) of x (D entries each) into dst, normalised; rows from Tlen on are zero.  All threads of `nthr` (a multiple
+// of D / 4, whole warps).
+template <int D, bool NORM>
+__device__ __forceinline__ void load_rows(const float* __restrict__ x, float* dst, int t0, int n, int Tlen, int thr, int nthr) {
+  constexpr int PR = D / 4;      // lanes per row
+  for (int i = thr; i < n * PR; i += nthr) {
+    const int row = t0 + i / PR;
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (row < Tlen) a = ld4(x + (size_t)row * D + (i % PR) * 4);
+    if (NORM) {
+      float ss = a.x * a.x + a.y * a.y + a.z * a.z + a.w * a.w;
+#pragma unroll
+      for (int off = 1; off < PR; off <<= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
+      const float r = rsqrt_or_zero(ss);
+      a.x *= r; a.y *= r; a.z *= r; a.w *= r;
+    }
+    *reinterpret_cast<float4*>(dst + i * 4) = a;
+  }
+}
+
+template <int DK, int DV>
+__global__ void __launch_bounds__((n_features(DK) + 31) / 32 * 32)
+state_loc_kernel(const float* __restrict__ k, const float* __restrict__ v, float* __restrict__ S, int Tlen, int n_chunks) {
+  constexpr int NF = n_features(DK), SP = state_stride(DV), NTHR = (NF + 31) / 32 * 32, TB = 64;
+  __shared__ __align__(16) float ks[TB * DK], vs[TB * DV];
+  const int c = blockIdx.x, bh = blockIdx.y, tid = threadIdx.x;
+  int a = 0, rem = tid < NF ? tid : 0;
+  while (rem >= DK - a) {
+    rem -= DK - a;
+    ++a;
+  }
+  const int b = a + rem;
+  float acc[DV], den = 0.f;
+#pragma unroll
+  for (int i = 0; i < DV; ++i) acc[i] = 0.f;
+  for (int t0 = c * CHUNK; t0 < (c + 1) * CHUNK; t0 += TB) {
+    __syncthreads();
+    load_rows<DK, true>(k + (size_t)bh * Tlen * DK, ks, t0, TB, Tlen, tid, NTHR);
+    load_rows<DV, false>(v + (size_t)bh * Tlen * DV, vs, t0, TB, Tlen, tid, NTHR);
+    __syncthreads();
+#pragma unroll 4
+    for (int t = 0; t < TB; ++t) {
+      const float w = ks[t * DK + a] * ks[t * DK + b];
+      den += w;
+#pragma unroll
+      for (int i = 0; i < DV; i += 4) {
+        const float4 x = ld4(vs + t * DV + i);
+        acc[i] = fmaf(w, x.x, acc[i]);
+        acc[i + 1] = fmaf(w, x.y, acc[i + 1]);
+        acc[i + 2] = fmaf(w, x.z, acc[i + 2]);
+        acc[i + 3] = fmaf(w, x.w, acc[i + 3]);
+      }
+    }
+  }
+  if (tid >= NF) return;
+  const float m = a == b ? 1.f : 2.f;
+  float* dst = S + (((size_t)bh * n_chunks + c + 1) * NF + tid) * SP;
+#pragma unroll
+  for (int i = 0; i < DV; i += 4) *reinterpret_cast<float4*>(dst + i) = make_float4(m * acc[i], m * acc[i + 1], m * acc[i + 2], m * acc[i + 3]);
+  *reinterpret_cast<float4*>(dst + DV) = make_float4(m * den, 0.f, 0.f, 0.f);
+}
+
+// S[1 .. n_chunks - 1] of every head: running sums; n4 = float4s per state, eight loads in flight
+__global__ void __launch_bounds__(128) state_prefix_kernel(float4* __restrict__ S, int n4, int n_chunks) {
+  cudaGridDependencySynchronize();
+  const int i = blockIdx.x * 128 + threadIdx.x;
+  if (i >= n4) return;
+  float4* p = S + (size_t)blockIdx.y * n_chunks * n4 + i;
+  float4 run = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int c0 = 1; c0 < n_chunks; c0 += 8) {
+    float4 x[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (c0 + u < n_chunks) x[u] = p[(size_t)(c0 + u) * n4];
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (c0 + u < n_chunks) {
+        run.x += x[u].x; run.y += x[u].y; run.z += x[u].z; run.w += x[u].w;
+        p[(size_t)(c0 + u) * n4] = run;
+      }
+  }
+}
+
+template <int DK, int DV> constexpr int attend_smem_floats() {
+  const int tiles = QB * DK + NW * 32 * (DK + DV), red = NW * (DV + 1) * QB;
+  return tiles > red ? tiles : red;
+}
+
+template <int DK, int DV>
+__global__ void __launch_bounds__(NW * 32) attend_kernel(const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ v,
+                                                         float* __restrict__ out, const float* __restrict__ S, int Tlen, int chunk,
+                                                         int n_chunks) {
+  constexpr int NF = n_features(DK), SP = state_stride(DV);
+  extern __shared__ __align__(16) float sm[];
+  float* qs = sm;                                          // [DK][QB]
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  float* kt = sm + QB * DK + warp * 32 * (DK + DV);        // this warp's tile: k_hat [32][DK], v [32][DV]
+  float* vt = kt + 32 * DK;
+  const int q0 = ((int)gridDim.x - 1 - (int)blockIdx.x) * QB, bh = blockIdx.y;     // last blocks first
+  const float* kh = k + (size_t)bh * Tlen * DK;
+  const float* vh = v + (size_t)bh * Tlen * DV;
+  const float* qh = q + (size_t)bh * Tlen * DK;
+  if (S != nullptr) cudaGridDependencySynchronize();
+
+  for (int i = tid; i < QB * DK; i += NW * 32) {
+    const int row = i / DK, a = i % DK;
+    qs[a * QB + row] = q0 + row < Tlen ? qh[(size_t)(q0 + row) * DK + a] : 0.f;
+  }
+  __syncthreads();
+  float qa[DK], qb[DK], na[DV], nb[DV], da = 0.f, db = 0.f;      // queries q0 + lane and q0 + 32 + lane
+#pragma unroll
+  for (int i = 0; i < DK; ++i) {
+    qa[i] = qs[i * QB + lane];
+    qb[i] = qs[i * QB + 32 + lane];
+  }
+#pragma unroll
+  for (int i = 0; i < DV; ++i) na[i] = nb[i] = 0.f;
+  auto add = [&](const float* row, float wa, float wb) {
+#pragma unroll
+    for (int i = 0; i < DV; i += 4) {
+      const float4 x = ld4(row + i);
+      na[i] = fmaf(wa, x.x, na[i]);
+      na[i + 1] = fmaf(wa, x.y, na[i + 1]);
+      na[i + 2] = fmaf(wa, x.z, na[i + 2]);
+      na[i + 3] = fmaf(wa, x.w, na[i + 3]);
+      nb[i] = fmaf(wb, x.x, nb[i]);
+      nb[i + 1] = fmaf(wb, x.y, nb[i + 1]);
+      nb[i + 2] = fmaf(wb, x.z, nb[i + 2]);
+      nb[i + 3] = fmaf(wb, x.w, nb[i + 3]);
+    }
+  };
+  // ---- the state before the chunk ----
+  const int c = q0 / chunk;
+  if (c > 0) {
+    const float* Sc = S + ((size_t)bh * n_chunks + c) * NF * SP;
+    const int f0 = NF * warp / NW, f1 = NF * (warp + 1) / NW;
+    int a = 0, rem = f0;
+    while (rem >= DK - a) {
+      rem -= DK - a;
+      ++a;
+    }
+    int b = a + rem;
+    float xa = qs[a * QB + lane], xb = qs[a * QB + 32 + lane];
+    // sixteen rows at a time through this warp's tile buffer, the next sixteen on their way meanwhile
+    constexpr int RB = 16, N4 = RB * SP / 4, PL = (N4 + 31) / 32;
+    float4 pre[PL];
+    auto fetch = [&](int f) {
+      const int n4 = (f1 - f < RB ? f1 - f : RB) * SP / 4;
+#pragma unroll
+      for (int i = 0; i < PL; ++i)
+        if (lane + 32 * i < n4) pre[i] = ld4(Sc + (size_t)f * SP + (lane + 32 * i) * 4);
+    };
+    fetch(f0);
+    for (int fb = f0; fb < f1; fb += RB) {
+      __syncwarp();
+#pragma unroll
+      for (int i = 0; i < PL; ++i)
+        if (lane + 32 * i < N4) *reinterpret_cast<float4*>(kt + (lane + 32 * i) * 4) = pre[i];
+      __syncwarp();
+      if (fb + RB < f1) fetch(fb + RB);
+      const int n = f1 - fb < RB ? f1 - fb : RB;
+#pragma unroll 2
+      for (int r = 0; r < n; ++r) {
+        const float wa = xa * qs[b * QB + lane], wb = xb * qs[b * QB + 32 + lane];
+        const float* row = kt + r * SP;
+        add(row, wa, wb);
+        const float z = row[DV];
+        da = fmaf(wa, z, da);
+        db = fmaf(wb, z, db);
+        if (++b == DK) {
+          b = ++a;
+          if (a < DK) {
+            xa = qs[a * QB + lane];
+            xb = qs[a * QB + 32 + lane];
+          }
+        }
+      }
+    }
+  }
+  // ---- the keys of the chunk, tiles of 32 ----
+  const int k_end = min(q0 + QB, Tlen);
+  for (int t0 = c * chunk + warp * 32; t0 < k_end; t0 += NW * 32) {
+    __syncwarp();
+    load_rows<DK, true>(kh, kt, t0, 32, Tlen, lane, 32);
+    load_rows<DV, false>(vh, vt, t0, 32, Tlen, lane, 32);
+    __syncwarp();
+    const bool diag = t0 + 31 > q0;
+#pragma unroll 2
+    for (int t = 0; t < 32; ++t) {
+      float sa = 0.f, sb = 0.f;
+#pragma unroll
+      for (int i = 0; i < DK; i += 4) {
+        const float4 x = ld4(kt + t * DK + i);
+        sa = fmaf(qa[i], x.x, sa);
+        sa = fmaf(qa[i + 1], x.y, sa);
+        sa = fmaf(qa[i + 2], x.z, sa);
+        sa = fmaf(qa[i + 3], x.w, sa);
+        sb = fmaf(qb[i], x.x, sb);
+        sb = fmaf(qb[i + 1], x.y, sb);
+        sb = fmaf(qb[i + 2], x.z, sb);
+        sb = fmaf(qb[i + 3], x.w, sb);
+      }
+      float wa = sa * sa, wb = sb * sb;
+      if (diag) {
+        if (t0 + t > q0 + lane) wa = 0.f;
+        if (t0 + t > q0 + 32 + lane) wb = 0.f;
+      }
+      da += wa;
+      db += wb;
+      add(vt + t * DV, wa, wb);
+    }
+  }
+  // ---- the warps' shares, in order ----
+  __syncthreads();
+  float* red = sm + warp * (DV + 1) * QB;                  // [warp][DV + 1][QB]
+#pragma unroll
+  for (int i = 0; i < DV; ++i) {
+    red[i * QB + lane] = na[i];
+    red[i * QB + 32 + lane] = nb[i];
+  }
+  red[DV * QB + lane] = da;
+  red[DV * QB + 32 + lane] = db;
+  __syncthreads();
+  const int row = tid & (QB - 1), part = tid / QB;         // four threads per query
+  float den = 0.f;
+#pragma unroll
+  for (int w = 0; w < NW; ++w) den += sm[(w * (DV + 1) + DV) * QB + row];
+  const float inv = den > 0.f ? 1.f / den : 0.f;
+  if (q0 + row >= Tlen) return;
+  constexpr int CPT = DV / 4;                              // columns per thread
+  float* dst = out + ((size_t)bh * Tlen + q0 + row) * DV + part * CPT;
+#pragma unroll
+  for (int i = 0; i < CPT; i += 4) {
+    float x[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int w = 0; w < NW; ++w)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) x[e] += sm[(w * (DV + 1) + part * CPT + i + e) * QB + row];
+    *reinterpret_cast<float4*>(dst + i) = make_float4(x[0] * inv, x[1] * inv, x[2] * inv, x[3] * inv);
+  }
+}
+
+int one_chunk_tokens(int d_k) { return d_k == 16 ? 1024 : 1536; }
+
+template <int DK, int DV> void run(const Problem& p, float* S, LaunchCtx& ctx) {
+  const int BH = p.B * p.H;
+  const float *q = static_cast<const float*>(p.q), *k = static_cast<const float*>(p.k), *v = static_cast<const float*>(p.v);
+  const bool states = p.T > one_chunk_tokens(DK);
+  const int chunk = states ? CHUNK : (p.T + QB - 1) / QB * QB, n_chunks = (p.T + chunk - 1) / chunk;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.stream = ctx.stream;
+  bool ok = true;
+  if (states) {
+    state_loc_kernel<DK, DV><<<dim3(n_chunks - 1, BH), (n_features(DK) + 31) / 32 * 32, 0, ctx.stream>>>(k, v, S, p.T, n_chunks);
+    note_launch(ctx);
+    const int n4 = n_features(DK) * state_stride(DV) / 4;
+    cfg.gridDim = dim3((n4 + 127) / 128, BH);
+    cfg.blockDim = dim3(128);
+    cfg.numAttrs = 1;
+    ok = cudaLaunchKernelEx(&cfg, state_prefix_kernel, reinterpret_cast<float4*>(S), n4, n_chunks) == cudaSuccess;
+    ctx.launches += ok;
+  }
+  constexpr int smem = attend_smem_floats<DK, DV>() * (int)sizeof(float);
+  cfg.gridDim = dim3((p.T + QB - 1) / QB, BH);
+  cfg.blockDim = dim3(NW * 32);
+  cfg.dynamicSmemBytes = smem;
+  cfg.numAttrs = states ? 1 : 0;
+  ok = ok && cudaFuncSetAttribute(attend_kernel<DK, DV>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
+       cudaLaunchKernelEx(&cfg, attend_kernel<DK, DV>, q, k, v, static_cast<float*>(p.out), (const float*)(states ? S : nullptr), p.T, chunk,
+                          n_chunks) == cudaSuccess;
+  if (!ok) {
+    cudaGetLastError();
+    ctx.status = KATA_ERR_CUDA;
+    return;
+  }
+  ++ctx.launches;
+}
+
+}  // namespace
+
+bool simt_attend_supported(const Problem& p) {
+  return p.dtype == KATA_F32 && p.feature_order == 2 && p.groups == 1 && p.d_k <= 32 && p.d_v <= 32;
+}
+
+size_t simt_attend_workspace_bytes(const Problem& p) {
+  if (p.T <= one_chunk_tokens(p.d_k)) return 0;
+  return (size_t)p.B * p.H * ((p.T + CHUNK - 1) / CHUNK) * n_features(p.d_k) * state_stride(p.d_v) * sizeof(float);
+}
+
+void simt_attend(const Problem& p, float* ws, LaunchCtx& ctx) {
+  if (p.d_k == 16) {
+    if (p.d_v == 16) run<16, 16>(p, ws, ctx); else run<16, 32>(p, ws, ctx);
+  } else {
+    if (p.d_v == 16) run<32, 16>(p, ws, ctx); else run<32, 32>(p, ws, ctx);
+  }
+}
+
+}  // namespace kata

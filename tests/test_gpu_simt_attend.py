@@ -1,0 +1,28 @@
+"""GPU parity of the fp32 chunked form on narrow rows (chunk states of 256 tokens, blocks of 64 queries, tiles of 32 keys):
+edges of the blocks, of the chunks and of the lengths that run as one chunk."""
+import pytest
+
+from paper_2607_17419_b200 import binding as kb
+from paper_2607_17419_b200 import inputs
+
+from helpers import check, dev_tensors, oracle_full, to_numpy64
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("dk,dv", [(16, 16), (16, 32), (32, 16), (32, 32)])
+@pytest.mark.parametrize("T", [1, 31, 33, 64, 65, 1024, 1025, 1536, 1537, 2049, 2111])
+def test_simt_attend(dk, dv, T):
+    import torch
+    w = inputs.gaussian_workload(f"sa_{dk}_{dv}_{T}", "f32", 1, 2, T, dk, dv, 64, 7000 + T + dk)
+    for arr in (w.k_ref, w.k_dev):
+        arr[0, 0, [0, T - 1]] = 0               # a first key of zero: normaliser 0, output 0
+    q, k, v = dev_tensors(w)
+    o = kb.kata_fwd_chunked(q, k, v)
+    torch.cuda.synchronize()
+    assert kb.kata_last_impl() == kb.KATA_IMPL_SIMT
+    assert kb.kata_last_launch_count() == (3 if T > (1024 if dk == 16 else 1536) else 1)
+    assert torch.equal(o, kb.kata_fwd_chunked(q, k, v)), "fixed summation order"
+    assert torch.all(o[0, 0, 0] == 0)
+    for (b, h), r in oracle_full(w).items():
+        check(to_numpy64(o)[b, h], r, "f32", f"T={T} d={dk},{dv} head {h}")
