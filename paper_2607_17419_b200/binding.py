@@ -8,8 +8,11 @@ fails, an exception is raised.
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 from typing import Optional
+
+import torch
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(HERE, "libkata.so")
@@ -106,25 +109,42 @@ def status_string(status: int) -> str:
     return lib().kata_status_string(status).decode()
 
 
+_OPTS_SIZE = ctypes.sizeof(KataOpts)
+
+
 def make_opts(dtype: int, *, feature_order: int = 2, state_layout: int = KATA_LAYOUT_DIRECT,
               inter_chunk: int = KATA_SEQUENTIAL, impl: int = KATA_IMPL_AUTO, scan_group: int = 0,
               feature_groups: int = 0,
               workspace: int = 0, workspace_bytes: int = 0, s_pre: int = 0, z_pre: int = 0,
               device_status: int = 0, stream: int = 0, s_init: int = 0, z_init: int = 0) -> KataOpts:
-    o = KataOpts()
-    o.struct_size = ctypes.sizeof(KataOpts)
-    o.dtype, o.feature_order, o.state_layout = dtype, feature_order, state_layout
-    o.inter_chunk, o.impl, o.scan_group = inter_chunk, impl, scan_group
-    o.feature_groups = feature_groups
-    o.workspace, o.workspace_bytes = workspace or None, workspace_bytes
-    o.s_pre, o.z_pre = s_pre or None, z_pre or None
-    o.device_status, o.stream = device_status or None, stream or None
-    o.s_init, o.z_init = s_init or None, z_init or None
-    return o
+    # (one constructor call: setting the fields one by one costs 3 us of a 10 us call)
+    return KataOpts(_OPTS_SIZE, dtype, feature_order, state_layout, inter_chunk, impl, scan_group, feature_groups,
+                    workspace or None, workspace_bytes, s_pre or None, z_pre or None, device_status or None, stream or None,
+                    s_init or None, z_init or None)
 
 
 def kata_workspace_bytes(fn: int, B, H, T, d_k, d_v, C, opts: KataOpts) -> int:
     return int(lib().kata_workspace_bytes(fn, B, H, T, d_k, d_v, C, ctypes.byref(opts)))
+
+
+@functools.lru_cache(maxsize=4096)
+def _scratch_bytes(fn: int, B, H, T, d_k, d_v, C, dtype, order, layout, inter, impl, scan_group, groups, state_in: bool,
+                   state_out: bool, in_place: bool) -> int:
+    """kata_workspace_bytes as what it is: a function of the sizes, the options and which state pointers are set."""
+    o = make_opts(dtype, feature_order=order, state_layout=layout, inter_chunk=inter, impl=impl, scan_group=scan_group,
+                  feature_groups=groups, s_pre=256 if state_out else 0, z_pre=256 if state_out else 0,
+                  s_init=(256 if in_place else 512) if state_in else 0, z_init=(256 if in_place else 512) if state_in else 0)
+    return kata_workspace_bytes(fn, B, H, T, d_k, d_v, C, o)
+
+
+def _scratch(ws, fn: int, sizes, o: KataOpts, device) -> None:
+    """Point the options at scratch of the size the call needs."""
+    need = _scratch_bytes(fn, *sizes, o.dtype, o.feature_order, o.state_layout, o.inter_chunk, o.impl, o.scan_group,
+                          o.feature_groups, bool(o.s_init or o.z_init), bool(o.s_pre or o.z_pre),
+                          o.z_init is not None and o.z_init == o.z_pre)
+    ptr, size = (ws if ws is not None else _default_ws).get(need, device)
+    if size:
+        o.workspace, o.workspace_bytes = ptr, size
 
 
 def kata_scan_plan(fn: int, B, H, T, d_k, d_v, C, opts: KataOpts):
@@ -152,7 +172,6 @@ def kata_selftest_wait_timeout(device_status, report, max_polls: int = 1000, str
     `device_status` is an int32 CUDA tensor of one element (or None), `report` one of eight (the last is the flag in
     global memory that the flag wait is tried on: 0 on entry).  Returns the status code.
     """
-    import torch
     if stream is None:
         stream = torch.cuda.current_stream().cuda_stream
     return int(lib().kata_selftest_wait_timeout(device_status.data_ptr() if device_status is not None else None,
@@ -179,13 +198,19 @@ _FN_NAMES = {KATA_FN_QUADRATIC: "kata_fwd_quadratic", KATA_FN_CHUNKED: "kata_fwd
              KATA_FN_CHUNK_STATE_SCAN: "kata_chunk_state_scan"}
 
 
+_DTYPE_CODES = {torch.float32: KATA_F32, torch.bfloat16: KATA_BF16}
+
+
 def _dtype_code(t) -> int:
-    import torch
-    if t.dtype == torch.float32:
-        return KATA_F32
-    if t.dtype == torch.bfloat16:
-        return KATA_BF16
-    raise TypeError(f"unsupported dtype {t.dtype}")
+    try:
+        return _DTYPE_CODES[t.dtype]
+    except KeyError:
+        raise TypeError(f"unsupported dtype {t.dtype}") from None
+
+
+def _stream(device) -> int:
+    """Handle of torch's current stream on the device (without the stream object: 2 us of a 10 us call)."""
+    return torch._C._cuda_getCurrentRawStream(device.index)
 
 
 class Workspace:
@@ -195,12 +220,12 @@ class Workspace:
         self.buf = None
 
     def get(self, nbytes: int, device):
-        import torch
         if nbytes == 0:
             return 0, 0
-        if self.buf is None or self.buf.numel() < nbytes or self.buf.device != device:
-            self.buf = torch.empty(nbytes, dtype=torch.uint8, device=device)
-        return self.buf.data_ptr(), self.buf.numel()
+        buf = self.buf
+        if buf is None or buf.numel() < nbytes or buf.device != device:
+            self.buf = buf = torch.empty(nbytes, dtype=torch.uint8, device=device)
+        return buf.data_ptr(), buf.numel()
 
 
 _default_ws = Workspace()
@@ -208,7 +233,6 @@ _default_ws = Workspace()
 
 def _call(fn: int, q, k, v, out, C: int, *, host_io: bool = False, workspace: Optional[Workspace] = None,
           s_pre=None, z_pre=None, s_init=None, z_init=None, device_status=None, stream=None, **opt_kw):
-    import torch
     if not (q.is_contiguous() and k.is_contiguous() and v.is_contiguous()):
         raise ValueError("q, k, v must be contiguous [B,H,T,d]")
     B, H, T, d_k = q.shape
@@ -217,17 +241,14 @@ def _call(fn: int, q, k, v, out, C: int, *, host_io: bool = False, workspace: Op
         out = torch.empty_like(v)
     dev = torch.device("cuda", torch.cuda.current_device()) if host_io else q.device
     if stream is None:
-        stream = torch.cuda.current_stream(dev).cuda_stream
+        stream = _stream(dev)
     opts = make_opts(_dtype_code(q), stream=stream,
                      s_pre=s_pre.data_ptr() if s_pre is not None else 0,
                      z_pre=z_pre.data_ptr() if z_pre is not None else 0,
                      s_init=s_init.data_ptr() if s_init is not None else 0,
                      z_init=z_init.data_ptr() if z_init is not None else 0,
                      device_status=device_status.data_ptr() if device_status is not None else 0, **opt_kw)
-    need = kata_workspace_bytes(fn | (KATA_FN_HOST_IO if host_io else 0), B, H, T, d_k, d_v, C, opts)
-    ws = workspace if workspace is not None else _default_ws
-    ptr, size = ws.get(need, dev)
-    opts.workspace, opts.workspace_bytes = ptr or None, size
+    _scratch(workspace, fn | (KATA_FN_HOST_IO if host_io else 0), (B, H, T, d_k, d_v, C), opts, dev)
     args = (q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(), B, H, T, d_k, d_v, C, ctypes.byref(opts))
     if host_io:
         st = lib().kata_fwd_host(fn, *args)
@@ -274,7 +295,6 @@ def decode_n_psi(d_k: int, feature_order: int = 2, state_layout: int = KATA_LAYO
 def kata_decode_step(q, k, v, S, Z, out=None, *, workspace: Optional[Workspace] = None, stream=None, **opt_kw):
     """One decode token per (b,h): q,k [B,H,d_k], v [B,H,d_v]; fp32 state S [B,H,n_psi,d_v], Z [B,H,n_psi] is
     updated in place.  Returns out [B,H,d_v]."""
-    import torch
     B, H, d_k = q.shape
     d_v = v.shape[-1]
     if not (q.is_contiguous() and k.is_contiguous() and v.is_contiguous() and S.is_contiguous() and Z.is_contiguous()):
@@ -284,15 +304,12 @@ def kata_decode_step(q, k, v, S, Z, out=None, *, workspace: Optional[Workspace] 
     if out is None:
         out = torch.empty_like(v)
     if stream is None:
-        stream = torch.cuda.current_stream(q.device).cuda_stream
+        stream = _stream(q.device)
     opts = make_opts(_dtype_code(q), stream=stream, **opt_kw)
     n_psi = decode_n_psi(d_k, opts.feature_order, opts.state_layout, opts.feature_groups)
-    if tuple(S.shape) != (B, H, n_psi, d_v) or tuple(Z.shape) != (B, H, n_psi):
+    if S.shape != (B, H, n_psi, d_v) or Z.shape != (B, H, n_psi):
         raise ValueError(f"state shapes must be {(B, H, n_psi, d_v)} and {(B, H, n_psi)}")
-    need = kata_workspace_bytes(KATA_FN_DECODE_STEP, B, H, 1, d_k, d_v, 0, opts)
-    ws = workspace if workspace is not None else _default_ws
-    ptr, size = ws.get(need, q.device)
-    opts.workspace, opts.workspace_bytes = ptr or None, size
+    _scratch(workspace, KATA_FN_DECODE_STEP, (B, H, 1, d_k, d_v, 0), opts, q.device)
     st = lib().kata_decode_step(q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(), S.data_ptr(), Z.data_ptr(),
                                 B, H, d_k, d_v, ctypes.byref(opts))
     if st != 0:
@@ -304,7 +321,6 @@ def kata_bwd_quadratic(q, k, v, dout, dq=None, dk=None, dv=None, *, workspace: O
                        stream=None, **opt_kw):
     """Gradients of sum(dout * out) with respect to q, k, v (q,k [B,H,T,d_k]; v,dout [B,H,T,d_v]); the forward
     is recomputed.  Returns (dq, dk, dv) in the dtype of the inputs."""
-    import torch
     if not (q.is_contiguous() and k.is_contiguous() and v.is_contiguous() and dout.is_contiguous()):
         raise ValueError("q, k, v, dout must be contiguous [B,H,T,d]")
     B, H, T, d_k = q.shape
@@ -313,12 +329,9 @@ def kata_bwd_quadratic(q, k, v, dout, dq=None, dk=None, dv=None, *, workspace: O
     dk = torch.empty_like(k) if dk is None else dk
     dv = torch.empty_like(v) if dv is None else dv
     if stream is None:
-        stream = torch.cuda.current_stream(q.device).cuda_stream
+        stream = _stream(q.device)
     opts = make_opts(_dtype_code(q), stream=stream, **opt_kw)
-    need = kata_workspace_bytes(KATA_FN_BWD_QUADRATIC, B, H, T, d_k, d_v, 0, opts)
-    ws = workspace if workspace is not None else _default_ws
-    ptr, size = ws.get(need, q.device)
-    opts.workspace, opts.workspace_bytes = ptr or None, size
+    _scratch(workspace, KATA_FN_BWD_QUADRATIC, (B, H, T, d_k, d_v, 0), opts, q.device)
     st = lib().kata_bwd_quadratic(q.data_ptr(), k.data_ptr(), v.data_ptr(), dout.data_ptr(), dq.data_ptr(),
                                   dk.data_ptr(), dv.data_ptr(), B, H, T, d_k, d_v, ctypes.byref(opts))
     if st != 0:
@@ -330,7 +343,6 @@ def kata_bwd_chunked(q, k, v, dout, dq=None, dk=None, dv=None, C: int = 64, *, w
                      stream=None, **opt_kw):
     """The same gradients as ``kata_bwd_quadratic`` by the O(T) two-pass linear-state backward.  Returns (dq, dk, dv)
     in the dtype of the inputs."""
-    import torch
     if not (q.is_contiguous() and k.is_contiguous() and v.is_contiguous() and dout.is_contiguous()):
         raise ValueError("q, k, v, dout must be contiguous [B,H,T,d]")
     B, H, T, d_k = q.shape
@@ -339,12 +351,9 @@ def kata_bwd_chunked(q, k, v, dout, dq=None, dk=None, dv=None, C: int = 64, *, w
     dk = torch.empty_like(k) if dk is None else dk
     dv = torch.empty_like(v) if dv is None else dv
     if stream is None:
-        stream = torch.cuda.current_stream(q.device).cuda_stream
+        stream = _stream(q.device)
     opts = make_opts(_dtype_code(q), stream=stream, **opt_kw)
-    need = kata_workspace_bytes(KATA_FN_BWD_CHUNKED, B, H, T, d_k, d_v, C, opts)
-    ws = workspace if workspace is not None else _default_ws
-    ptr, size = ws.get(need, q.device)
-    opts.workspace, opts.workspace_bytes = ptr or None, size
+    _scratch(workspace, KATA_FN_BWD_CHUNKED, (B, H, T, d_k, d_v, C), opts, q.device)
     st = lib().kata_bwd_chunked(q.data_ptr(), k.data_ptr(), v.data_ptr(), dout.data_ptr(), dq.data_ptr(),
                                 dk.data_ptr(), dv.data_ptr(), B, H, T, d_k, d_v, C, ctypes.byref(opts))
     if st != 0:
@@ -362,11 +371,10 @@ def kata_chunk_state_scan_static(q, k, v, out, C: int = 64, *, scan_group: int =
     Unlike the other wrappers this one never touches torch's allocator: ``out`` must be passed in, and
     no workspace is requested.  Calls that overlap on the GPU share (and race on) the one scratch array.
     """
-    import torch
     B, H, T, d_k = q.shape
     d_v = v.shape[-1]
     if stream is None:
-        stream = torch.cuda.current_stream(q.device).cuda_stream
+        stream = _stream(q.device)
     opts = make_opts(_dtype_code(q), stream=stream, scan_group=scan_group, impl=impl, feature_order=feature_order)
     st = lib().kata_chunk_state_scan_static(q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(), B, H, T, d_k, d_v,
                                             C, ctypes.byref(opts))

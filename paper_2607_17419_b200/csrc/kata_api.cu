@@ -301,17 +301,9 @@ bool stream_kernel_forced() {
 }
 
 int check_arch() {
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) {
-    cudaGetLastError();
-    return KATA_ERR_CUDA;
-  }
-  int major = 0;
-  if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess) {
-    cudaGetLastError();
-    return KATA_ERR_CUDA;
-  }
-  return major == 10 ? KATA_OK : KATA_ERR_ARCH;
+  static std::atomic<int> known[kMaxDevices];
+  const int major = device_fact(cudaDevAttrComputeCapabilityMajor, known);
+  return major < 0 ? KATA_ERR_CUDA : major == 10 ? KATA_OK : KATA_ERR_ARCH;
 }
 
 // Validation shared by every entry point; fills the problem, the plan and the workspace need.

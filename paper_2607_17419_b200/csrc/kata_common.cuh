@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "../../include/kata.h"
 
 namespace kata {
@@ -37,6 +39,50 @@ inline void note_launch(LaunchCtx& ctx) {
     cudaGetLastError();
     ctx.status = KATA_ERR_CUDA;
   }
+}
+
+// Facts of the current device that do not change, read once per device: a small call is mostly host time (a query or an
+// attribute call is 0.2 to 1 us, a launch 3).
+constexpr int kMaxDevices = 64;
+inline int device_ordinal() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) {
+    cudaGetLastError();
+    return -1;
+  }
+  return dev;
+}
+inline int device_fact(cudaDeviceAttr what, std::atomic<int>* known) {      // -1: the query failed
+  const int dev = device_ordinal();
+  if (dev < 0) return -1;
+  if (dev < kMaxDevices) {
+    const int v = known[dev].load(std::memory_order_relaxed);
+    if (v > 0) return v;
+  }
+  int v = 0;
+  if (cudaDeviceGetAttribute(&v, what, dev) != cudaSuccess) {
+    cudaGetLastError();
+    return -1;
+  }
+  if (dev < kMaxDevices) known[dev].store(v, std::memory_order_relaxed);
+  return v;
+}
+inline int sm_count() {
+  static std::atomic<int> known[kMaxDevices];
+  const int v = device_fact(cudaDevAttrMultiProcessorCount, known);
+  return v > 0 ? v : 148;
+}
+// Lets kernel K use `bytes` of dynamic shared memory on the current device (set once per kernel and device).
+template <auto K> bool allow_smem(int bytes) {
+  static std::atomic<int> set[kMaxDevices];
+  const int dev = device_ordinal();
+  if (dev >= 0 && dev < kMaxDevices && set[dev].load(std::memory_order_acquire) == bytes) return true;
+  if (cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  if (dev >= 0 && dev < kMaxDevices) set[dev].store(bytes, std::memory_order_release);
+  return true;
 }
 
 struct Problem {

@@ -15,7 +15,6 @@
 namespace kata {
 namespace {
 
-constexpr int DEC_THREADS = 256;
 constexpr int DEC_ROWS = 256;     // feature rows per CTA
 
 // feature pair (a,b) and scale of row r.  With g feature blocks (blockwise PSD map) the rows of the blocks follow
@@ -45,7 +44,7 @@ __device__ __forceinline__ void feature_pair(int r, int d, int layout, int order
   b += gb * m;
 }
 
-template <typename T, int DV>
+template <typename T, int DV, int DEC_THREADS>
 __global__ void __launch_bounds__(DEC_THREADS) decode_update_kernel(const T* __restrict__ q, const T* __restrict__ k,
                                                                     const T* __restrict__ v, float* __restrict__ S,
                                                                     float* __restrict__ Z, float* __restrict__ part,
@@ -56,7 +55,9 @@ __global__ void __launch_bounds__(DEC_THREADS) decode_update_kernel(const T* __r
   const int bh = blockIdx.y, slab = blockIdx.x, n_slabs = gridDim.x;
   const int tid = threadIdx.x;
   // Launched with programmatic stream serialisation: the CTAs may be resident before the kernel ahead in the stream
-  // (the producer of q, k, v, or the previous step's finish kernel, which still reads `part`) has ended.
+  // (the producer of q, k, v, or the previous step's finish kernel, which still reads `part`) has ended, and let the kernel
+  // behind become resident at once.
+  cudaTriggerProgrammaticLaunchCompletion();
   cudaGridDependencySynchronize();
   // k_hat = k / ||k|| (zero row -> zero feature); the query norm cancels in the readout and is not applied
   if (tid < 64) {
@@ -190,11 +191,14 @@ template <typename T, int DV>
 void launch(const void* q, const void* k, const void* v, void* out, float* S, float* Z, float* part, int BH, int d_k,
             int n_psi, int layout, int order, int groups, LaunchCtx& ctx) {
   const int n_slabs = decode_slabs(n_psi);
+  // Threads of a CTA: 256, or 512 while that leaves SMs with one CTA or two (measured, us a step, 256 / 512 threads: 4 heads of
+  // 4096 feature rows 10.4 / 7.6, 16 heads 11.3 / 10.9, 64 heads 28.6 / 28.3, 256 heads 95.7 / 102.3).
+  const bool wide = (long long)n_slabs * BH <= 296;
   // both kernels may become resident before the kernel ahead of them has ended (each waits inside: the update kernel
   // at its top, the finish kernel after its own prologue)
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(n_slabs, BH);
-  cfg.blockDim = dim3(DEC_THREADS);
+  cfg.blockDim = dim3(wide ? 512 : 256);
   cfg.dynamicSmemBytes = 0;
   cfg.stream = ctx.stream;
   cudaLaunchAttribute attr[1];
@@ -205,7 +209,7 @@ void launch(const void* q, const void* k, const void* v, void* out, float* S, fl
   const float* part_c = part;
   const T *qc = static_cast<const T*>(q), *kc = static_cast<const T*>(k), *vc = static_cast<const T*>(v);
   T* oc = static_cast<T*>(out);
-  if (cudaLaunchKernelEx(&cfg, decode_update_kernel<T, DV>, qc, kc, vc, S, Z, part, d_k, n_psi, layout, order, groups) != cudaSuccess) {
+  if (cudaLaunchKernelEx(&cfg, wide ? decode_update_kernel<T, DV, 512> : decode_update_kernel<T, DV, 256>, qc, kc, vc, S, Z, part, d_k, n_psi, layout, order, groups) != cudaSuccess) {
     cudaGetLastError();
     ctx.status = KATA_ERR_CUDA;
     return;

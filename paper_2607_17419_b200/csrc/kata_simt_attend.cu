@@ -296,7 +296,7 @@ template <int DK, int DV> void run(const Problem& p, float* S, LaunchCtx& ctx) {
   cfg.blockDim = dim3(NW * 32);
   cfg.dynamicSmemBytes = smem;
   cfg.numAttrs = states ? 1 : 0;
-  ok = ok && cudaFuncSetAttribute(attend_kernel<DK, DV>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
+  ok = ok && allow_smem<attend_kernel<DK, DV>>(smem) &&
        cudaLaunchKernelEx(&cfg, attend_kernel<DK, DV>, q, k, v, static_cast<float*>(p.out), (const float*)(states ? S : nullptr), p.T, chunk,
                           n_chunks) == cudaSuccess;
   if (!ok) {

@@ -644,16 +644,13 @@ void tc_attend(const Problem& p, const __nv_bfloat16* rscale, const AttendStates
     return;
   }
   auto kern = p.groups == 1 ? tc_attend_kernel<1> : p.groups == 2 ? tc_attend_kernel<2> : tc_attend_kernel<4>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_ALLOC) != cudaSuccess) {
-    cudaGetLastError();
+  if (!(p.groups == 1   ? allow_smem<tc_attend_kernel<1>>((int)SMEM_ALLOC)
+        : p.groups == 2 ? allow_smem<tc_attend_kernel<2>>((int)SMEM_ALLOC)
+                        : allow_smem<tc_attend_kernel<4>>((int)SMEM_ALLOC))) {
     ctx.status = KATA_ERR_CUDA;
     return;
   }
-  int dev = 0, sms = 148;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-    cudaGetLastError();
-    sms = 148;
-  }
+  const int sms = sm_count();
   const long long n_items = (long long)BH * n_pairs;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(n_items < sms ? n_items : sms));   // persistent: one CTA per SM

@@ -780,11 +780,7 @@ __global__ void __launch_bounds__(256) bwd_rscale_kernel(const __nv_bfloat16* __
 template <int MODE, int G, int NS>
 bool launch_bwd(const CUtensorMap& x1, const CUtensorMap& x2, const CUtensorMap& y1, const CUtensorMap& y2, const BArgs& a, LaunchCtx& ctx) {
   auto kern = tc_bwd_kernel<MODE, G, NS>;
-  int dev = 0, sms = 148;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-    cudaGetLastError();
-    sms = 148;
-  }
+  const int sms = sm_count();
   const long long n_items = (long long)a.BH * ((a.Tlen + MT - 1) / MT);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(n_items < sms ? n_items : sms));   // persistent: one CTA per SM
@@ -796,7 +792,7 @@ bool launch_bwd(const CUtensorMap& x1, const CUtensorMap& x2, const CUtensorMap&
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_ALLOC) != cudaSuccess ||
+  if (!allow_smem<tc_bwd_kernel<MODE, G, NS>>((int)SMEM_ALLOC) ||
       cudaLaunchKernelEx(&cfg, kern, x1, x2, y1, y2, a) != cudaSuccess) {
     cudaGetLastError();
     ctx.status = KATA_ERR_CUDA;

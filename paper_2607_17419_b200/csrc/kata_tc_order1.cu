@@ -538,8 +538,7 @@ void tc_order1(const Problem& p, const ScanPlan& plan, bool use_scan, int C, flo
     ctx.status = KATA_ERR_CUDA;
     return;
   }
-  if (cudaFuncSetAttribute(tc_order1_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_ALLOC) != cudaSuccess) {
-    cudaGetLastError();
+  if (!allow_smem<tc_order1_kernel>((int)SMEM_ALLOC)) {
     ctx.status = KATA_ERR_CUDA;
     return;
   }
@@ -572,11 +571,7 @@ void tc_order1(const Problem& p, const ScanPlan& plan, bool use_scan, int C, flo
     a.anchor_state = bufB;
     a.flags = flags;
     a.ticket = reinterpret_cast<unsigned*>(flags + (size_t)BH * NG);
-    int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-      cudaGetLastError();
-      sms = 148;
-    }
+    const int sms = sm_count();
     const unsigned total = (unsigned)BH * NG;
     tc_order1_kernel<<<dim3(total < (unsigned)sms ? total : (unsigned)sms), NTHREADS, SMEM_ALLOC, ctx.stream>>>(tmQ, tmK, tmV, a);
     note_launch(ctx);

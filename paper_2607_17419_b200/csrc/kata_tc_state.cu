@@ -509,8 +509,9 @@ void tc_states(const Problem& p, const __nv_bfloat16* rscale, const StatePlan& p
     return;
   }
   auto kern = p.groups == 1 ? tc_state_kernel<1> : p.groups == 2 ? tc_state_kernel<2> : tc_state_kernel<4>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_ALLOC) != cudaSuccess) {
-    cudaGetLastError();
+  if (!(p.groups == 1   ? allow_smem<tc_state_kernel<1>>((int)SMEM_ALLOC)
+        : p.groups == 2 ? allow_smem<tc_state_kernel<2>>((int)SMEM_ALLOC)
+                        : allow_smem<tc_state_kernel<4>>((int)SMEM_ALLOC))) {
     ctx.status = KATA_ERR_CUDA;
     return;
   }
