@@ -4,20 +4,21 @@
 //   state_loc_kernel     S_loc = sum_t w psi(k_hat_t) [v_t, 1] over a chunk: thread = feature pair a <= b (w = 2 off the
 //                        diagonal: the lift is symmetric), its DV + 1 sums in registers, rows broadcast from shared memory
 //   state_prefix_kernel  running sum over the chunks, in order
-//   attend_kernel        lane = two queries; the eight warps of a CTA share out the feature rows of the state and the tiles
+//   attend_kernel        lane = two queries; the warps of a CTA share out the feature rows of the state and the tiles
 //                        of 32 keys, rows broadcast from shared memory (16 bytes per load feed 8 FMAs), and add their
 //                        numerators and normalisers in a fixed order at the end
 // What bounds it: FMAs.  The walk over the chunks of a head by one CTA (kata_simt_chunked.cu) was a chain of 21 us per 64
 // tokens; 2 heads x 512 tokens of 16 entries took 171 us.
 // Chunk length: at 16 entries a query costs 34 FMAs per key of its chunk and 2.3 k for the state, at 32 66 and 17 k: the
 // lengths up to which one chunk is the cheaper are about 1000 and 1500.
+#include <type_traits>
+
 #include "kata_common.cuh"
 
 namespace kata {
 namespace {
 
 constexpr int QB = 64;           // queries per CTA
-constexpr int NW = 8;            // warps per CTA
 constexpr int CHUNK = 256;       // tokens per chunk
 
 __host__ __device__ constexpr int n_features(int d) { return d * (d + 1) / 2; }
@@ -108,12 +109,12 @@ __global__ void __launch_bounds__(128) state_prefix_kernel(float4* __restrict__ 
   }
 }
 
-template <int DK, int DV> constexpr int attend_smem_floats() {
+template <int DK, int DV, int NW> constexpr int attend_smem_floats() {
   const int tiles = QB * DK + NW * 32 * (DK + DV), red = NW * (DV + 1) * QB;
   return tiles > red ? tiles : red;
 }
 
-template <int DK, int DV>
+template <int DK, int DV, int NW>          // NW warps share out the key tiles and state rows of a block
 __global__ void __launch_bounds__(NW * 32) attend_kernel(const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ v,
                                                          float* __restrict__ out, const float* __restrict__ S, int Tlen, int chunk,
                                                          int n_chunks) {
@@ -212,21 +213,22 @@ __global__ void __launch_bounds__(NW * 32) attend_kernel(const float* __restrict
     load_rows<DV, false>(vh, vt, t0, 32, Tlen, lane, 32);
     __syncwarp();
     const bool diag = t0 + 31 > q0;
-#pragma unroll 2
+#pragma unroll 4
     for (int t = 0; t < 32; ++t) {
-      float sa = 0.f, sb = 0.f;
+      float4 a4 = make_float4(0.f, 0.f, 0.f, 0.f), b4 = a4;      // (four partial sums: a chain of DK FMAs would set the pace)
 #pragma unroll
       for (int i = 0; i < DK; i += 4) {
         const float4 x = ld4(kt + t * DK + i);
-        sa = fmaf(qa[i], x.x, sa);
-        sa = fmaf(qa[i + 1], x.y, sa);
-        sa = fmaf(qa[i + 2], x.z, sa);
-        sa = fmaf(qa[i + 3], x.w, sa);
-        sb = fmaf(qb[i], x.x, sb);
-        sb = fmaf(qb[i + 1], x.y, sb);
-        sb = fmaf(qb[i + 2], x.z, sb);
-        sb = fmaf(qb[i + 3], x.w, sb);
+        a4.x = fmaf(qa[i], x.x, a4.x);
+        a4.y = fmaf(qa[i + 1], x.y, a4.y);
+        a4.z = fmaf(qa[i + 2], x.z, a4.z);
+        a4.w = fmaf(qa[i + 3], x.w, a4.w);
+        b4.x = fmaf(qb[i], x.x, b4.x);
+        b4.y = fmaf(qb[i + 1], x.y, b4.y);
+        b4.z = fmaf(qb[i + 2], x.z, b4.z);
+        b4.w = fmaf(qb[i + 3], x.w, b4.w);
       }
+      const float sa = (a4.x + a4.y) + (a4.z + a4.w), sb = (b4.x + b4.y) + (b4.z + b4.w);
       float wa = sa * sa, wb = sb * sb;
       if (diag) {
         if (t0 + t > q0 + lane) wa = 0.f;
@@ -248,7 +250,8 @@ __global__ void __launch_bounds__(NW * 32) attend_kernel(const float* __restrict
   red[DV * QB + lane] = da;
   red[DV * QB + 32 + lane] = db;
   __syncthreads();
-  const int row = tid & (QB - 1), part = tid / QB;         // four threads per query
+  const int row = tid & (QB - 1), part = tid / QB;         // four threads per query (of the first 256)
+  if (part >= 4) return;
   float den = 0.f;
 #pragma unroll
   for (int w = 0; w < NW; ++w) den += sm[(w * (DV + 1) + DV) * QB + row];
@@ -291,14 +294,20 @@ template <int DK, int DV> void run(const Problem& p, float* S, LaunchCtx& ctx) {
     ok = cudaLaunchKernelEx(&cfg, state_prefix_kernel, reinterpret_cast<float4*>(S), n4, n_chunks) == cudaSuccess;
     ctx.launches += ok;
   }
-  constexpr int smem = attend_smem_floats<DK, DV>() * (int)sizeof(float);
   cfg.gridDim = dim3((p.T + QB - 1) / QB, BH);
-  cfg.blockDim = dim3(NW * 32);
-  cfg.dynamicSmemBytes = smem;
   cfg.numAttrs = states ? 1 : 0;
-  ok = ok && allow_smem<attend_kernel<DK, DV>>(smem) &&
-       cudaLaunchKernelEx(&cfg, attend_kernel<DK, DV>, q, k, v, static_cast<float*>(p.out), (const float*)(states ? S : nullptr), p.T, chunk,
-                          n_chunks) == cudaSuccess;
+  auto attend = [&](auto nw) {
+    constexpr int NW = decltype(nw)::value, smem = attend_smem_floats<DK, DV, NW>() * (int)sizeof(float);
+    cfg.blockDim = dim3(NW * 32);
+    cfg.dynamicSmemBytes = smem;
+    return allow_smem<attend_kernel<DK, DV, NW>>(smem) &&
+           cudaLaunchKernelEx(&cfg, attend_kernel<DK, DV, NW>, q, k, v, static_cast<float*>(p.out), (const float*)(states ? S : nullptr),
+                              p.T, chunk, n_chunks) == cudaSuccess;
+  };
+  // sixteen warps where there are few blocks (rows of 16 leave registers for them): 2 heads x 512 tokens 15.6 us with eight
+  // warps, 13.4 with sixteen; 256 heads x 1024 tokens 349 and 419
+  const bool few = DK == 16 && DV == 16 && (long long)cfg.gridDim.x * cfg.gridDim.y <= 148;
+  ok = ok && (few ? attend(std::integral_constant<int, DK == 16 && DV == 16 ? 16 : 8>{}) : attend(std::integral_constant<int, 8>{}));
   if (!ok) {
     cudaGetLastError();
     ctx.status = KATA_ERR_CUDA;

@@ -89,26 +89,35 @@ enum {
   BAR_COUNT = 43
 };
 
-// Pre-pass: r = 1 / ||k||^2 per key row (0 for a zero row), one warp per 4 rows (8 lanes x 16 bytes per row).
+// Pre-pass: r = 1 / ||k||^2 per key row (0 for a zero row); eight lanes of 16 bytes per row, four rows per lane in flight
+// (memory-bound; one row per lane: RSFIG).
+constexpr int RS_ROWS = 4;
 __global__ void __launch_bounds__(256) rscale_kernel(const __nv_bfloat16* __restrict__ k, __nv_bfloat16* __restrict__ rscale,
                                                      size_t n_rows, int d) {
-  const size_t row = (size_t)blockIdx.x * 32 + (threadIdx.x >> 3);
+  const size_t row0 = (size_t)blockIdx.x * (32 * RS_ROWS) + (threadIdx.x >> 3);
   const int part = threadIdx.x & 7;
-  if (row >= n_rows) return;
-  uint4 kraw = make_uint4(0u, 0u, 0u, 0u);
-  if (part * 8 < d) kraw = *reinterpret_cast<const uint4*>(k + row * d + part * 8);
-  const uint32_t kw[4] = {kraw.x, kraw.y, kraw.z, kraw.w};
-  float ss = 0.f;
+  uint4 raw[RS_ROWS];
 #pragma unroll
-  for (int e = 0; e < 4; ++e) {
-    const float lo = __uint_as_float(kw[e] << 16), hi = __uint_as_float(kw[e] & 0xFFFF0000u);
-    ss = fmaf(lo, lo, ss);
-    ss = fmaf(hi, hi, ss);
+  for (int i = 0; i < RS_ROWS; ++i) {
+    const size_t row = row0 + i * 32;
+    raw[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (row < n_rows && part * 8 < d) raw[i] = *reinterpret_cast<const uint4*>(k + row * d + part * 8);
   }
-  ss += __shfl_xor_sync(0xffffffffu, ss, 1);
-  ss += __shfl_xor_sync(0xffffffffu, ss, 2);
-  ss += __shfl_xor_sync(0xffffffffu, ss, 4);
-  if (part == 0) rscale[row] = __float2bfloat16_rn(inv_or_zero(ss));
+#pragma unroll
+  for (int i = 0; i < RS_ROWS; ++i) {
+    const uint32_t kw[4] = {raw[i].x, raw[i].y, raw[i].z, raw[i].w};
+    float ss = 0.f;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const float lo = __uint_as_float(kw[e] << 16), hi = __uint_as_float(kw[e] & 0xFFFF0000u);
+      ss = fmaf(lo, lo, ss);
+      ss = fmaf(hi, hi, ss);
+    }
+    ss += __shfl_xor_sync(0xffffffffu, ss, 1);
+    ss += __shfl_xor_sync(0xffffffffu, ss, 2);
+    ss += __shfl_xor_sync(0xffffffffu, ss, 4);
+    if (part == 0 && row0 + i * 32 < n_rows) rscale[row0 + i * 32] = __float2bfloat16_rn(inv_or_zero(ss));
+  }
 }
 
 __device__ __forceinline__ uint32_t mul_bf16x2(uint32_t a, uint32_t b) {
@@ -618,7 +627,7 @@ size_t tc_quadratic_workspace_bytes(const Problem& p) { return ((size_t)p.B * p.
 
 void tc_rscale(const Problem& p, __nv_bfloat16* rscale, LaunchCtx& ctx) {
   const size_t n_rows = (size_t)p.B * p.H * p.T;
-  rscale_kernel<<<(unsigned)((n_rows + 31) / 32), 256, 0, ctx.stream>>>(static_cast<const __nv_bfloat16*>(p.k), rscale, n_rows, p.d_k);
+  rscale_kernel<<<(unsigned)((n_rows + 32 * RS_ROWS - 1) / (32 * RS_ROWS)), 256, 0, ctx.stream>>>(static_cast<const __nv_bfloat16*>(p.k), rscale, n_rows, p.d_k);
   note_launch(ctx);
 }
 

@@ -12,19 +12,20 @@
 //            through shared memory.
 //   update   [S | Z] += A [V | 1]   A from TMEM, B = the value tile as it is and a constant column of ones, N = 80,
 //            two accumulators of 128 rows
-// The accumulators hold one chunk; between chunks eight warps add them to a running sum in registers (fp32, one state
-// row per thread) and write it out in bf16 (the state before the next chunk, pair weights included), while the update goes
-// on in the other pair of accumulators.
+// The accumulators carry the sum over all chunks so far (fp32); between chunks eight warps copy them out, one state row per
+// thread: the state before the next chunk in bf16, pair weights included.  The builders run up to five half tiles ahead, so
+// the MMAs that wait for the copy catch up.
 //
-// What bounds it: shared memory.  Per tile and CTA: 640 cycles of MMA, and at 128 B per cycle 256 for the TMA writes, 320
-// for the value operand, about 460 for the builders' fragment loads, scales and shuffles.  Built in shared memory and read
-// by the MMAs from there, as products of token rows, the A operand alone took 1024.
+// What bounds it.  Per tile and CTA: 640 cycles of MMA, and the shared-memory port at 128 B per cycle: 256 for the TMA
+// writes, 320 for the value operand, about 340 for the builders' fragments and broadcasts.  Built in shared memory and read
+// by the MMAs from there, as products of token rows, the A operand alone took 1024.  A builder warp takes about 1000 cycles
+// for a half tile, half of it latency, so four sets of four take turns (two sets: 1460 cycles a tile).
 //
 // When the heads alone do not fill the GPU the chunk axis is cut into segments: every segment sums from zero and writes
 // fp32, and state_fix_kernel adds the segments before it and rounds.
 //
-// Warps (640 threads): 0 TMA producer, 1 MMA issuer, 2 key scales, 4-11 builders (quadrant = warp % 4, two sets taking
-// alternate halves of the tiles), 12-19 running sums.  All waits are bounded.
+// Warps (896 threads): 0 TMA producer, 1 MMA issuer, 2 key scales, 4-19 builders (quadrant = warp % 4, four sets taking
+// every fourth half tile), 20-27 copies.  All waits are bounded.
 #include <cuda.h>
 #include <type_traits>
 
@@ -41,19 +42,20 @@ using namespace umma;
 constexpr int D = 64;
 constexpr int CT = 128;          // tokens per tile
 constexpr int NSTAGE = 4;
-constexpr int NSLOT = 3;         // A operand: slots of 64 tokens x 256 features
-constexpr int NTHREADS = 640;
-constexpr int WARP_BLD0 = 4, WARP_SUM0 = 12;
+constexpr int NSLOT = 5;         // A operand: slots of 64 tokens x 256 features
+constexpr int NSET = 4;          // sets of builder warps
+constexpr int NTHREADS = 896;
+constexpr int WARP_BLD0 = 4, WARP_CPY0 = 20;
 
-constexpr uint32_t COL_ACC = 0;          // 2 (chunk parity) x 2 (tile of 128 rows) x 80
-constexpr uint32_t COL_A = 320;          // NSLOT x 2 x 32
+constexpr uint32_t COL_ACC = 0;          // 2 (tiles of 128 rows) x 80
+constexpr uint32_t COL_A = 160;          // NSLOT x 2 x 32
 constexpr uint32_t TMEM_COLS = 512;
 
 constexpr uint32_t STAGE_BYTES = 32768;                     // key tile, value tile
 constexpr uint32_t OFF_ONES = NSTAGE * STAGE_BYTES;         // 16 rows of [1, 0 ...]: columns 64.. of the values
 constexpr uint32_t OFF_RV = OFF_ONES + 2048;                // NSTAGE x 128 bf16 key scales, in the builders' order
-constexpr uint32_t OFF_SCR = OFF_RV + NSTAGE * 256;         // 8 builder warps x 2 KB: scaled fragments of run h
-constexpr uint32_t OFF_BAR = OFF_SCR + 8 * 2048;
+constexpr uint32_t OFF_SCR = OFF_RV + NSTAGE * 256;         // 16 builder warps x 2 KB: scaled fragments of run h
+constexpr uint32_t OFF_BAR = OFF_SCR + 16 * 2048;
 constexpr uint32_t SMEM_BYTES = OFF_BAR + 256;
 constexpr uint32_t SMEM_ALLOC = SMEM_BYTES + 1024;
 static_assert(SMEM_ALLOC > 116 * 1024, "one CTA per SM is assumed (the CTA allocates all of TMEM)");
@@ -61,12 +63,12 @@ static_assert(SMEM_ALLOC > 116 * 1024, "one CTA per SM is assumed (the CTA alloc
 enum {
   BAR_FULL = 0,      // [NSTAGE] tiles (TMA bytes) and their key scales (scale warp) landed
   BAR_EMPTY = 4,     // [NSTAGE] stage free: 256 builders and the issuer's commit
-  BAR_AFULL = 12,    // [NSLOT] operand slot built (128)
-  BAR_AEMPTY = 15,   // [NSLOT] ... and consumed
-  BAR_CFULL = 18,    // [2] accumulators of a chunk are complete
-  BAR_CFREE = 20,    // [2] ... and have been read (256)
-  BAR_DRAIN = 22,
-  BAR_COUNT = 23
+  BAR_AFULL = 8,     // [NSLOT] operand slot built (128)
+  BAR_AEMPTY = 13,   // [NSLOT] ... and consumed
+  BAR_CFULL = 18,    // the MMAs of a chunk are complete
+  BAR_CFREE = 19,    // the accumulators have been read, or set to the state handed in (256)
+  BAR_DRAIN = 20,
+  BAR_COUNT = 21
 };
 
 struct SArgs {
@@ -102,7 +104,7 @@ template <int G> __device__ __forceinline__ size_t public_rows(int packed) {
 
 template <int N> __device__ __forceinline__ void regs_release() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
 template <int N> __device__ __forceinline__ void regs_take() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
-static_assert(384 * 80 + 256 * 120 <= 640 * 96, "register budget");
+static_assert(128 * 40 + 512 * 80 + 256 * 72 <= 896 * 72, "register budget");
 
 __device__ __forceinline__ uint32_t mul_bf16x2(uint32_t a, uint32_t b) {
   const __nv_bfloat162 p = __hmul2(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));
@@ -145,21 +147,20 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
   const int n_tiles_all = (args.Tlen + CT - 1) / CT;
   const int t_beg = c_beg * args.chunk_tiles, t_end = min(c_end * args.chunk_tiles, n_tiles_all);
   const int n = t_end - t_beg;                    // tiles of this CTA
+  const bool first = c_beg == 0 && args.s_init != nullptr;      // starts from the state handed in
 
   if (tid == 0) {
     abort_s = 0;
     for (int i = 0; i < NSTAGE; ++i) {
       mbar_init(bar(BAR_FULL + i), 2);
-      mbar_init(bar(BAR_EMPTY + i), 257);
+      mbar_init(bar(BAR_EMPTY + i), 257);      // 256 threads of the two sets that read a tile, and the MMAs
     }
     for (int i = 0; i < NSLOT; ++i) {
       mbar_init(bar(BAR_AFULL + i), 128);
       mbar_init(bar(BAR_AEMPTY + i), 1);
     }
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(bar(BAR_CFULL + i), 1);
-      mbar_init(bar(BAR_CFREE + i), 256);
-    }
+    mbar_init(bar(BAR_CFULL), 1);
+    mbar_init(bar(BAR_CFREE), 256);
     mbar_init(bar(BAR_DRAIN), 1);
     fence_mbar_init();
     tma_prefetch_desc(&tmK);
@@ -179,7 +180,7 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
   bool ok = true;
 
   if (warp == 0) {
-    regs_release<80>();
+    regs_release<40>();
     // =========================== TMA producer ===========================
     if (elect_one()) {
       for (int j = 0; j < n && ok; ++j) {
@@ -192,19 +193,19 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
       }
     }
   } else if (warp == 1) {
-    regs_release<80>();
+    regs_release<40>();
     // =========================== update issuer ===========================
     if (elect_one()) {
       const uint32_t idesc = instr_desc(kFmtBF16, kFmtBF16, 0, 1, 128, 80);
       const uint32_t ones = smem_u32(base + OFF_ONES);
       int chunk_i = 0, in_chunk = 0;     // chunk of this segment, tile inside it
+      const int first_free = first ? 1 : 0;
       for (int j = 0; j < n && ok; ++j) {
         const int s = j % NSTAGE;
         ok = wait_or_abort(bar(BAR_FULL + s), (j / NSTAGE) & 1, abort_flag);
-        if (ok && in_chunk == 0 && chunk_i >= 2)       // the sums of two chunks back have left these accumulators
-          ok = wait_or_abort(bar(BAR_CFREE + (chunk_i & 1)), ((chunk_i >> 1) - 1) & 1, abort_flag);
+        if (ok && in_chunk == 0 && chunk_i + first_free >= 1)       // the accumulators have been copied out, or set
+          ok = wait_or_abort(bar(BAR_CFREE), (chunk_i + first_free - 1) & 1, abort_flag);
         const uint32_t va = smem_u32(stage(s)) + 16384;
-        const uint32_t acc_t = tb + COL_ACC + (chunk_i & 1) * 160;
 #pragma unroll
         for (int th = 0; th < 2; ++th) {
           const int hs = 2 * j + th, slot = hs % NSLOT;
@@ -216,22 +217,22 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks) {
               const uint32_t b = va + (th * 4 + ks) * 2048;
-              mma_f16_ts(acc_t + m * 80, tb + COL_A + slot * 64 + m * 32 + ks * 8, smem_desc(b, ones - b, 1024, kSwizzle128B), idesc,
-                         (in_chunk > 0 || th > 0 || ks > 0) ? 1u : 0u);
+              mma_f16_ts(tb + COL_ACC + m * 80, tb + COL_A + slot * 64 + m * 32 + ks * 8, smem_desc(b, ones - b, 1024, kSwizzle128B), idesc,
+                         (first || j > 0 || th > 0 || ks > 0) ? 1u : 0u);
             }
           mma_commit(bar(BAR_AEMPTY + slot));
         }
         if (!ok) break;
         mma_commit(bar(BAR_EMPTY + s));
         if (++in_chunk == args.chunk_tiles || j + 1 == n) {
-          mma_commit(bar(BAR_CFULL + (chunk_i & 1)));
+          mma_commit(bar(BAR_CFULL));
           in_chunk = 0;
           ++chunk_i;
         }
       }
     }
   } else if (warp == 2) {
-    regs_release<80>();
+    regs_release<40>();
     // =========================== key scales, from the pre-pass to shared memory ===========================
     cudaGridDependencySynchronize();
     const unsigned short* rs = reinterpret_cast<const unsigned short*>(args.rscale) + (size_t)bh * args.Tlen;
@@ -262,11 +263,11 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
       if (lane == 0) mbar_arrive(bar(BAR_FULL + s));
     }
   } else if (warp == 3) {
-    regs_release<80>();
-  } else if (warp < WARP_SUM0) {
-    regs_release<80>();
+    regs_release<40>();
+  } else if (warp < WARP_CPY0) {
+    regs_take<80>();
     // =========================== builders ===========================
-    const int q4 = warp & 3, th = (warp - WARP_BLD0) >> 2;
+    const int q4 = warp & 3, set = (warp - WARP_BLD0) >> 2, th = set & 1;   // half of the tiles j with j % 2 = set / 2
     const int pa = 4 * slice + (q4 >> 1), pb = pa + 2;
     const int ga = kPairs.g[pa], gb = kPairs.g[pb], ha = kPairs.h[pa], hb = kPairs.h[pb];
     const uint32_t scr = smem_u32(base + OFF_SCR) + (warp - WARP_BLD0) * 2048, scr_w = scr + lane * 16;
@@ -278,7 +279,7 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     // (two copies of the loop: the pairs share the run h or have one each)
     auto build = [&](auto two) {
       constexpr bool TWO = decltype(two)::value;
-      for (int j = 0; j < n && ok; ++j) {
+      for (int j = set >> 1; j < n && ok; j += NSET / 2) {
         const int s = j % NSTAGE, hs = 2 * j + th, slot = hs % NSLOT;
         ok = wait_or_abort(bar(BAR_FULL + s), (j / NSTAGE) & 1, abort_flag);
         if (!ok) break;
@@ -334,90 +335,99 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     };
     if (ha != hb) build(std::true_type{}); else build(std::false_type{});
   } else {
-    regs_take<120>();
-    // =========================== running sums: one state row per thread ===========================
-    const int q4 = warp & 3, m = (warp - WARP_SUM0) >> 2;
+    // =========================== copies: one state row per thread ===========================
+    const int q4 = warp & 3, m = (warp - WARP_CPY0) >> 2;
     const int row = slice * 256 + m * 128 + q4 * 32 + lane;
     const int p = 4 * slice + 2 * m + (q4 >> 1), e = (q4 & 1) * 32 + lane;
     const int a = 8 * kPairs.g[p] + (e & 7), b = 8 * kPairs.h[p] + (e >> 3);
     const bool mirror = kPairs.g[p] != kPairs.h[p];          // the pair also stands for (b, a)
     const float wgt = mirror ? 2.f : 1.f;
-    float sum[64], zsum = 0.f;
-#pragma unroll
-    for (int i = 0; i < 64; ++i) sum[i] = 0.f;
     const int prow = public_row<G>(min(a, b), max(a, b), args.packed);
     const size_t n_pub = public_rows<G>(args.packed);
-    const bool first = c_beg == 0 && args.s_init != nullptr;
+    const uint32_t ta = tmem_addr(tb, q4 * 32, COL_ACC + m * 80);
+    // bf16 state of chunk c: columns [col, col + 32) from x, and Z
+    auto put_state = [&](int c, int col, const float (&x)[32]) {
+      uint4* dst = reinterpret_cast<uint4*>(args.s + (((size_t)bh * args.n_chunks + c) * ROWS + row) * D + col);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        dst[i] = make_uint4(pack_bf16(x[8 * i] * wgt, x[8 * i + 1] * wgt), pack_bf16(x[8 * i + 2] * wgt, x[8 * i + 3] * wgt),
+                            pack_bf16(x[8 * i + 4] * wgt, x[8 * i + 5] * wgt), pack_bf16(x[8 * i + 6] * wgt, x[8 * i + 7] * wgt));
+    };
+    auto put_z = [&](int c, float z) { args.z[((size_t)bh * args.n_chunks + c) * ROWS + row] = __float2bfloat16_rn(z * wgt); };
+    auto put_f32 = [&](float* dst, const float (&x)[32], float f) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) reinterpret_cast<float4*>(dst)[i] = make_float4(x[4 * i] * f, x[4 * i + 1] * f, x[4 * i + 2] * f, x[4 * i + 3] * f);
+    };
     if (first) {
+      // the state handed in: into the accumulators, and out in bf16 for chunk 0
       const float inv = (args.packed && a != b) ? 0.70710678118654752440f : 1.f;   // packed rows off the diagonal carry sqrt(2)
       const float4* src = reinterpret_cast<const float4*>(args.s_init + ((size_t)bh * n_pub + prow) * D);
 #pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        const float4 x = src[i];
-        sum[4 * i] = x.x * inv; sum[4 * i + 1] = x.y * inv; sum[4 * i + 2] = x.z * inv; sum[4 * i + 3] = x.w * inv;
+      for (int col = 0; col < 64; col += 32) {
+        float x[32];
+        uint32_t u[32];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const float4 y = src[col / 4 + i];
+          x[4 * i] = y.x * inv; x[4 * i + 1] = y.y * inv; x[4 * i + 2] = y.z * inv; x[4 * i + 3] = y.w * inv;
+        }
+#pragma unroll
+        for (int i = 0; i < 32; ++i) u[i] = __float_as_uint(x[i]);
+        tmem_st32(ta + col, u);
+        put_state(0, col, x);
       }
-      zsum = args.z_init[(size_t)bh * n_pub + prow] * inv;
+      const float z = args.z_init[(size_t)bh * n_pub + prow] * inv;
+      uint32_t u[16] = {__float_as_uint(z)};
+      tmem_st16(ta + 64, u);
+      put_z(0, z);
+      tmem_wait_st();
+      tc_fence_before();
+      mbar_arrive(bar(BAR_CFREE));
     }
     // (advanced in place: no thread writes before all have read; a row is read and written by one CTA)
     if (args.s_init != nullptr && args.s_final != nullptr) asm volatile("bar.sync 1, 256;" ::: "memory");
-    // the state before chunk c, in bf16
-    auto write_state = [&](int c) {
-      const size_t slot = (size_t)bh * args.n_chunks + c;
-      uint4* dst = reinterpret_cast<uint4*>(args.s + (slot * ROWS + row) * D);
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        uint4 x;
-        x.x = pack_bf16(sum[8 * i] * wgt, sum[8 * i + 1] * wgt);
-        x.y = pack_bf16(sum[8 * i + 2] * wgt, sum[8 * i + 3] * wgt);
-        x.z = pack_bf16(sum[8 * i + 4] * wgt, sum[8 * i + 5] * wgt);
-        x.w = pack_bf16(sum[8 * i + 6] * wgt, sum[8 * i + 7] * wgt);
-        dst[i] = x;
-      }
-      args.z[slot * ROWS + row] = __float2bfloat16_rn(zsum * wgt);
-    };
-    if (first) write_state(0);
     for (int c = c_beg, i = 0; c < c_end && ok; ++c, ++i) {
-      ok = wait_or_abort(bar(BAR_CFULL + (i & 1)), (i >> 1) & 1, abort_flag);
+      ok = wait_or_abort(bar(BAR_CFULL), i & 1, abort_flag);
       if (!ok) break;
       tc_fence_after();
-      const uint32_t ta = tmem_addr(tb, q4 * 32, COL_ACC + (i & 1) * 160 + m * 80);
+      const bool last = c + 1 == args.n_chunks, fin = last && args.s_final != nullptr;
+      uint32_t u[32], zz[4];
 #pragma unroll
-      for (int col = 0; col < 64; col += 16) {
-        uint32_t x[16];
-        tmem_ld16(ta + col, x);
-        tmem_wait_ld(x);
+      for (int col = 0; col < 64; col += 32) {
+        tmem_ld32(ta + col, u);
+        if (col == 0) tmem_ld4(ta + 64, zz);
+        tmem_wait_ld(u);
+        if (col == 0) tmem_wait_ld(zz);
+        if (col == 32) {
+          tc_fence_before();
+          mbar_arrive(bar(BAR_CFREE));
+        }
+        float x[32];
 #pragma unroll
-        for (int y = 0; y < 16; ++y) sum[col + y] += __uint_as_float(x[y]);
+        for (int y = 0; y < 32; ++y) x[y] = __uint_as_float(u[y]);
+        if (args.s_loc != nullptr) put_f32(args.s_loc + (((size_t)bh * args.n_chunks + c) * ROWS + row) * D + col, x, 1.f);
+        else if (!last) put_state(c + 1, col, x);
+        if (fin) {
+          // both triangles of a direct state; inside a diagonal block both (a, b) and (b, a) have a thread of their own
+          float* dst = args.s_final + (size_t)bh * n_pub * D + col;
+          if (args.packed) {
+            if (mirror || a <= b) put_f32(dst + (size_t)prow * D, x, a != b ? 1.41421356237309504880f : 1.f);
+          } else {
+            put_f32(dst + (size_t)public_row<G>(a, b, 0) * D, x, 1.f);
+            if (mirror) put_f32(dst + (size_t)public_row<G>(b, a, 0) * D, x, 1.f);
+          }
+        }
       }
-      uint32_t zz[4];
-      tmem_ld4(ta + 64, zz);
-      tmem_wait_ld(zz);
-      zsum += __uint_as_float(zz[0]);
-      tc_fence_before();
-      mbar_arrive(bar(BAR_CFREE + (i & 1)));
-      if (args.s_loc != nullptr) {
-        const size_t slot = (size_t)bh * args.n_chunks + c;
-        float4* dst = reinterpret_cast<float4*>(args.s_loc + (slot * ROWS + row) * D);
-#pragma unroll
-        for (int y = 0; y < 16; ++y) dst[y] = make_float4(sum[4 * y], sum[4 * y + 1], sum[4 * y + 2], sum[4 * y + 3]);
-        args.z_loc[slot * ROWS + row] = zsum;
-      } else if (c + 1 < args.n_chunks) {
-        write_state(c + 1);
-      }
-    }
-    if (ok && args.s_final != nullptr) {
-      // both triangles of a direct state; inside a diagonal block both (a, b) and (b, a) have a thread of their own
-      auto put = [&](int r, float f) {
-        float4* dst = reinterpret_cast<float4*>(args.s_final + ((size_t)bh * n_pub + r) * D);
-#pragma unroll
-        for (int y = 0; y < 16; ++y) dst[y] = make_float4(sum[4 * y] * f, sum[4 * y + 1] * f, sum[4 * y + 2] * f, sum[4 * y + 3] * f);
-        args.z_final[(size_t)bh * n_pub + r] = zsum * f;
-      };
-      if (args.packed) {
-        if (mirror || a <= b) put(prow, a != b ? 1.41421356237309504880f : 1.f);
-      } else {
-        put(public_row<G>(a, b, 0), 1.f);
-        if (mirror) put(public_row<G>(b, a, 0), 1.f);
+      const float z = __uint_as_float(zz[0]);
+      if (args.s_loc != nullptr) args.z_loc[((size_t)bh * args.n_chunks + c) * ROWS + row] = z;
+      else if (!last) put_z(c + 1, z);
+      if (fin) {
+        if (args.packed) {
+          if (mirror || a <= b) args.z_final[(size_t)bh * n_pub + prow] = a != b ? z * 1.41421356237309504880f : z;
+        } else {
+          args.z_final[(size_t)bh * n_pub + public_row<G>(a, b, 0)] = z;
+          if (mirror) args.z_final[(size_t)bh * n_pub + public_row<G>(b, a, 0)] = z;
+        }
       }
     }
   }
