@@ -20,11 +20,11 @@
  *     DEVICE pointers (except in kata_fwd_host), element type opts->dtype (fp32 or bf16).
  *   - All accumulation, the running state (S,Z) and the normaliser are fp32; out is rounded
  *     to the element type (round-to-nearest-even).  On the bf16 tensor-core kernels the OPERANDS of the matrix
- *     products are bf16: the chunked forms read the running state through a bf16 copy taken once per tile of 128
- *     tokens (S and Z are accumulated in fp32, but psi(q)^T S and psi(q)^T Z see them rounded), the intra-tile
- *     weights (q.k)^2 are rounded to bf16 before they multiply the values, and the key scale 1/||k||^2 is rounded to
- *     bf16 (the chunked forms multiply it into the values, v/||k||^2 rounded again; the quadratic form into the
- *     weights, rounded again, whose row sum is then the normaliser).  The convex weights of the output gate therefore sum to 1 only to
+ *     products are bf16: the chunked forms read the running state through a bf16 copy taken once per chunk (S and Z are
+ *     accumulated in fp32, but psi(q)^T S and psi(q)^T Z see them, and psi(q), rounded; psi(k) is a product of bf16 entries
+ *     and of the key scale, rounded twice), the weights (q.k)^2 inside a chunk and in the quadratic form are rounded to bf16
+ *     before they multiply the values, and the key scale 1/||k||^2 is rounded to bf16 and multiplied into the weights,
+ *     rounded again, whose row sum is then the normaliser.  The convex weights of the output gate therefore sum to 1 only to
  *     about 2^-8, and a normaliser that is tiny against its terms (a query nearly orthogonal to every key before it)
  *     can come out <= 0 from the rounded operands, in which case out = 0 as for an exact zero.  All of it stays
  *     inside the 2e-2 tolerance of the bf16 tests.
@@ -42,7 +42,8 @@
  *     other on the stream and in the same workspace (kata_workspace_bytes gives the largest slab's need), as
  *     long as no state pointer is set; the other entry points, and these with state pointers, return
  *     KATA_ERR_UNSUPPORTED_SHAPE beyond 65535 heads.  The tensor-core (tcgen05) kernels cover bf16 with d_k = d_v = 64; narrower bf16
- *     rows are zero-padded to 64 entries in the workspace and run on the same kernels (the result is the same
+ *     rows run on the same kernels as rows zero-padded to 64 entries (read that way, or in the scan forms and the
+ *     backward copied to the workspace; the result is the same
  *     function: dot products and norms do not change) unless feature_groups > 1 or a state is handed over, whose
  *     layouts depend on the true width; everything else runs on the fp32 SIMT kernels.
  *   - Return value: KATA_OK (0) or a negative kata_status.  Errors detectable on the host
@@ -50,9 +51,8 @@
  *     that expires writes KATA_ERR_DEVICE_TIMEOUT to *opts->device_status (if non-null),
  *     visible after the caller synchronises the stream; the kernel still terminates.  How long a launch
  *     that has stalled takes to end: the waits of its warps run out side by side and a warp enters no further
- *     wait once one has failed, so it is one limit, not their sum -- 0.1 s on the streaming, quadratic, backward
- *     and first-order kernels (a limit on time), and on the feature-split chunked kernel 4 M polls of at most 1 us
- *     each (between 0.1 s and 4 s) plus at most 2 s for a CTA that waits for the other CTAs of its head.
+ *     wait once one has failed, so it is one limit, not their sum -- 0.1 s (a limit on time; on the streaming and first-order kernels a
+ *     poll count that lasts between 0.1 s and 4 s).
  */
 #ifndef KATA_H_
 #define KATA_H_
@@ -109,7 +109,9 @@ enum { KATA_FN_QUADRATIC = 0, KATA_FN_CHUNKED = 1, KATA_FN_CHUNK_STATE_SCAN = 2,
  *                 group in parallel (section "Tree-scan inter-chunk reduction").  INTER_AUTO lets the
  *                 library choose: SCAN where the heads alone leave most of the GPU idle and the
  *                 sequence is long enough for the scan form's extra pass to pay (a model of the
- *                 tensor-core kernel's time in whole waves of CTAs decides); SEQUENTIAL otherwise,
+ *                 streaming kernels' time in whole waves of CTAs decides; from 16384 tokens x heads on the chunk-state
+ *                 kernels then cut the chunk axis into segments of their own instead of running the scan form's
+ *                 passes); SEQUENTIAL otherwise,
  *                 on the fp32 kernels, for feature_order 1 (whose tensor-core path makes this choice
  *                 by itself) and whenever a state is handed in or out.  Both forms give the same
  *                 result up to the rounding order of the state sums.
@@ -181,11 +183,12 @@ int kata_fwd_quadratic(const void* q, const void* k, const void* v, void* out,
  *   D = Psi(Q_[c]) Z_[c] + P 1,  O_[c] = diag(D)^-1 N
  * (section "Chunkwise forward").  O(T) work, fp32 state.  opts->inter_chunk selects how
  * the inter-chunk recurrence is traversed; both give the same result up to fp32
- * re-association.  Workspace: kata_workspace_bytes(KATA_FN_CHUNKED, ...); the sequential walk on the tensor-core
- * path (bf16, d_k = d_v = 64, feature_order 2, no state pointers) splits the state of a head over
- * nine CTAs (five, six or ten with feature_groups 2 or 4) and needs about 0.15 KB per token, head and CTA there (scaled values, key scales, the CTAs' shares of the
- * output and a counter per tile); the environment variable KATA_CHUNKED_KERNEL=stream selects the one-CTA-per-value-
- * slice streaming kernel instead (no workspace; for comparisons).
+ * re-association.  Workspace: kata_workspace_bytes(KATA_FN_CHUNKED, ...).  The sequential form on the tensor-core path
+ * (bf16, feature_order 2) writes the state before every chunk of 512 or 1024 tokens to the workspace and then answers
+ * blocks of 256 queries from that state and the keys of their chunk; sequences too short for that to pay run as one chunk,
+ * which is the quadratic form.  fp32 rows of 16 or 32 entries without state pointers work the same way on plain FMAs (chunks
+ * of 256).  The environment variable KATA_CHUNKED_KERNEL=stream selects the one-CTA-per-value-slice streaming kernel
+ * instead on the tensor-core path (no workspace; for comparisons).
  */
 int kata_fwd_chunked(const void* q, const void* k, const void* v, void* out,
                      int B, int H, int T, int d_k, int d_v, int C, const kata_opts* opts);
@@ -243,13 +246,15 @@ int kata_bwd_quadratic(const void* q, const void* k, const void* v, const void* 
  * pass (S = sum psi(k_hat) v^T, Z = sum psi(k_hat)), recomputes out_t and its normaliser and produces dq; a reverse
  * sweep carries the state sum psi(q_hat_t) [dout_t / D_t, (dout_t . out_t) / D_t] of the tokens behind and produces dk
  * and dv; the terms inside a chunk come from its C x C causal scores.  Arguments, layouts and error values as for
- * kata_bwd_quadratic; C must be 64.  fp32 arithmetic on plain FMAs for both element types (bf16 tensors are widened on
- * load and rounded once on store), every sum in a fixed order (bit-reproducible).  Supported: feature_order 2,
- * feature_groups 1, d_k in {16, 32, 64}, d_v a multiple of 8 up to 64 (KATA_ERR_UNSUPPORTED_SHAPE otherwise,
- * also for opts->impl = KATA_IMPL_TENSOR); inter_chunk, scan_group, state_layout are ignored; s_pre/z_pre/s_init/
- * z_init must be null.  Rows whose normaliser is 0 and zero rows of q or k get zero gradients.
- * Workspace: kata_workspace_bytes(KATA_FN_BWD_CHUNKED, B, H, T, d_k, d_v, 64, opts) bytes, about
- * 4 (2 d_k + d_v + (d_v / 8)(d_k + 1) + 2) bytes per token and head (2.9 KB at d_k = d_v = 64).
+ * kata_bwd_quadratic; C must be 64.  fp32 arithmetic for both element types (bf16 tensors are widened on load and rounded
+ * once on store), every sum in a fixed order (bit-reproducible).  Supported: feature_order 2, feature_groups 1, d_k in
+ * {16, 32, 64}, d_v a multiple of 8 up to 64 (KATA_ERR_UNSUPPORTED_SHAPE otherwise); inter_chunk, scan_group, state_layout
+ * are ignored; s_pre/z_pre/s_init/z_init must be null.  Rows whose normaliser is 0 and zero rows of q or k get zero
+ * gradients.  bf16 with d_k = d_v = 64 and 512 <= T <= 16384, unless opts->impl = KATA_IMPL_SIMT: the tensor-core kernels of
+ * kata_bwd_quadratic with the weights carried in three bf16 terms (24 bits) -- O(T^2) work, less at these lengths, the same
+ * precision; opts->impl = KATA_IMPL_TENSOR returns KATA_ERR_UNSUPPORTED_SHAPE outside that range.
+ * Workspace: kata_workspace_bytes(KATA_FN_BWD_CHUNKED, B, H, T, d_k, d_v, 64, opts) bytes: 12 bytes per token and head on the
+ * tensor cores, else about 4 (2 d_k + d_v + (d_v / 8)(d_k + 1) + 2) (2.9 KB at d_k = d_v = 64).
  */
 int kata_bwd_chunked(const void* q, const void* k, const void* v, const void* dout, void* dq, void* dk, void* dv,
                      int B, int H, int T, int d_k, int d_v, int C, const kata_opts* opts);
@@ -265,8 +270,8 @@ int kata_bwd_chunked(const void* q, const void* k, const void* v, const void* do
  * computed, each piece starting from the state the previous one left ("Linear attention as a recurrence").  The
  * caller's stream waits for all of it -- also when a piece fails: the error is returned only after the caller's
  * stream has been made to wait for every copy already queued on the library's streams -- so the contract above is
- * unchanged.  The result is the same function as the one-pass call; the pieces run on the streaming kernel, which
- * rounds at other places than the feature-split kernel of the one-pass call (both inside the bf16 tolerance).
+ * unchanged.  The result is the same function as the one-pass call, rounded at other places (the chunks of a piece start
+ * with the piece).
  * This route creates two streams and seven events per device on first use and keeps them; calls that take it are
  * serialised inside the library by a process-wide mutex; host memory that is not pinned makes the copies synchronous.
  * The paper has no counterpart; this is the end-to-end path measured by the benchmark.
@@ -324,7 +329,8 @@ int kata_host_plan(int fn, int B, int H, int T, int d_k, int d_v, int C, const k
                    int* piece_tokens);
 
 /* Number of scan groups, chunks per group and rounds of the scan over the group states (doubling rounds; anchor hops on
- * the first-order tensor-core path) the library would use; beyond 65535 heads, those of a full slab of heads.  For
+ * the first-order tensor-core path) of the scan form the library would use (for inter_chunk = AUTO the form that the model
+ * of the streaming kernels prefers; see kata_opts for what runs in its place); beyond 65535 heads, those of a full slab of heads.  For
  * reporting and tests. */
 int kata_scan_plan(int fn, int B, int H, int T, int d_k, int d_v, int C, const kata_opts* opts,
                    int* n_groups, int* chunks_per_group, int* scan_rounds);

@@ -1,16 +1,15 @@
 // Chunked KATA forward in fp32 on plain FMAs for rows of 16 or 32 entries (full lift, no state handed over): the states
-// before chunks of 256 tokens, all chunks in parallel, then blocks of 64 queries over the state and the keys of their
+// before chunks of 256 tokens, all chunks in parallel, then blocks of 32 or 64 queries over the state and the keys of their
 // chunk.  Short sequences are one chunk: one launch, the quadratic form.
 //   state_loc_kernel     S_loc = sum_t w psi(k_hat_t) [v_t, 1] over a chunk: thread = feature pair a <= b (w = 2 off the
 //                        diagonal: the lift is symmetric), its DV + 1 sums in registers, rows broadcast from shared memory
 //   state_prefix_kernel  running sum over the chunks, in order
-//   attend_kernel        lane = two queries; the warps of a CTA share out the feature rows of the state and the tiles
+//   attend_kernel        lane = one or two queries; the warps of a CTA share out the feature rows of the state and the tiles
 //                        of 32 keys, rows broadcast from shared memory (16 bytes per load feed 8 FMAs), and add their
 //                        numerators and normalisers in a fixed order at the end
 // What bounds it: FMAs.  The walk over the chunks of a head by one CTA (kata_simt_chunked.cu) was a chain of 21 us per 64
-// tokens; 2 heads x 512 tokens of 16 entries took 171 us.
-// Chunk length: at 16 entries a query costs 34 FMAs per key of its chunk and 2.3 k for the state, at 32 66 and 17 k: the
-// lengths up to which one chunk is the cheaper are about 1000 and 1500.
+// tokens: 2 heads x 512 tokens of 16 entries took 171 us, now 9; 16 x 16000 5378, now 242 (rows of 32: 12842, now 1197).
+// Chunk length: at 16 entries a query costs 34 FMAs per key of its chunk and 2.3 k for the state, at 32 66 and 17 k.
 #include <type_traits>
 
 #include "kata_common.cuh"
@@ -18,7 +17,6 @@
 namespace kata {
 namespace {
 
-constexpr int QB = 64;           // queries per CTA
 constexpr int CHUNK = 256;       // tokens per chunk
 
 __host__ __device__ constexpr int n_features(int d) { return d * (d + 1) / 2; }
@@ -109,16 +107,17 @@ __global__ void __launch_bounds__(128) state_prefix_kernel(float4* __restrict__ 
   }
 }
 
-template <int DK, int DV, int NW> constexpr int attend_smem_floats() {
-  const int tiles = QB * DK + NW * 32 * (DK + DV), red = NW * (DV + 1) * QB;
+template <int DK, int DV, int NW, int QPL> constexpr int attend_smem_floats() {
+  const int tiles = 32 * QPL * DK + NW * 32 * (DK + DV), red = NW * (DV + 1) * 32 * QPL;
   return tiles > red ? tiles : red;
 }
 
-template <int DK, int DV, int NW>          // NW warps share out the key tiles and state rows of a block
+// QPL queries per lane (a block is 32 QPL queries); NW warps share out its key tiles and state rows
+template <int DK, int DV, int NW, int QPL>
 __global__ void __launch_bounds__(NW * 32) attend_kernel(const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ v,
                                                          float* __restrict__ out, const float* __restrict__ S, int Tlen, int chunk,
                                                          int n_chunks) {
-  constexpr int NF = n_features(DK), SP = state_stride(DV);
+  constexpr int NF = n_features(DK), SP = state_stride(DV), QB = 32 * QPL;
   extern __shared__ __align__(16) float sm[];
   float* qs = sm;                                          // [DK][QB]
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -131,30 +130,30 @@ __global__ void __launch_bounds__(NW * 32) attend_kernel(const float* __restrict
   if (S != nullptr) cudaGridDependencySynchronize();
 
   for (int i = tid; i < QB * DK; i += NW * 32) {
-    const int row = i / DK, a = i % DK;
-    qs[a * QB + row] = q0 + row < Tlen ? qh[(size_t)(q0 + row) * DK + a] : 0.f;
+    const int row = i % QB, a = i / QB;
+    qs[i] = q0 + row < Tlen ? qh[(size_t)(q0 + row) * DK + a] : 0.f;
   }
   __syncthreads();
-  float qa[DK], qb[DK], na[DV], nb[DV], da = 0.f, db = 0.f;      // queries q0 + lane and q0 + 32 + lane
+  float qr[QPL][DK], num[QPL][DV], den[QPL];               // queries q0 + 32 u + lane
 #pragma unroll
-  for (int i = 0; i < DK; ++i) {
-    qa[i] = qs[i * QB + lane];
-    qb[i] = qs[i * QB + 32 + lane];
+  for (int u = 0; u < QPL; ++u) {
+    den[u] = 0.f;
+#pragma unroll
+    for (int i = 0; i < DK; ++i) qr[u][i] = qs[i * QB + 32 * u + lane];
+#pragma unroll
+    for (int i = 0; i < DV; ++i) num[u][i] = 0.f;
   }
-#pragma unroll
-  for (int i = 0; i < DV; ++i) na[i] = nb[i] = 0.f;
-  auto add = [&](const float* row, float wa, float wb) {
+  auto add = [&](const float* row, const float (&w)[QPL]) {
 #pragma unroll
     for (int i = 0; i < DV; i += 4) {
       const float4 x = ld4(row + i);
-      na[i] = fmaf(wa, x.x, na[i]);
-      na[i + 1] = fmaf(wa, x.y, na[i + 1]);
-      na[i + 2] = fmaf(wa, x.z, na[i + 2]);
-      na[i + 3] = fmaf(wa, x.w, na[i + 3]);
-      nb[i] = fmaf(wb, x.x, nb[i]);
-      nb[i + 1] = fmaf(wb, x.y, nb[i + 1]);
-      nb[i + 2] = fmaf(wb, x.z, nb[i + 2]);
-      nb[i + 3] = fmaf(wb, x.w, nb[i + 3]);
+#pragma unroll
+      for (int u = 0; u < QPL; ++u) {
+        num[u][i] = fmaf(w[u], x.x, num[u][i]);
+        num[u][i + 1] = fmaf(w[u], x.y, num[u][i + 1]);
+        num[u][i + 2] = fmaf(w[u], x.z, num[u][i + 2]);
+        num[u][i + 3] = fmaf(w[u], x.w, num[u][i + 3]);
+      }
     }
   };
   // ---- the state before the chunk ----
@@ -168,7 +167,9 @@ __global__ void __launch_bounds__(NW * 32) attend_kernel(const float* __restrict
       ++a;
     }
     int b = a + rem;
-    float xa = qs[a * QB + lane], xb = qs[a * QB + 32 + lane];
+    float xa[QPL];
+#pragma unroll
+    for (int u = 0; u < QPL; ++u) xa[u] = qs[a * QB + 32 * u + lane];
     // sixteen rows at a time through this warp's tile buffer, the next sixteen on their way meanwhile
     constexpr int RB = 16, N4 = RB * SP / 4, PL = (N4 + 31) / 32;
     float4 pre[PL];
@@ -189,17 +190,20 @@ __global__ void __launch_bounds__(NW * 32) attend_kernel(const float* __restrict
       const int n = f1 - fb < RB ? f1 - fb : RB;
 #pragma unroll 2
       for (int r = 0; r < n; ++r) {
-        const float wa = xa * qs[b * QB + lane], wb = xb * qs[b * QB + 32 + lane];
         const float* row = kt + r * SP;
-        add(row, wa, wb);
         const float z = row[DV];
-        da = fmaf(wa, z, da);
-        db = fmaf(wb, z, db);
+        float w[QPL];
+#pragma unroll
+        for (int u = 0; u < QPL; ++u) {
+          w[u] = xa[u] * qs[b * QB + 32 * u + lane];
+          den[u] = fmaf(w[u], z, den[u]);
+        }
+        add(row, w);
         if (++b == DK) {
           b = ++a;
           if (a < DK) {
-            xa = qs[a * QB + lane];
-            xb = qs[a * QB + 32 + lane];
+#pragma unroll
+            for (int u = 0; u < QPL; ++u) xa[u] = qs[a * QB + 32 * u + lane];
           }
         }
       }
@@ -215,47 +219,47 @@ __global__ void __launch_bounds__(NW * 32) attend_kernel(const float* __restrict
     const bool diag = t0 + 31 > q0;
 #pragma unroll 4
     for (int t = 0; t < 32; ++t) {
-      float4 a4 = make_float4(0.f, 0.f, 0.f, 0.f), b4 = a4;      // (four partial sums: a chain of DK FMAs would set the pace)
+      float4 s4[QPL];                                      // (four partial sums: a chain of DK FMAs would set the pace)
+#pragma unroll
+      for (int u = 0; u < QPL; ++u) s4[u] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
       for (int i = 0; i < DK; i += 4) {
         const float4 x = ld4(kt + t * DK + i);
-        a4.x = fmaf(qa[i], x.x, a4.x);
-        a4.y = fmaf(qa[i + 1], x.y, a4.y);
-        a4.z = fmaf(qa[i + 2], x.z, a4.z);
-        a4.w = fmaf(qa[i + 3], x.w, a4.w);
-        b4.x = fmaf(qb[i], x.x, b4.x);
-        b4.y = fmaf(qb[i + 1], x.y, b4.y);
-        b4.z = fmaf(qb[i + 2], x.z, b4.z);
-        b4.w = fmaf(qb[i + 3], x.w, b4.w);
+#pragma unroll
+        for (int u = 0; u < QPL; ++u) {
+          s4[u].x = fmaf(qr[u][i], x.x, s4[u].x);
+          s4[u].y = fmaf(qr[u][i + 1], x.y, s4[u].y);
+          s4[u].z = fmaf(qr[u][i + 2], x.z, s4[u].z);
+          s4[u].w = fmaf(qr[u][i + 3], x.w, s4[u].w);
+        }
       }
-      const float sa = (a4.x + a4.y) + (a4.z + a4.w), sb = (b4.x + b4.y) + (b4.z + b4.w);
-      float wa = sa * sa, wb = sb * sb;
-      if (diag) {
-        if (t0 + t > q0 + lane) wa = 0.f;
-        if (t0 + t > q0 + 32 + lane) wb = 0.f;
+      float w[QPL];
+#pragma unroll
+      for (int u = 0; u < QPL; ++u) {
+        const float s = (s4[u].x + s4[u].y) + (s4[u].z + s4[u].w);
+        w[u] = s * s;
+        if (diag && t0 + t > q0 + 32 * u + lane) w[u] = 0.f;
+        den[u] += w[u];
       }
-      da += wa;
-      db += wb;
-      add(vt + t * DV, wa, wb);
+      add(vt + t * DV, w);
     }
   }
   // ---- the warps' shares, in order ----
   __syncthreads();
   float* red = sm + warp * (DV + 1) * QB;                  // [warp][DV + 1][QB]
 #pragma unroll
-  for (int i = 0; i < DV; ++i) {
-    red[i * QB + lane] = na[i];
-    red[i * QB + 32 + lane] = nb[i];
-  }
-  red[DV * QB + lane] = da;
-  red[DV * QB + 32 + lane] = db;
-  __syncthreads();
-  const int row = tid & (QB - 1), part = tid / QB;         // four threads per query (of the first 256)
-  if (part >= 4) return;
-  float den = 0.f;
+  for (int u = 0; u < QPL; ++u) {
 #pragma unroll
-  for (int w = 0; w < NW; ++w) den += sm[(w * (DV + 1) + DV) * QB + row];
-  const float inv = den > 0.f ? 1.f / den : 0.f;
+    for (int i = 0; i < DV; ++i) red[i * QB + 32 * u + lane] = num[u][i];
+    red[DV * QB + 32 * u + lane] = den[u];
+  }
+  __syncthreads();
+  const int row = tid % QB, part = tid / QB;               // four threads per query
+  if (part >= 4) return;
+  float dsum = 0.f;
+#pragma unroll
+  for (int w = 0; w < NW; ++w) dsum += sm[(w * (DV + 1) + DV) * QB + row];
+  const float inv = dsum > 0.f ? 1.f / dsum : 0.f;
   if (q0 + row >= Tlen) return;
   constexpr int CPT = DV / 4;                              // columns per thread
   float* dst = out + ((size_t)bh * Tlen + q0 + row) * DV + part * CPT;
@@ -270,13 +274,15 @@ __global__ void __launch_bounds__(NW * 32) attend_kernel(const float* __restrict
   }
 }
 
-int one_chunk_tokens(int d_k) { return d_k == 16 ? 1024 : 1536; }
+// measured, us, one chunk / chunks of 256: rows of 16, one head x 1024 tokens 19 / 34, 256 heads 349 / 247; rows of 32, one
+// head x 1400 46 / 76, 128 heads x 1536 872 / 950
+int one_chunk_tokens(const Problem& p) { return p.d_k == 32 ? 1536 : (long long)p.B * p.H * p.T <= 16384 ? 1024 : 512; }
 
 template <int DK, int DV> void run(const Problem& p, float* S, LaunchCtx& ctx) {
   const int BH = p.B * p.H;
   const float *q = static_cast<const float*>(p.q), *k = static_cast<const float*>(p.k), *v = static_cast<const float*>(p.v);
-  const bool states = p.T > one_chunk_tokens(DK);
-  const int chunk = states ? CHUNK : (p.T + QB - 1) / QB * QB, n_chunks = (p.T + chunk - 1) / chunk;
+  const bool states = p.T > one_chunk_tokens(p);
+  const int chunk = states ? CHUNK : (p.T + 63) / 64 * 64, n_chunks = (p.T + chunk - 1) / chunk;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -294,20 +300,24 @@ template <int DK, int DV> void run(const Problem& p, float* S, LaunchCtx& ctx) {
     ok = cudaLaunchKernelEx(&cfg, state_prefix_kernel, reinterpret_cast<float4*>(S), n4, n_chunks) == cudaSuccess;
     ctx.launches += ok;
   }
-  cfg.gridDim = dim3((p.T + QB - 1) / QB, BH);
   cfg.numAttrs = states ? 1 : 0;
-  auto attend = [&](auto nw) {
-    constexpr int NW = decltype(nw)::value, smem = attend_smem_floats<DK, DV, NW>() * (int)sizeof(float);
+  auto attend = [&](auto nw, auto qpl) {
+    constexpr int NW = decltype(nw)::value, QPL = decltype(qpl)::value;
+    constexpr int smem = attend_smem_floats<DK, DV, NW, QPL>() * (int)sizeof(float);
+    cfg.gridDim = dim3((p.T + 32 * QPL - 1) / (32 * QPL), BH);
     cfg.blockDim = dim3(NW * 32);
     cfg.dynamicSmemBytes = smem;
-    return allow_smem<attend_kernel<DK, DV, NW>>(smem) &&
-           cudaLaunchKernelEx(&cfg, attend_kernel<DK, DV, NW>, q, k, v, static_cast<float*>(p.out), (const float*)(states ? S : nullptr),
-                              p.T, chunk, n_chunks) == cudaSuccess;
+    return allow_smem<attend_kernel<DK, DV, NW, QPL>>(smem) &&
+           cudaLaunchKernelEx(&cfg, attend_kernel<DK, DV, NW, QPL>, q, k, v, static_cast<float*>(p.out),
+                              (const float*)(states ? S : nullptr), p.T, chunk, n_chunks) == cudaSuccess;
   };
-  // sixteen warps where there are few blocks (rows of 16 leave registers for them): 2 heads x 512 tokens 15.6 us with eight
-  // warps, 13.4 with sixteen; 256 heads x 1024 tokens 349 and 419
-  const bool few = DK == 16 && DV == 16 && (long long)cfg.gridDim.x * cfg.gridDim.y <= 148;
-  ok = ok && (few ? attend(std::integral_constant<int, DK == 16 && DV == 16 ? 16 : 8>{}) : attend(std::integral_constant<int, 8>{}));
+  // Two queries per lane feed two FMAs per word loaded; where that makes fewer blocks than SMs, one query per lane and, if
+  // the registers allow it, sixteen warps (2 heads x 512 tokens of 16 entries: 15.6 us of GPU time,
+  // 13.4 with sixteen warps, 9.1 with one query per lane as well; 256 heads x 1024 tokens the other way round: 349 and 419).
+  using std::integral_constant;
+  const bool few = (long long)((p.T + 63) / 64) * BH <= 148;
+  ok = ok && (few ? attend(integral_constant<int, DK == 16 && DV == 16 ? 16 : 8>{}, integral_constant<int, 1>{})
+                  : attend(integral_constant<int, 8>{}, integral_constant<int, 2>{}));
   if (!ok) {
     cudaGetLastError();
     ctx.status = KATA_ERR_CUDA;
@@ -323,7 +333,7 @@ bool simt_attend_supported(const Problem& p) {
 }
 
 size_t simt_attend_workspace_bytes(const Problem& p) {
-  if (p.T <= one_chunk_tokens(p.d_k)) return 0;
+  if (p.T <= one_chunk_tokens(p)) return 0;
   return (size_t)p.B * p.H * ((p.T + CHUNK - 1) / CHUNK) * n_features(p.d_k) * state_stride(p.d_v) * sizeof(float);
 }
 

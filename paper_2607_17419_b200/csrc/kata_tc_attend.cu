@@ -82,7 +82,7 @@ enum {
   BAR_PFULL = 16,    // [half][sub] the builders are done with the sub-buffer (128)
   BAR_FFULL = 20,    // [half][sub][piece] features of a state tile in TMEM (128)
   BAR_SFREE = 28,    // [half][sub][piece] ... and consumed
-  BAR_QT = 36,       // [2] query tile in TMEM (256)
+  BAR_QT = 36,       // [2] query tile in TMEM (128)
   BAR_ODONE = 38,    // [2] the MMAs of an item are complete: [O | D] is final
   BAR_OFREE = 40,    // [2] [O | D] has been read (256): the next item may overwrite it
   BAR_DRAIN = 42,
@@ -90,10 +90,11 @@ enum {
 };
 
 // Pre-pass: r = 1 / ||k||^2 per key row (0 for a zero row); eight lanes of 16 bytes per row, four rows per lane in flight
-// (memory-bound; one row per lane: RSFIG).
+// (memory-bound; 33.5 MB of keys: 8.7 us with one row per lane, 6.9 with four).
 constexpr int RS_ROWS = 4;
 __global__ void __launch_bounds__(256) rscale_kernel(const __nv_bfloat16* __restrict__ k, __nv_bfloat16* __restrict__ rscale,
                                                      size_t n_rows, int d) {
+  cudaTriggerProgrammaticLaunchCompletion();   // the kernel behind sets itself up meanwhile
   const size_t row0 = (size_t)blockIdx.x * (32 * RS_ROWS) + (threadIdx.x >> 3);
   const int part = threadIdx.x & 7;
   uint4 raw[RS_ROWS];
@@ -209,7 +210,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     mbar_init(bar(BAR_QFULL), 1);
     mbar_init(bar(BAR_QEMPTY), 512);
     for (int i = 0; i < 2; ++i) {
-      mbar_init(bar(BAR_QT + i), 256);
+      mbar_init(bar(BAR_QT + i), 128);
       mbar_init(bar(BAR_ODONE + i), 1);
       mbar_init(bar(BAR_OFREE + i), 256);
     }
@@ -248,6 +249,9 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
   tc_fence_after();
   const uint32_t tb = tmem_base_s;
   bool ok = true;
+  // A programmatic dependent launch behind the state kernel, which may run for long: everybody waits for it here, where no
+  // limit on time applies.  (Without states only warp 3 waits, for the key scales.)
+  if (args.first_state < args.n_chunks) cudaGridDependencySynchronize();
 
   if (warp == 0) {
     regs_release<64>();
@@ -256,8 +260,6 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       uint32_t it = 0;                                   // tiles loaded so far, over all items
       int ni = 0;
       Item w;
-      // the kernel is a programmatic dependent launch: the states are the work of the kernel before it
-      if (args.first_state < args.n_chunks) cudaGridDependencySynchronize();
       for (int n = 0; ok && next_item(n, w); ++n, ++ni) {
         ok = wait_or_abort(bar(BAR_QEMPTY), (ni & 1) ^ 1, abort_flag);
         if (!ok) break;
@@ -380,7 +382,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     regs_release<64>();
     // =========================== per tile: r = 1 / ||k||^2 of its keys, or its column of Z, to shared memory ===========================
     // (the key scale multiplies the weights, so the values are used as they are; a zero key row has r = 0: zero
-    // feature).  A programmatic dependent launch: this warp and the producer wait for the kernels before.
+    // feature).
     cudaGridDependencySynchronize();
     uint32_t it = 0;
     Item w;
@@ -436,18 +438,22 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     const uint32_t qrow_s = smem_u32(base + OFF_Q) + h * 16384;
     // 16 bytes (eight features) of this thread's query row, from the item's tile in shared memory
     auto qrun = [&](int c) { return lds128(qrow_s + sw128_offset(rowl, c)); };
-    // the query tile of an item into TMEM: this thread's row, 32 of its features
+    // The query tile of an item into TMEM, by the warps of the second sub-buffer: the scores of an item's last tile are
+    // issued sub-buffer 0 first, so only they know that no score MMA reads the tile of the item before any more.
     auto copy_q = [&](int ni, const Item& w) {
       ok = ok && wait_or_abort(bar(BAR_QFULL), ni & 1, abort_flag);
       if (!ok) return;
-      if (h == 0 || w.nk_b > 0) {
-        uint32_t r[16];
+      if (ch == 1 && (h == 0 || w.nk_b > 0)) {
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const uint4 x = qrun(ch * 4 + c);
-          r[4 * c] = x.x; r[4 * c + 1] = x.y; r[4 * c + 2] = x.z; r[4 * c + 3] = x.w;
+        for (int hf = 0; hf < 2; ++hf) {
+          uint32_t r[16];
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            const uint4 x = qrun(hf * 4 + c);
+            r[4 * c] = x.x; r[4 * c + 1] = x.y; r[4 * c + 2] = x.z; r[4 * c + 3] = x.w;
+          }
+          tmem_st16(tmem_addr(tb, q4 * 32, COL_Q + h * 32 + hf * 16), r);
         }
-        tmem_st16(tmem_addr(tb, q4 * 32, COL_Q + h * 32 + ch * 16), r);
         tmem_wait_st();
         tc_fence_before();
         mbar_arrive(bar(BAR_QT + h));
@@ -571,7 +577,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         mbar_arrive(bar(BAR_PFULL + 2 * h + ch));
       }
       if (!ok) break;
-      // the next item's queries go to TMEM before the wait for this item's last MMAs (its score MMAs are all through)
+      // the next item's queries go to TMEM before the wait for this item's last MMAs
       const int bh = w.bh;
       ++n;
       more = next_item(n, w);

@@ -106,7 +106,7 @@ enum {
   BAR_SFULL = 16,    // [2] scores in TMEM
   BAR_SFREE = 18,    // [2] the score buffer may take new scores (its weight warps; where weights lie over scores, the output MMAs)
   BAR_PFULL = 20,    // [2] weights stored, scalars read (CS x 128 threads)
-  BAR_PFREE = 22,    // [2] weights consumed
+  BAR_PFREE = 22,    // [2] weights consumed, or (first sweep) the step seen by the output issuer
   BAR_ODONE = 24,    // the accumulators of an item are complete
   BAR_OFREE = 25,    // ... and have been read (256 threads)
   BAR_XT = 26,       // [2] fixed tiles of an item in TMEM (256 threads)
@@ -160,6 +160,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
   __shared__ int abort_s;
   volatile int* abort_flag = &abort_s;
 
+  cudaTriggerProgrammaticLaunchCompletion();                      // (dk, dv start on the SMs that dq leaves)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int n_m = (args.Tlen + MT - 1) / MT;                      // fixed tiles of a head
   const int n_stream = (args.Tlen + NT - 1) / NT;                 // streamed tiles of the whole sequence
@@ -222,6 +223,9 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
   tc_fence_after();
   const uint32_t tb = tmem_base_s;
   bool ok = true;
+  // A programmatic dependent launch.  dk, dv start while dq runs on other SMs and wait for it here, where no limit on time
+  // applies; dq waits for its pre-pass where it reads the key scales.
+  if (MODE == MODE_DKV) cudaGridDependencySynchronize();
 
   if (warp == 0) {
     if (SETS == 4) regs_release<64>();
@@ -313,7 +317,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
           ok = wait_or_abort(bar(BAR_PFULL + b), (t / NBUF) & 1, abort_flag);
           if (!ok) break;
           if (MODE == MODE_DQ && j < w.ntiles) {         // (the first sweep only sums the row scalars)
-            if (!SEP) mbar_arrive(bar(BAR_SFREE + b));
+            mbar_arrive(bar((SEP ? BAR_PFREE : BAR_SFREE) + b));
             mbar_arrive(bar(BAR_EMPTY + s));
             continue;
           }
@@ -348,8 +352,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
   } else if (warp == 3) {
     if (SETS == 4) regs_release<64>();
     // =========================== scalars of the streamed rows, two tiles ahead ===========================
-    // A programmatic dependent launch: only this warp reads what the kernel before it wrote.
-    cudaGridDependencySynchronize();
+    if (MODE == MODE_DQ) cudaGridDependencySynchronize();
     constexpr int RPL = NT / 32;                       // rows per lane
     constexpr int FPR = MODE == MODE_DQ ? 1 : 2;       // floats per row
     const float* src = MODE == MODE_DQ ? args.rk : args.stats;
@@ -426,7 +429,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
       mbar_arrive(bar(BAR_XT + xb));
       if (MODE == MODE_DQ) mbar_arrive(bar(BAR_XEMPTY + xb));
     };
-    uint32_t t0 = 0, n_out = 0;                  // steps of the items before; steps with outputs of this set's buffer
+    uint32_t t0 = 0, n_out = 0;                  // steps of the items before; steps of this set's buffer
     int ni = 0;
     Item w, wn;
     int n = 0, nn = 0;
@@ -507,7 +510,12 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
           sum_d += d2.x + d2.y;
           sum_m += m2.x + m2.y;
           }
-          end();                                 // nothing is stored
+          // (nothing is stored, but the output issuer must have seen this buffer's step before: a parity cannot tell two
+          // phases of BAR_PFULL apart)
+          if (SEP && n_out > 0) ok = wait_or_abort(bar(BAR_PFREE + grp), (n_out - 1) & 1, abort_flag);
+          if (!ok) break;
+          ++n_out;
+          end();
         }
         if (!ok) break;
         // the sets' shares of a row meet, in a fixed order
@@ -759,6 +767,7 @@ size_t align256(size_t n) { return (n + 255) / 256 * 256; }
 
 // Pre-pass: one warp per 4 key rows (8 lanes x 16 bytes per row).  r = 1 / ||k||^2 (fp32).
 __global__ void __launch_bounds__(256) bwd_rscale_kernel(const __nv_bfloat16* __restrict__ k, float* __restrict__ rk, size_t n_rows) {
+  cudaTriggerProgrammaticLaunchCompletion();
   const size_t row = (size_t)blockIdx.x * 32 + (threadIdx.x >> 3);
   const int part = threadIdx.x & 7;
   if (row >= n_rows) return;

@@ -141,6 +141,7 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
   static constexpr PairTable<G> kPairs{};
   constexpr int ROWS = PairTable<G>::kRows;
 
+  cudaTriggerProgrammaticLaunchCompletion();      // the kernel behind starts on the SMs that this one leaves
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int slice = blockIdx.x, bh = blockIdx.y;
   const int c_beg = blockIdx.z * args.seg_chunks, c_end = min(c_beg + args.seg_chunks, args.walk_chunks);
@@ -455,6 +456,7 @@ __global__ void __launch_bounds__(256) state_fix_kernel(const float* __restrict_
                                                         int seg_chunks, float* __restrict__ s_final, float* __restrict__ z_final, int packed) {
   constexpr int ROWS = PairTable<G>::kRows;
   static constexpr PairTable<G> kPairs{};
+  cudaTriggerProgrammaticLaunchCompletion();
   cudaGridDependencySynchronize();
   const int bh = blockIdx.y, idx = blockIdx.x * 256 + threadIdx.x, row = idx >> 4, c4 = idx & 15;   // ROWS is a multiple of 16
   const int p = row >> 6, e = row & 63;

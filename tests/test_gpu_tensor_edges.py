@@ -127,3 +127,26 @@ def test_queries_nearly_orthogonal_to_every_key(form):
         check(g[b, h], r, "bf16", f"near-orthogonal/{form} head ({b},{h})")
         check(g[b, h][probes], r[probes], "bf16", f"near-orthogonal/{form} probe rows, head ({b},{h})")
         assert np.all(np.abs(g[b, h][probes]).max(axis=1) > 0), "a probe row came out as 0: its normaliser was lost"
+
+
+@pytest.mark.parametrize("T", [130, 325, 421])
+def test_many_short_heads(T):
+    """Hundreds of heads of a few tiles: every CTA of the persistent forward and backward kernels runs through many short
+    items, so that the hand-over from one item to the next is what is timed.  Heads against the definition, and the same
+    bits from every run."""
+    import torch
+    B, H = 40, 16
+    w = inputs.gaussian_workload(f"short_{T}", "bf16", B, H, T, 64, 64, 64, 950 + T)
+    q, k, v = dev_tensors(w)
+    g = torch.from_numpy(inputs.normal(3, 7, B * H * T * 64).reshape(B, H, T, 64)).to(torch.bfloat16).cuda()
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    run_all = lambda: (kb.kata_fwd_quadratic(q, k, v, device_status=st), *kb.kata_bwd_quadratic(q, k, v, g, device_status=st))
+    first = run_all()
+    for _ in range(30):
+        assert all(torch.equal(a, b) for a, b in zip(first, run_all()))
+    assert int(st.item()) == 0
+    for (b, h), r in oracle_full(w, heads=[(0, 0), (17, 5), (B - 1, H - 1)]).items():
+        check(to_numpy64(first[0])[b, h], r, "bf16", f"T={T} head ({b},{h})")
+        refs = ko.kata_quadratic_bwd(w.q_ref[b, h], w.k_ref[b, h], w.v_ref[b, h], to_numpy64(g[b, h]))
+        for name, got, ref in zip(("dq", "dk", "dv"), first[1:], refs):
+            assert np.max(np.abs(to_numpy64(got[b, h]) - ref)) <= 2e-2 * max(1.0, np.abs(ref).max()), (name, b, h)
