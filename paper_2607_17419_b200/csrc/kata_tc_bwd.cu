@@ -89,7 +89,7 @@ constexpr uint32_t OFF_X = 0;                      // 2 x (two fixed tiles of 12
 constexpr uint32_t OFF_ST = 65536;                 // stages: two streamed tiles of up to 8 KB
 constexpr uint32_t STAGE_BYTES = 16384;
 constexpr uint32_t OFF_SC = OFF_ST + NSTAGE * STAGE_BYTES;   // per stage 512 bytes of scalars of the streamed rows:
-                                                             // r_i (MODE_DQ) or (1/D_t, dout_t . o_t) (MODE_DKV)
+                                                             // r_i (MODE_DQ) or 1/D_t and -dout_t . o_t (MODE_DKV)
 constexpr uint32_t OFF_PART = OFF_SC + NSTAGE * 512;         // 2 (item parity) x 4 sets x 128 float2: the sums of a row meet here
 constexpr uint32_t OFF_BAR = OFF_PART + 8192;
 constexpr uint32_t SMEM_BYTES = OFF_BAR + 256;
@@ -385,7 +385,10 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
         if (!ok) break;
 #pragma unroll
         for (int e = 0; e < RPL * FPR; ++e) {
-          reinterpret_cast<float*>(sc(s))[lane * RPL * FPR + e] = v0[e];
+          // MODE_DKV: (1/D, 1/D, -dout.o, -dout.o) of a pair of rows, the operands of the packed multiplies and adds
+          const int i = lane * RPL * FPR + e, row = i >> 1;
+          if (MODE == MODE_DQ) reinterpret_cast<float*>(sc(s))[i] = v0[e];
+          else reinterpret_cast<float*>(sc(s))[(row >> 1) * 4 + (i & 1) * 2 + (row & 1)] = (i & 1) ? -v0[e] : v0[e];
           v0[e] = v1[e];
           v1[e] = v2[e];
         }
@@ -569,10 +572,10 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
                   const float4 r4 = cs[c / 4];
                   e2 = __fmul2_rn(__fmul2_rn(__fadd2_rn(c2, make_float2(-del_row, -del_row)), (c & 2) ? make_float2(r4.z, r4.w) : make_float2(r4.x, r4.y)), s2);
                 } else {
-                  const float4 st = cs[c / 2];                                  // (1/D, dout.o) of two queries
-                  const float2 t2 = __fmul2_rn(s2, make_float2(st.x, st.z));    // s / D
+                  const float4 st = cs[c / 2];                                  // 1/D and -dout.o of two queries
+                  const float2 t2 = __fmul2_rn(s2, make_float2(st.x, st.y));    // s / D
                   p2 = __fmul2_rn(t2, s2);
-                  e2 = __fmul2_rn(__fadd2_rn(c2, make_float2(-st.y, -st.w)), t2);
+                  e2 = __fmul2_rn(__fadd2_rn(c2, make_float2(st.z, st.w)), t2);
                 }
                 if constexpr (decltype(masked)::value) {
                   if (dead(c)) { e2.x = 0.f; p2.x = 0.f; }
@@ -608,7 +611,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
                 f = __fmul2_rn(__fadd2_rn(c2, make_float2(-del_row, -del_row)), (c & 2) ? make_float2(r4.z, r4.w) : make_float2(r4.x, r4.y));
               } else {
                 const float4 st = cs[c / 2];
-                f = __fmul2_rn(__fadd2_rn(c2, make_float2(-st.y, -st.w)), make_float2(st.x, st.z));
+                f = __fmul2_rn(__fadd2_rn(c2, make_float2(st.z, st.w)), make_float2(st.x, st.y));
               }
               if constexpr (decltype(masked)::value) {
                 if (dead(c)) f.x = 0.f;
@@ -643,7 +646,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
 #pragma unroll
               for (int c = 0; c < 32; c += 2) {
                 const float4 st = cs[c / 2];
-                float2 p2 = __fmul2_rn(ss[c / 2], make_float2(st.x, st.z));
+                float2 p2 = __fmul2_rn(ss[c / 2], make_float2(st.x, st.y));
                 if constexpr (decltype(masked)::value) {
                   if (dead(c)) p2.x = 0.f;
                   if (dead(c + 1)) p2.y = 0.f;
