@@ -287,9 +287,11 @@ tc_order1_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     }
   } else if (warp == W_MMA_A) {
     // =========================== scores P = Q K^T ===========================
-    // Four issuer warps, one per MMA group of a tile: the groups of a tile do not depend on one another, and a
-    // thread that waits for one group's operands should not hold up the next group's MMAs.  Every lane waits, one issues (a warp of
-    // waiters is woken sooner than a single waiting lane).
+    // Four issuer warps, one per MMA group of a tile: the groups of a tile do not depend on one another, and a thread that
+    // waits for one group's operands should not hold up the next group's MMAs.  Every lane waits, lane 0 issues (a warp of
+    // waiters is woken sooner than a single waiting lane).  Issued by an elected lane, with the descriptors in uniform
+    // registers, the MMAs of a group enter the pipe in one run and the groups get in one another's way: 16 heads x 131072
+    // tokens in one pass 1320 us instead of 1230, 64 x 32768 329 instead of 323.
     if (wo) {
       const uint32_t idQK = instr_desc(kFmtBF16, kFmtBF16, 0, 0, 128, 128);
       const uint64_t dk = smem_desc(0, 16, 1024, kSwizzle128B);
@@ -298,7 +300,7 @@ tc_order1_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         ok = wait_or_abort_counted(bar(BAR_FULL + s), (j / NSTAGE) & 1, abort_flag) &&
              wait_or_abort_counted(bar(BAR_P_EMPTY + b), ((j >> 1) & 1) ^ 1, abort_flag);
         if (!ok) break;
-        if (elect_one()) {
+        if (lane == 0) {
           const uint32_t qa = smem_u32(qtile(s)), ka = smem_u32(ktile(s));
           tc_fence_after();
 #pragma unroll
@@ -324,7 +326,7 @@ tc_order1_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       // the accumulators are free once the snapshot of the previous state has left TMEM
       if (ok && upd && wo && j > 0) ok = wait_or_abort_counted(bar(BAR_SNAP_LD), (j - 1) & 1, abort_flag);
       if (!ok) break;
-      if (elect_one()) {
+      if (lane == 0) {
         const uint32_t ka = smem_u32(ktile(s)), va = smem_u32(vtile(s));
         if (upd) {
           tc_fence_after();
@@ -354,7 +356,7 @@ tc_order1_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         // the snapshot after tile j - 1 went to buffer j & 1; it is that buffer's ((j - 1) / 2)-th
         if (ok && j > 0) ok = wait_or_abort_counted(bar(BAR_SNAP_ST + (j & 1)), ((j - 1) >> 1) & 1, abort_flag);
         if (!ok) break;
-        if (elect_one()) {
+        if (lane == 0) {
           if (resume || j > 0) {
             const uint32_t qa = smem_u32(qtile(s));
             tc_fence_after();
@@ -379,7 +381,7 @@ tc_order1_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
              wait_or_abort_counted(bar(BAR_P_FULL + b), (j >> 1) & 1, abort_flag) &&
              wait_or_abort_counted(bar(BAR_R_DONE + b), (j >> 1) & 1, abort_flag);
         if (!ok) break;
-        if (elect_one()) {
+        if (lane == 0) {
           const uint32_t va = smem_u32(vtile(s));
           tc_fence_after();
 #pragma unroll
@@ -507,7 +509,7 @@ tc_order1_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if ((warp == W_MMA_A || warp == W_MMA_B || warp == W_MMA_U || warp == W_MMA_R) && elect_one()) {
+  if ((warp == W_MMA_A || warp == W_MMA_B || warp == W_MMA_U || warp == W_MMA_R) && lane == 0) {
     mma_commit(bar(BAR_DRAIN));
     mbar_wait(bar(BAR_DRAIN), 0);
   }
