@@ -169,7 +169,9 @@ struct StateBuffers {
   float* z_final;
   int layout;
 };
-int tc_state_rows(int groups);
+int tc_state_rows(const Problem& p);
+// Rows of up to 32 entries (full map): the tensor-core kernels skip the empty half of the features.
+inline bool tc_narrow(const Problem& p) { return p.groups == 1 && p.d_k <= 32; }
 void tc_states(const Problem& p, const __nv_bfloat16* rscale, const StatePlan& plan, const StateBuffers& buf, int* device_status,
                LaunchCtx& ctx);
 // Outputs of blocks of 256 queries: over the keys of their chunk and the state before it (zero-initialise for the

@@ -4,7 +4,8 @@
 // The 64 features of a row are cut into 8 runs of 8; the pair (g, h), h <= g, is the 64 products u[8g+i] u[8h+j].
 // (q.k)^2 = sum over the pairs of w <Q_gh, K_gh> with w = 1 for g = h and 2 otherwise (the lift is symmetric); the
 // blockwise map keeps the pairs inside a feature group.  36, 20 and 12 pairs for 1, 2 and 4 groups: multiples of four,
-// so the feature axis falls into slices of 256 rows.  Inside a pair, row 8 j + i is the product (8g+i, 8h+j).
+// so the feature axis falls into slices of 256 rows.  Rows of up to 32 entries have only the first four runs: 10 pairs of
+// the full map, and two empty ones.  Inside a pair, row 8 j + i is the product (8g+i, 8h+j).
 // Order of the pairs: the pairs 4s and 4s+2, and 4s+1 and 4s+3, share h wherever the counts allow it, because one warp of
 // the state kernel builds those two and then fetches the factors of run h once.
 #pragma once
@@ -12,9 +13,9 @@
 
 namespace kata {
 
-template <int G> struct PairTable {
-  static constexpr int kRuns = 8 / G;                       // runs of 8 features per group
-  static constexpr int kPairs = G * kRuns * (kRuns + 1) / 2;
+template <int G, int R = 8> struct PairTable {
+  static constexpr int kRuns = R / G;                       // runs of 8 features per group
+  static constexpr int kPairs = (G * kRuns * (kRuns + 1) / 2 + 3) / 4 * 4;
   static constexpr int kSlices = kPairs / 4;                // slices of 256 state rows
   static constexpr int kRows = kPairs * 64;
   uint8_t g[kPairs], h[kPairs];
@@ -41,6 +42,7 @@ template <int G> struct PairTable {
         }
       }
     for (int i = 0; i + 1 < n_single; i += 2) put(single_g[i], single_h[i], single_g[i + 1], single_h[i + 1]);
+    if (2 * couple < kPairs) put(R, R, R + 1 < 8 ? R + 1 : R, R);      // (narrow rows: two pairs of empty runs)
   }
 };
 

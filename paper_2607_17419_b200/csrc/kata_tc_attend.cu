@@ -20,7 +20,9 @@
 //   epilogue out = O / D  (0 where that is 0)      the gate/normalise step of the readout
 // There is no running maximum and no rescaling: the weights are polynomial.  The query norm cancels between
 // numerator and denominator and is never applied.  In the quadratic form the d^2-wide feature state is never formed.
-// Rows narrower than 64 entries are read by TMA boxes of 64 columns, whose columns beyond the row are zero.
+// Rows narrower than 64 entries are read by TMA boxes of 64 columns, whose columns beyond the row are zero; with up to 32
+// entries (R = 4 runs of 8) the empty half of the features is left out: 12 block pairs instead of 36, two score steps
+// instead of four (8 heads x 16 x 6000 tokens of 32 entries 501 -> 312 us, 16 x 60000 828 -> 486).
 //
 // What bounds it and why this split.  A key tile is 576 cycles of MMA per half (4 x N=128, 8 x N=80) and a chain
 // scores -> builders -> apply of about 1700, most of it hand-offs.  Four chains run side by side: two halves times two
@@ -150,10 +152,10 @@ struct AArgs {
   const unsigned short* z;       // [BH][n_chunks][state rows] bf16: Z before each chunk
 };
 
-// G = feature groups of the blockwise map: a key tile holds KT = 128 / G keys, and the 128 score columns of a buffer
+// R = runs of 8 features that a row may have.  G = feature groups of the blockwise map: a key tile holds KT = 128 / G keys, and the 128 score columns of a buffer
 // hold, for each half of those keys, the G per-group score blocks Q_a K_a^T side by side (group a in columns [a KT/2,
 // a KT/2 + KT/2) of the sub-buffer); the weight of a key is the sum over the groups of the squared scores.
-template <int G>
+template <int G, int R>
 __global__ void __launch_bounds__(NTHREADS, 1)
 tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                  const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmS, const AArgs args) {
@@ -169,7 +171,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
   constexpr int KT = KTILE / G;                   // keys per tile
   constexpr int KH = KT / 2;                      // keys of a sub-tile
   constexpr int KPL = KT / 32;                    // keys per lane of the scale warp
-  constexpr int NST = PairTable<G>::kSlices;      // state tiles
+  constexpr int NST = PairTable<G, R>::kSlices;      // state tiles
 
   // Work items.  Rank -> (block of its chunk, chunk, head): the last blocks of the chunks (the most key tiles) first,
   // among them the chunks in descending order, so that chunk 0, which reads no state, comes last.  The n-th item of a CTA:
@@ -311,7 +313,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         auto open = [&](uint32_t g_it, int c) {
           const uint32_t st = smem_u32(stage(g_it % NSTAGE));
 #pragma unroll
-          for (int ks = 0; ks < 4; ++ks)   // 16 features per step; group ks / (4 / G) accumulates over its own steps
+          for (int ks = 0; ks < R / 2; ++ks)   // 16 features per step; group ks / (4 / G) accumulates over its own steps
             mma_f16_ts(tS + c * 64 + (ks / (4 / G)) * KH, tQ + ks * 8, at(dk, st + c * KH * 128 + ks * 32), id_s, (ks % (4 / G)) > 0);
           mma_commit(bar(BAR_SFULL + 2 * h + c));
         };
@@ -472,7 +474,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       it += w.n_tiles;
       if (nk > 0 && w.ns > 0) {
         // ---- the features of this query row, 256 per tile, this warp's two pairs of runs ----
-        static constexpr PairTable<G> kPairs{};
+        static constexpr PairTable<G, R> kPairs{};
 #pragma unroll 1
         for (int t = 0; t < NST && ok; ++t, ++n_st) {
 #pragma unroll 1
@@ -650,7 +652,7 @@ void tc_attend(const Problem& p, const __nv_bfloat16* rscale, const AttendStates
     a.n_chunks = st.n_chunks;
     a.first_state = st.first_state;
     a.z = reinterpret_cast<const unsigned short*>(st.z);
-    maps = maps && make_tile_map(&tmS, st.s, BH * st.n_chunks, tc_state_rows(p.groups), 256);
+    maps = maps && make_tile_map(&tmS, st.s, BH * st.n_chunks, tc_state_rows(p), 256);
   } else {
     tmS = tmK;
   }
@@ -658,10 +660,12 @@ void tc_attend(const Problem& p, const __nv_bfloat16* rscale, const AttendStates
     ctx.status = KATA_ERR_CUDA;
     return;
   }
-  auto kern = p.groups == 1 ? tc_attend_kernel<1> : p.groups == 2 ? tc_attend_kernel<2> : tc_attend_kernel<4>;
-  if (!(p.groups == 1   ? allow_smem<tc_attend_kernel<1>>((int)SMEM_ALLOC)
-        : p.groups == 2 ? allow_smem<tc_attend_kernel<2>>((int)SMEM_ALLOC)
-                        : allow_smem<tc_attend_kernel<4>>((int)SMEM_ALLOC))) {
+  const bool narrow = tc_narrow(p);
+  auto kern = p.groups == 2 ? tc_attend_kernel<2, 8> : p.groups == 4 ? tc_attend_kernel<4, 8> : narrow ? tc_attend_kernel<1, 4> : tc_attend_kernel<1, 8>;
+  if (!(p.groups == 2   ? allow_smem<tc_attend_kernel<2, 8>>((int)SMEM_ALLOC)
+        : p.groups == 4 ? allow_smem<tc_attend_kernel<4, 8>>((int)SMEM_ALLOC)
+        : narrow        ? allow_smem<tc_attend_kernel<1, 4>>((int)SMEM_ALLOC)
+                        : allow_smem<tc_attend_kernel<1, 8>>((int)SMEM_ALLOC))) {
     ctx.status = KATA_ERR_CUDA;
     return;
   }

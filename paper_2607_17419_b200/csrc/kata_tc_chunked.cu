@@ -18,7 +18,7 @@ struct ChunkBuffers {
   size_t r, s, z, s_loc, z_loc, total;
 };
 ChunkBuffers chunk_buffers(const Problem& p, const StatePlan& plan, bool states) {
-  const size_t BH = (size_t)p.B * p.H, slots = BH * plan.n_chunks, rows = (size_t)tc_state_rows(p.groups);
+  const size_t BH = (size_t)p.B * p.H, slots = BH * plan.n_chunks, rows = (size_t)tc_state_rows(p);
   ChunkBuffers b{};
   b.r = 0;
   b.s = align256(BH * p.T * 2);
@@ -37,12 +37,14 @@ ChunkBuffers chunk_buffers(const Problem& p, const StatePlan& plan, bool states)
 //   full lift   T = 6000: 75 / 99, 587 / 645, 49 / 44     T = 8192: 119 / 130, 1148 / 900, 65 / 54
 //   two groups  T = 2000: 31 / 38, 147 / 152, 30 / 37     T = 4096: 53 / 60, 450 / 315, 51 / 39
 //   four groups T = 2000: 45 / 42, 193 / 161, 43 / 41
+//   rows of 32 entries (a third of the state)  T = 3000: 32 / 48, 151 / 155     T = 4096: 42 / 46, 237 / 208, 36 / 32     T = 6000: 77 / 67, 470 / 312
+//   (a wave of blocks that is not full costs the chunks more: their line lies higher with few heads)
 // Chunks of 1024: 16 heads x 131072 tokens 2.26 ms; 512: 2.30, 2048: 2.44 (shorter chunks write and read more state, longer
 // ones have more key tiles).  Halved where even one chunk per CTA leaves SMs idle (3 heads x 2048 tokens with the state
 // handed out: 43 -> 38 us).
 StatePlan tc_chunk_plan(const Problem& p, bool state_in, bool state_out) {
-  const int BH = p.B * p.H, slices = tc_state_rows(p.groups) / 256;
-  const int quad_tokens = p.groups == 1 ? 7168 : p.groups == 2 ? 3072 : 1536;
+  const int BH = p.B * p.H, slices = tc_state_rows(p) / 256;
+  const int quad_tokens = tc_narrow(p) ? (BH < 64 ? 4352 : 3584) : p.groups == 1 ? 7168 : p.groups == 2 ? 3072 : 1536;
   StatePlan plan{};
   int L = 1024;
   if (!state_in && !state_out && p.T <= quad_tokens) L = (p.T + 255) / 256 * 256;

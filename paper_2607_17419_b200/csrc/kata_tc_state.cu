@@ -128,7 +128,7 @@ __device__ __forceinline__ void sts128(uint32_t addr, const uint32_t (&r)[4]) {
   asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
 }
 
-template <int G>
+template <int G, int R>
 __global__ void __launch_bounds__(NTHREADS, 1)
 tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, const SArgs args) {
   extern __shared__ unsigned char smem_raw[];
@@ -138,8 +138,8 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
   __shared__ uint32_t tmem_base_s;
   __shared__ int abort_s;
   volatile int* abort_flag = &abort_s;
-  static constexpr PairTable<G> kPairs{};
-  constexpr int ROWS = PairTable<G>::kRows;
+  static constexpr PairTable<G, R> kPairs{};
+  constexpr int ROWS = PairTable<G, R>::kRows;
 
   cudaTriggerProgrammaticLaunchCompletion();      // the kernel behind starts on the SMs that this one leaves
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -450,12 +450,12 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
 // (the first one's starts from the state handed in); after the last chunk, the state handed out.
 // One thread per (head, state row, four value columns) walks the chunks; eight loads in flight.  Memory-bound: 256 bytes
 // read and 128 written per chunk and state row.
-template <int G>
+template <int G, int R>
 __global__ void __launch_bounds__(256) state_fix_kernel(const float* __restrict__ s_loc, const float* __restrict__ z_loc,
                                                         __nv_bfloat16* __restrict__ s, __nv_bfloat16* __restrict__ z, int n_chunks,
                                                         int seg_chunks, float* __restrict__ s_final, float* __restrict__ z_final, int packed) {
-  constexpr int ROWS = PairTable<G>::kRows;
-  static constexpr PairTable<G> kPairs{};
+  constexpr int ROWS = PairTable<G, R>::kRows;
+  static constexpr PairTable<G, R> kPairs{};
   cudaTriggerProgrammaticLaunchCompletion();
   cudaGridDependencySynchronize();
   const int bh = blockIdx.y, idx = blockIdx.x * 256 + threadIdx.x, row = idx >> 4, c4 = idx & 15;   // ROWS is a multiple of 16
@@ -510,7 +510,9 @@ __global__ void __launch_bounds__(256) state_fix_kernel(const float* __restrict_
 
 }  // namespace
 
-int tc_state_rows(int groups) { return groups == 1 ? PairTable<1>::kRows : groups == 2 ? PairTable<2>::kRows : PairTable<4>::kRows; }
+int tc_state_rows(const Problem& p) {
+  return p.groups == 2 ? PairTable<2>::kRows : p.groups == 4 ? PairTable<4>::kRows : tc_narrow(p) ? PairTable<1, 4>::kRows : PairTable<1>::kRows;
+}
 
 void tc_states(const Problem& p, const __nv_bfloat16* rscale, const StatePlan& plan, const StateBuffers& buf, int* device_status,
                LaunchCtx& ctx) {
@@ -520,10 +522,12 @@ void tc_states(const Problem& p, const __nv_bfloat16* rscale, const StatePlan& p
     ctx.status = KATA_ERR_CUDA;
     return;
   }
-  auto kern = p.groups == 1 ? tc_state_kernel<1> : p.groups == 2 ? tc_state_kernel<2> : tc_state_kernel<4>;
-  if (!(p.groups == 1   ? allow_smem<tc_state_kernel<1>>((int)SMEM_ALLOC)
-        : p.groups == 2 ? allow_smem<tc_state_kernel<2>>((int)SMEM_ALLOC)
-                        : allow_smem<tc_state_kernel<4>>((int)SMEM_ALLOC))) {
+  const bool narrow = tc_narrow(p);
+  auto kern = p.groups == 2 ? tc_state_kernel<2, 8> : p.groups == 4 ? tc_state_kernel<4, 8> : narrow ? tc_state_kernel<1, 4> : tc_state_kernel<1, 8>;
+  if (!(p.groups == 2   ? allow_smem<tc_state_kernel<2, 8>>((int)SMEM_ALLOC)
+        : p.groups == 4 ? allow_smem<tc_state_kernel<4, 8>>((int)SMEM_ALLOC)
+        : narrow        ? allow_smem<tc_state_kernel<1, 4>>((int)SMEM_ALLOC)
+                        : allow_smem<tc_state_kernel<1, 8>>((int)SMEM_ALLOC))) {
     ctx.status = KATA_ERR_CUDA;
     return;
   }
@@ -545,7 +549,7 @@ void tc_states(const Problem& p, const __nv_bfloat16* rscale, const StatePlan& p
   a.n_chunks = plan.n_chunks;
   a.walk_chunks = buf.s_final != nullptr ? plan.n_chunks : plan.n_chunks - 1;
   a.seg_chunks = plan.seg_chunks;
-  const int slices = tc_state_rows(p.groups) / 256;
+  const int slices = tc_state_rows(p) / 256;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(slices, BH, plan.segments);
   cfg.blockDim = dim3(NTHREADS);
@@ -563,8 +567,8 @@ void tc_states(const Problem& p, const __nv_bfloat16* rscale, const StatePlan& p
   }
   ++ctx.launches;
   if (!segmented) return;
-  auto fix = p.groups == 1 ? state_fix_kernel<1> : p.groups == 2 ? state_fix_kernel<2> : state_fix_kernel<4>;
-  cfg.gridDim = dim3(tc_state_rows(p.groups) / 16, BH);
+  auto fix = p.groups == 2 ? state_fix_kernel<2, 8> : p.groups == 4 ? state_fix_kernel<4, 8> : narrow ? state_fix_kernel<1, 4> : state_fix_kernel<1, 8>;
+  cfg.gridDim = dim3(tc_state_rows(p) / 16, BH);
   cfg.blockDim = dim3(256);
   cfg.dynamicSmemBytes = 0;
   if (cudaLaunchKernelEx(&cfg, fix, (const float*)buf.s_loc, (const float*)buf.z_loc, buf.s, buf.z, plan.n_chunks, plan.seg_chunks,

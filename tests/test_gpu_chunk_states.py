@@ -40,6 +40,21 @@ def test_chunked_without_state(g, H, T, d):
     check(np.stack([gpu[b, h, t] for b, h, t in picks]), oracle_rows(w, picks, feature_of(g)), "bf16", f"M{g} T={T} H={H} d={d}")
 
 
+# rows of up to 32 entries: four of the eight runs of features, two block pairs of the last slice empty
+@pytest.mark.parametrize("H,T,dk,dv", [(1, 4353, 32, 32), (64, 3601, 32, 32), (2, 5121, 16, 64), (3, 4608, 32, 64), (2, 4400, 16, 16)])
+def test_narrow_rows(H, T, dk, dv):
+    import torch
+    w = inputs.gaussian_workload(f"narrow_{H}_{T}_{dk}_{dv}", "bf16", 1, H, T, dk, dv, 64, 5200 + T)
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    o = kb.kata_fwd_chunked(*dev_tensors(w), device_status=st)
+    torch.cuda.synchronize()
+    assert kb.kata_last_impl() == kb.KATA_IMPL_TENSOR and int(st.item()) == 0
+    assert kb.kata_last_launch_count() in (3, 4)
+    picks = sample_picks(w, 64, T) + [(0, H - 1, t) for c in (512, 1024, 2048, 3072, 3584) for t in (c - 1, c, c + 127, c + 128) if t < T]
+    gpu = to_numpy64(o)
+    check(np.stack([gpu[b, h, t] for b, h, t in picks]), oracle_rows(w, picks, "psd_direct"), "bf16", f"narrow {dk}x{dv} T={T} H={H}")
+
+
 @pytest.mark.parametrize("layout", ["psd_direct", "psd_packed"])
 @pytest.mark.parametrize("g,H,cuts", [(1, 2, (513, 1537)), (1, 20, (100, 612)), (2, 3, (1024, 1025)), (4, 2, (700, 2300))])
 def test_state_in_and_out(layout, g, H, cuts):
