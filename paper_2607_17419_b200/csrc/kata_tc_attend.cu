@@ -149,6 +149,7 @@ struct AArgs {
   int chunk_pairs;               // ... of a chunk (the quadratic form: n_pairs)
   int n_chunks;
   int first_state;               // first chunk that has a state before it
+  int by_chunk;                  // order of the items: the blocks of a chunk one after the other
   const unsigned short* z;       // [BH][n_chunks][state rows] bf16: Z before each chunk
 };
 
@@ -177,6 +178,11 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
   // among them the chunks in descending order, so that chunk 0, which reads no state, comes last.  The n-th item of a CTA:
   // rounds of gridDim.x items, dealt forwards and backwards in turn, so that the CTA that got the heaviest item of one
   // round gets the lightest of the next.
+  // With two dozen items per CTA and more (by_chunk) the blocks of a chunk follow one another instead, so that its state is
+  // read from memory once and by the other blocks from L2; the deal keeps a CTA's share even (block p in one round, the
+  // mirrored one in the next).  With fewer items the last round weighs more.  Heaviest first / by chunk, us: 16 heads x 131072
+  // tokens 2305 / 2182, 32 x 32768 1114 / 1073, 128 x 8192 1007 / 982; 16 x 32768 (14 items per CTA) 545 / 558, 128 x 4096 with
+  // two groups 348 / 352.
   struct Item {
     int bh, chunk, q0;            // head, chunk, first query
     int k0;                       // first key tile (in tiles of KT keys)
@@ -191,8 +197,14 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       const long long id = (long long)n * gridDim.x + ((n & 1) ? (int)gridDim.x - 1 - (int)blockIdx.x : (int)blockIdx.x);
       if ((long long)n * gridDim.x >= n_ranks) return false;
       if (id >= n_ranks) continue;
-      const int p = args.chunk_pairs - 1 - (int)id / per_block;
-      const int rem = (int)id % per_block;
+      int p, rem;
+      if (args.by_chunk) {
+        rem = (int)id / args.chunk_pairs;
+        p = args.chunk_pairs - 1 - (int)id % args.chunk_pairs;
+      } else {
+        p = args.chunk_pairs - 1 - (int)id / per_block;
+        rem = (int)id % per_block;
+      }
       it.chunk = args.n_chunks - 1 - rem / args.BH;
       it.bh = rem % args.BH;
       const int pair = it.chunk * args.chunk_pairs + p;
@@ -644,13 +656,14 @@ void tc_attend(const Problem& p, const __nv_bfloat16* rscale, const AttendStates
   CUtensorMap tmQ, tmK, tmV, tmS;
   const int kt = KTILE / p.groups;
   const int n_pairs = (p.T + 2 * QT - 1) / (2 * QT);
-  AArgs a{static_cast<__nv_bfloat16*>(p.out), rscale, device_status, p.T, p.d_v, BH, n_pairs, n_pairs, 1, 1, nullptr};
+  AArgs a{static_cast<__nv_bfloat16*>(p.out), rscale, device_status, p.T, p.d_v, BH, n_pairs, n_pairs, 1, 1, 0, nullptr};
   bool maps = make_tile_map(&tmQ, p.q, BH, p.T, QT, p.d_k) && make_tile_map(&tmK, p.k, BH, p.T, kt, p.d_k) &&
               make_tile_map(&tmV, p.v, BH, p.T, kt, p.d_v);
   if (st.n_chunks > 0) {
     a.chunk_pairs = st.chunk_tokens / (2 * QT);
     a.n_chunks = st.n_chunks;
     a.first_state = st.first_state;
+    a.by_chunk = (long long)BH * st.n_chunks * a.chunk_pairs >= 24LL * sm_count() ? 1 : 0;
     a.z = reinterpret_cast<const unsigned short*>(st.z);
     maps = maps && make_tile_map(&tmS, st.s, BH * st.n_chunks, tc_state_rows(p), 256);
   } else {
