@@ -47,11 +47,11 @@ def quadratic_flops(B, H, T, d=64, dv=64):
 
 
 def load_traffic(T: int):
-    """DRAM bytes per launch of the dominant kernel, scaled linearly in T from the ncu capture recorded beside its
+    """DRAM bytes per step of the two large kernels, scaled linearly in T from the ncu capture recorded beside its
     summary under profiles/ (null if the record is missing)."""
-    path = os.path.join(ROOT, "profiles", "tc_split_kernel_c4_T32768_traffic.json")
+    path = os.path.join(ROOT, "profiles", "tc_chunk_kernels_c4_T32768_traffic.json")
     if not os.path.exists(path):
-        return None, "kata::tc_split_kernel (tcgen05 feature-split chunked forward)"
+        return None, "kata::tc_state_kernel + kata::tc_attend_kernel (tcgen05 chunk states and outputs)"
     with open(path) as f:
         rec = json.load(f)
     scale = T / rec["T"]
@@ -266,8 +266,8 @@ def run_ours(args):
     f1.record(stream)
     barrier()
     e2e_ms_total = f0.elapsed_time(f1)
-    # the host route works in pieces that hand the state over and runs them on the streaming kernel, the device call
-    # on the feature-split kernel: the same function, rounded at different places
+    # the host route works in pieces that hand the state over, whose chunks begin elsewhere than those of the one call:
+    # the same function, rounded at different places
     diff = (ho.to(dev).float() - out.float()).abs().amax(dim=-1)
     assert bool((diff <= 3e-2 * out.float().abs().amax(dim=-1).clamp_min(1e-3)).all()), "host route and device call disagree"
 
@@ -585,8 +585,9 @@ def measure_extra(kb, inputs, dev, stream, q, k, v, out, peaks):
         dqb, dkb, dvb = torch.empty_like(qb), torch.empty_like(kb_), torch.empty_like(vb)
         ms_c = timed(lambda: kb.kata_bwd_chunked(qb, kb_, vb, gb, dqb, dkb, dvb), reps=3, warm=1)
         lc = kb.kata_last_launch_count()
+        impl_c = "tensor" if kb.kata_last_impl() == kb.KATA_IMPL_TENSOR else "simt"
         ms_q = timed(lambda: kb.kata_bwd_quadratic(qb, kb_, vb, gb, dqb, dkb, dvb), reps=3, warm=1)
-        res[f"bwd_chunked_H16_T{Tb}"] = dict(ms=ms_c, tokens_per_s=Tb / (ms_c * 1e-3), launches=lc, impl="simt",
+        res[f"bwd_chunked_H16_T{Tb}"] = dict(ms=ms_c, tokens_per_s=Tb / (ms_c * 1e-3), launches=lc, impl=impl_c,
                                              bwd_quadratic_ms=ms_q, speedup_over_quadratic=ms_q / ms_c)
         if cross is None and ms_c < ms_q:
             cross = Tb
