@@ -39,7 +39,7 @@ ChunkBuffers chunk_buffers(const Problem& p, const StatePlan& plan, bool states)
 //   four groups T = 2000: 45 / 42, 193 / 161, 43 / 41
 //   rows of 32 entries (a third of the state)  T = 3000: 32 / 48, 151 / 155     T = 4096: 42 / 46, 237 / 208, 36 / 32     T = 6000: 77 / 67, 470 / 312
 //   (a wave of blocks that is not full costs the chunks more: their line lies higher with few heads)
-// Chunks of 1024: 16 heads x 131072 tokens 2.26 ms; 512: 2.30, 2048: 2.44 (shorter chunks write and read more state, longer
+// Chunks of 1024: 16 heads x 131072 tokens 2.08 ms; 768: 2.10, 512: 2.17, 2048 about 2.3 (shorter chunks write and read more state, longer
 // ones have more key tiles).  Halved where even one chunk per CTA leaves SMs idle (3 heads x 2048 tokens with the state
 // handed out: 43 -> 38 us).
 StatePlan tc_chunk_plan(const Problem& p, bool state_in, bool state_out) {
