@@ -79,17 +79,27 @@ class ClockSampler:
         self.rows = []
         self.proc = None
         self.thread = None
+        self.skip = 0          # samples from before the timed region
 
     def start(self):
         try:
             self.proc = subprocess.Popen(
                 ["nvidia-smi", f"--id={self.gpu}", f"--query-gpu={self.FIELDS}", "--format=csv,noheader,nounits",
-                 "-lms", "100"], stdout=subprocess.PIPE, stderr=subprocess.DEVNULL, text=True)
+                 "-lms", "20"], stdout=subprocess.PIPE, stderr=subprocess.DEVNULL, text=True)
         except OSError:
             self.proc = None
             return
         self.thread = threading.Thread(target=self._read, daemon=True)
         self.thread.start()
+
+    def wait_first(self, limit_s=3.0):
+        """nvidia-smi takes longer to start than a short timed region lasts: wait for its first line, and drop it."""
+        t0 = time.time()
+        while self.proc is not None and not self.rows and time.time() - t0 < limit_s:
+            time.sleep(0.01)
+
+    def mark(self):
+        self.skip = len(self.rows)
 
     def _read(self):
         for line in self.proc.stdout:
@@ -106,7 +116,7 @@ class ClockSampler:
             self.proc.kill()
         sm, smax, reasons = [], [], set()
         names = ["hw_slowdown", "hw_thermal_slowdown", "sw_thermal_slowdown", "sw_power_cap"]
-        for r in self.rows:
+        for r in self.rows[self.skip:]:
             if len(r) < 8:
                 continue
             try:
@@ -233,8 +243,13 @@ def run_ours(args):
     sampler = ClockSampler(local_rank)
     if rank == 0:
         sampler.start()
+        sampler.wait_first()
+    barrier()
+    for _ in range(3):                   # the wait let the GPU go idle
+        step()
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     barrier()
+    sampler.mark()
     e0.record(stream)
     for _ in range(args.steps):
         step()
@@ -250,6 +265,11 @@ def run_ours(args):
         b.record(stream)
     barrier()
     single = sorted(a.elapsed_time(b) for a, b in pairs)
+    if rank == 0:                        # a short run may end between two samples: the same step until there is one
+        t0 = time.time()
+        while sampler.proc is not None and len(sampler.rows) <= sampler.skip and time.time() - t0 < 1.0:
+            step()
+            torch.cuda.synchronize()
     clocks = sampler.stop() if rank == 0 else None
 
     # ---- end to end: pinned host buffers through kata_fwd_host, copies inside the timed region ----
