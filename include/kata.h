@@ -24,7 +24,8 @@
  *     accumulated in fp32, but psi(q)^T S and psi(q)^T Z see them, and psi(q), rounded; psi(k) is a product of bf16 entries
  *     and of the key scale, rounded twice), the weights (q.k)^2 inside a chunk and in the quadratic form are rounded to bf16
  *     before they multiply the values, and the key scale 1/||k||^2 is rounded to bf16 and multiplied into the weights,
- *     rounded again, whose row sum is then the normaliser.  The convex weights of the output gate therefore sum to 1 only to
+ *     rounded again, whose row sum is then the normaliser (kata_fwd_chunked with a state handed over or with feature groups
+ *     multiplies by the fp32 scale before it rounds, once).  The convex weights of the output gate therefore sum to 1 only to
  *     about 2^-8, and a normaliser that is tiny against its terms (a query nearly orthogonal to every key before it)
  *     can come out <= 0 from the rounded operands, in which case out = 0 as for an exact zero.  All of it stays
  *     inside the 2e-2 tolerance of the bf16 tests.

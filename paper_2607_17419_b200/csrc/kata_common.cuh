@@ -150,8 +150,13 @@ void decode_step(const void* q, const void* k, const void* v, void* out, float* 
 bool tc_supported(const Problem& p, int fn);
 size_t tc_quadratic_workspace_bytes(const Problem& p);
 void tc_quadratic(const Problem& p, void* workspace, int* device_status, LaunchCtx& ctx);
-// r = 1 / ||k||^2 [BH][T] (bf16), which the kernels below take
-void tc_rscale(const Problem& p, __nv_bfloat16* rscale, LaunchCtx& ctx);
+// r = 1 / ||k||^2 [BH][T], which the kernels below take: fp32 (chunk states, exact_scales) or bf16 (the quadratic form, whose
+// scratch is two bytes per key)
+struct KeyScales {
+  float* f32;
+  __nv_bfloat16* bf16;         // when f32 is null
+};
+void tc_rscale(const Problem& p, const KeyScales& r, LaunchCtx& ctx);
 // States before the chunks (kata_tc_state.cu), for tc_attend.
 struct StatePlan {
   int chunk_tokens;            // a multiple of 256
@@ -172,7 +177,7 @@ struct StateBuffers {
 int tc_state_rows(const Problem& p);
 // Rows of up to 32 entries (full map): the tensor-core kernels skip the empty half of the features.
 inline bool tc_narrow(const Problem& p) { return p.groups == 1 && p.d_k <= 32; }
-void tc_states(const Problem& p, const __nv_bfloat16* rscale, const StatePlan& plan, const StateBuffers& buf, int* device_status,
+void tc_states(const Problem& p, const float* rscale, const StatePlan& plan, const StateBuffers& buf, int* device_status,
                LaunchCtx& ctx);
 // Outputs of blocks of 256 queries: over the keys of their chunk and the state before it (zero-initialise for the
 // quadratic form: one chunk, no state).
@@ -181,8 +186,9 @@ struct AttendStates {
   const __nv_bfloat16* z;      // [BH][n_chunks][rows]: its normaliser, likewise
   int n_chunks, chunk_tokens;  // chunk_tokens: a multiple of 256
   int first_state;             // first chunk that has a state before it (0 or 1)
+  bool exact_scales;           // weights times the fp32 key scales, rounded once
 };
-void tc_attend(const Problem& p, const __nv_bfloat16* rscale, const AttendStates& st, int* device_status, LaunchCtx& ctx);
+void tc_attend(const Problem& p, const KeyScales& r, const AttendStates& st, int* device_status, LaunchCtx& ctx);
 void tc_chunked_stream(const Problem& p, int* device_status, LaunchCtx& ctx);
 // Chunked form on the chunk-state and attend kernels (kata_tc_chunked.cu).  n_chunks = 1 without state pointers: the
 // quadratic form alone.

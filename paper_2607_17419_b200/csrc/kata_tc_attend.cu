@@ -14,7 +14,8 @@
 //   key tiles of 128 keys, from the start of the chunk (quadratic form: of the sequence) up to the diagonal:
 //     scores   S = Q K_j^T            A = the query tile in TMEM, B = the key tile (TMA, 128B swizzle)
 //     weights  P = r S^2 (causal mask on the diagonal tiles)  packed fp32x2 multiplies on the TMEM read-back, rounded
-//                                     to bf16, times r, stored back over the scores
+//                                     to bf16, times r, stored back over the scores; with exact key scales (XR) times
+//                                     r in fp32 and rounded once
 //     apply    [O | D] += P [V | 1]   A = P from TMEM, B = the value tile and a constant column of ones (MN-major,
 //                                     N = 80): the normaliser is column 64 of the same accumulator
 //   epilogue out = O / D  (0 where that is 0)      the gate/normalise step of the readout
@@ -67,8 +68,8 @@ constexpr uint32_t STAGE_BYTES = 32768;             // K tile 16 KB, V tile 16 K
 constexpr uint32_t OFF_ST = 32768;
 constexpr uint32_t OFF_ONES = OFF_ST + NSTAGE * STAGE_BYTES;   // 16 rows of [1, 0 ...]: columns 64.. of the values
 constexpr uint32_t OFF_Z = OFF_ONES + 2048;                    // columns 64.. of a state: 256 rows of 128 bytes, stage s in bytes [32 s, 32 s + 32)
-constexpr uint32_t OFF_RV = OFF_Z + 32768;                     // NSTAGE x 128 bf16: 1 / ||k||^2 of the keys of a tile
-constexpr uint32_t OFF_BAR = OFF_RV + NSTAGE * 256;
+constexpr uint32_t OFF_RV = OFF_Z + 32768;                     // NSTAGE x 128 bf16 or fp32: 1 / ||k||^2 of the keys of a tile
+constexpr uint32_t OFF_BAR = OFF_RV + NSTAGE * 512;
 constexpr uint32_t SMEM_BYTES = OFF_BAR + 512;
 constexpr uint32_t SMEM_ALLOC = SMEM_BYTES + 1024;
 static_assert(SMEM_ALLOC > 116 * 1024, "one CTA per SM is assumed (the CTA allocates all of TMEM)");
@@ -94,8 +95,8 @@ enum {
 // Pre-pass: r = 1 / ||k||^2 per key row (0 for a zero row); eight lanes of 16 bytes per row, four rows per lane in flight
 // (memory-bound; 33.5 MB of keys: 8.7 us with one row per lane, 6.9 with four).
 constexpr int RS_ROWS = 4;
-__global__ void __launch_bounds__(256) rscale_kernel(const __nv_bfloat16* __restrict__ k, __nv_bfloat16* __restrict__ rscale,
-                                                     size_t n_rows, int d) {
+__global__ void __launch_bounds__(256) rscale_kernel(const __nv_bfloat16* __restrict__ k, float* __restrict__ r_f32,
+                                                     __nv_bfloat16* __restrict__ r_bf16, size_t n_rows, int d) {
   cudaTriggerProgrammaticLaunchCompletion();   // the kernel behind sets itself up meanwhile
   const size_t row0 = (size_t)blockIdx.x * (32 * RS_ROWS) + (threadIdx.x >> 3);
   const int part = threadIdx.x & 7;
@@ -119,7 +120,10 @@ __global__ void __launch_bounds__(256) rscale_kernel(const __nv_bfloat16* __rest
     ss += __shfl_xor_sync(0xffffffffu, ss, 1);
     ss += __shfl_xor_sync(0xffffffffu, ss, 2);
     ss += __shfl_xor_sync(0xffffffffu, ss, 4);
-    if (part == 0 && row0 + i * 32 < n_rows) rscale[row0 + i * 32] = __float2bfloat16_rn(inv_or_zero(ss));
+    if (part == 0 && row0 + i * 32 < n_rows) {
+      const float r = inv_or_zero(ss);
+      if (r_f32 != nullptr) r_f32[row0 + i * 32] = r; else r_bf16[row0 + i * 32] = __float2bfloat16_rn(r);
+    }
   }
 }
 
@@ -140,7 +144,8 @@ template <int N> __device__ __forceinline__ void regs_take() { asm volatile("set
 
 struct AArgs {
   __nv_bfloat16* out;
-  const __nv_bfloat16* rscale;   // [BH][T] bf16: 1 / ||k||^2 (pre-pass)
+  const float* r_f32;            // [BH][T]: 1 / ||k||^2 (pre-pass)
+  const __nv_bfloat16* r_bf16;   // ... where r_f32 is null
   int* device_status;
   int Tlen;
   int d_v;
@@ -153,10 +158,15 @@ struct AArgs {
   const unsigned short* z;       // [BH][n_chunks][state rows] bf16: Z before each chunk
 };
 
+// XR = exact key scales: the weights are r s^2 rounded to bf16 once, instead of s^2, r and their product.  Taken by the chunked
+// form with a state handed in or out and with feature groups, whose outputs were 3 to 8 % further from the 64-bit result (2-norm)
+// than on the kernels that answer the short calls of the same kinds (2.9e-3 there; 2.2e-3 to 2.4e-3 with exact scales).  One packed multiply
+// and twice the reads of r per pair: 4 x 16 heads x 4096 tokens of the quadratic form 126 -> 136 us, where nothing calls for
+// it; 2 x 16 x 3001 with the state 109 -> 111.
 // R = runs of 8 features that a row may have.  G = feature groups of the blockwise map: a key tile holds KT = 128 / G keys, and the 128 score columns of a buffer
 // hold, for each half of those keys, the G per-group score blocks Q_a K_a^T side by side (group a in columns [a KT/2,
 // a KT/2 + KT/2) of the sub-buffer); the weight of a key is the sum over the groups of the squared scores.
-template <int G, int R>
+template <int G, int R, bool XR>
 __global__ void __launch_bounds__(NTHREADS, 1)
 tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                  const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmS, const AArgs args) {
@@ -401,9 +411,9 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     uint32_t it = 0;
     Item w;
     for (int n = 0; ok && next_item(n, w); ++n) {
-      const unsigned short* rs = reinterpret_cast<const unsigned short*>(args.rscale) + (size_t)w.bh * args.Tlen;
+      const size_t head = (size_t)w.bh * args.Tlen;
       const unsigned short* zs = args.z + ((size_t)w.bh * args.n_chunks + w.chunk) * (NST * 256);
-      auto load = [&](int j, unsigned short (&x)[8]) {            // tile j: r of KPL keys, or Z of 8 rows, per lane
+      auto load = [&](int j, uint32_t (&x)[8]) {                  // tile j: r of KPL keys (fp32 or bf16), or Z of 8 rows (bf16), per lane
         if (j < w.ns) {
 #pragma unroll
           for (int e = 0; e < 8; ++e) x[e] = zs[j * 256 + e * 32 + lane];
@@ -411,15 +421,18 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
 #pragma unroll
           for (int e = 0; e < KPL; ++e) {
             const int key = (w.k0 + j - w.ns) * KT + lane * KPL + e;
-            x[e] = (j < w.n_tiles && key < args.Tlen) ? rs[key] : (unsigned short)0;
+            const bool in = j < w.n_tiles && key < args.Tlen;
+            if (XR) x[e] = in ? __float_as_uint(args.r_f32[head + key]) : 0u;
+            else if (args.r_f32 != nullptr) x[e] = in ? pack_bf16(args.r_f32[head + key], 0.f) : 0u;
+            else x[e] = in ? reinterpret_cast<const unsigned short*>(args.r_bf16)[head + key] : 0u;
           }
         }
       };
-      unsigned short x[8] = {};
+      uint32_t x[8] = {};
       load(0, x);
       for (int j = 0; j < w.n_tiles && ok; ++j, ++it) {
         const int s = it % NSTAGE;
-        unsigned short nx[8] = {};
+        uint32_t nx[8] = {};
         load(j + 1, nx);                // one tile ahead: the global-load latency stays off the ring
         ok = wait_or_abort(bar(BAR_EMPTY + s), ((it / NSTAGE) & 1) ^ 1, abort_flag);
         if (!ok) break;
@@ -427,12 +440,15 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
 #pragma unroll
           for (int e = 0; e < 8; ++e) {
             const int row = e * 32 + lane;
-            *reinterpret_cast<unsigned short*>(base + OFF_Z + (row >> 4) * 2048 + sw128_offset(row & 15, 2 * s)) = x[e];
+            *reinterpret_cast<unsigned short*>(base + OFF_Z + (row >> 4) * 2048 + sw128_offset(row & 15, 2 * s)) = (unsigned short)x[e];
           }
           fence_async_smem();
         } else {
 #pragma unroll
-          for (int e = 0; e < KPL; ++e) reinterpret_cast<unsigned short*>(base + OFF_RV + s * 256)[lane * KPL + e] = x[e];
+          for (int e = 0; e < KPL; ++e) {
+            if (XR) reinterpret_cast<uint32_t*>(base + OFF_RV + s * 512)[lane * KPL + e] = x[e];
+            else reinterpret_cast<unsigned short*>(base + OFF_RV + s * 512)[lane * KPL + e] = (unsigned short)x[e];
+          }
         }
 #pragma unroll
         for (int e = 0; e < 8; ++e) x[e] = nx[e];
@@ -525,7 +541,8 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
           // this warp weighs keys [ch KT/2, ch KT/2 + KT/2) of the tile: one column run per group
           const int key0 = (w.k0 + j) * KT + ch * KH;
           uint32_t y[G][KH], pk[KH / 2];
-          const uint32_t* rw = reinterpret_cast<const uint32_t*>(base + OFF_RV + s * 256) + ch * (KH / 2);   // r of this warp's keys, in pairs
+          const uint32_t rbase = smem_u32(base + OFF_RV) + s * 512 + ch * (KH * 4);   // fp32 r of this warp's keys, 4 per load
+          const uint32_t* rw = reinterpret_cast<const uint32_t*>(base + OFF_RV + s * 512) + ch * (KH / 2);   // bf16 r, in pairs
 #pragma unroll
           for (int g = 0; g < G; ++g) {
             if constexpr (KH == 32) tmem_ld32(tS + g * KH, y[g]); else tmem_ld16(tS + g * KH, y[g]);
@@ -535,42 +552,51 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
           // two copies of the loop, chosen once per tile: the causal test exists on the diagonal tiles only
           auto weigh_g = [&](auto masked) {
 #pragma unroll
-            for (int c = 0; c < KH; c += 2) {
-              float2 x = make_float2(0.f, 0.f);
+            for (int c0 = 0; c0 < KH; c0 += 4) {
+              uint4 t4 = make_uint4(0u, 0u, 0u, 0u);
+              if (XR) t4 = lds128(rbase + c0 * 4);
+              const float rr[4] = {__uint_as_float(t4.x), __uint_as_float(t4.y), __uint_as_float(t4.z), __uint_as_float(t4.w)};
 #pragma unroll
-              for (int g = 0; g < G; ++g) {
-                const float2 sv = make_float2(__uint_as_float(y[g][c]), __uint_as_float(y[g][c + 1]));
-                x = __ffma2_rn(sv, sv, x);
+              for (int c = c0; c < c0 + 4; c += 2) {
+                float2 x = make_float2(0.f, 0.f);
+#pragma unroll
+                for (int g = 0; g < G; ++g) {
+                  const float2 sv = make_float2(__uint_as_float(y[g][c]), __uint_as_float(y[g][c + 1]));
+                  x = __ffma2_rn(sv, sv, x);
+                }
+                if (XR) x = __fmul2_rn(x, make_float2(rr[c - c0], rr[c - c0 + 1]));
+                if constexpr (decltype(masked)::value) {
+                  if (key0 + c > qrow) x.x = 0.f;
+                  if (key0 + c + 1 > qrow) x.y = 0.f;
+                }
+                pk[c / 2] = XR ? pack_bf16(x.x, x.y) : mul_bf16x2(pack_bf16(x.x, x.y), rw[c / 2]);
               }
-              if constexpr (decltype(masked)::value) {
-                if (key0 + c > qrow) x.x = 0.f;
-                if (key0 + c + 1 > qrow) x.y = 0.f;
-              }
-              pk[c / 2] = mul_bf16x2(pack_bf16(x.x, x.y), rw[c / 2]);
             }
           };
           if (diag) weigh_g(std::true_type{}); else weigh_g(std::false_type{});
           // the weights overwrite this warp's own score columns of group 0
           if constexpr (KH == 32) tmem_st16(tS, pk); else tmem_st8(tS, pk);
         } else {
-          const uint32_t rbase = smem_u32(base + OFF_RV) + s * 256 + ch * 128;   // r of this warp's 64 keys, 8 per load
+          const uint32_t rbase = smem_u32(base + OFF_RV) + s * 512 + ch * (XR ? 256 : 128);   // r of this warp's 64 keys, 16 bytes per load
           const int key0 = (w.k0 + j) * KT + ch * 64;
           uint32_t ya[32], yb[32], pk[16];
           auto weigh = [&](const uint32_t (&y)[32], int col0, auto masked) {
+            constexpr int RPL = XR ? 4 : 8;                    // keys per load
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const uint4 t4 = lds128(rbase + (col0 / 8 + i) * 16);
+            for (int i = 0; i < 32 / RPL; ++i) {
+              const uint4 t4 = lds128(rbase + (col0 / RPL + i) * 16);
               const uint32_t rr[4] = {t4.x, t4.y, t4.z, t4.w};
 #pragma unroll
-              for (int e = 0; e < 8; e += 2) {
-                const int jj = 8 * i + e;
+              for (int e = 0; e < RPL; e += 2) {
+                const int jj = RPL * i + e;
                 const float2 sv = make_float2(__uint_as_float(y[jj]), __uint_as_float(y[jj + 1]));
                 float2 x = __fmul2_rn(sv, sv);
+                if constexpr (XR) x = __fmul2_rn(x, make_float2(__uint_as_float(rr[e]), __uint_as_float(rr[e + 1])));
                 if constexpr (decltype(masked)::value) {
                   if (key0 + col0 + jj > qrow) x.x = 0.f;
                   if (key0 + col0 + jj + 1 > qrow) x.y = 0.f;
                 }
-                pk[jj / 2] = mul_bf16x2(pack_bf16(x.x, x.y), rr[e / 2]);
+                pk[jj / 2] = XR ? pack_bf16(x.x, x.y) : mul_bf16x2(pack_bf16(x.x, x.y), rr[e / 2]);
               }
             }
           };
@@ -645,18 +671,19 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
 // workspace: r [BH][T] bf16
 size_t tc_quadratic_workspace_bytes(const Problem& p) { return ((size_t)p.B * p.H * p.T * 2 + 255) / 256 * 256; }
 
-void tc_rscale(const Problem& p, __nv_bfloat16* rscale, LaunchCtx& ctx) {
+void tc_rscale(const Problem& p, const KeyScales& r, LaunchCtx& ctx) {
   const size_t n_rows = (size_t)p.B * p.H * p.T;
-  rscale_kernel<<<(unsigned)((n_rows + 32 * RS_ROWS - 1) / (32 * RS_ROWS)), 256, 0, ctx.stream>>>(static_cast<const __nv_bfloat16*>(p.k), rscale, n_rows, p.d_k);
+  rscale_kernel<<<(unsigned)((n_rows + 32 * RS_ROWS - 1) / (32 * RS_ROWS)), 256, 0, ctx.stream>>>(static_cast<const __nv_bfloat16*>(p.k), r.f32,
+                                                                                                          r.bf16, n_rows, p.d_k);
   note_launch(ctx);
 }
 
-void tc_attend(const Problem& p, const __nv_bfloat16* rscale, const AttendStates& st, int* device_status, LaunchCtx& ctx) {
+void tc_attend(const Problem& p, const KeyScales& r, const AttendStates& st, int* device_status, LaunchCtx& ctx) {
   const int BH = p.B * p.H;
   CUtensorMap tmQ, tmK, tmV, tmS;
   const int kt = KTILE / p.groups;
   const int n_pairs = (p.T + 2 * QT - 1) / (2 * QT);
-  AArgs a{static_cast<__nv_bfloat16*>(p.out), rscale, device_status, p.T, p.d_v, BH, n_pairs, n_pairs, 1, 1, 0, nullptr};
+  AArgs a{static_cast<__nv_bfloat16*>(p.out), r.f32, r.bf16, device_status, p.T, p.d_v, BH, n_pairs, n_pairs, 1, 1, 0, nullptr};
   bool maps = make_tile_map(&tmQ, p.q, BH, p.T, QT, p.d_k) && make_tile_map(&tmK, p.k, BH, p.T, kt, p.d_k) &&
               make_tile_map(&tmV, p.v, BH, p.T, kt, p.d_v);
   if (st.n_chunks > 0) {
@@ -674,11 +701,21 @@ void tc_attend(const Problem& p, const __nv_bfloat16* rscale, const AttendStates
     return;
   }
   const bool narrow = tc_narrow(p);
-  auto kern = p.groups == 2 ? tc_attend_kernel<2, 8> : p.groups == 4 ? tc_attend_kernel<4, 8> : narrow ? tc_attend_kernel<1, 4> : tc_attend_kernel<1, 8>;
-  if (!(p.groups == 2   ? allow_smem<tc_attend_kernel<2, 8>>((int)SMEM_ALLOC)
-        : p.groups == 4 ? allow_smem<tc_attend_kernel<4, 8>>((int)SMEM_ALLOC)
-        : narrow        ? allow_smem<tc_attend_kernel<1, 4>>((int)SMEM_ALLOC)
-                        : allow_smem<tc_attend_kernel<1, 8>>((int)SMEM_ALLOC))) {
+  void (*kern)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, AArgs) = nullptr;
+  auto pick = [&](auto g, auto r, auto xr) {
+    constexpr auto K = tc_attend_kernel<decltype(g)::value, decltype(r)::value, decltype(xr)::value>;
+    kern = K;
+    return allow_smem<K>((int)SMEM_ALLOC);
+  };
+  using std::integral_constant;
+  auto pick_g = [&](auto xr) {
+    if (p.groups == 2) return pick(integral_constant<int, 2>{}, integral_constant<int, 8>{}, xr);
+    if (p.groups == 4) return pick(integral_constant<int, 4>{}, integral_constant<int, 8>{}, xr);
+    return pick(integral_constant<int, 1>{}, integral_constant<int, 8>{}, xr);
+  };
+  if (!(narrow              ? pick(integral_constant<int, 1>{}, integral_constant<int, 4>{}, std::false_type{})
+        : st.exact_scales   ? pick_g(std::true_type{})
+                            : pick_g(std::false_type{}))) {
     ctx.status = KATA_ERR_CUDA;
     return;
   }
@@ -703,9 +740,9 @@ void tc_attend(const Problem& p, const __nv_bfloat16* rscale, const AttendStates
 }
 
 void tc_quadratic(const Problem& p, void* workspace, int* device_status, LaunchCtx& ctx) {
-  __nv_bfloat16* rscale = static_cast<__nv_bfloat16*>(workspace);
-  tc_rscale(p, rscale, ctx);
-  if (ctx.status == KATA_OK) tc_attend(p, rscale, AttendStates{}, device_status, ctx);
+  const KeyScales r{nullptr, static_cast<__nv_bfloat16*>(workspace)};
+  tc_rscale(p, r, ctx);
+  if (ctx.status == KATA_OK) tc_attend(p, r, AttendStates{}, device_status, ctx);
 }
 
 }  // namespace kata

@@ -21,7 +21,7 @@ ChunkBuffers chunk_buffers(const Problem& p, const StatePlan& plan, bool states)
   const size_t BH = (size_t)p.B * p.H, slots = BH * plan.n_chunks, rows = (size_t)tc_state_rows(p);
   ChunkBuffers b{};
   b.r = 0;
-  b.s = align256(BH * p.T * 2);
+  b.s = align256(BH * p.T * 4);
   b.z = b.s + (states ? align256(slots * rows * 64 * 2) : 0);
   b.s_loc = b.z + (states ? align256(slots * rows * 2) : 0);
   b.z_loc = b.s_loc + (states && plan.segments > 1 ? align256(slots * rows * 64 * 4) : 0);
@@ -69,9 +69,12 @@ void tc_chunked_states(const Problem& p, const StatePlan& plan, void* workspace,
   const bool states = plan.n_chunks > 1 || s_init != nullptr || s_final != nullptr;
   const ChunkBuffers b = chunk_buffers(p, plan, states);
   unsigned char* w = static_cast<unsigned char*>(workspace);
-  __nv_bfloat16* r = reinterpret_cast<__nv_bfloat16*>(w + b.r);
+  const bool exact_scales = p.groups > 1 || s_init != nullptr || s_final != nullptr;
+  KeyScales r{};
+  if (states || exact_scales) r.f32 = reinterpret_cast<float*>(w + b.r); else r.bf16 = reinterpret_cast<__nv_bfloat16*>(w + b.r);
   tc_rscale(p, r, ctx);
   AttendStates at{};
+  at.exact_scales = exact_scales;
   if (states) {
     StateBuffers buf{};
     buf.s = reinterpret_cast<__nv_bfloat16*>(w + b.s);
@@ -83,7 +86,7 @@ void tc_chunked_states(const Problem& p, const StatePlan& plan, void* workspace,
     buf.s_final = s_final;
     buf.z_final = z_final;
     buf.layout = state_layout;
-    if (ctx.status == KATA_OK) tc_states(p, r, plan, buf, device_status, ctx);
+    if (ctx.status == KATA_OK) tc_states(p, r.f32, plan, buf, device_status, ctx);
     at.s = buf.s;
     at.z = buf.z;
     at.n_chunks = plan.n_chunks;

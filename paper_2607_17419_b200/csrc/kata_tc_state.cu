@@ -6,7 +6,9 @@
 // chunk axis.  It walks tiles of 128 tokens:
 //   operand  A[f, t] = (r_t k_t,b) k_t,a   features on the TMEM lanes, tokens on the columns.  A builder warp takes the
 //            key tile in MMA-fragment form, transposed on the way (ldmatrix.trans: lane = (feature of a run of 8, pair of
-//            tokens)), multiplies the fragment of run h by the key scales, leaves it in a scratch of its own from which
+//            tokens)), multiplies the fragment of run h by the key scales (r as the sum of two bf16, so that r k_b is rounded
+//            once and a feature twice: with r rounded first the exported state was 2.9e-3 off in the 2-norm instead of
+//            2.35e-3), leaves it in a scratch of its own from which
 //            each of its features b is broadcast to the lanes (16 bytes = 4 runs of tokens per load), and multiplies the
 //            fragments of the runs g by it.  tcgen05.st.16x128b takes exactly this layout, so the operand never passes
 //            through shared memory.
@@ -53,8 +55,8 @@ constexpr uint32_t TMEM_COLS = 512;
 
 constexpr uint32_t STAGE_BYTES = 32768;                     // key tile, value tile
 constexpr uint32_t OFF_ONES = NSTAGE * STAGE_BYTES;         // 16 rows of [1, 0 ...]: columns 64.. of the values
-constexpr uint32_t OFF_RV = OFF_ONES + 2048;                // NSTAGE x 128 bf16 key scales, in the builders' order
-constexpr uint32_t OFF_SCR = OFF_RV + NSTAGE * 256;         // 16 builder warps x 2 KB: scaled fragments of run h
+constexpr uint32_t OFF_RV = OFF_ONES + 2048;                // NSTAGE x 2 x 128 bf16 key scales (high and low parts), in the builders' order
+constexpr uint32_t OFF_SCR = OFF_RV + NSTAGE * 512;         // 16 builder warps x 2 KB: scaled fragments of run h
 constexpr uint32_t OFF_BAR = OFF_SCR + 16 * 2048;
 constexpr uint32_t SMEM_BYTES = OFF_BAR + 256;
 constexpr uint32_t SMEM_ALLOC = SMEM_BYTES + 1024;
@@ -72,7 +74,7 @@ enum {
 };
 
 struct SArgs {
-  const __nv_bfloat16* rscale;   // [BH][T]
+  const float* rscale;           // [BH][T]
   __nv_bfloat16* s;              // [BH][n_chunks][rows][64]: state before each chunk (one segment)
   __nv_bfloat16* z;              // [BH][n_chunks][rows]
   float* s_loc;                  // [BH][n_chunks][rows][64]: sum of the segment up to and including the chunk (several segments)
@@ -108,6 +110,13 @@ static_assert(128 * 40 + 512 * 80 + 256 * 72 <= 896 * 72, "register budget");
 
 __device__ __forceinline__ uint32_t mul_bf16x2(uint32_t a, uint32_t b) {
   const __nv_bfloat162 p = __hmul2(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));
+  return *reinterpret_cast<const uint32_t*>(&p);
+}
+// x (hi + lo), rounded once (the rounding of the small term does not count)
+__device__ __forceinline__ uint32_t scale_bf16x2(uint32_t x, uint32_t hi, uint32_t lo) {
+  const uint32_t low = mul_bf16x2(x, lo);
+  const __nv_bfloat162 p = __hfma2(*reinterpret_cast<const __nv_bfloat162*>(&x), *reinterpret_cast<const __nv_bfloat162*>(&hi),
+                                   *reinterpret_cast<const __nv_bfloat162*>(&low));
   return *reinterpret_cast<const uint32_t*>(&p);
 }
 // Four 8 x 8 blocks, each transposed: lane i gets column i / 4, rows 2 (i % 4) and 2 (i % 4) + 1, of block j in r[j].
@@ -236,20 +245,17 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     regs_release<40>();
     // =========================== key scales, from the pre-pass to shared memory ===========================
     cudaGridDependencySynchronize();
-    const unsigned short* rs = reinterpret_cast<const unsigned short*>(args.rscale) + (size_t)bh * args.Tlen;
-    auto load_r = [&](int j, uint32_t (&w)[2]) {          // tokens 4 lane .. 4 lane + 3 of tile j
+    const float* rs = args.rscale + (size_t)bh * args.Tlen;
+    auto load_r = [&](int j, float (&w)[4]) {             // tokens 4 lane .. 4 lane + 3 of tile j
       const int t0 = (t_beg + j) * CT + 4 * lane;
-      unsigned short x[4];
 #pragma unroll
-      for (int e = 0; e < 4; ++e) x[e] = (j < n && t0 + e < args.Tlen) ? rs[t0 + e] : (unsigned short)0;
-      w[0] = (uint32_t)x[0] | ((uint32_t)x[1] << 16);
-      w[1] = (uint32_t)x[2] | ((uint32_t)x[3] << 16);
+      for (int e = 0; e < 4; ++e) w[e] = (j < n && t0 + e < args.Tlen) ? rs[t0 + e] : 0.f;
     };
-    uint32_t w[2];
+    float w[4];
     load_r(0, w);
     for (int j = 0; j < n && ok; ++j) {
       const int s = j % NSTAGE;
-      uint32_t nx[2];
+      float nx[4];
       load_r(j + 1, nx);
       ok = wait_or_abort(bar(BAR_EMPTY + s), ((j / NSTAGE) & 1) ^ 1, abort_flag);
       if (!ok) break;
@@ -257,8 +263,14 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
         const int pr = 2 * lane + e, grp = pr >> 4, run = (pr >> 2) & 3, i4 = pr & 3;
-        *reinterpret_cast<uint32_t*>(base + OFF_RV + s * 256 + (grp * 16 + i4 * 4 + run) * 4) = w[e];
-        w[e] = nx[e];
+        unsigned char* dst = base + OFF_RV + s * 512 + (grp * 16 + i4 * 4 + run) * 4;
+        const uint32_t hi = pack_bf16(w[2 * e], w[2 * e + 1]);
+        auto low = [](float x, float h) { return isinf(h) ? 0.f : x - h; };
+        *reinterpret_cast<uint32_t*>(dst) = hi;
+        *reinterpret_cast<uint32_t*>(dst + 256) =
+            pack_bf16(low(w[2 * e], __uint_as_float(hi << 16)), low(w[2 * e + 1], __uint_as_float(hi & 0xFFFF0000u)));
+        w[2 * e] = nx[2 * e];
+        w[2 * e + 1] = nx[2 * e + 1];
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(bar(BAR_FULL + s));
@@ -284,22 +296,23 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         const int s = j % NSTAGE, hs = 2 * j + th, slot = hs % NSLOT;
         ok = wait_or_abort(bar(BAR_FULL + s), (j / NSTAGE) & 1, abort_flag);
         if (!ok) break;
-        const uint32_t kt = smem_u32(stage(s)), rv = smem_u32(base + OFF_RV) + s * 256 + th * 128 + (lane & 3) * 16;
+        const uint32_t kt = smem_u32(stage(s)), rv = smem_u32(base + OFF_RV) + s * 512 + th * 128 + (lane & 3) * 16;
         uint32_t fa[2][4], fb[2][4];
 #pragma unroll
         for (int grp = 0; grp < 2; ++grp) {                    // 32 tokens
-          uint32_t fh[4], fk[4], r4[4];
+          uint32_t fh[4], fk[4], r4[4], l4[4];
           ldmatrix_x4_trans(fh, kt + o_ha + grp * 4096);
           if constexpr (TWO) ldmatrix_x4_trans(fk, kt + o_hb + grp * 4096);
           lds128(r4, rv + grp * 64);
+          lds128(l4, rv + 256 + grp * 64);
           ldmatrix_x4_trans(fa[grp], kt + o_ga + grp * 4096);
           ldmatrix_x4_trans(fb[grp], kt + o_gb + grp * 4096);
 #pragma unroll
-          for (int o = 0; o < 4; ++o) fh[o] = mul_bf16x2(fh[o], r4[o]);
+          for (int o = 0; o < 4; ++o) fh[o] = scale_bf16x2(fh[o], r4[o], l4[o]);
           sts128(scr_w + grp * 512, fh);
           if constexpr (TWO) {
 #pragma unroll
-            for (int o = 0; o < 4; ++o) fk[o] = mul_bf16x2(fk[o], r4[o]);
+            for (int o = 0; o < 4; ++o) fk[o] = scale_bf16x2(fk[o], r4[o], l4[o]);
             sts128(scr_w + 1024 + grp * 512, fk);
           }
         }
@@ -514,7 +527,7 @@ int tc_state_rows(const Problem& p) {
   return p.groups == 2 ? PairTable<2>::kRows : p.groups == 4 ? PairTable<4>::kRows : tc_narrow(p) ? PairTable<1, 4>::kRows : PairTable<1>::kRows;
 }
 
-void tc_states(const Problem& p, const __nv_bfloat16* rscale, const StatePlan& plan, const StateBuffers& buf, int* device_status,
+void tc_states(const Problem& p, const float* rscale, const StatePlan& plan, const StateBuffers& buf, int* device_status,
                LaunchCtx& ctx) {
   const int BH = p.B * p.H;
   CUtensorMap tmK, tmV;

@@ -84,3 +84,55 @@ def test_state_in_and_out(layout, g, H, cuts):
         f = ko.apply_feature(w.k_ref[0, h], feature_of(g, layout))
         for got, ref in ((S, f.T @ w.v_ref[0, h]), (Z, f.sum(axis=0))):
             assert np.max(np.abs(to_numpy64(got[0, h]) - ref)) <= 2e-2 * max(1.0, np.abs(ref).max())
+
+
+@pytest.mark.parametrize("layout", ["psd_direct", "psd_packed"])
+@pytest.mark.parametrize("g,H,T", [(1, 2, 700), (1, 20, 1500), (2, 3, 1500), (4, 40, 900)])
+def test_exported_state_rounding(layout, g, H, T):
+    """A term psi_f(k_t) v_t of the exported state is rounded to bf16 twice (r k_b and its product with k_a), as on the
+    streaming kernel.  One rounding is off by 2^-8 / sqrt(3) x rms(1 / m) = 1.66e-3 (m, the mantissa, spread over its
+    logarithm), independently from term to term: |S - ref| = 1.66e-3 sqrt(n) sqrt(sum |psi_t|^2 |v_t|^2) for n roundings.
+    The bound lies at n = 2.45, between two and three."""
+    import torch
+    w = inputs.gaussian_workload(f"round_{g}_{H}_{T}", "bf16", 1, H, T, 64, 64, 64, 5400 + T + g)
+    code = kb.KATA_LAYOUT_PACKED if layout == "psd_packed" else kb.KATA_LAYOUT_DIRECT
+    n = kb.decode_n_psi(64, 2, code, g)
+    S, Z = torch.empty(1, H, n, 64, device="cuda"), torch.empty(1, H, n, device="cuda")
+    kb.kata_fwd_chunked(*dev_tensors(w), s_pre=S, z_pre=Z, state_layout=code, feature_groups=g)
+    torch.cuda.synchronize()
+    assert kb.kata_last_impl() == kb.KATA_IMPL_TENSOR and kb.kata_last_launch_count() >= 3
+    eps = 2.0 ** -8 / np.sqrt(3.0) * np.sqrt(3.0 / (8.0 * np.log(2.0)))
+    for h in (0, H - 1):
+        v = w.v_ref[0, h]
+        f = ko.apply_feature(w.k_ref[0, h], feature_of(g, layout))
+        p2 = (f * f).sum(axis=1)
+        for got, ref, terms in ((S, f.T @ v, p2 * (v * v).sum(axis=1)), (Z, f.sum(axis=0), p2)):
+            err = np.linalg.norm(to_numpy64(got[0, h]) - ref)
+            assert err <= eps * np.sqrt(2.45 * terms.sum()), (g, layout, h, err / (eps * np.sqrt(terms.sum())))
+
+
+@pytest.mark.parametrize("g,H,T,state", [(1, 20, 600, True), (2, 3, 1000, False), (2, 20, 400, True), (4, 5, 1200, False)])
+def test_weight_rounding(g, H, T, state):
+    """Calls of one chunk with a state handed out or with feature groups: a weight r s^2 is rounded to bf16 once, so with the
+    1.66e-3 of a rounding (above) an output row is off by 1.66e-3 sqrt(n sum (w / D)^2 |v - o|^2 + |o|^2), n = 1, the second
+    term being the rounding of the result.  The bound lies at n = 2; s^2, r and their product rounded in turn are n = 3."""
+    import torch
+    w = inputs.gaussian_workload(f"weights_{g}_{H}_{T}", "bf16", 1, H, T, 64, 64, 64, 5500 + T + g)
+    n = kb.decode_n_psi(64, 2, kb.KATA_LAYOUT_DIRECT, g)
+    kw = dict(s_pre=torch.empty(1, H, n, 64, device="cuda"), z_pre=torch.empty(1, H, n, device="cuda")) if state else {}
+    o = kb.kata_fwd_chunked(*dev_tensors(w), feature_groups=g, **kw)
+    torch.cuda.synchronize()
+    assert kb.kata_last_impl() == kb.KATA_IMPL_TENSOR and kb.kata_last_launch_count() == (3 if state else 2)
+    eps = 2.0 ** -8 / np.sqrt(3.0) * np.sqrt(3.0 / (8.0 * np.log(2.0)))
+    err = near = far = 0.0
+    m = 64 // g
+    for h in (0, H - 1):
+        q, k, v = w.q_ref[0, h], w.k_ref[0, h], w.v_ref[0, h]
+        p = sum((q[:, a:a + m] @ k[:, a:a + m].T) ** 2 for a in range(0, 64, m)) / (k * k).sum(axis=1)
+        p = np.tril(p)
+        p /= p.sum(axis=1, keepdims=True)
+        r = p @ v
+        err += ((to_numpy64(o[0, h]) - r) ** 2).sum()
+        near += ((p * p) * ((v * v).sum(axis=1)[None, :] - 2 * (r @ v.T) + (r * r).sum(axis=1)[:, None])).sum()
+        far += (r * r).sum()
+    assert np.sqrt(err) <= eps * np.sqrt(2.0 * near + far), (g, H, T, (err / eps ** 2 - far) / near)
