@@ -71,12 +71,14 @@ template <int MODE, int G, int NS> struct Geo {
   static constexpr uint32_t COL_ACC = SEP ? 256 + NBUF * EW : 384;        // accumulators: 64 or 128 columns
   static constexpr int NTHREADS = 128 + SETS * 128;
   static_assert(NBUF * BW <= (SEP ? 256u : COL_ACC) && COL_ACC + (MODE == MODE_DQ ? 64 : 128) <= (XT ? COL_X : 512u), "TMEM columns");
-  // first column of the bf16 weights of a buffer: their own, or over scores that are already in registers
-  __host__ __device__ static constexpr uint32_t p_col(int b, int term) {
-    return SEP ? 256 + b * EW : b * BW + (NS == 3 ? (term == 0 ? 0u : term == 1 ? 128u : 160u) : CB);
+  // first of the 16 columns of the bf16 weights of 32 streamed rows (run ch of a buffer): columns of their own, or over scores
+  // that the same warp has in its registers (three terms: P and E of a term side by side, over the run's columns of S, of C
+  // and of the 64 more, so that no set touches what the other still reads)
+  __host__ __device__ static constexpr uint32_t p_col(int b, int term, int ch) {
+    return SEP ? 256 + b * EW + ch * 16 : b * BW + (NS == 3 ? term * 64 + ch * 32 : CB + ch * 16);
   }
-  __host__ __device__ static constexpr uint32_t e_col(int b, int g, int term) {
-    return SEP ? 256 + b * EW + (MODE == MODE_DQ ? 32 * term : 32) : b * BW + (NS == 3 ? (term == 0 ? 64u : term == 1 ? 32u : 96u) : g * NT);
+  __host__ __device__ static constexpr uint32_t e_col(int b, int g, int term, int ch) {
+    return SEP ? 256 + b * EW + (MODE == MODE_DQ ? 32 * term : 32) + ch * 16 : b * BW + (NS == 3 ? term * 64 + ch * 32 + 16 : g * NT + ch * 16);
   }
 };
 
@@ -111,7 +113,8 @@ enum {
   BAR_OFREE = 25,    // ... and have been read (256 threads)
   BAR_XT = 26,       // [2] fixed tiles of an item in TMEM (256 threads)
   BAR_DRAIN = 28,
-  BAR_COUNT = 29
+  BAR_MEET = 29,     // MODE_DQ: the sums of an item are in shared memory (all weight threads)
+  BAR_COUNT = 30
 };
 
 struct BArgs {
@@ -208,6 +211,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
     mbar_init(bar(BAR_ODONE), 1);
     mbar_init(bar(BAR_OFREE), 256);
     mbar_init(bar(BAR_DRAIN), 2);
+    mbar_init(bar(BAR_MEET), SETS * 128);
     fence_mbar_init();
     tma_prefetch_desc(&tmX1);
     tma_prefetch_desc(&tmX2);
@@ -331,7 +335,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
             for (int term = 0; term < NS; ++term)
 #pragma unroll
               for (int ks = 0; ks < NT / 16; ++ks)      // dv~ += P^T dout
-                mma_f16_ts(tb + COL_ACC, tb + geo::p_col(b, term) + ks * 8, at(dmn, yb + ks * 2048), id_o, (acc || term > 0 || ks > 0) ? 1u : 0u);
+                mma_f16_ts(tb + COL_ACC, tb + geo::p_col(b, term, ks / 2) + (ks & 1) * 8, at(dmn, yb + ks * 2048), id_o, (acc || term > 0 || ks > 0) ? 1u : 0u);
           }
           constexpr uint32_t col = COL_ACC + (MODE == MODE_DKV ? 64 : 0);
 #pragma unroll
@@ -340,7 +344,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
             for (int term = 0; term < NS; ++term)
 #pragma unroll
               for (int ks = 0; ks < NT / 16; ++ks)      // dq += E K, u += E^T Q
-                mma_f16_ts(tb + col + g * MG, tb + geo::e_col(b, g, term) + ks * 8, at(dmn, ya + ks * 2048 + g * MG * 2), id_g,
+                mma_f16_ts(tb + col + g * MG, tb + geo::e_col(b, g, term, ks / 2) + (ks & 1) * 8, at(dmn, ya + ks * 2048 + g * MG * 2), id_g,
                            (acc || term > 0 || ks > 0) ? 1u : 0u);
           acc = 1;
           mma_commit(bar((SEP ? BAR_PFREE : BAR_SFREE) + b));
@@ -404,13 +408,6 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
     const int ch0 = set % CS;                    // ... and its columns of every block (CPW runs of 32)
     const int rowl = q4 * 32 + lane;             // row of the fixed tile (= TMEM lane)
     const uint32_t lanes = tmem_addr(tb, q4 * 32, 0), buf = lanes + grp * BW, accu = lanes + COL_ACC;
-    // the sets of a buffer have read what the weights of the other are about to overwrite
-    auto both_read = [&]() {
-      if (SEP || CS == 1) return;
-      tc_fence_before();
-      asm volatile("bar.sync %0, 64;" ::"r"(2 + grp * 4 + (int)q4) : "memory");
-      tc_fence_after();
-    };
     // fixed tiles of item i from shared memory to TMEM: set 0 the first, set 1 the second
     auto copy_x = [&](int i) {
       const int xb = i & 1;
@@ -521,10 +518,12 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
           end();
         }
         if (!ok) break;
-        // the sets' shares of a row meet, in a fixed order
+        // the sets' shares of a row meet, in a fixed order (a bounded wait: a set that has given up does not come)
         float2* part = reinterpret_cast<float2*>(base + OFF_PART) + (ni & 1) * 512 + rowl;
         part[set * MT] = make_float2(sum_d, sum_m);
-        asm volatile("bar.sync 1, %0;" ::"n"(SETS * 128) : "memory");
+        mbar_arrive(bar(BAR_MEET));
+        ok = wait_or_abort(bar(BAR_MEET), ni & 1, abort_flag);
+        if (!ok) break;
         float dt = 0.f, mt = 0.f;
 #pragma unroll
         for (int g = 0; g < SETS; ++g) {
@@ -554,7 +553,6 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
         tmem_wait_ld(cv);
         read_done();
         if constexpr (G == 1) {
-          both_read();
           // the outputs of two steps back have read this buffer's weights
           if (SEP && n_out > 0) ok = wait_or_abort(bar(BAR_PFREE + grp), (n_out - 1) & 1, abort_flag);
           if (!ok) break;
@@ -593,8 +591,8 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
               }
 #pragma unroll
               for (int i = 0; i < NS; ++i) {
-                tmem_st8(lanes + geo::e_col(grp, 0, i) + ch * 16 + c0 / 2, pe[i]);
-                if constexpr (MODE == MODE_DKV) tmem_st8(lanes + geo::p_col(grp, i) + ch * 16 + c0 / 2, pp[i]);
+                tmem_st8(lanes + geo::e_col(grp, 0, i, ch) + c0 / 2, pe[i]);
+                if constexpr (MODE == MODE_DKV) tmem_st8(lanes + geo::p_col(grp, i, ch) + c0 / 2, pp[i]);
               }
             }
           };
@@ -637,8 +635,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
               const float2 e2 = __fmul2_rn(make_float2(__uint_as_float(cv[c]), __uint_as_float(cv[c + 1])), s2);
               pk[c / 2] = pack_bf16(e2.x, e2.y);
             }
-            both_read();
-            tmem_st16(lanes + geo::e_col(grp, g, 0) + ch * 16, pk);
+            tmem_st16(lanes + geo::e_col(grp, g, 0, ch), pk);
           }
           if constexpr (MODE == MODE_DKV) {
             // p = sum_g s_g^2 / D_t
@@ -655,7 +652,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
               }
             };
             if (diag) weights(std::true_type{}); else weights(std::false_type{});
-            tmem_st16(lanes + geo::p_col(grp, 0) + ch * 16, pk);
+            tmem_st16(lanes + geo::p_col(grp, 0, ch), pk);
           }
         }
         }
