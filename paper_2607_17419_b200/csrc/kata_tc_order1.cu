@@ -42,7 +42,7 @@ constexpr int SROWS = 80;          // state rows kept: 64 value columns, the nor
 constexpr int W_MMA_A = 1, W_MMA_B = 2, W_MMA_U = 3, W_SNAP0 = 4, W_MMA_R = 7, W_BLD0 = 8;
 
 constexpr uint32_t COL_S = 0;      // 64 fp32: [S | Z]^T, lanes = (v, z, 0..), columns = feature a
-constexpr uint32_t COL_P = 64;     // 2 x 128 fp32 scores; the bf16 weights overwrite columns [0,64) of a buffer
+constexpr uint32_t COL_P = 64;     // 2 x 128 fp32 scores; the bf16 weights overwrite columns [0,32) and [64,96) of a buffer
 constexpr uint32_t COL_O = 320;    // 2 x 80: 64 outputs, column 64 = normaliser
 constexpr uint32_t TMEM_COLS = 512;
 
@@ -386,7 +386,7 @@ tc_order1_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
           tc_fence_after();
 #pragma unroll
           for (int ks = 0; ks < 8; ++ks)
-            mma_f16_ts(tb + COL_O + b * 80, tb + COL_P + b * 128 + ks * 8,
+            mma_f16_ts(tb + COL_O + b * 80, tb + COL_P + b * 128 + (ks >> 2) * 64 + (ks & 3) * 8,
                        smem_desc(va + ks * 2048, ones - va, 1024, kSwizzle128B), idPV, (resume || j > 0 || ks > 0) ? 1u : 0u);
           mma_commit(bar(BAR_P_EMPTY + b));
           mma_commit(bar(BAR_O_FULL + b));
@@ -490,12 +490,8 @@ tc_order1_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         pk[c / 2] = pack_bf16(k0 <= rowl ? __uint_as_float(ya[c]) : 0.f, k0 + 1 <= rowl ? __uint_as_float(ya[c + 1]) : 0.f);
         pk[16 + c / 2] = pack_bf16(k1 <= rowl ? __uint_as_float(yb[c]) : 0.f, k1 + 1 <= rowl ? __uint_as_float(yb[c + 1]) : 0.f);
       }
-      // the weights overwrite score columns [0,64) of the buffer, which the column-half-0 warp of this
-      // quadrant reads: both warps of the quadrant must have their scores in registers first
-      tc_fence_before();
-      asm volatile("bar.sync %0, 64;" ::"r"(1 + (int)q4) : "memory");
-      tc_fence_after();
-      tmem_st32(tmem_addr(tb, q4 * 32, COL_P + b * 128 + ch * 32), pk);
+      // the weights of a column half overwrite its own scores, which are in this thread's registers
+      tmem_st32(scol, pk);
       tmem_wait_st();
       tc_fence_before();
       mbar_arrive(bar(BAR_P_FULL + b));
