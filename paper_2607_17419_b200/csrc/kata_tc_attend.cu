@@ -163,10 +163,13 @@ struct AArgs {
 // than on the kernels that answer the short calls of the same kinds (2.9e-3 there; 2.2e-3 to 2.4e-3 with exact scales).  One packed multiply
 // and twice the reads of r per pair: 4 x 16 heads x 4096 tokens of the quadratic form 126 -> 136 us, where nothing calls for
 // it; 2 x 16 x 3001 with the state 109 -> 111.
+// SPLIT = a work item is 128 queries without a state: both halves hold the same query tile, half A takes the even and half B the
+// odd key tiles, and the epilogue adds their [O | D] (the weights are polynomial: partial sums simply add).  For calls of few
+// blocks; see tc_attend.
 // R = runs of 8 features that a row may have.  G = feature groups of the blockwise map: a key tile holds KT = 128 / G keys, and the 128 score columns of a buffer
 // hold, for each half of those keys, the G per-group score blocks Q_a K_a^T side by side (group a in columns [a KT/2,
 // a KT/2 + KT/2) of the sub-buffer); the weight of a key is the sum over the groups of the squared scores.
-template <int G, int R, bool XR>
+template <int G, int R, bool XR, bool SPLIT>
 __global__ void __launch_bounds__(NTHREADS, 1)
 tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                  const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmS, const AArgs args) {
@@ -219,6 +222,14 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       it.bh = rem % args.BH;
       const int pair = it.chunk * args.chunk_pairs + p;
       if (pair >= args.n_pairs) continue;
+      if (SPLIT) {
+        it.q0 = pair * QT;
+        it.k0 = it.ns = 0;
+        it.n_tiles = (p + 1) * G;
+        it.nk_b = it.n_tiles / 2;
+        it.nk_a = it.n_tiles - it.nk_b;
+        return true;
+      }
       it.q0 = pair * 2 * QT;
       it.k0 = it.chunk * args.chunk_pairs * 2 * G;
       it.nk_a = (2 * p + 1) * G;
@@ -236,7 +247,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     for (int i = 0; i < 2; ++i) {
       mbar_init(bar(BAR_QT + i), 128);
       mbar_init(bar(BAR_ODONE + i), 1);
-      mbar_init(bar(BAR_OFREE + i), 256);
+      mbar_init(bar(BAR_OFREE + i), SPLIT ? 512 : 256);
     }
     for (int i = 0; i < 4; ++i) {
       mbar_init(bar(BAR_SFULL + i), 1);
@@ -287,9 +298,10 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       for (int n = 0; ok && next_item(n, w); ++n, ++ni) {
         ok = wait_or_abort(bar(BAR_QEMPTY), (ni & 1) ^ 1, abort_flag);
         if (!ok) break;
-        mbar_arrive_expect_tx(bar(BAR_QFULL), w.nk_b > 0 ? 32768 : 16384);
+        const bool two = !SPLIT && w.nk_b > 0;           // query tiles
+        mbar_arrive_expect_tx(bar(BAR_QFULL), two ? 32768 : 16384);
         tma_load_3d(base + OFF_Q, &tmQ, bar(BAR_QFULL), 0, w.q0, w.bh);
-        if (w.nk_b > 0) tma_load_3d(base + OFF_Q + 16384, &tmQ, bar(BAR_QFULL), 0, w.q0 + QT, w.bh);
+        if (two) tma_load_3d(base + OFF_Q + 16384, &tmQ, bar(BAR_QFULL), 0, w.q0 + QT, w.bh);
         for (int j = 0; j < w.n_tiles && ok; ++j, ++it) {
           const int s = it % NSTAGE;
           ok = wait_or_abort(bar(BAR_EMPTY + s), ((it / NSTAGE) & 1) ^ 1, abort_flag);
@@ -350,6 +362,39 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
           }
           return true;
         };
+        if constexpr (SPLIT) {
+          // every other tile is this half's; the others are passed on as they land (a parity cannot tell two phases of a
+          // stage apart, so both halves see every tile)
+          const uint32_t end = it + w.n_tiles;
+          auto pass = [&](uint32_t g_it) -> bool {
+            if (!landed(g_it)) return false;
+            mbar_arrive(bar(BAR_EMPTY + g_it % NSTAGE));
+            return true;
+          };
+          if (h == 1) ok = pass(it++);
+          if (nk > 0) {
+            ok = ok && wait_or_abort(bar(BAR_QT + h), n_done & 1, abort_flag) && landed(it);
+            if (ok) {
+              tc_fence_after();
+              open(it, 0);
+              open(it, 1);
+            }
+            for (int j = 0; j < nk && ok; ++j, it += 2, ++cnt) {
+              const bool next = j + 1 < nk;
+              ok = (!next || (pass(it + 1) && landed(it + 2))) && close(it, 0);
+              if (ok && next) open(it + 2, 0);
+              ok = ok && close(it, 1);
+              if (!ok) break;
+              mma_commit(bar(BAR_EMPTY + it % NSTAGE));
+              if (next) open(it + 2, 1);
+              else if (it + 1 < end) ok = pass(it + 1);
+            }
+            if (ok) mma_commit(bar(BAR_ODONE + h));
+            ++n_done;
+          }
+          it = end;
+          continue;
+        }
         if (nt > 0) ok = wait_or_abort(bar(BAR_QT + h), n_done & 1, abort_flag) && (w.ns > 0 || landed(it));
         if (nt > 0 && ok) {
           tc_fence_after();
@@ -465,7 +510,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     const int ch = (bw >> 2) & 1;                // sub-buffer: the first or second half of the keys (features) of a tile
     const int rowl = q4 * 32 + lane;             // query row inside the tile (= TMEM lane)
     const uint32_t tS = tmem_addr(tb, q4 * 32, COL_S + h * 128 + ch * 64), tO = tmem_addr(tb, q4 * 32, COL_O + h * 80);
-    const uint32_t qrow_s = smem_u32(base + OFF_Q) + h * 16384;
+    const uint32_t qrow_s = smem_u32(base + OFF_Q) + (SPLIT ? 0 : h * 16384);
     // 16 bytes (eight features) of this thread's query row, from the item's tile in shared memory
     auto qrun = [&](int c) { return lds128(qrow_s + sw128_offset(rowl, c)); };
     // The query tile of an item into TMEM, by the warps of the second sub-buffer: the scores of an item's last tile are
@@ -492,12 +537,13 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     };
     uint32_t it = 0, cnt = 0, n_st = 0;
     int n_done = 0, ni = 0, n = 0;
+    int n_done_b = 0;                            // SPLIT: items with tiles for half B (n_done: all)
     Item w;
     bool more = next_item(n, w);
     if (more) copy_q(0, w);
     for (; more && ok; ++ni) {
       const int nk = h == 0 ? w.nk_a : w.nk_b;
-      const int qrow = w.q0 + h * QT + rowl;
+      const int qrow = w.q0 + (SPLIT ? 0 : h * QT) + rowl;
       const uint32_t it0 = it;
       it += w.n_tiles;
       if (nk > 0 && w.ns > 0) {
@@ -531,15 +577,16 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       }
       if (w.ns > 0) mbar_arrive(bar(BAR_QEMPTY));
       for (int j = 0; j < nk && ok; ++j, ++cnt) {
-        const uint32_t g_it = it0 + w.ns + j;
+        const int kj = SPLIT ? 2 * j + h : j;         // key tile of the item
+        const uint32_t g_it = it0 + w.ns + kj;
         const int s = g_it % NSTAGE;
         ok = wait_or_abort(bar(BAR_SFULL + 2 * h + ch), cnt & 1, abort_flag);
         if (!ok) break;
         tc_fence_after();
-        const bool diag = j >= nk - G;
+        const bool diag = kj >= (SPLIT ? w.n_tiles : nk) - G;
         if constexpr (G > 1) {
           // this warp weighs keys [ch KT/2, ch KT/2 + KT/2) of the tile: one column run per group
-          const int key0 = (w.k0 + j) * KT + ch * KH;
+          const int key0 = (w.k0 + kj) * KT + ch * KH;
           uint32_t y[G][KH], pk[KH / 2];
           const uint32_t rbase = smem_u32(base + OFF_RV) + s * 512 + ch * (KH * 4);   // fp32 r of this warp's keys, 4 per load
           const uint32_t* rw = reinterpret_cast<const uint32_t*>(base + OFF_RV + s * 512) + ch * (KH / 2);   // bf16 r, in pairs
@@ -578,7 +625,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
           if constexpr (KH == 32) tmem_st16(tS, pk); else tmem_st8(tS, pk);
         } else {
           const uint32_t rbase = smem_u32(base + OFF_RV) + s * 512 + ch * (XR ? 256 : 128);   // r of this warp's 64 keys, 16 bytes per load
-          const int key0 = (w.k0 + j) * KT + ch * 64;
+          const int key0 = (w.k0 + kj) * KT + ch * 64;
           uint32_t ya[32], yb[32], pk[16];
           auto weigh = [&](const uint32_t (&y)[32], int col0, auto masked) {
             constexpr int RPL = XR ? 4 : 8;                    // keys per load
@@ -619,9 +666,45 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       if (!ok) break;
       // the next item's queries go to TMEM before the wait for this item's last MMAs
       const int bh = w.bh;
+      const bool with_b = w.nk_b > 0;
       ++n;
       more = next_item(n, w);
       if (more) copy_q(ni + 1, w);
+      if constexpr (SPLIT) {
+        // ---- epilogue: the halves' [O | D] of these queries added, 16 columns per thread ----
+        const uint32_t oa = tmem_addr(tb, q4 * 32, COL_O), c16 = (2 * h + ch) * 16;
+        ok = ok && wait_or_abort(bar(BAR_ODONE), n_done & 1, abort_flag) &&
+             (!with_b || wait_or_abort(bar(BAR_ODONE + 1), n_done_b & 1, abort_flag));
+        if (!ok) break;
+        ++n_done;
+        n_done_b += with_b ? 1 : 0;
+        tc_fence_after();
+        uint32_t x[16], y[16], dx[4], dy[4];
+        tmem_ld16(oa + c16, x);
+        tmem_ld4(oa + 64, dx);
+        tmem_ld16(oa + 80 + c16, y);
+        tmem_ld4(oa + 80 + 64, dy);
+        tmem_wait_ld(x);
+        tmem_wait_ld(y);
+        tmem_wait_ld(dx);
+        tmem_wait_ld(dy);
+        tc_fence_before();
+        mbar_arrive(bar(BAR_OFREE));
+        if (with_b) mbar_arrive(bar(BAR_OFREE + 1));
+        const float den = __uint_as_float(dx[0]) + (with_b ? __uint_as_float(dy[0]) : 0.f);
+        const float inv = den > 0.f ? 1.f / den : 0.f;
+        if (qrow < args.Tlen) {
+          __nv_bfloat16* dst = args.out + ((size_t)bh * args.Tlen + qrow) * args.d_v + c16;
+          auto sum = [&](int c) { return (__uint_as_float(x[c]) + (with_b ? __uint_as_float(y[c]) : 0.f)) * inv; };
+#pragma unroll
+          for (int jj = 0; jj < 16; jj += 8) {
+            if ((int)c16 + jj >= args.d_v) break;
+            *reinterpret_cast<uint4*>(dst + jj) = make_uint4(pack_bf16(sum(jj), sum(jj + 1)), pack_bf16(sum(jj + 2), sum(jj + 3)),
+                                                             pack_bf16(sum(jj + 4), sum(jj + 5)), pack_bf16(sum(jj + 6), sum(jj + 7)));
+          }
+        }
+        continue;
+      }
       if (nk == 0) continue;
       // ---- epilogue: out = O / D ----
       ok = ok && wait_or_abort(bar(BAR_ODONE + h), n_done & 1, abort_flag);
@@ -682,7 +765,17 @@ void tc_attend(const Problem& p, const KeyScales& r, const AttendStates& st, int
   const int BH = p.B * p.H;
   CUtensorMap tmQ, tmK, tmV, tmS;
   const int kt = KTILE / p.groups;
-  const int n_pairs = (p.T + 2 * QT - 1) / (2 * QT);
+  // No states and not more blocks of 256 queries than SMs: the call lasts as long as its longest block, so the halves of a CTA
+  // share out the keys of one block of 128 queries instead (SPLIT).  From four tiles of the longest half on; shorter ones gain
+  // nothing, and with more blocks the tiles that only one half uses cost more than the finer deal gives (with feature groups,
+  // whose tiles cost more weighing per byte, the line lies a third higher).  Measured, us, blocks of 256 / split:
+  //   one head x 8192 55 / 37, with two groups 86 / 56, with four 147 / 90; 6 x 4096 (96 blocks) 34.5 / 24.7, 8 x 4096 (128)
+  //   34.9 / 26.5, 24 x 1500 (144) 18.7 / 18.5, 37 x 1024 (148) 16.4 / 16.4; 12 x 4096 (192) 35.0 / 36.9, 64 x 4096 131 / 169
+  //   two groups 12 x 4096 (192) 51.2 / 47.2, 37 x 1500 (222) 24.8 / 26.7; four groups 80.8 / 73.0, 37.0 / 39.0
+  //   short: 64 x 512 12.4 / 14.4
+  const int n_blocks = (p.T + 2 * QT - 1) / (2 * QT);
+  const bool split = st.n_chunks == 0 && n_blocks >= 2 && n_blocks * p.groups >= 4 && 3LL * BH * n_blocks <= (p.groups > 1 ? 4 : 3) * sm_count();
+  const int n_pairs = split ? (p.T + QT - 1) / QT : n_blocks;
   AArgs a{static_cast<__nv_bfloat16*>(p.out), r.f32, r.bf16, device_status, p.T, p.d_v, BH, n_pairs, n_pairs, 1, 1, 0, nullptr};
   bool maps = make_tile_map(&tmQ, p.q, BH, p.T, QT, p.d_k) && make_tile_map(&tmK, p.k, BH, p.T, kt, p.d_k) &&
               make_tile_map(&tmV, p.v, BH, p.T, kt, p.d_v);
@@ -703,9 +796,10 @@ void tc_attend(const Problem& p, const KeyScales& r, const AttendStates& st, int
   const bool narrow = tc_narrow(p);
   void (*kern)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, AArgs) = nullptr;
   auto pick = [&](auto g, auto r, auto xr) {
-    constexpr auto K = tc_attend_kernel<decltype(g)::value, decltype(r)::value, decltype(xr)::value>;
-    kern = K;
-    return allow_smem<K>((int)SMEM_ALLOC);
+    constexpr auto K = tc_attend_kernel<decltype(g)::value, decltype(r)::value, decltype(xr)::value, false>;
+    constexpr auto KS = tc_attend_kernel<decltype(g)::value, decltype(r)::value, decltype(xr)::value, true>;
+    kern = split ? KS : K;
+    return split ? allow_smem<KS>((int)SMEM_ALLOC) : allow_smem<K>((int)SMEM_ALLOC);
   };
   using std::integral_constant;
   auto pick_g = [&](auto xr) {

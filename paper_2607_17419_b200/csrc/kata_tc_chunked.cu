@@ -33,12 +33,13 @@ ChunkBuffers chunk_buffers(const Problem& p, const StatePlan& plan, bool states)
 // Chunk length and segments.
 // No state pointers and a short sequence: one chunk, the quadratic form alone.  Per tile of 128 tokens and head the chunk
 // states cost about 9 us of one SM to build and 7 to read (full lift), a key tile 0.55: the quadratic form wins until the
-// average query sees about 29 key tiles.  Measured, us, quadratic / chunks of 1024, for 16, 128 and 3 heads:
-//   full lift   T = 6000: 75 / 99, 587 / 645, 49 / 44     T = 8192: 119 / 130, 1148 / 900, 65 / 54
-//   two groups  T = 2000: 31 / 38, 147 / 152, 30 / 37     T = 4096: 53 / 60, 450 / 315, 51 / 39
-//   four groups T = 2000: 45 / 42, 193 / 161, 43 / 41
-//   rows of 32 entries (a third of the state)  T = 3000: 32 / 48, 151 / 155     T = 4096: 42 / 46, 237 / 208, 36 / 32     T = 6000: 77 / 67, 470 / 312
-//   (a wave of blocks that is not full costs the chunks more: their line lies higher with few heads)
+// average query sees about 29 key tiles.  Measured, us, quadratic / chunks of 1024, for 3, 16 and 128 heads:
+//   full lift   T = 6000: 31 / 41, 75 / 92, 580 / 693     T = 7168: 35 / 51, 99 / 103, 784 / 835     T = 8192: 39 / 51, 123 / 123, 1172 / 936
+//   two groups  T = 2500: 23 / 29, 37 / 47, 168 / 203     T = 3000: 26 / 29, 42 / 47, 236 / 227     T = 4096: 33 / 31, 53 / 58, 408 / 341
+//   four groups T = 1500: 23 / 31, 24 / 35, 104 / 138     T = 2000: 29 / 31, 29 / 37, 166 / 147
+//   rows of 32 entries (a third of the state)  T = 3000: 19 / 25, 28 / 41, 139 / 153     T = 4096: 25 / 26, 35 / 41, 232 / 211     T = 6000: 32 / 28, 67 / 61, 498 / 321
+//   (few heads, whose blocks split the keys between the halves of a CTA, would take the quadratic form further: 3 heads up to
+//   10000 tokens 45 / 53; the line is one for all heads)
 // Chunks of 1024: 16 heads x 131072 tokens 2.08 ms; 768: 2.10, 512: 2.17, 2048 about 2.3 (shorter chunks write and read more state, longer
 // ones have more key tiles).  Halved where even one chunk per CTA leaves SMs idle (3 heads x 2048 tokens with the state
 // handed out: 43 -> 38 us).
