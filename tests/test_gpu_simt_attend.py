@@ -26,3 +26,17 @@ def test_simt_attend(dk, dv, T):
     assert torch.all(o[0, 0, 0] == 0)
     for (b, h), r in oracle_full(w).items():
         check(to_numpy64(o)[b, h], r, "f32", f"T={T} d={dk},{dv} head {h}")
+
+
+@pytest.mark.parametrize("dk,T", [(16, 900), (16, 1200), (32, 1700)])
+@pytest.mark.parametrize("scale", [1e-21, 1e18])
+def test_queries_of_any_norm(dk, T, scale):
+    """The norm of a query cancels: queries whose squares leave the range of fp32 give the answer of the unscaled ones (their
+    squared norms, 1.6e-41 and up, do not leave it)."""
+    import torch
+    w = inputs.gaussian_workload(f"sa_norm_{dk}_{T}", "f32", 1, 2, T, dk, dk, 64, 7100 + T)
+    q, k, v = dev_tensors(w)
+    o = kb.kata_fwd_chunked(q * scale, k, v)
+    torch.cuda.synchronize()
+    for (b, h), r in oracle_full(w).items():
+        check(to_numpy64(o)[b, h], r, "f32", f"T={T} d={dk} scale {scale} head {h}")
