@@ -254,7 +254,7 @@ int kata_bwd_quadratic(const void* q, const void* k, const void* v, const void* 
  * gradients.  bf16 with d_k = d_v = 64 and 512 <= T <= 16384, unless opts->impl = KATA_IMPL_SIMT: the tensor-core kernels of
  * kata_bwd_quadratic with the weights carried in three bf16 terms (24 bits) -- O(T^2) work, less at these lengths, the same
  * precision; opts->impl = KATA_IMPL_TENSOR returns KATA_ERR_UNSUPPORTED_SHAPE outside that range.
- * Workspace: kata_workspace_bytes(KATA_FN_BWD_CHUNKED, B, H, T, d_k, d_v, 64, opts) bytes: 12 bytes per token and head on the
+ * Workspace: kata_workspace_bytes(KATA_FN_BWD_CHUNKED, B, H, T, d_k, d_v, 64, opts) bytes: 276 bytes per token and head on the
  * tensor cores, else about 4 (2 d_k + d_v + (d_v / 8)(d_k + 1) + 2) (2.9 KB at d_k = d_v = 64).
  */
 int kata_bwd_chunked(const void* q, const void* k, const void* v, const void* dout, void* dq, void* dk, void* dv,

@@ -20,7 +20,9 @@
 //
 // NS = bf16 terms of the weights P and E.  One: kata_bwd_quadratic.  Three (24 bits: fp32 weights; every other operand is
 // a bf16 input, exact, and every sum fp32): kata_bwd_chunked on sequences short enough for the quadratic form, whose
-// contract is fp32 arithmetic.
+// contract is fp32 arithmetic.  Its rows of q and k come as copies scaled by powers of two (exact) to largest entries of 1 to 2,
+// so that rows of any norm whose square fp32 holds give the gradients that the walk over the chunks, which normalises
+// them, gives; the gradients are scaled back where they are stored.
 //
 // What bounds it.  A step (128 x 64 pairs) is 256 to 384 cycles of score MMAs and 128 (dq) or 256 (dk, dv) of output MMAs;
 // the rest is hand-offs, about 300 cycles each from one thread's arrival through the MMAs to the next thread's first
@@ -122,6 +124,7 @@ struct BArgs {
   __nv_bfloat16* out1;       // MODE_DKV: dv
   float* stats;              // [BH][T][2]: 1 / D_t, dout_t . o_t (written by MODE_DQ, read by MODE_DKV)
   const float* rk;           // [BH][T]: 1 / ||k_i||^2
+  const float* row_scale;    // NS = 3: [BH][T] power of two that the row of q (MODE_DQ) or k (MODE_DKV) was scaled by
   int* device_status;
   int Tlen;
   int BH;
@@ -228,8 +231,8 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
   const uint32_t tb = tmem_base_s;
   bool ok = true;
   // A programmatic dependent launch.  dk, dv start while dq runs on other SMs and wait for it here, where no limit on time
-  // applies; dq waits for its pre-pass where it reads the key scales.
-  if (MODE == MODE_DKV) cudaGridDependencySynchronize();
+  // applies; dq waits for its pre-pass where it reads the key scales, or, where that writes the rows it loads, here.
+  if (MODE == MODE_DKV || NS == 3) cudaGridDependencySynchronize();
 
   if (warp == 0) {
     if (SETS == 4) regs_release<64>();
@@ -699,6 +702,11 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
         const float f = 2.f * inv_row;
 #pragma unroll
         for (int c = 0; c < 32; ++c) x[c] = f * __uint_as_float(a0[c]);
+        if constexpr (NS == 3) {
+          const float back = grow < args.Tlen ? args.row_scale[(size_t)cur.bh * args.Tlen + grow] : 0.f;
+#pragma unroll
+          for (int c = 0; c < 32; ++c) x[c] *= back;
+        }
         if (grow < args.Tlen) store32(args.out0 + row_off + set * 32, x);
       } else {
         // set 0: dk = r (2 u - r (k . 2 u) k);  set 1: dv = r dv~
@@ -732,6 +740,8 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
         }
         const float r = inv_or_zero(n2);
         const float proj = r * dot;
+        float back = 1.f;
+        if constexpr (NS == 3) back = set == 0 && grow < args.Tlen ? args.row_scale[(size_t)cur.bh * args.Tlen + grow] : 1.f;
 #pragma unroll 1
         for (int half = 0; half < 2; ++half) {
           float x[32];
@@ -740,7 +750,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
           tmem_wait_ld(a0);
 #pragma unroll
           for (int c = 0; c < 32; ++c)
-            x[c] = set == 0 ? 2.f * r * (__uint_as_float(a0[c]) - proj * kf[c]) : r * __uint_as_float(a0[c]);
+            x[c] = set == 0 ? 2.f * r * (__uint_as_float(a0[c]) - proj * kf[c]) * back : r * __uint_as_float(a0[c]);
           if (grow < args.Tlen) store32((set == 0 ? args.out0 : args.out1) + row_off + half * 32, x);
         }
         tc_fence_before();
@@ -786,6 +796,56 @@ __global__ void __launch_bounds__(256) bwd_rscale_kernel(const __nv_bfloat16* __
   if (part == 0) rk[row] = inv_or_zero(ss);
 }
 
+// The pre-pass of the three-term weights: also copies of the rows of k (blockIdx.y = 0) and q (1) scaled by the power of two that
+// brings the largest entry to [1, 2), and that power; r is that of the scaled key.  An entry that the scaling takes below the
+// smallest bf16 is 2^-126 of the row's largest.  Memory-bound, four rows per lane in flight.
+constexpr int SCALE_ROWS = 4;
+__global__ void __launch_bounds__(256) bwd_scale_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ q,
+                                                        __nv_bfloat16* __restrict__ ks, __nv_bfloat16* __restrict__ qs, float* __restrict__ fk,
+                                                        float* __restrict__ fq, float* __restrict__ rk, size_t n_rows) {
+  cudaTriggerProgrammaticLaunchCompletion();
+  const size_t row0 = (size_t)blockIdx.x * (32 * SCALE_ROWS) + (threadIdx.x >> 3);
+  const int part = threadIdx.x & 7;
+  const bool is_q = blockIdx.y != 0;
+  const unsigned lanes = 0xFFu << (threadIdx.x & 24);       // the eight lanes of a row
+  uint4 raw[SCALE_ROWS];
+#pragma unroll
+  for (int i = 0; i < SCALE_ROWS; ++i) {
+    const size_t row = row0 + i * 32;
+    raw[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (row < n_rows) raw[i] = *reinterpret_cast<const uint4*>((is_q ? q : k) + row * D + part * 8);
+  }
+#pragma unroll
+  for (int i = 0; i < SCALE_ROWS; ++i) {
+    const size_t row = row0 + i * 32;
+    const uint32_t w[4] = {raw[i].x, raw[i].y, raw[i].z, raw[i].w};
+    uint32_t top = 0;                                       // largest exponent field of the row
+#pragma unroll
+    for (int e = 0; e < 4; ++e) top = max(top, max(w[e] & 0x7F80u, (w[e] >> 16) & 0x7F80u));
+#pragma unroll
+    for (int off = 1; off < 8; off <<= 1) top = max(top, __shfl_xor_sync(lanes, top, off));
+    const uint32_t ex = min(max(top >> 7, 1u), 253u);
+    const float f = __uint_as_float((254u - ex) << 23);     // 2^(127 - ex)
+    uint32_t s[4];
+    float ss = 0.f;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const float2 x = unpack_bf16(w[e]);
+      s[e] = pack_bf16(x.x * f, x.y * f);
+      const float2 y = unpack_bf16(s[e]);
+      ss = fmaf(y.x, y.x, ss);
+      ss = fmaf(y.y, y.y, ss);
+    }
+#pragma unroll
+    for (int off = 1; off < 8; off <<= 1) ss += __shfl_xor_sync(lanes, ss, off);
+    if (row >= n_rows) continue;
+    *reinterpret_cast<uint4*>((is_q ? qs : ks) + row * D + part * 8) = make_uint4(s[0], s[1], s[2], s[3]);
+    if (part != 0) continue;
+    (is_q ? fq : fk)[row] = f;
+    if (!is_q) rk[row] = inv_or_zero(ss);
+  }
+}
+
 template <int MODE, int G, int NS>
 bool launch_bwd(const CUtensorMap& x1, const CUtensorMap& x2, const CUtensorMap& y1, const CUtensorMap& y2, const BArgs& a, LaunchCtx& ctx) {
   auto kern = tc_bwd_kernel<MODE, G, NS>;
@@ -811,13 +871,29 @@ bool launch_bwd(const CUtensorMap& x1, const CUtensorMap& x2, const CUtensorMap&
   return true;
 }
 
+// Scratch: r, the row scalars, and with three terms the scaled rows and their powers of two.
+struct BwdScratch {
+  float* rk;                  // [BH][T]
+  float* stats;               // [BH][T][2]
+  __nv_bfloat16 *qs, *ks;     // [BH][T][64]
+  float *fq, *fk;             // [BH][T]
+};
+
 // r, then dq and the row scalars, then dk and dv (which read the scalars)
 template <int G, int NS>
-void run_bwd(const Problem& p, const void* dout, void* dq, void* dk, void* dv, float* rk, float* stats, int* device_status, LaunchCtx& ctx) {
+void run_bwd(Problem p, const void* dout, void* dq, void* dk, void* dv, const BwdScratch& w, int* device_status, LaunchCtx& ctx) {
   const int BH = p.B * p.H;
   const size_t rows = (size_t)BH * p.T;
   constexpr int NT = Geo<MODE_DQ, G, NS>::NT;
-  bwd_rscale_kernel<<<(unsigned)((rows + 31) / 32), 256, 0, ctx.stream>>>(static_cast<const __nv_bfloat16*>(p.k), rk, rows);
+  const __nv_bfloat16 *q = static_cast<const __nv_bfloat16*>(p.q), *k = static_cast<const __nv_bfloat16*>(p.k);
+  const unsigned blocks = (unsigned)((rows + 31) / 32);
+  if (NS == 3) {
+    bwd_scale_kernel<<<dim3((blocks + SCALE_ROWS - 1) / SCALE_ROWS, 2), 256, 0, ctx.stream>>>(k, q, w.ks, w.qs, w.fk, w.fq, w.rk, rows);
+    p.q = w.qs;
+    p.k = w.ks;
+  } else {
+    bwd_rscale_kernel<<<blocks, 256, 0, ctx.stream>>>(k, w.rk, rows);
+  }
   note_launch(ctx);
   CUtensorMap qf, gf, kf, vf, qs, gs, ks, vs;     // fixed tiles of 128 rows, streamed tiles of NT
   if (!make_tile_map(&qf, p.q, BH, p.T, MT) || !make_tile_map(&gf, dout, BH, p.T, MT) || !make_tile_map(&kf, p.k, BH, p.T, MT) ||
@@ -826,9 +902,9 @@ void run_bwd(const Problem& p, const void* dout, void* dq, void* dk, void* dv, f
     ctx.status = KATA_ERR_CUDA;
     return;
   }
-  BArgs a{static_cast<__nv_bfloat16*>(dq), nullptr, stats, rk, device_status, p.T, BH};
+  BArgs a{static_cast<__nv_bfloat16*>(dq), nullptr, w.stats, w.rk, w.fq, device_status, p.T, BH};
   if (!launch_bwd<MODE_DQ, G, NS>(qf, gf, ks, vs, a, ctx)) return;
-  BArgs b{static_cast<__nv_bfloat16*>(dk), static_cast<__nv_bfloat16*>(dv), stats, rk, device_status, p.T, BH};
+  BArgs b{static_cast<__nv_bfloat16*>(dk), static_cast<__nv_bfloat16*>(dv), w.stats, w.rk, w.fk, device_status, p.T, BH};
   launch_bwd<MODE_DKV, G, NS>(kf, vf, qs, gs, b, ctx);
 }
 
@@ -844,24 +920,36 @@ size_t tc_bwd_workspace_bytes(const Problem& p) {
 void tc_bwd_quadratic(const Problem& p, const void* dout, void* dq, void* dk, void* dv, void* workspace, int* device_status,
                       LaunchCtx& ctx) {
   const size_t rows = (size_t)p.B * p.H * p.T;
-  float* rk = static_cast<float*>(workspace);
-  float* stats = reinterpret_cast<float*>(static_cast<unsigned char*>(workspace) + align256(rows * sizeof(float)));
-  if (p.groups == 1) run_bwd<1, 1>(p, dout, dq, dk, dv, rk, stats, device_status, ctx);
-  else if (p.groups == 2) run_bwd<2, 1>(p, dout, dq, dk, dv, rk, stats, device_status, ctx);
-  else run_bwd<4, 1>(p, dout, dq, dk, dv, rk, stats, device_status, ctx);
+  BwdScratch w{};
+  w.rk = static_cast<float*>(workspace);
+  w.stats = reinterpret_cast<float*>(static_cast<unsigned char*>(workspace) + align256(rows * sizeof(float)));
+  if (p.groups == 1) run_bwd<1, 1>(p, dout, dq, dk, dv, w, device_status, ctx);
+  else if (p.groups == 2) run_bwd<2, 1>(p, dout, dq, dk, dv, w, device_status, ctx);
+  else run_bwd<4, 1>(p, dout, dq, dk, dv, w, device_status, ctx);
 }
 
 // The gradients with fp32 weights (three bf16 terms): kata_bwd_chunked on sequences short enough for the quadratic form.
 size_t tc_bwd_exact_workspace_bytes(const Problem& p) {
   const size_t rows = (size_t)p.B * p.H * p.T;
-  return align256(rows * sizeof(float)) + align256(rows * 2 * sizeof(float));
+  return 3 * align256(rows * sizeof(float)) + align256(rows * 2 * sizeof(float)) + 2 * align256(rows * D * 2);
 }
 
 void tc_bwd_exact(const Problem& p, const void* dout, void* dq, void* dk, void* dv, void* workspace, int* device_status, LaunchCtx& ctx) {
   const size_t rows = (size_t)p.B * p.H * p.T;
-  float* rk = static_cast<float*>(workspace);
-  float* stats = reinterpret_cast<float*>(static_cast<unsigned char*>(workspace) + align256(rows * sizeof(float)));
-  run_bwd<1, 3>(p, dout, dq, dk, dv, rk, stats, device_status, ctx);
+  unsigned char* w8 = static_cast<unsigned char*>(workspace);
+  auto take = [&](size_t bytes) {
+    unsigned char* at = w8;
+    w8 += align256(bytes);
+    return at;
+  };
+  BwdScratch w{};
+  w.rk = reinterpret_cast<float*>(take(rows * sizeof(float)));
+  w.stats = reinterpret_cast<float*>(take(rows * 2 * sizeof(float)));
+  w.fq = reinterpret_cast<float*>(take(rows * sizeof(float)));
+  w.fk = reinterpret_cast<float*>(take(rows * sizeof(float)));
+  w.qs = reinterpret_cast<__nv_bfloat16*>(take(rows * D * 2));
+  w.ks = reinterpret_cast<__nv_bfloat16*>(take(rows * D * 2));
+  run_bwd<1, 3>(p, dout, dq, dk, dv, w, device_status, ctx);
 }
 
 }  // namespace kata

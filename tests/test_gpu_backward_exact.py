@@ -43,3 +43,25 @@ def test_backward_exact(T, zero):
             for what, x in (("tensor", got), ("plain", other)):
                 err = np.abs(to_numpy64(x[0, h]) - r)
                 assert np.all(err <= 2.0 ** -8 * np.abs(r) + 1e-5 * np.abs(r).max()), (name, what, T, float(err.max()))
+
+
+def test_rows_of_any_norm():
+    """Rows scaled by powers of two (exact in bf16) whose squared norms fp32 holds, though not their products: out does not
+    change, and the gradients are those of the unscaled rows divided by the powers, to the bit."""
+    import torch
+    T = 577
+    w = inputs.gaussian_workload("bwdx_norm", "bf16", 1, 2, T, 64, 64, 64, 6900)
+    q, k, v = dev_tensors(w)
+    g, _ = dout_for(w, 6)
+    k[0, 0, [0, 130]] = 0
+    q[0, 1, 7] = 0
+    base = kb.kata_bwd_chunked(q, k, v, g)
+    gen = torch.Generator(device="cuda").manual_seed(1)
+    for lo, hi in ((-55, -50), (40, 55), (-55, 55)):
+        fq, fk = (torch.exp2(torch.randint(lo, hi, (1, 2, T, 1), device="cuda", generator=gen).float()) for _ in range(2))
+        qs, ks = (q.float() * fq).bfloat16(), (k.float() * fk).bfloat16()
+        dq, dk, dv = kb.kata_bwd_chunked(qs, ks, v, g)
+        torch.cuda.synchronize()
+        assert kb.kata_last_impl() == kb.KATA_IMPL_TENSOR
+        for name, got, ref in (("dq", dq.float() * fq, base[0]), ("dk", dk.float() * fk, base[1]), ("dv", dv.float(), base[2])):
+            assert torch.equal(got, ref.float()), (name, lo, hi)
