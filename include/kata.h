@@ -188,8 +188,10 @@ int kata_fwd_quadratic(const void* q, const void* k, const void* v, void* out,
  * (bf16, feature_order 2) writes the state before every chunk of 512 or 1024 tokens to the workspace and then answers
  * blocks of 256 queries from that state and the keys of their chunk; sequences too short for that to pay run as one chunk,
  * which is the quadratic form.  fp32 rows of 16 or 32 entries without state pointers work the same way on plain FMAs (chunks
- * of 256).  The environment variable KATA_CHUNKED_KERNEL=stream selects the one-CTA-per-value-slice streaming kernel
- * instead on the tensor-core path (no workspace; for comparisons).
+ * of 256).  Less scratch than kata_workspace_bytes says, or none, is enough for the calls that kernels with less serve: with a
+ * state handed in or out (none; in place a copy of the normaliser state), fp32 rows without a state (none), inter_chunk = AUTO
+ * (the scan form's); they run on those kernels then.  The environment variable KATA_CHUNKED_KERNEL=stream selects the
+ * one-CTA-per-value-slice streaming kernel instead on the tensor-core path (no workspace; for comparisons).
  */
 int kata_fwd_chunked(const void* q, const void* k, const void* v, void* out,
                      int B, int H, int T, int d_k, int d_v, int C, const kata_opts* opts);

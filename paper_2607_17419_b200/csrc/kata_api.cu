@@ -353,8 +353,11 @@ Problem kernel_problem(const Prepared& r) {
   return pp;
 }
 
+// small_scratch: kernels that need less scratch, for a caller who brings less than kata_workspace_bytes says.  From 1: the
+// streaming kernels for a state handed in or out and for the scan form, the walk over the chunks in fp32 (no scratch, or that of
+// the scan passes), and chunks of 1024 tokens where shorter ones would be quicker.  2: the sequential form for AUTO as well.
 int prepare(int fn, const void* q, const void* k, const void* v, void* out, int B, int H, int T, int d_k,
-            int d_v, int C, const kata_opts* opts, bool need_ptrs, Prepared& r) {
+            int d_v, int C, const kata_opts* opts, bool need_ptrs, Prepared& r, int small_scratch = 0) {
   int st = read_opts(opts, r.o);
   if (st != KATA_OK) return st;
   st = check_shape(fn, B, H, T, d_k, d_v, C);
@@ -388,7 +391,7 @@ int prepare(int fn, const void* q, const void* k, const void* v, void* out, int 
     Opts scan = r.o;
     scan.inter_chunk = KATA_SCAN;
     r.o.inter_chunk = KATA_SEQUENTIAL;
-    if (C == kChunk && want_tensor(fn, kp, r.o) && want_tensor(fn, kp, scan) && tensor_scan_pays(B * H, (T + C - 1) / C)) {
+    if (small_scratch < 2 && C == kChunk && want_tensor(fn, kp, r.o) && want_tensor(fn, kp, scan) && tensor_scan_pays(B * H, (T + C - 1) / C)) {
       r.o.inter_chunk = KATA_SCAN;
       auto_scan = true;
     }
@@ -409,19 +412,19 @@ int prepare(int fn, const void* q, const void* k, const void* v, void* out, int 
     if (st != KATA_OK) return st;
     r.inner_bytes = inner_workspace(fn, r.plan, kp, r.state_elems);
     const bool state_in = r.o.s_init != nullptr, state_out = r.o.s_pre != nullptr;
-    r.simt_att = fn == KATA_FN_CHUNKED && !r.tensor && r.o.inter_chunk == KATA_SEQUENTIAL && !state_in && !state_out &&
+    r.simt_att = !small_scratch && fn == KATA_FN_CHUNKED && !r.tensor && r.o.inter_chunk == KATA_SEQUENTIAL && !state_in && !state_out &&
                  simt_attend_supported(r.p);
     if (r.simt_att) {
       r.inner_bytes = align_up(simt_attend_workspace_bytes(r.p));
       return KATA_OK;
     }
     r.states = fn == KATA_FN_CHUNKED && r.tensor && r.p.feature_order == 2 && !stream_kernel_forced() &&
-               ((r.o.inter_chunk == KATA_SEQUENTIAL && (!(state_in || state_out) || !short_state_call(B * H, T))) ||
-                (auto_scan && (long long)B * H * T >= kStreamScanTokens));
+               ((r.o.inter_chunk == KATA_SEQUENTIAL && (!(state_in || state_out) || (!small_scratch && !short_state_call(B * H, T)))) ||
+                (auto_scan && !small_scratch && (long long)B * H * T >= kStreamScanTokens));
     if (r.states) {
       r.pad = false;
       Problem sp = r.p;
-      r.sp = tc_chunk_plan(sp, state_in, state_out);
+      r.sp = tc_chunk_plan(sp, state_in, state_out, small_scratch > 0);
       r.inner_bytes = align_up(tc_chunk_workspace_bytes(sp, r.sp, state_in, state_out));
       if (r.p.groups == 1 && !state_in && !state_out) {
         const size_t least = published_chunked_bytes(B * H, T);
@@ -535,6 +538,10 @@ int entry(int fn, const void* q, const void* k, const void* v, void* out, int B,
   }
   Prepared r;
   int st = prepare(fn, q, k, v, out, B, H, T, d_k, d_v, C, opts, true, r);
+  for (int small = 1; small <= 2 && st == KATA_OK && r.inner_bytes > 0 &&
+                      (r.o.workspace == nullptr || r.o.workspace_bytes < r.inner_bytes ||
+                       (reinterpret_cast<uintptr_t>(r.o.workspace) & (kAlign - 1)) != 0); ++small)
+    st = prepare(fn, q, k, v, out, B, H, T, d_k, d_v, C, opts, true, r, small);
   if (st != KATA_OK) return st;
   if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(out)) return KATA_ERR_ALIGNMENT;
   if (r.o.s_pre != nullptr && (!aligned16(r.o.s_pre) || !aligned16(r.o.z_pre))) return KATA_ERR_ALIGNMENT;
@@ -822,6 +829,10 @@ int kata_fwd_host(int fn, const void* q_host, const void* k_host, const void* v_
   if (st != KATA_OK) return st;
   if (r.o.s_pre != nullptr && (!aligned16(r.o.s_pre) || !aligned16(r.o.z_pre))) return KATA_ERR_ALIGNMENT;
   if (r.o.s_init != nullptr && (!aligned16(r.o.s_init) || !aligned16(r.o.z_init))) return KATA_ERR_ALIGNMENT;
+  for (int small = 1; small <= 2 && r.o.workspace_bytes < staging_layout(r.p, r.inner_bytes).total; ++small) {
+    st = prepare(fn, q_host, k_host, v_host, out_host, B, H, T, d_k, d_v, C, opts, true, r, small);
+    if (st != KATA_OK) return st;
+  }
   const Staging s = staging_layout(r.p, r.inner_bytes);
   if (r.o.workspace == nullptr || r.o.workspace_bytes < s.total) return KATA_ERR_WORKSPACE_TOO_SMALL;
   if ((reinterpret_cast<uintptr_t>(r.o.workspace) & (kAlign - 1)) != 0) return KATA_ERR_ALIGNMENT;

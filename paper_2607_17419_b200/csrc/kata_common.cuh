@@ -192,7 +192,7 @@ void tc_attend(const Problem& p, const KeyScales& r, const AttendStates& st, int
 void tc_chunked_stream(const Problem& p, int* device_status, LaunchCtx& ctx);
 // Chunked form on the chunk-state and attend kernels (kata_tc_chunked.cu).  n_chunks = 1 without state pointers: the
 // quadratic form alone.
-StatePlan tc_chunk_plan(const Problem& p, bool state_in, bool state_out);
+StatePlan tc_chunk_plan(const Problem& p, bool state_in, bool state_out, bool small_scratch);
 size_t tc_chunk_workspace_bytes(const Problem& p, const StatePlan& plan, bool state_in, bool state_out);
 void tc_chunked_states(const Problem& p, const StatePlan& plan, void* workspace, int* device_status, const float* s_init,
                        const float* z_init, float* s_final, float* z_final, int state_layout, LaunchCtx& ctx);

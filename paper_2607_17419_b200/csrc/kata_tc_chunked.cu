@@ -43,13 +43,13 @@ ChunkBuffers chunk_buffers(const Problem& p, const StatePlan& plan, bool states)
 // Chunks of 1024: 16 heads x 131072 tokens 2.08 ms; 768: 2.10, 512: 2.17, 2048 about 2.3 (shorter chunks write and read more state, longer
 // ones have more key tiles).  Halved where even one chunk per CTA leaves SMs idle (3 heads x 2048 tokens with the state
 // handed out: 43 -> 38 us).
-StatePlan tc_chunk_plan(const Problem& p, bool state_in, bool state_out) {
+StatePlan tc_chunk_plan(const Problem& p, bool state_in, bool state_out, bool small_scratch) {
   const int BH = p.B * p.H, slices = tc_state_rows(p) / 256;
   const int quad_tokens = tc_narrow(p) ? (BH < 64 ? 4352 : 3584) : p.groups == 1 ? 7168 : p.groups == 2 ? 3072 : 1536;
   StatePlan plan{};
   int L = 1024;
   if (!state_in && !state_out && p.T <= quad_tokens) L = (p.T + 255) / 256 * 256;
-  else if ((long long)BH * slices * ((p.T + L - 1) / L) < 148) L = 512;
+  else if (!small_scratch && (long long)BH * slices * ((p.T + L - 1) / L) < 148) L = 512;
   plan.chunk_tokens = L;
   plan.n_chunks = (p.T + L - 1) / L;
   const int walk = state_out ? plan.n_chunks : plan.n_chunks - 1;
