@@ -130,7 +130,7 @@ enum { KATA_FN_QUADRATIC = 0, KATA_FN_CHUNKED = 1, KATA_FN_CHUNK_STATE_SCAN = 2,
  *                 waits on other CTAs are bounded (2 s); a CTA that gives up marks its group so that the
  *                 CTAs behind it give up at once.
  *  workspace      device scratch of at least kata_workspace_bytes(...) bytes, 256-byte aligned;
- *                 may be null when that size is 0.
+ *                 may be null when that size is 0.  Calls that may overlap on the GPU need a workspace each.
  *  s_pre, z_pre   optional device outputs (fp32), both null or both non-null.
  *                 kata_chunk_state_scan: s_pre [B,H,N_C,n_psi,d_v], z_pre [B,H,N_C,n_psi], N_C = ceil(T/C),
  *                 the exclusive prefix chunk states, entry 0 along N_C being zero.

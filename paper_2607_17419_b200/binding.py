@@ -7,9 +7,11 @@ fails, an exception is raised.
 """
 from __future__ import annotations
 
+import collections
 import ctypes
 import functools
 import os
+import threading
 from typing import Optional
 
 import torch
@@ -137,14 +139,23 @@ def _scratch_bytes(fn: int, B, H, T, d_k, d_v, C, dtype, order, layout, inter, i
     return kata_workspace_bytes(fn, B, H, T, d_k, d_v, C, o)
 
 
-def _scratch(ws, fn: int, sizes, o: KataOpts, device) -> None:
-    """Point the options at scratch of the size the call needs."""
+def _scratch(ws, fn: int, sizes, o: KataOpts, device):
+    """Point the options at scratch of the size the call needs; the caller holds what is returned until the call is made."""
     need = _scratch_bytes(fn, *sizes, o.dtype, o.feature_order, o.state_layout, o.inter_chunk, o.impl, o.scan_group,
                           o.feature_groups, bool(o.s_init or o.z_init), bool(o.s_pre or o.z_pre),
                           o.z_init is not None and o.z_init == o.z_pre)
-    ptr, size = (ws if ws is not None else _default_ws).get(need, device)
-    if size:
-        o.workspace, o.workspace_bytes = ptr, size
+    if ws is not None:
+        ptr, size = ws.get(need, device)
+        if size:
+            o.workspace, o.workspace_bytes = ptr, size
+        return ws
+    if need == 0:
+        return None
+    held = _default_scratch.bufs.get((device.index, o.stream))
+    if held is None or held[2] < need or torch._C._cuda_isCurrentStreamCapturing():
+        held = _default_scratch.new(need, device, o.stream)
+    o.workspace, o.workspace_bytes = held[1], held[2]
+    return held
 
 
 def kata_scan_plan(fn: int, B, H, T, d_k, d_v, C, opts: KataOpts):
@@ -228,7 +239,34 @@ class Workspace:
         return buf.data_ptr(), buf.numel()
 
 
-_default_ws = Workspace()
+class _StreamScratch(threading.local):
+    """Scratch of the calls that bring no Workspace: a buffer per thread, device and stream, so that calls on different
+    streams or threads never share one.  The buffers belong to their streams in torch's allocator (one that is replaced is
+    used again behind the calls that still read it), the oldest of more than KEEP goes back to it, and all of a thread's go
+    with the thread.  A call under graph capture gets a buffer of its own from the graph's pool (a capture that torch did not
+    begin has no pool: bring a Workspace)."""
+
+    KEEP = 16
+
+    def __init__(self):
+        self.bufs = {}                  # (device index, stream) -> (buffer, its address, its size)
+
+    def new(self, nbytes: int, device, stream: Optional[int]):
+        if (stream or 0) == _stream(device):
+            buf = torch.empty(nbytes, dtype=torch.uint8, device=device)
+        else:
+            with torch.cuda.stream(torch.cuda.ExternalStream(stream or 0, device=device)):
+                buf = torch.empty(nbytes, dtype=torch.uint8, device=device)
+        held = (buf, buf.data_ptr(), nbytes)
+        if not torch.cuda.is_current_stream_capturing():
+            self.bufs.pop((device.index, stream), None)
+            self.bufs[device.index, stream] = held
+            if len(self.bufs) > self.KEEP:
+                del self.bufs[next(iter(self.bufs))]
+        return held
+
+
+_default_scratch = _StreamScratch()
 
 
 def _call(fn: int, q, k, v, out, C: int, *, host_io: bool = False, workspace: Optional[Workspace] = None,
@@ -248,7 +286,7 @@ def _call(fn: int, q, k, v, out, C: int, *, host_io: bool = False, workspace: Op
                      s_init=s_init.data_ptr() if s_init is not None else 0,
                      z_init=z_init.data_ptr() if z_init is not None else 0,
                      device_status=device_status.data_ptr() if device_status is not None else 0, **opt_kw)
-    _scratch(workspace, fn | (KATA_FN_HOST_IO if host_io else 0), (B, H, T, d_k, d_v, C), opts, dev)
+    held = _scratch(workspace, fn | (KATA_FN_HOST_IO if host_io else 0), (B, H, T, d_k, d_v, C), opts, dev)
     args = (q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(), B, H, T, d_k, d_v, C, ctypes.byref(opts))
     if host_io:
         st = lib().kata_fwd_host(fn, *args)
@@ -309,7 +347,7 @@ def kata_decode_step(q, k, v, S, Z, out=None, *, workspace: Optional[Workspace] 
     n_psi = decode_n_psi(d_k, opts.feature_order, opts.state_layout, opts.feature_groups)
     if S.shape != (B, H, n_psi, d_v) or Z.shape != (B, H, n_psi):
         raise ValueError(f"state shapes must be {(B, H, n_psi, d_v)} and {(B, H, n_psi)}")
-    _scratch(workspace, KATA_FN_DECODE_STEP, (B, H, 1, d_k, d_v, 0), opts, q.device)
+    held = _scratch(workspace, KATA_FN_DECODE_STEP, (B, H, 1, d_k, d_v, 0), opts, q.device)
     st = lib().kata_decode_step(q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(), S.data_ptr(), Z.data_ptr(),
                                 B, H, d_k, d_v, ctypes.byref(opts))
     if st != 0:
@@ -331,7 +369,7 @@ def kata_bwd_quadratic(q, k, v, dout, dq=None, dk=None, dv=None, *, workspace: O
     if stream is None:
         stream = _stream(q.device)
     opts = make_opts(_dtype_code(q), stream=stream, **opt_kw)
-    _scratch(workspace, KATA_FN_BWD_QUADRATIC, (B, H, T, d_k, d_v, 0), opts, q.device)
+    held = _scratch(workspace, KATA_FN_BWD_QUADRATIC, (B, H, T, d_k, d_v, 0), opts, q.device)
     st = lib().kata_bwd_quadratic(q.data_ptr(), k.data_ptr(), v.data_ptr(), dout.data_ptr(), dq.data_ptr(),
                                   dk.data_ptr(), dv.data_ptr(), B, H, T, d_k, d_v, ctypes.byref(opts))
     if st != 0:
@@ -353,7 +391,7 @@ def kata_bwd_chunked(q, k, v, dout, dq=None, dk=None, dv=None, C: int = 64, *, w
     if stream is None:
         stream = _stream(q.device)
     opts = make_opts(_dtype_code(q), stream=stream, **opt_kw)
-    _scratch(workspace, KATA_FN_BWD_CHUNKED, (B, H, T, d_k, d_v, C), opts, q.device)
+    held = _scratch(workspace, KATA_FN_BWD_CHUNKED, (B, H, T, d_k, d_v, C), opts, q.device)
     st = lib().kata_bwd_chunked(q.data_ptr(), k.data_ptr(), v.data_ptr(), dout.data_ptr(), dq.data_ptr(),
                                 dk.data_ptr(), dv.data_ptr(), B, H, T, d_k, d_v, C, ctypes.byref(opts))
     if st != 0:
