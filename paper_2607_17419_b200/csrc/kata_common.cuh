@@ -1,6 +1,7 @@
 // Shared device/host helpers of the KATA kernels (element-type access, status plumbing).
 #pragma once
 
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -72,16 +73,37 @@ inline int sm_count() {
   const int v = device_fact(cudaDevAttrMultiProcessorCount, known);
   return v > 0 ? v : 148;
 }
-// Lets kernel K use `bytes` of dynamic shared memory on the current device (set once per kernel and device).
+// Number of the current context, never given twice in a process; 0: unknown.
+inline unsigned long long context_id() {
+  typedef CUresult (*GetId)(CUcontext, unsigned long long*);
+  static const GetId fn = []() -> GetId {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPoint("cuCtxGetId", &p, cudaEnableDefault, &q) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    return reinterpret_cast<GetId>(p);
+  }();
+  unsigned long long id = 0;
+  return fn != nullptr && fn(nullptr, &id) == CUDA_SUCCESS ? id : 0;
+}
+// Lets kernel K use `bytes` (always the same) of dynamic shared memory.  The setting is the context's: remembered with its number,
+// so that a context made after another was destroyed, or made current in its place, gets it too.
 template <auto K> bool allow_smem(int bytes) {
-  static std::atomic<int> set[kMaxDevices];
+  static std::atomic<unsigned long long> set[kMaxDevices];
   const int dev = device_ordinal();
-  if (dev >= 0 && dev < kMaxDevices && set[dev].load(std::memory_order_acquire) == bytes) return true;
+  const bool known = dev >= 0 && dev < kMaxDevices;
+  unsigned long long ctx = known ? context_id() : 0;
+  if (ctx != 0 && set[dev].load(std::memory_order_acquire) == ctx) return true;
   if (cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  if (dev >= 0 && dev < kMaxDevices) set[dev].store(bytes, std::memory_order_release);
+  if (known) {
+    if (ctx == 0) ctx = context_id();          // (the call above made it)
+    set[dev].store(ctx, std::memory_order_release);
+  }
   return true;
 }
 
