@@ -151,9 +151,10 @@ def _scratch(ws, fn: int, sizes, o: KataOpts, device):
         return ws
     if need == 0:
         return None
-    held = _default_scratch.bufs.get((device.index, o.stream))
-    if held is None or held[2] < need or torch._C._cuda_isCurrentStreamCapturing():
-        held = _default_scratch.new(need, device, o.stream)
+    stream = o.stream                   # (None: the legacy default stream, which cannot be captured)
+    held = _default_scratch.bufs.get((device.index, stream))
+    if held is None or held[2] < need or (stream is not None and torch._C._cuda_isCurrentStreamCapturing()):
+        held = _default_scratch.new(need, device, stream)
     o.workspace, o.workspace_bytes = held[1], held[2]
     return held
 
