@@ -112,7 +112,7 @@ enum { KATA_FN_QUADRATIC = 0, KATA_FN_CHUNKED = 1, KATA_FN_CHUNK_STATE_SCAN = 2,
  *                 sequence is long enough for the scan form's extra pass to pay (a model of the
  *                 streaming kernels' time in whole waves of CTAs decides; from 16384 tokens x heads on the chunk-state
  *                 kernels then cut the chunk axis into segments of their own instead of running the scan form's
- *                 passes); SEQUENTIAL otherwise,
+ *                 passes, unless scan_group is set); SEQUENTIAL otherwise,
  *                 on the fp32 kernels, for feature_order 1 (whose tensor-core path makes this choice
  *                 by itself) and whenever a state is handed in or out.  Both forms give the same
  *                 result up to the rounding order of the state sums.

@@ -420,7 +420,7 @@ int prepare(int fn, const void* q, const void* k, const void* v, void* out, int 
     }
     r.states = fn == KATA_FN_CHUNKED && r.tensor && r.p.feature_order == 2 && !stream_kernel_forced() &&
                ((r.o.inter_chunk == KATA_SEQUENTIAL && (!(state_in || state_out) || (!small_scratch && !short_state_call(B * H, T)))) ||
-                (auto_scan && !small_scratch && (long long)B * H * T >= kStreamScanTokens));
+                (auto_scan && !small_scratch && r.o.scan_group == 0 && (long long)B * H * T >= kStreamScanTokens));
     if (r.states) {
       r.pad = false;
       Problem sp = r.p;

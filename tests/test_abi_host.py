@@ -112,8 +112,8 @@ def test_scan_workspace_and_plan(L):
     assert kb.kata_workspace_bytes(kb.KATA_FN_QUADRATIC, 4, 16, 4096, 64, 64, 64, o) == 4 * 16 * 4096 * 2
     o32 = kb.make_opts(kb.KATA_F32)
     assert kb.kata_workspace_bytes(kb.KATA_FN_QUADRATIC, 4, 16, 4096, 64, 64, 64, o32) == 0
-    # sequential walk of the feature-split kernel: tile counters and the ticket, the scaled values and key scales of
-    # the pre-pass, nine shares of 17 KB per head and tile of 128 tokens
+    # sequential form: the published need (sized for nine shares of 17 KB per head and tile of 128 tokens, scaled values, key
+    # scales and counters), which the chunk states stay under at this size
     al = lambda x: (x + 255) // 256 * 256
     BH, T, nt = 8 * 16, 4096, 32
     assert kb.kata_workspace_bytes(kb.KATA_FN_CHUNKED, 8, 16, 4096, 64, 64, 64, o) == \
@@ -153,6 +153,11 @@ def test_inter_chunk_auto_and_tensor_groups(L):
     bad = kb.make_opts(kb.KATA_BF16, inter_chunk=3)
     with pytest.raises(kb.KataError):
         plan(1, 1, 1024, bad)
+    # a group size that is asked for is kept under AUTO too: the scan form's passes, with their scratch
+    for T in (8192, 32768, 131072):
+        sized = [kb.kata_workspace_bytes(kb.KATA_FN_CHUNKED, 1, 1, T, 64, 64, 64, kb.make_opts(kb.KATA_BF16, inter_chunk=mode, scan_group=24))
+                 for mode in (kb.KATA_INTER_AUTO, kb.KATA_SCAN)]
+        assert sized[0] == sized[1] > 0, T
     # explicit scan form on the tensor cores: groups of whole 128-token tiles, the last pass in whole waves
     scan = kb.make_opts(kb.KATA_BF16, inter_chunk=kb.KATA_SCAN)
     ng, g, _ = plan(1, 16, 131072, scan)
