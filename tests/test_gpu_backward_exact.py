@@ -65,3 +65,43 @@ def test_rows_of_any_norm():
         assert kb.kata_last_impl() == kb.KATA_IMPL_TENSOR
         for name, got, ref in (("dq", dq.float() * fq, base[0]), ("dk", dk.float() * fk, base[1]), ("dv", dv.float(), base[2])):
             assert torch.equal(got, ref.float()), (name, lo, hi)
+
+
+@pytest.mark.parametrize("B,H,T", [(8, 16, 513), (8, 16, 577), (3, 40, 700)])
+def test_many_heads(B, H, T):
+    """Several items per CTA of both kernels (five to six tiles of 128 rows per head and 120 or 128 heads: four to five items each):
+    the hand-over from one item to the next.  First, middle and last heads against the oracle, and the same bits every time."""
+    import torch
+    w = inputs.gaussian_workload(f"bwdx_heads_{B}_{H}_{T}", "bf16", B, H, T, 64, 64, 64, 6200 + T)
+    q, k, v = dev_tensors(w)
+    g = torch.from_numpy(inputs.normal(3, 8, B * H * T * 64).reshape(B, H, T, 64)).to(torch.bfloat16).cuda()
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    grads = kb.kata_bwd_chunked(q, k, v, g, device_status=st)
+    for _ in range(10):
+        assert all(torch.equal(a, b) for a, b in zip(grads, kb.kata_bwd_chunked(q, k, v, g, device_status=st)))
+    torch.cuda.synchronize()
+    assert kb.kata_last_impl() == kb.KATA_IMPL_TENSOR and int(st.item()) == 0
+    for b, h in ((0, 0), (B // 2, H // 3), (B - 1, H - 1)):
+        refs = ko.kata_quadratic_bwd(w.q_ref[b, h], w.k_ref[b, h], w.v_ref[b, h], to_numpy64(g[b, h]))
+        for name, got, r in zip(("dq", "dk", "dv"), grads, refs):
+            err = np.abs(to_numpy64(got[b, h]) - r)
+            assert np.all(err <= 2.0 ** -8 * np.abs(r) + 1e-5 * np.abs(r).max()), (name, b, h, float(err.max()))
+
+
+@pytest.mark.parametrize("T,impl", [(16384, "tensor"), (16385, "simt"), (511, "simt"), (512, "tensor")])
+def test_ends_of_the_range(T, impl):
+    """The last length of either route and the first of the other, sampled rows (dq row by row; dk and dv with every query
+    behind the key) to the same bound."""
+    import torch
+    w = inputs.gaussian_workload(f"bwdx_end_{T}", "bf16", 1, 1, T, 64, 64, 64, 6300 + T)
+    q, k, v = dev_tensors(w)
+    g, g_ref = dout_for(w, 7)
+    grads = kb.kata_bwd_chunked(q, k, v, g)
+    torch.cuda.synchronize()
+    assert kb.kata_last_impl() == (kb.KATA_IMPL_TENSOR if impl == "tensor" else kb.KATA_IMPL_SIMT)
+    rows = [0, 1, 127, 128, T // 2, T - 129, T - 2, T - 1]
+    refs = ko.kata_bwd_rows(w.q_ref[0, 0], w.k_ref[0, 0], w.v_ref[0, 0], g_ref[0, 0], rows, rows)
+    for name, got, r in zip(("dq", "dk", "dv"), grads, refs):
+        full = to_numpy64(got[0, 0])
+        err = np.abs(full[rows] - r)
+        assert np.all(err <= 2.0 ** -8 * np.abs(r) + 1e-5 * np.abs(full).max()), (name, T, float(err.max()))

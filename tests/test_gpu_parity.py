@@ -113,7 +113,7 @@ def test_inter_chunk_auto_takes_the_scan_form_for_one_long_head():
     q, k, v = dev_tensors(w)
     o = kb.kata_fwd_chunked(q, k, v, inter_chunk=kb.KATA_INTER_AUTO)
     torch.cuda.synchronize()
-    # the sequential walk of the feature-split kernel: the key-scale pre-pass and the kernel
+    # the sequential form, one chunk at this length: the key-scale pre-pass and the attend kernel
     assert kb.kata_last_launch_count() == 2
     for (b, h), r in oracle_full(w, heads=[(0, 3)]).items():
         check(to_numpy64(o)[b, h], r, "bf16", "auto -> sequential")

@@ -1,5 +1,5 @@
-"""GPU parity of the fp32 chunked form on narrow rows (chunk states of 256 tokens, blocks of 64 queries, tiles of 32 keys):
-edges of the blocks, of the chunks and of the lengths that run as one chunk."""
+"""GPU parity of the fp32 chunked form on narrow rows (chunk states of 256 tokens, blocks of 32 or 64 queries, tiles of 32
+keys): edges of the blocks, of the chunks and of the lengths that run as one chunk."""
 import pytest
 
 from paper_2607_17419_b200 import binding as kb
@@ -40,3 +40,22 @@ def test_queries_of_any_norm(dk, T, scale):
     torch.cuda.synchronize()
     for (b, h), r in oracle_full(w).items():
         check(to_numpy64(o)[b, h], r, "f32", f"T={T} d={dk} scale {scale} head {h}")
+
+
+@pytest.mark.parametrize("dk,dv", [(16, 16), (16, 32), (32, 16), (32, 32)])
+@pytest.mark.parametrize("T", [65, 511, 513, 1025, 1537, 2049])
+def test_two_queries_per_lane(dk, dv, T):
+    """Enough heads that blocks of 64 queries outnumber the SMs: two queries per lane, with one chunk and with several."""
+    import torch
+    H = 80
+    assert (T + 63) // 64 * H > 148
+    w = inputs.gaussian_workload(f"sa2_{dk}_{dv}_{T}", "f32", 1, H, T, dk, dv, 64, 7200 + T + dk)
+    q, k, v = dev_tensors(w)
+    o = kb.kata_fwd_chunked(q, k, v)
+    torch.cuda.synchronize()
+    assert kb.kata_last_impl() == kb.KATA_IMPL_SIMT
+    one_chunk = 1536 if dk == 32 else 1024 if H * T <= 16384 else 512
+    assert kb.kata_last_launch_count() == (3 if T > one_chunk else 1)
+    assert torch.equal(o, kb.kata_fwd_chunked(q, k, v)), "fixed summation order"
+    for (b, h), r in oracle_full(w, heads=[(0, 0), (0, H // 2), (0, H - 1)]).items():
+        check(to_numpy64(o[b, h]), r, "f32", f"T={T} d={dk},{dv} head {h}")
