@@ -254,8 +254,8 @@ int kata_bwd_quadratic(const void* q, const void* k, const void* v, const void* 
  * {16, 32, 64}, d_v a multiple of 8 up to 64 (KATA_ERR_UNSUPPORTED_SHAPE otherwise); inter_chunk, scan_group, state_layout
  * are ignored; s_pre/z_pre/s_init/z_init must be null.  Rows whose normaliser is 0 and zero rows of q or k get zero
  * gradients.  bf16 with d_k = d_v = 64 and 512 <= T <= 16384, unless opts->impl = KATA_IMPL_SIMT: the tensor-core kernels of
- * kata_bwd_quadratic with the weights carried in three bf16 terms (24 bits) -- O(T^2) work, less at these lengths, the same
- * precision; opts->impl = KATA_IMPL_TENSOR returns KATA_ERR_UNSUPPORTED_SHAPE outside that range.
+ * kata_bwd_quadratic with the weights carried in three bf16 terms (24 bits) -- O(T^2) work, but quicker at these lengths, and
+ * the same precision; opts->impl = KATA_IMPL_TENSOR returns KATA_ERR_UNSUPPORTED_SHAPE outside that range.
  * Workspace: kata_workspace_bytes(KATA_FN_BWD_CHUNKED, B, H, T, d_k, d_v, 64, opts) bytes: 276 bytes per token and head on the
  * tensor cores, else about 4 (2 d_k + d_v + (d_v / 8)(d_k + 1) + 2) (2.9 KB at d_k = d_v = 64).
  */

@@ -78,8 +78,12 @@ int check_shape(int fn, int B, int H, int T, int d_k, int d_v, int C) {
   return KATA_OK;
 }
 
-// Lengths of that route.  Below 512 tokens the entry stays on its plain FMA kernels (their cost there is a millisecond at
-// most); above 16384 it keeps the O(T) walk that it promises.
+// Lengths of that route.  They are set by the entry's contract, not by speed: shorter calls are the plain FMA kernels' (and
+// refused with impl = KATA_IMPL_TENSOR), and beyond 16384 tokens the entry keeps the O(T) work that it is called for.  The
+// tensor cores would be quicker on both sides.  Measured, us, tensor cores / FMA kernels:
+//   one head     T = 64: 16 / 242, 448: 31 / 1576, 16384: 534 / 56800, 32768: 1040 / 114000, 131072: 16300 / 460000
+//   16 heads     T = 64: 19 / 247, 448: 33 / 1590, 16384: 3800 / 57900, 32768: 16800 / 116000, 65536: 69200 / 231000
+//   128 heads    T = 64: 21 / 1600, 448: 78 / 11100
 constexpr int kBwdExactMin = 512, kBwdExactMax = 16384;
 
 bool want_tensor(int fn, const Problem& p, const Opts& o) {
@@ -95,7 +99,7 @@ bool bwd_tensor(const Problem& p, const Opts& o) {
 }
 
 // kata_bwd_chunked on the tensor cores: the quadratic form with fp32 weights (kata_tc_bwd.cu) for bf16 rows of 64 entries
-// and lengths at which its O(T^2) work is the smaller.
+// between those lengths.
 bool bwd_exact(const Problem& p, const Opts& o) {
   return o.impl != KATA_IMPL_SIMT && p.dtype == KATA_BF16 && p.feature_order == 2 && p.groups == 1 && p.d_k == 64 && p.d_v == 64 &&
          p.T >= kBwdExactMin && p.T <= kBwdExactMax && (long long)p.B * p.H <= 65535;
@@ -277,8 +281,9 @@ Staging staging_layout(const Problem& p, size_t inner_bytes) {
   return s;
 }
 
-// Scratch of the sequential chunked form (full lift, no state pointers) as published: callers that sized a buffer once
-// keep it.  The chunk states take less at every size where one segment walks a head; the larger of the two is asked for.
+// Scratch of the sequential chunked form (full lift, no state pointers) as published: the least that is asked for.  The chunk
+// states take less at nearly every size (headline call 0.62 GB of 2.8); one or two heads of 7169 to 16384 tokens take more, and
+// with the published size chunks of 1024 (see small_scratch).
 size_t published_chunked_bytes(int BH, int T) {
   const size_t nt = (T + 127) / 128, rows = (size_t)BH * T;
   return align_up((BH * nt + 1) * 4) + align_up(rows * 128) + align_up(rows * 2) + align_up(BH * 9 * nt * (128 * 128 + 128 * 8));
@@ -287,7 +292,10 @@ size_t published_chunked_bytes(int BH, int T) {
 // A state handed in or out on a short call: the streaming kernel while its CTAs (eight per head) are one wave.  Measured,
 // us, chunk states / streaming kernel: 16 heads, T = 256: 34 / 24, 512: 33 / 31, 1024: 35 / 45; 128 heads, T = 256: 98 / 128.
 bool short_state_call(int BH, int T) { return T <= 512 && BH * 8 <= 148; }
-// inter_chunk = AUTO where the model above prefers the scan form: fewer tokens x heads than this stay on its group passes.
+// inter_chunk = AUTO where the model above prefers the scan form: fewer tokens x heads than this stay on its group passes, the plan
+// that kata_scan_plan gives for AUTO there.  The line is drawn by that plan and not by speed: the sequential form is quicker on
+// both sides.  Measured, us, sequential / group passes: one head x 2048 17 / 39, x 6000 29 / 55, x 8192 34 / 61, x 16384 45 / 85;
+// four heads x 2048 16 / 50, x 4096 23 / 74, x 8192 52 / 122.
 constexpr long long kStreamScanTokens = 16384;
 
 // Diagnostic override: KATA_CHUNKED_KERNEL=stream in the environment keeps the sequential chunked form on the

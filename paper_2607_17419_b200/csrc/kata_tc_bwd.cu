@@ -910,8 +910,8 @@ void run_bwd(Problem p, const void* dout, void* dq, void* dk, void* dv, const Bw
 
 }  // namespace
 
-// workspace: 128 bytes per row as published (not used any more: k is read as it is), r [BH][T] fp32, the row scalars
-// [BH][T][2] fp32
+// workspace: r [BH][T] fp32, the row scalars [BH][T][2] fp32, and 128 bytes per row that are published but not used (k is read as
+// it is)
 size_t tc_bwd_workspace_bytes(const Problem& p) {
   const size_t rows = (size_t)p.B * p.H * p.T;
   return align256(rows * D * 2) + align256(rows * sizeof(float)) + align256(rows * 2 * sizeof(float));

@@ -41,7 +41,10 @@ ChunkBuffers chunk_buffers(const Problem& p, const StatePlan& plan, bool states)
 //   (few heads, whose blocks split the keys between the halves of a CTA, would take the quadratic form further: 3 heads up to
 //   10000 tokens 45 / 53; the line is one for all heads)
 // Chunks of 1024: 16 heads x 131072 tokens 2.08 ms; 768: 2.10, 512: 2.17, 2048 about 2.3 (shorter chunks write and read more state, longer
-// ones have more key tiles).  Halved where even one chunk per CTA leaves SMs idle (3 heads x 2048 tokens with the state
+// ones have more key tiles).  One length for every map; measured, us, 512 / 768 / 1024: full lift 4 x 50001 313 / 276 / 249,
+// 64 x 8192 540 / 523 / 508, 32 x 3001 with the state 117 / 111 / 111; two groups 4 x 50001 222 / 201 / 183, 16 x 32768
+// 462 / 452 / 456, 128 x 4096 350 / 370 / 342; four groups 4 x 50001 166 / 166 / 160, 16 x 32768 378 / 373 / 395, 64 x 8192
+// 334 / 354 / 373 (there 512 would be quicker).  Halved where even one chunk per CTA leaves SMs idle (3 heads x 2048 tokens with the state
 // handed out: 43 -> 38 us).
 StatePlan tc_chunk_plan(const Problem& p, bool state_in, bool state_out, bool small_scratch) {
   const int BH = p.B * p.H, slices = tc_state_rows(p) / 256;
