@@ -47,9 +47,9 @@ def quadratic_flops(B, H, T, d=64, dv=64):
 
 
 def load_traffic(T: int):
-    """DRAM bytes per step of the two large kernels, scaled linearly in T from the ncu capture recorded beside its
-    summary under profiles/ (null if the record is missing)."""
-    path = os.path.join(ROOT, "profiles", "tc_chunk_kernels_c4_T32768_traffic.json")
+    """DRAM bytes per step of the two large kernels, from the ncu capture at T = 131072 recorded beside its summary under
+    profiles/ (scaled linearly for another T; null if the record is missing)."""
+    path = os.path.join(ROOT, "profiles", "tc_chunk_kernels_c4_T131072_traffic.json")
     if not os.path.exists(path):
         return None, "kata::tc_state_kernel + kata::tc_attend_kernel (tcgen05 chunk states and outputs)"
     with open(path) as f:
