@@ -25,6 +25,11 @@
 // entries (R = 4 runs of 8) the empty half of the features is left out: 12 block pairs instead of 36, two score steps
 // instead of four (8 heads x 16 x 6000 tokens of 32 entries 501 -> 312 us, 16 x 60000 828 -> 486).
 //
+// The issuers' descriptors are sums of a constant and a stage's offset, and what is checked once an item or a tile is checked
+// outside the loop over the sub-buffers: an issuer shares its scheduler with four builder warps, and every instruction of its
+// waits a few cycles for a slot (per sub-buffer of 64 keys a wait, 8 MMAs and a commit, some 370 cycles of which the pipe has
+// use for 288; 64 heads x 4096 tokens 128.9 -> 124.1 us).
+//
 // What bounds it and why this split.  A key tile is 576 cycles of MMA per half (4 x N=128, 8 x N=80) and a chain
 // scores -> builders -> apply of about 1700, most of it hand-offs.  Four chains run side by side: two halves times two
 // sub-buffers of 64 score columns each.  Both halves share every key, value and state tile, which halves the tile
@@ -335,6 +340,9 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       const uint32_t ones = smem_u32(base + OFF_ONES), zcol = smem_u32(base + OFF_Z);
       // MN-major, 128B swizzle: 8 rows per 1024-byte atom (SBO), columns 64.. in the constant block (LBO)
       auto bdesc = [&](uint32_t addr, uint32_t extra) { return smem_desc(addr, extra - addr, 1024, kSwizzle128B); };
+      // ... moved by a number of bytes: the start address goes up and the distance to the constant block down
+      auto move = [](uint64_t desc, uint32_t bytes) { return desc + (uint64_t)(bytes >> 4) * (1ull - (1ull << 16)); };
+      const uint64_t dv0 = bdesc(smem_u32(stage(0)) + 16384, ones), dk0 = at(dk, smem_u32(stage(0)));
       uint32_t it = 0, cnt = 0, n_st = 0;   // tiles, key tiles of this half, its state tiles
       int n_done = 0;                       // items of this half so far
       Item w;
@@ -343,23 +351,21 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         const int nt = nk > 0 ? w.ns + nk : 0;      // tiles of this half
         uint32_t acc = 0;
         auto landed = [&](uint32_t g_it) { return wait_or_abort(bar(BAR_FULL + g_it % NSTAGE), (g_it / NSTAGE) & 1, abort_flag); };
-        auto o_free = [&]() { return acc != 0 || n_done == 0 || wait_or_abort(bar(BAR_OFREE + h), (n_done - 1) & 1, abort_flag); };
+        auto o_free = [&]() { return n_done == 0 || wait_or_abort(bar(BAR_OFREE + h), (n_done - 1) & 1, abort_flag); };
         auto open = [&](uint32_t g_it, int c) {
-          const uint32_t st = smem_u32(stage(g_it % NSTAGE));
+          const uint64_t d = dk0 + ((g_it % NSTAGE) * STAGE_BYTES + c * KH * 128) / 16;
 #pragma unroll
           for (int ks = 0; ks < R / 2; ++ks)   // 16 features per step; group ks / (4 / G) accumulates over its own steps
-            mma_f16_ts(tS + c * 64 + (ks / (4 / G)) * KH, tQ + ks * 8, at(dk, st + c * KH * 128 + ks * 32), id_s, (ks % (4 / G)) > 0);
+            mma_f16_ts(tS + c * 64 + (ks / (4 / G)) * KH, tQ + ks * 8, d + ks * 2, id_s, (ks % (4 / G)) > 0);
           mma_commit(bar(BAR_SFULL + 2 * h + c));
         };
         auto close = [&](uint32_t g_it, int c) -> bool {
-          if (!wait_or_abort(bar(BAR_PFULL + 2 * h + c), cnt & 1, abort_flag) || !o_free()) return false;
+          if (!wait_or_abort(bar(BAR_PFULL + 2 * h + c), cnt & 1, abort_flag)) return false;
           tc_fence_after();
-          const uint32_t va = smem_u32(stage(g_it % NSTAGE)) + 16384 + c * KH * 128;
+          const uint64_t d = move(dv0, (g_it % NSTAGE) * STAGE_BYTES + c * KH * 128);
 #pragma unroll
-          for (int ks = 0; ks < KH / 16; ++ks) {
-            mma_f16_ts(tO, tS + c * 64 + ks * 8, bdesc(va + ks * 2048, ones), id_p, acc);
-            acc = 1;
-          }
+          for (int ks = 0; ks < KH / 16; ++ks) mma_f16_ts(tO, tS + c * 64 + ks * 8, move(d, ks * 2048), id_p, ks > 0 ? 1u : acc);
+          acc = 1;
           return true;
         };
         if constexpr (SPLIT) {
@@ -378,6 +384,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
               tc_fence_after();
               open(it, 0);
               open(it, 1);
+              ok = o_free();
             }
             for (int j = 0; j < nk && ok; ++j, it += 2, ++cnt) {
               const bool next = j + 1 < nk;
@@ -401,8 +408,8 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
           if (w.ns > 0) {
 #pragma unroll 1
             for (int t = 0; t < NST && ok; ++t, ++it, ++n_st) {
-              ok = landed(it) && o_free() && (t + 1 < NST || landed(it + 1));
-              const uint32_t sa = smem_u32(stage(it % NSTAGE)), za = zcol + (it % NSTAGE) * 32;
+              ok = landed(it) && (t > 0 || o_free()) && (t + 1 < NST || landed(it + 1));
+              const uint64_t ds = bdesc(smem_u32(stage(it % NSTAGE)), zcol + (it % NSTAGE) * 32);
 #pragma unroll
               for (int c = 0; c < 2; ++c) {
 #pragma unroll
@@ -411,11 +418,9 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                   if (!ok) break;
                   tc_fence_after();
 #pragma unroll
-                  for (int ks = 0; ks < 4; ++ks) {
-                    const uint32_t blk = (c * 8 + pp * 4 + ks) * 2048;     // 16 rows
-                    mma_f16_ts(tO, tS + c * 64 + pp * 32 + ks * 8, bdesc(sa + blk, za + blk), id_p, acc);
-                    acc = 1;
-                  }
+                  for (int ks = 0; ks < 4; ++ks)             // 16 rows per 2 KB, of the state and of Z
+                    mma_f16_ts(tO, tS + c * 64 + pp * 32 + ks * 8, ds + (c * 8 + pp * 4 + ks) * 128, id_p, c + pp + ks > 0 ? 1u : acc);
+                  acc = 1;
                   mma_commit(bar(BAR_SFREE + 4 * h + 2 * c + pp));
                 }
                 if (!ok) break;
@@ -426,6 +431,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
           } else {
             open(it, 0);
             open(it, 1);
+            ok = o_free();
           }
         }
         for (int j = 0; j < nk && ok; ++j, ++it, ++cnt) {
@@ -626,36 +632,35 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         } else {
           const uint32_t rbase = smem_u32(base + OFF_RV) + s * 512 + ch * (XR ? 256 : 128);   // r of this warp's 64 keys, 16 bytes per load
           const int key0 = (w.k0 + kj) * KT + ch * 64;
-          uint32_t ya[32], yb[32], pk[16];
-          auto weigh = [&](const uint32_t (&y)[32], int col0, auto masked) {
-            constexpr int RPL = XR ? 4 : 8;                    // keys per load
-#pragma unroll
-            for (int i = 0; i < 32 / RPL; ++i) {
-              const uint4 t4 = lds128(rbase + (col0 / RPL + i) * 16);
-              const uint32_t rr[4] = {t4.x, t4.y, t4.z, t4.w};
-#pragma unroll
-              for (int e = 0; e < RPL; e += 2) {
-                const int jj = RPL * i + e;
-                const float2 sv = make_float2(__uint_as_float(y[jj]), __uint_as_float(y[jj + 1]));
-                float2 x = __fmul2_rn(sv, sv);
-                if constexpr (XR) x = __fmul2_rn(x, make_float2(__uint_as_float(rr[e]), __uint_as_float(rr[e + 1])));
-                if constexpr (decltype(masked)::value) {
-                  if (key0 + col0 + jj > qrow) x.x = 0.f;
-                  if (key0 + col0 + jj + 1 > qrow) x.y = 0.f;
-                }
-                pk[jj / 2] = XR ? pack_bf16(x.x, x.y) : mul_bf16x2(pack_bf16(x.x, x.y), rr[e / 2]);
-              }
-            }
-          };
+          // 32 columns at a time, each half behind a load of its own: a warp that runs through a hundred independent
+          // instructions holds its scheduler, and the issuers, whose few instructions the MMAs wait for, get their slots when
+          // it stalls (64 heads x 4096 tokens 124.1 -> 121.3 us; 16 columns at a time 123.4)
           auto weigh_tile = [&](auto masked) {
-            tmem_ld32(tS, ya);
-            tmem_ld32(tS + 32, yb);
-            tmem_wait_ld(ya);
-            tmem_wait_ld(yb);
-            weigh(ya, 0, masked);
-            tmem_st16(tS, pk);          // over this warp's own scores, which are in registers
-            weigh(yb, 32, masked);
-            tmem_st16(tS + 16, pk);
+            constexpr int CW = 32, RPL = XR ? 4 : 8;             // columns at a time, keys per load of r
+#pragma unroll
+            for (int c0 = 0; c0 < 64; c0 += CW) {
+              uint32_t y[CW], pk[CW / 2];
+              tmem_ld32(tS + c0, y);
+              tmem_wait_ld(y);
+#pragma unroll
+              for (int i = 0; i < CW / RPL; ++i) {
+                const uint4 t4 = lds128(rbase + (c0 / RPL + i) * 16);
+                const uint32_t rr[4] = {t4.x, t4.y, t4.z, t4.w};
+#pragma unroll
+                for (int e = 0; e < RPL; e += 2) {
+                  const int jj = RPL * i + e;
+                  const float2 sv = make_float2(__uint_as_float(y[jj]), __uint_as_float(y[jj + 1]));
+                  float2 x = __fmul2_rn(sv, sv);
+                  if constexpr (XR) x = __fmul2_rn(x, make_float2(__uint_as_float(rr[e]), __uint_as_float(rr[e + 1])));
+                  if constexpr (decltype(masked)::value) {
+                    if (key0 + c0 + jj > qrow) x.x = 0.f;
+                    if (key0 + c0 + jj + 1 > qrow) x.y = 0.f;
+                  }
+                  pk[jj / 2] = XR ? pack_bf16(x.x, x.y) : mul_bf16x2(pack_bf16(x.x, x.y), rr[e / 2]);
+                }
+              }
+              tmem_st16(tS + c0 / 2, pk);          // over scores that are in this warp's registers
+            }
           };
           if (diag) weigh_tile(std::true_type{}); else weigh_tile(std::false_type{});
         }
