@@ -1,5 +1,6 @@
-"""Thin ctypes binding over libkata.so (argument marshalling only; every step runs in the CUDA
-library).  Function names mirror the C ABI of include/kata.h.
+"""Thin binding over libkata.so (argument marshalling only; every step runs in the CUDA
+library).  Function names mirror the C ABI of include/kata.h.  The ordinary tensor call goes through a native module
+(csrc/kata_torch.cpp), every other one, and every error, through ctypes here.
 
 Tensors are torch CUDA tensors (or pinned host tensors for ``kata_fwd_host``); torch is used for
 device memory and streams only.  There is no CPU fallback: if the library is missing or a call
@@ -105,6 +106,22 @@ def lib() -> ctypes.CDLL:
     L.kata_selftest_wait_timeout.restype = i
     _lib = L
     return L
+
+
+_native = None
+
+
+def native():
+    """The native module with the tensor calls, or NotImplemented from it for a call that is left to this file (loaded once)."""
+    global _native
+    if _native is None:
+        lib()
+        try:
+            from . import _kata_torch
+        except ImportError as e:
+            raise RuntimeError(f"_kata_torch.so does not load ({e}): build it with `python -m paper_2607_17419_b200.build`") from e
+        _native = _kata_torch
+    return _native
 
 
 def status_string(status: int) -> str:
@@ -272,6 +289,12 @@ _default_scratch = _StreamScratch()
 
 def _call(fn: int, q, k, v, out, C: int, *, host_io: bool = False, workspace: Optional[Workspace] = None,
           s_pre=None, z_pre=None, s_init=None, z_init=None, device_status=None, stream=None, **opt_kw):
+    if workspace is None and stream is None and not host_io:
+        r = (_native or native()).forward(fn, _default_scratch, q, k, v, out, C, s_pre, z_pre, s_init, z_init, device_status, opt_kw)
+        if type(r) is int:
+            raise KataError(r, _FN_NAMES[fn])
+        if r is not NotImplemented:
+            return r
     if not (q.is_contiguous() and k.is_contiguous() and v.is_contiguous()):
         raise ValueError("q, k, v must be contiguous [B,H,T,d]")
     B, H, T, d_k = q.shape
@@ -334,6 +357,12 @@ def decode_n_psi(d_k: int, feature_order: int = 2, state_layout: int = KATA_LAYO
 def kata_decode_step(q, k, v, S, Z, out=None, *, workspace: Optional[Workspace] = None, stream=None, **opt_kw):
     """One decode token per (b,h): q,k [B,H,d_k], v [B,H,d_v]; fp32 state S [B,H,n_psi,d_v], Z [B,H,n_psi] is
     updated in place.  Returns out [B,H,d_v]."""
+    if workspace is None and stream is None:
+        r = (_native or native()).decode(_default_scratch, q, k, v, S, Z, out, opt_kw)
+        if type(r) is int:
+            raise KataError(r, "kata_decode_step")
+        if r is not NotImplemented:
+            return r
     B, H, d_k = q.shape
     d_v = v.shape[-1]
     if not (q.is_contiguous() and k.is_contiguous() and v.is_contiguous() and S.is_contiguous() and Z.is_contiguous()):
@@ -360,6 +389,12 @@ def kata_bwd_quadratic(q, k, v, dout, dq=None, dk=None, dv=None, *, workspace: O
                        stream=None, **opt_kw):
     """Gradients of sum(dout * out) with respect to q, k, v (q,k [B,H,T,d_k]; v,dout [B,H,T,d_v]); the forward
     is recomputed.  Returns (dq, dk, dv) in the dtype of the inputs."""
+    if workspace is None and stream is None:
+        r = (_native or native()).backward(KATA_FN_BWD_QUADRATIC, _default_scratch, q, k, v, dout, dq, dk, dv, 0, opt_kw)
+        if type(r) is int:
+            raise KataError(r, "kata_bwd_quadratic")
+        if r is not NotImplemented:
+            return r
     if not (q.is_contiguous() and k.is_contiguous() and v.is_contiguous() and dout.is_contiguous()):
         raise ValueError("q, k, v, dout must be contiguous [B,H,T,d]")
     B, H, T, d_k = q.shape
@@ -382,6 +417,12 @@ def kata_bwd_chunked(q, k, v, dout, dq=None, dk=None, dv=None, C: int = 64, *, w
                      stream=None, **opt_kw):
     """The same gradients as ``kata_bwd_quadratic`` by the O(T) two-pass linear-state backward.  Returns (dq, dk, dv)
     in the dtype of the inputs."""
+    if workspace is None and stream is None:
+        r = (_native or native()).backward(KATA_FN_BWD_CHUNKED, _default_scratch, q, k, v, dout, dq, dk, dv, C, opt_kw)
+        if type(r) is int:
+            raise KataError(r, "kata_bwd_chunked")
+        if r is not NotImplemented:
+            return r
     if not (q.is_contiguous() and k.is_contiguous() and v.is_contiguous() and dout.is_contiguous()):
         raise ValueError("q, k, v, dout must be contiguous [B,H,T,d]")
     B, H, T, d_k = q.shape

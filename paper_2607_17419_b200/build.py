@@ -8,6 +8,7 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libkata.so")
+HOST = os.path.join(HERE, "_kata_torch.so")      # the binding's tensor calls (csrc/kata_torch.cpp)
 SOURCES = ["kata_api.cu", "kata_simt_quadratic.cu", "kata_simt_bwd.cu", "kata_simt_bwd_chunked.cu", "kata_simt_chunked.cu", "kata_simt_order1.cu", "kata_simt_attend.cu", "kata_tc.cu", "kata_tc_chunked.cu",
     "kata_tc_stream.cu", "kata_tc_stream_export.cu", "kata_tc_stream_restart.cu", "kata_tc_stream_state.cu", "kata_tc_attend.cu", "kata_tc_state.cu", "kata_tc_bwd.cu", "kata_tc_order1.cu", "kata_decode.cu", "kata_static.cu", "kata_selftest.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -20,15 +21,34 @@ def _nvcc() -> str:
 
 
 def needs_build() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(HOST):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(HOST))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(HERE, "..", "include", "kata.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def _host_command(obj: str) -> list:
+    """Compiler call for the binding's native module."""
+    import sysconfig
+
+    import torch
+    inc = os.path.join(os.path.dirname(torch.__file__), "include")
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    return ["g++", "-O2", "-std=c++17", "-fPIC", "-fvisibility=hidden", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+            "-isystem", inc, "-isystem", os.path.join(inc, "torch", "csrc", "api", "include"), "-isystem", os.path.join(cuda, "include"),
+            "-isystem", sysconfig.get_path("include"), "-c", os.path.join(CSRC, "kata_torch.cpp"), "-o", obj]
+
+
+def _host_link(obj: str) -> list:
+    import torch
+    lib = os.path.join(os.path.dirname(torch.__file__), "lib")
+    return ["g++", "-shared", "-o", HOST, obj, "-L" + HERE, "-l:libkata.so", "-Wl,-rpath,$ORIGIN", "-L" + lib, "-lc10", "-lc10_cuda", "-ltorch_cpu",
+            "-ltorch_python"]
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile every .cu into objects (in parallel) and link libkata.so next to this file."""
+    """Compile every .cu into objects (in parallel) and link libkata.so next to this file, and the binding's native module."""
     if not force and not needs_build():
         return LIB
     objdir = os.path.join(HERE, "build")
@@ -43,6 +63,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
         if verbose:
             cmd.insert(1, "-Xptxas=-v")
         procs.append((src, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
+    host_obj = os.path.join(objdir, "kata_torch.host.o")
+    procs.append(("kata_torch.cpp", subprocess.Popen(_host_command(host_obj), stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
     failed = False
     for src, pr in procs:
         out, _ = pr.communicate()
@@ -52,6 +74,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if failed:
         raise RuntimeError("nvcc failed")
     subprocess.check_call([_nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-shared", "-o", LIB, *objs])
+    subprocess.check_call(_host_link(host_obj))
     return LIB
 
 
