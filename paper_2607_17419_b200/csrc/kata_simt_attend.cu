@@ -7,12 +7,18 @@
 //   attend_kernel        lane = one or two queries; the warps of a CTA share out the feature rows of the state and the tiles
 //                        of 32 keys, rows broadcast from shared memory (16 bytes per load feed 8 FMAs), and add their
 //                        numerators and normalisers in a fixed order at the end
+// Few blocks: a cluster of CTAs shares the keys and the rows of one block, in tiles of 8 keys (2 heads x 512 tokens of 16
+// entries: 32 blocks, whose warps walked 32 keys each, four to a scheduler, 8.9 us; as 128 CTAs 4.4).
 // What bounds it: FMAs.  The walk over the chunks of a head by one CTA (kata_simt_chunked.cu) was a chain of 21 us per 64
-// tokens: 2 heads x 512 tokens of 16 entries took 171 us, now 9; 16 x 16000 5378, now 242 (rows of 32: 12842, now 1197).
+// tokens: 2 heads x 512 tokens of 16 entries took 171 us, now 4.4; 16 x 16000 5378, now 242 (rows of 32: 12842, now 1197).
 // Chunk length: at 16 entries a query costs 34 FMAs per key of its chunk and 2.3 k for the state, at 32 66 and 17 k.
+#include <cooperative_groups.h>
+
 #include <type_traits>
 
 #include "kata_common.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace kata {
 namespace {
@@ -107,27 +113,34 @@ __global__ void __launch_bounds__(128) state_prefix_kernel(float4* __restrict__ 
   }
 }
 
-template <int DK, int DV, int NW, int QPL> constexpr int attend_smem_floats() {
+template <int DK, int DV, int NW, int QPL, int CL> __host__ __device__ constexpr int attend_smem_floats() {
   const int tiles = 32 * QPL * DK + NW * 32 * (DK + DV), red = NW * (DV + 1) * 32 * QPL;
-  return tiles > red ? tiles : red;
+  return (tiles > red ? tiles : red) + (CL > 1 ? CL * (DV + 1) * 32 * QPL : 0);
 }
 
 // QPL queries per lane (a block is 32 QPL queries); NW warps share out its key tiles and state rows.  (One query per lane: two
 // blocks per SM, rows of 32 with 132 registers lost the second and 16 heads x 512 tokens went from 27 to 33 us.)
-template <int DK, int DV, int NW, int QPL>
+// CL > 1: a cluster of CL CTAs does this for a block, in key tiles of TK, and adds its CTAs' sums in the shared memory of the
+// first.
+template <int DK, int DV, int NW, int QPL, int CL>
 __global__ void __launch_bounds__(NW * 32, DK == 32 && DV == 32 && QPL == 1 ? 2 : 0) attend_kernel(const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ v,
                                                          float* __restrict__ out, const float* __restrict__ S, int Tlen, int chunk,
                                                          int n_chunks) {
   constexpr int NF = n_features(DK), SP = state_stride(DV), QB = 32 * QPL;
-  extern __shared__ __align__(16) float sm[];
+  constexpr int TK = CL > 1 ? 8 : 32;                      // keys per tile
+  constexpr int GW = NW * CL;                              // warps that share a block
+  extern __shared__ __align__(16) float smem[];
+  float* sm = smem;
   float* qs = sm;                                          // [DK][QB]
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   float* kt = sm + QB * DK + warp * 32 * (DK + DV);        // this warp's tile: k_hat [32][DK], v [32][DV]
   float* vt = kt + 32 * DK;
-  const int q0 = ((int)gridDim.x - 1 - (int)blockIdx.x) * QB, bh = blockIdx.y;     // last blocks first
+  const int rank = CL > 1 ? (int)blockIdx.x % CL : 0, gw = rank * NW + warp;       // (a cluster is CL neighbours on x)
+  const int q0 = ((int)gridDim.x / CL - 1 - (int)blockIdx.x / CL) * QB, bh = blockIdx.y;     // last blocks first
   const float* kh = k + (size_t)bh * Tlen * DK;
   const float* vh = v + (size_t)bh * Tlen * DV;
   const float* qh = q + (size_t)bh * Tlen * DK;
+  if (CL > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");     // this CTA has started
   if (S != nullptr) cudaGridDependencySynchronize();
 
   for (int i = tid; i < QB * DK; i += NW * 32) {
@@ -169,7 +182,7 @@ __global__ void __launch_bounds__(NW * 32, DK == 32 && DV == 32 && QPL == 1 ? 2 
   const int c = q0 / chunk;
   if (c > 0) {
     const float* Sc = S + ((size_t)bh * n_chunks + c) * NF * SP;
-    const int f0 = NF * warp / NW, f1 = NF * (warp + 1) / NW;
+    const int f0 = NF * gw / GW, f1 = NF * (gw + 1) / GW;
     int a = 0, rem = f0;
     while (rem >= DK - a) {
       rem -= DK - a;
@@ -218,16 +231,16 @@ __global__ void __launch_bounds__(NW * 32, DK == 32 && DV == 32 && QPL == 1 ? 2 
       }
     }
   }
-  // ---- the keys of the chunk, tiles of 32 ----
+  // ---- the keys of the chunk ----
   const int k_end = min(q0 + QB, Tlen);
-  for (int t0 = c * chunk + warp * 32; t0 < k_end; t0 += NW * 32) {
+  for (int t0 = c * chunk + gw * TK; t0 < k_end; t0 += GW * TK) {
     __syncwarp();
-    load_rows<DK, true>(kh, kt, t0, 32, Tlen, lane, 32);
-    load_rows<DV, false>(vh, vt, t0, 32, Tlen, lane, 32);
+    load_rows<DK, true>(kh, kt, t0, TK, Tlen, lane, 32);
+    load_rows<DV, false>(vh, vt, t0, TK, Tlen, lane, 32);
     __syncwarp();
-    const bool diag = t0 + 31 > q0;
+    const bool diag = t0 + TK - 1 > q0;
 #pragma unroll 4
-    for (int t = 0; t < 32; ++t) {
+    for (int t = 0; t < TK; ++t) {
       float4 s4[QPL];                                      // (four partial sums: a chain of DK FMAs would set the pace)
 #pragma unroll
       for (int u = 0; u < QPL; ++u) s4[u] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -263,11 +276,28 @@ __global__ void __launch_bounds__(NW * 32, DK == 32 && DV == 32 && QPL == 1 ? 2 
     red[DV * QB + 32 * u + lane] = den[u];
   }
   __syncthreads();
+  if constexpr (CL > 1) {
+    // the CTA's sums to the first CTA of the cluster, which adds them in the order of the ranks
+    float* all = sm + attend_smem_floats<DK, DV, NW, QPL, 1>();
+    cg::cluster_group cluster = cg::this_cluster();
+    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");                         // ... as have the others
+    float* dst = cluster.map_shared_rank(all, 0) + rank * (DV + 1) * QB;
+    for (int i = tid; i < (DV + 1) * QB; i += NW * 32) {
+      float x = 0.f;
+#pragma unroll
+      for (int w = 0; w < NW; ++w) x += sm[w * (DV + 1) * QB + i];
+      dst[i] = x;
+    }
+    cluster.sync();
+    if (rank != 0) return;
+    sm = all;
+  }
+  constexpr int NSUM = CL > 1 ? CL : NW;
   const int row = tid % QB, part = tid / QB;               // four threads per query
   if (part >= 4) return;
   float dsum = 0.f;
 #pragma unroll
-  for (int w = 0; w < NW; ++w) dsum += sm[(w * (DV + 1) + DV) * QB + row];
+  for (int w = 0; w < NSUM; ++w) dsum += sm[(w * (DV + 1) + DV) * QB + row];
   const float inv = dsum > 0.f ? 1.f / dsum : 0.f;
   if (q0 + row >= Tlen) return;
   constexpr int CPT = DV / 4;                              // columns per thread
@@ -276,15 +306,15 @@ __global__ void __launch_bounds__(NW * 32, DK == 32 && DV == 32 && QPL == 1 ? 2 
   for (int i = 0; i < CPT; i += 4) {
     float x[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-    for (int w = 0; w < NW; ++w)
+    for (int w = 0; w < NSUM; ++w)
 #pragma unroll
       for (int e = 0; e < 4; ++e) x[e] += sm[(w * (DV + 1) + part * CPT + i + e) * QB + row];
     *reinterpret_cast<float4*>(dst + i) = make_float4(x[0] * inv, x[1] * inv, x[2] * inv, x[3] * inv);
   }
 }
 
-// measured, us, one chunk / chunks of 256: rows of 16, one head x 1024 tokens 19 / 34, 256 heads 349 / 247; rows of 32, one
-// head x 1400 46 / 76, 128 heads x 1536 872 / 950
+// measured, us, one chunk / chunks of 256: rows of 16, one head x 1024 tokens 6 / 22, 256 heads 349 / 247; rows of 32, one
+// head x 1400 19 / 66, 128 heads x 1536 872 / 950
 int one_chunk_tokens(const Problem& p) { return p.d_k == 32 ? 1536 : (long long)p.B * p.H * p.T <= 16384 ? 1024 : 512; }
 
 template <int DK, int DV> void run(const Problem& p, float* S, LaunchCtx& ctx) {
@@ -293,7 +323,7 @@ template <int DK, int DV> void run(const Problem& p, float* S, LaunchCtx& ctx) {
   const bool states = p.T > one_chunk_tokens(p);
   const int chunk = states ? CHUNK : (p.T + 63) / 64 * 64, n_chunks = (p.T + chunk - 1) / chunk;
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
@@ -309,24 +339,43 @@ template <int DK, int DV> void run(const Problem& p, float* S, LaunchCtx& ctx) {
     ok = cudaLaunchKernelEx(&cfg, state_prefix_kernel, reinterpret_cast<float4*>(S), n4, n_chunks) == cudaSuccess;
     ctx.launches += ok;
   }
-  cfg.numAttrs = states ? 1 : 0;
-  auto attend = [&](auto nw, auto qpl) {
-    constexpr int NW = decltype(nw)::value, QPL = decltype(qpl)::value;
-    constexpr int smem = attend_smem_floats<DK, DV, NW, QPL>() * (int)sizeof(float);
-    cfg.gridDim = dim3((p.T + 32 * QPL - 1) / (32 * QPL), BH);
+  auto attend = [&](auto nw, auto qpl, auto cl) {
+    constexpr int NW = decltype(nw)::value, QPL = decltype(qpl)::value, CL = decltype(cl)::value;
+    constexpr int smem = attend_smem_floats<DK, DV, NW, QPL, CL>() * (int)sizeof(float);
+    cfg.numAttrs = states ? 1 : 0;
+    if (CL > 1) {
+      attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+      attr[cfg.numAttrs].val.clusterDim.x = CL;
+      attr[cfg.numAttrs].val.clusterDim.y = attr[cfg.numAttrs].val.clusterDim.z = 1;
+      ++cfg.numAttrs;
+    }
+    cfg.gridDim = dim3((p.T + 32 * QPL - 1) / (32 * QPL) * CL, BH);
     cfg.blockDim = dim3(NW * 32);
     cfg.dynamicSmemBytes = smem;
-    return allow_smem<attend_kernel<DK, DV, NW, QPL>>(smem) &&
-           cudaLaunchKernelEx(&cfg, attend_kernel<DK, DV, NW, QPL>, q, k, v, static_cast<float*>(p.out),
+    return allow_smem<attend_kernel<DK, DV, NW, QPL, CL>>(smem) &&
+           cudaLaunchKernelEx(&cfg, attend_kernel<DK, DV, NW, QPL, CL>, q, k, v, static_cast<float*>(p.out),
                               (const float*)(states ? S : nullptr), p.T, chunk, n_chunks) == cudaSuccess;
   };
   // Two queries per lane feed two FMAs per word loaded; where that makes fewer blocks than SMs, one query per lane and, if
   // the registers allow it, sixteen warps (2 heads x 512 tokens of 16 entries: 15.6 us of GPU time,
   // 13.4 with sixteen warps, 9.1 with one query per lane as well; 256 heads x 1024 tokens the other way round: 349 and 419).
+  // Blocks that leave SMs idle have a cluster of CTAs each, as many as fit at once (a CTA of sixteen warps fills an SM, of eight
+  // half of one), and where a block is long (1024 keys and more) two in any case.  Measured, us, CTAs per block 1 / 2 / 4 / 8: rows
+  // of 16, two heads x 512 (32 blocks) 8.9 / 5.9 / 4.4 / 10.3, one x 1024 (32) 15.7 / 9.1 / 6.1 / 10.7, two x 1024 (64) 15.8 / 9.2 / 9.7 /
+  // 17.7, eight x 512 (128) 9.2 / 10.6 / 15.1 / 31.3, four x 1024 (128) 15.8 / 14.2 / 18.0 / 31.5; rows of 32, one x 512 (16) 17.2 / 12.0 / 8.1 /
+  // 7.4, one x 1024 (32) 31.0 / 20.1 / 12.3 / 10.5, two x 1024 (64) 31.0 / 20.6 / 16.9 / 17.7, eight x 1024 (256) 45.8 / 42.2 / 45.9 / 65.4.
   using std::integral_constant;
   const bool few = (long long)((p.T + 63) / 64) * BH <= 148;
-  ok = ok && (few ? attend(integral_constant<int, DK == 16 && DV == 16 ? 16 : 8>{}, integral_constant<int, 1>{})
-                  : attend(integral_constant<int, 8>{}, integral_constant<int, 2>{}));
+  const long long blocks = (long long)((p.T + 31) / 32) * BH;
+  constexpr bool wide = DK == 16 && DV == 16;
+  constexpr integral_constant<int, wide ? 16 : 8> nw{};
+  constexpr integral_constant<int, 1> one{};
+  const long long slots = wide ? sm_count() : 2 * sm_count();
+  if (!few) ok = ok && attend(integral_constant<int, 8>{}, integral_constant<int, 2>{}, one);
+  else if (!wide && 8 * blocks <= slots) ok = ok && attend(nw, one, integral_constant<int, 8>{});
+  else if (4 * blocks <= slots) ok = ok && attend(nw, one, integral_constant<int, 4>{});
+  else if (2 * blocks <= slots || chunk >= 1024) ok = ok && attend(nw, one, integral_constant<int, 2>{});
+  else ok = ok && attend(nw, one, one);
   if (!ok) {
     cudaGetLastError();
     ctx.status = KATA_ERR_CUDA;

@@ -59,3 +59,23 @@ def test_two_queries_per_lane(dk, dv, T):
     assert torch.equal(o, kb.kata_fwd_chunked(q, k, v)), "fixed summation order"
     for (b, h), r in oracle_full(w, heads=[(0, 0), (0, H // 2), (0, H - 1)]).items():
         check(to_numpy64(o[b, h]), r, "f32", f"T={T} d={dk},{dv} head {h}")
+
+
+@pytest.mark.parametrize("dk,dv,H,T", [(16, 16, 1, 7), (16, 16, 1, 1001), (16, 16, 2, 575), (16, 16, 3, 801), (16, 16, 5, 1024), (16, 16, 9, 513),
+                                       (16, 16, 1, 2335), (16, 32, 1, 1000), (32, 16, 5, 400), (32, 32, 1, 9), (32, 32, 1, 1153), (32, 32, 2, 1160),
+                                       (32, 32, 5, 900), (32, 32, 9, 1100), (32, 32, 1, 1700)])
+def test_clusters_of_ctas_per_block(dk, dv, H, T):
+    """Few blocks: two, four or eight CTAs share the keys of a block in tiles of 8, and the rows of its state; both sides of the
+    counts of blocks at which the number changes."""
+    import torch
+    w = inputs.gaussian_workload(f"sac_{dk}_{dv}_{H}_{T}", "f32", 1, H, T, dk, dv, 64, 7300 + T + dk + H)
+    for arr in (w.k_ref, w.k_dev):
+        arr[0, 0, [0, T - 1]] = 0
+    q, k, v = dev_tensors(w)
+    o = kb.kata_fwd_chunked(q, k, v)
+    torch.cuda.synchronize()
+    assert kb.kata_last_impl() == kb.KATA_IMPL_SIMT
+    assert torch.equal(o, kb.kata_fwd_chunked(q, k, v)), "fixed summation order"
+    assert torch.all(o[0, 0, 0] == 0)
+    for (b, h), r in oracle_full(w, heads=[(0, 0), (0, H - 1)]).items():
+        check(to_numpy64(o)[b, h], r, "f32", f"T={T} d={dk},{dv} head {h}")
