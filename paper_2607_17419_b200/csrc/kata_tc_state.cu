@@ -18,10 +18,13 @@
 // thread: the state before the next chunk in bf16, pair weights included.  The builders run up to five half tiles ahead, so
 // the MMAs that wait for the copy catch up.
 //
-// What bounds it.  Per tile and CTA: 640 cycles of MMA, and the shared-memory port at 128 B per cycle: 256 for the TMA
-// writes, 320 for the value operand, about 340 for the builders' fragments and broadcasts.  Built in shared memory and read
-// by the MMAs from there, as products of token rows, the A operand alone took 1024.  A builder warp takes about 1000 cycles
-// for a half tile, half of it latency, so four sets of four take turns (two sets: 1460 cycles a tile).
+// What bounds it.  Per tile and CTA 640 cycles of MMA, and about 1600 at present: the load/store pipe delivers 128 bytes a cycle
+// to registers, and the builders' fragments (192), key scales (128), scaled runs (64) and broadcasts (270) take some 760 cycles
+// of it, beside 256 for the TMA writes and 320 for the value operand on the shared memory.  The states leave by TMA from
+// staging rows: stored by the copy warps, 16 bytes of a row per lane, they were another 344 cycles of that pipe per tile (16
+// heads x 32768: 446 k cycles of the kernel, 392 k now; 131072 2.20 -> 2.00 ms a call).  Built in shared memory and read by the
+// MMAs from there, as products of token rows, the A operand alone took 1024.  A builder warp takes about 1300 cycles for a half
+// tile, most of it latency, so four sets of four take turns (two sets: 1460 cycles a tile of the kernel of that time).
 //
 // When the heads alone do not fill the GPU the chunk axis is cut into segments: every segment sums from zero and writes
 // fp32, and state_fix_kernel adds the segments before it and rounds.
@@ -57,15 +60,17 @@ constexpr uint32_t STAGE_BYTES = 32768;                     // key tile, value t
 constexpr uint32_t OFF_ONES = NSTAGE * STAGE_BYTES;         // 16 rows of [1, 0 ...]: columns 64.. of the values
 constexpr uint32_t OFF_RV = OFF_ONES + 2048;                // NSTAGE x 2 x 128 bf16 key scales (high and low parts), in the builders' order
 constexpr uint32_t OFF_SCR = OFF_RV + NSTAGE * 512;         // 16 builder warps x 2 KB: scaled fragments of run h
-constexpr uint32_t OFF_BAR = OFF_SCR + 16 * 2048;
+constexpr uint32_t OFF_OUT = OFF_SCR + 16 * 2048;           // 8 copy warps x 32 state rows of 128 bytes, 128B swizzle
+constexpr uint32_t OFF_BAR = OFF_OUT + 8 * 4096;
+static_assert(OFF_OUT % 1024 == 0, "swizzle");
 constexpr uint32_t SMEM_BYTES = OFF_BAR + 256;
 constexpr uint32_t SMEM_ALLOC = SMEM_BYTES + 1024;
 static_assert(SMEM_ALLOC > 116 * 1024, "one CTA per SM is assumed (the CTA allocates all of TMEM)");
 
 enum {
   BAR_FULL = 0,      // [NSTAGE] tiles (TMA bytes) and their key scales (scale warp) landed
-  BAR_EMPTY = 4,     // [NSTAGE] stage free: 256 builders and the issuer's commit
-  BAR_AFULL = 8,     // [NSLOT] operand slot built (128)
+  BAR_EMPTY = 4,     // [NSTAGE] stage free: eight builder warps and the issuer's commit
+  BAR_AFULL = 8,     // [NSLOT] operand slot built (four warps)
   BAR_AEMPTY = 13,   // [NSLOT] ... and consumed
   BAR_CFULL = 18,    // the MMAs of a chunk are complete
   BAR_CFREE = 19,    // the accumulators have been read, or set to the state handed in (256)
@@ -137,9 +142,19 @@ __device__ __forceinline__ void sts128(uint32_t addr, const uint32_t (&r)[4]) {
   asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
 }
 
+// A tile from shared memory to global memory, as a bulk group of this thread's; bulk_wait_read: the groups before have read their
+// shared memory, bulk_wait: they are complete.
+__device__ __forceinline__ void tma_store_3d(const void* tmap, const void* smem_src, int c0, int c1, int c2) {
+  asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.tile.bulk_group [%0, {%2, %3, %4}], [%1];\n\tcp.async.bulk.commit_group;"
+               ::"l"(tmap), "r"(smem_u32(smem_src)), "r"(c0), "r"(c1), "r"(c2) : "memory");
+}
+__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+
 template <int G, int R>
 __global__ void __launch_bounds__(NTHREADS, 1)
-tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, const SArgs args) {
+tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmOut,
+                const SArgs args) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   auto bar = [&](int i) { return reinterpret_cast<uint64_t*>(base + OFF_BAR) + i; };
@@ -163,10 +178,10 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     abort_s = 0;
     for (int i = 0; i < NSTAGE; ++i) {
       mbar_init(bar(BAR_FULL + i), 2);
-      mbar_init(bar(BAR_EMPTY + i), 257);      // 256 threads of the two sets that read a tile, and the MMAs
+      mbar_init(bar(BAR_EMPTY + i), 9);        // eight warps of the two sets that read a tile, and the MMAs
     }
     for (int i = 0; i < NSLOT; ++i) {
-      mbar_init(bar(BAR_AFULL + i), 128);
+      mbar_init(bar(BAR_AFULL + i), 4);
       mbar_init(bar(BAR_AEMPTY + i), 1);
     }
     mbar_init(bar(BAR_CFULL), 1);
@@ -207,7 +222,10 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     // =========================== update issuer ===========================
     if (elect_one()) {
       const uint32_t idesc = instr_desc(kFmtBF16, kFmtBF16, 0, 1, 128, 80);
-      const uint32_t ones = smem_u32(base + OFF_ONES);
+      // 16 tokens per 2 KB; a step moves the start address up and the distance to the constant block down
+      const uint32_t v0 = smem_u32(stage(0)) + 16384;
+      const uint64_t dv = smem_desc(v0, smem_u32(base + OFF_ONES) - v0, 1024, kSwizzle128B);
+      auto move = [](uint64_t desc, uint32_t bytes) { return desc + (uint64_t)(bytes >> 4) * (1ull - (1ull << 16)); };
       int chunk_i = 0, in_chunk = 0;     // chunk of this segment, tile inside it
       const int first_free = first ? 1 : 0;
       for (int j = 0; j < n && ok; ++j) {
@@ -215,7 +233,8 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         ok = wait_or_abort(bar(BAR_FULL + s), (j / NSTAGE) & 1, abort_flag);
         if (ok && in_chunk == 0 && chunk_i + first_free >= 1)       // the accumulators have been copied out, or set
           ok = wait_or_abort(bar(BAR_CFREE), (chunk_i + first_free - 1) & 1, abort_flag);
-        const uint32_t va = smem_u32(stage(s)) + 16384;
+        const uint64_t ds = move(dv, s * STAGE_BYTES);
+        const uint32_t acc = first || j > 0 ? 1u : 0u;
 #pragma unroll
         for (int th = 0; th < 2; ++th) {
           const int hs = 2 * j + th, slot = hs % NSLOT;
@@ -225,11 +244,9 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
 #pragma unroll
           for (int m = 0; m < 2; ++m)
 #pragma unroll
-            for (int ks = 0; ks < 4; ++ks) {
-              const uint32_t b = va + (th * 4 + ks) * 2048;
-              mma_f16_ts(tb + COL_ACC + m * 80, tb + COL_A + slot * 64 + m * 32 + ks * 8, smem_desc(b, ones - b, 1024, kSwizzle128B), idesc,
-                         (first || j > 0 || th > 0 || ks > 0) ? 1u : 0u);
-            }
+            for (int ks = 0; ks < 4; ++ks)
+              mma_f16_ts(tb + COL_ACC + m * 80, tb + COL_A + slot * 64 + m * 32 + ks * 8, move(ds, (th * 4 + ks) * 2048), idesc,
+                         th > 0 || ks > 0 ? 1u : acc);
           mma_commit(bar(BAR_AEMPTY + slot));
         }
         if (!ok) break;
@@ -340,11 +357,13 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
           tmem_st_16x128b_x8(ta + ((uint32_t)(jp * 16) << 16), xa);
           tmem_st_16x128b_x8(ta + ((uint32_t)(jp * 16) << 16) + 32, xb);
         }
-        mbar_arrive(bar(BAR_EMPTY + s));                       // this thread's part of the key tile has been used
         tmem_wait_st();
         tc_fence_before();
-        mbar_arrive(bar(BAR_AFULL + slot));
-        __syncwarp();                                          // before the scratch is written again
+        __syncwarp();                                          // (also before the scratch is written again)
+        if (lane == 0) {
+          mbar_arrive(bar(BAR_AFULL + slot));
+          mbar_arrive(bar(BAR_EMPTY + s));                     // this warp's part of the key tile has been used
+        }
       }
     };
     if (ha != hb) build(std::true_type{}); else build(std::false_type{});
@@ -359,13 +378,35 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     const int prow = public_row<G>(min(a, b), max(a, b), args.packed);
     const size_t n_pub = public_rows<G>(args.packed);
     const uint32_t ta = tmem_addr(tb, q4 * 32, COL_ACC + m * 80);
-    // bf16 state of chunk c: columns [col, col + 32) from x, and Z
+    // bf16 state of chunk c, rows of this warp: columns [col, col + 32) from x into its staging rows, and with the second half
+    // all of them out by one TMA store
+    unsigned char* out_rows = base + OFF_OUT + (warp - WARP_CPY0) * 4096;
     auto put_state = [&](int c, int col, const float (&x)[32]) {
-      uint4* dst = reinterpret_cast<uint4*>(args.s + (((size_t)bh * args.n_chunks + c) * ROWS + row) * D + col);
+      if (col == 0) {
+        if (lane == 0) bulk_wait_read();           // the store of the chunk before has read the rows
+        __syncwarp();
+      }
 #pragma unroll
       for (int i = 0; i < 4; ++i)
-        dst[i] = make_uint4(pack_bf16(x[8 * i] * wgt, x[8 * i + 1] * wgt), pack_bf16(x[8 * i + 2] * wgt, x[8 * i + 3] * wgt),
-                            pack_bf16(x[8 * i + 4] * wgt, x[8 * i + 5] * wgt), pack_bf16(x[8 * i + 6] * wgt, x[8 * i + 7] * wgt));
+        *reinterpret_cast<uint4*>(out_rows + sw128_offset(lane, col / 8 + i)) =
+            make_uint4(pack_bf16(x[8 * i] * wgt, x[8 * i + 1] * wgt), pack_bf16(x[8 * i + 2] * wgt, x[8 * i + 3] * wgt),
+                       pack_bf16(x[8 * i + 4] * wgt, x[8 * i + 5] * wgt), pack_bf16(x[8 * i + 6] * wgt, x[8 * i + 7] * wgt));
+      if (col == 32) {
+        fence_async_smem();
+        __syncwarp();
+        if (lane == 0) tma_store_3d(&tmOut, out_rows, 0, row, bh * args.n_chunks + c);
+      }
+    };
+    // fp32 sum of the segment up to and including chunk c: 32 columns are as many bytes
+    auto put_local = [&](int c, int col, const float (&x)[32]) {
+      if (lane == 0) bulk_wait_read();
+      __syncwarp();
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        *reinterpret_cast<float4*>(out_rows + sw128_offset(lane, i)) = make_float4(x[4 * i], x[4 * i + 1], x[4 * i + 2], x[4 * i + 3]);
+      fence_async_smem();
+      __syncwarp();
+      if (lane == 0) tma_store_3d(&tmOut, out_rows, col, row, bh * args.n_chunks + c);
     };
     auto put_z = [&](int c, float z) { args.z[((size_t)bh * args.n_chunks + c) * ROWS + row] = __float2bfloat16_rn(z * wgt); };
     auto put_f32 = [&](float* dst, const float (&x)[32], float f) {
@@ -388,7 +429,11 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
 #pragma unroll
         for (int i = 0; i < 32; ++i) u[i] = __float_as_uint(x[i]);
         tmem_st32(ta + col, u);
-        put_state(0, col, x);
+        uint4* dst = reinterpret_cast<uint4*>(args.s + ((size_t)bh * args.n_chunks * ROWS + row) * D + col);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          dst[i] = make_uint4(pack_bf16(x[8 * i] * wgt, x[8 * i + 1] * wgt), pack_bf16(x[8 * i + 2] * wgt, x[8 * i + 3] * wgt),
+                              pack_bf16(x[8 * i + 4] * wgt, x[8 * i + 5] * wgt), pack_bf16(x[8 * i + 6] * wgt, x[8 * i + 7] * wgt));
       }
       const float z = args.z_init[(size_t)bh * n_pub + prow] * inv;
       uint32_t u[16] = {__float_as_uint(z)};
@@ -419,7 +464,7 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         float x[32];
 #pragma unroll
         for (int y = 0; y < 32; ++y) x[y] = __uint_as_float(u[y]);
-        if (args.s_loc != nullptr) put_f32(args.s_loc + (((size_t)bh * args.n_chunks + c) * ROWS + row) * D + col, x, 1.f);
+        if (args.s_loc != nullptr) put_local(c, col, x);
         else if (!last) put_state(c + 1, col, x);
         if (fin) {
           // both triangles of a direct state; inside a diagonal block both (a, b) and (b, a) have a thread of their own
@@ -446,6 +491,7 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     }
   }
 
+  if (warp >= WARP_CPY0 && lane == 0) bulk_wait();
   // ---------------- teardown ----------------
   if (!ok && args.device_status != nullptr) atomicExch(args.device_status, (int)KATA_ERR_DEVICE_TIMEOUT);
   tc_fence_before();
@@ -530,8 +576,11 @@ int tc_state_rows(const Problem& p) {
 void tc_states(const Problem& p, const float* rscale, const StatePlan& plan, const StateBuffers& buf, int* device_status,
                LaunchCtx& ctx) {
   const int BH = p.B * p.H;
-  CUtensorMap tmK, tmV;
-  if (!make_tile_map(&tmK, p.k, BH, p.T, CT, p.d_k) || !make_tile_map(&tmV, p.v, BH, p.T, CT, p.d_v)) {
+  const bool segmented = plan.segments > 1;
+  CUtensorMap tmK, tmV, tmOut;                    // (tmOut: what goes out per chunk, 128 bytes of 32 rows at a time)
+  if (!make_tile_map(&tmK, p.k, BH, p.T, CT, p.d_k) || !make_tile_map(&tmV, p.v, BH, p.T, CT, p.d_v) ||
+      !(segmented ? make_tile_map_f32(&tmOut, buf.s_loc, BH * plan.n_chunks, tc_state_rows(p), 32)
+                  : make_tile_map(&tmOut, buf.s, BH * plan.n_chunks, tc_state_rows(p), 32))) {
     ctx.status = KATA_ERR_CUDA;
     return;
   }
@@ -544,7 +593,6 @@ void tc_states(const Problem& p, const float* rscale, const StatePlan& plan, con
     ctx.status = KATA_ERR_CUDA;
     return;
   }
-  const bool segmented = plan.segments > 1;
   SArgs a{};
   a.rscale = rscale;
   a.s = buf.s;
@@ -573,7 +621,7 @@ void tc_states(const Problem& p, const float* rscale, const StatePlan& plan, con
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, kern, tmK, tmV, a) != cudaSuccess) {
+  if (cudaLaunchKernelEx(&cfg, kern, tmK, tmV, tmOut, a) != cudaSuccess) {
     cudaGetLastError();
     ctx.status = KATA_ERR_CUDA;
     return;

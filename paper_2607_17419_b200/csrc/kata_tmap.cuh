@@ -37,4 +37,17 @@ inline bool make_tile_map(CUtensorMap* tm, const void* ptr, int BH, int T, int r
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// [BH][T][64] fp32 tensor, box = 32 columns x rows x 1 head, 128B swizzle.
+inline bool make_tile_map_f32(CUtensorMap* tm, const void* ptr, int BH, int T, int rows) {
+  EncodeTiledFn fn = tensor_map_encoder();
+  if (fn == nullptr) return false;
+  cuuint64_t dims[3] = {64, (cuuint64_t)T, (cuuint64_t)BH};
+  cuuint64_t strides[2] = {256, (cuuint64_t)T * 256};
+  cuuint32_t box[3] = {32, (cuuint32_t)rows, 1};
+  cuuint32_t es[3] = {1, 1, 1};
+  return fn(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(ptr), dims, strides, box, es,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 }  // namespace kata
