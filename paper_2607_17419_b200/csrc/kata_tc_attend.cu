@@ -72,7 +72,7 @@ constexpr uint32_t OFF_Q = 0;                       // 2 x (128 x 64 bf16, 128B 
 constexpr uint32_t STAGE_BYTES = 32768;             // K tile 16 KB, V tile 16 KB
 constexpr uint32_t OFF_ST = 32768;
 constexpr uint32_t OFF_ONES = OFF_ST + NSTAGE * STAGE_BYTES;   // 16 rows of [1, 0 ...]: columns 64.. of the values
-constexpr uint32_t OFF_Z = OFF_ONES + 2048;                    // columns 64.. of a state: 256 rows of 128 bytes, stage s in bytes [32 s, 32 s + 32)
+constexpr uint32_t OFF_Z = OFF_ONES + 2048;                    // columns 64.. of a state: 256 rows of 128 bytes, 32 of them per stage
 constexpr uint32_t OFF_RV = OFF_Z + 32768;                     // NSTAGE x 128 bf16 or fp32: 1 / ||k||^2 of the keys of a tile
 constexpr uint32_t OFF_BAR = OFF_RV + NSTAGE * 512;
 constexpr uint32_t SMEM_BYTES = OFF_BAR + 512;
@@ -174,7 +174,9 @@ struct AArgs {
 // R = runs of 8 features that a row may have.  G = feature groups of the blockwise map: a key tile holds KT = 128 / G keys, and the 128 score columns of a buffer
 // hold, for each half of those keys, the G per-group score blocks Q_a K_a^T side by side (group a in columns [a KT/2,
 // a KT/2 + KT/2) of the sub-buffer); the weight of a key is the sum over the groups of the squared scores.
-template <int G, int R, bool XR, bool SPLIT>
+// VC = value columns: 64, or 32 for rows of values of up to 32 entries, whose tiles have rows of 64 bytes (64B swizzle) and whose
+// apply and state MMAs N = 32 + 16 instead of 64 + 16 (128 heads x 2048 tokens of 32 entries 66.0 -> 62.3 us).
+template <int G, int R, bool XR, bool SPLIT, int VC>
 __global__ void __launch_bounds__(NTHREADS, 1)
 tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                  const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmS, const AArgs args) {
@@ -191,6 +193,11 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
   constexpr int KH = KT / 2;                      // keys of a sub-tile
   constexpr int KPL = KT / 32;                    // keys per lane of the scale warp
   constexpr int NST = PairTable<G, R>::kSlices;      // state tiles
+  constexpr uint32_t VROW = VC * 2;               // bytes of a row of a value or state tile
+  // byte offset of (row, 16-byte chunk) in such a tile, as TMA and the MMA descriptors swizzle it
+  // where the Z columns of a stage begin: 32 bytes of every row, for four stages (two, and the other two behind them)
+  auto z_stage = [](uint32_t s) { return VC == 64 ? s * 32 : (s >> 1) * 16384 + (s & 1) * 32; };
+  auto v_offset = [](uint32_t row, uint32_t chunk) { return VC == 64 ? sw128_offset(row, chunk) : row * 64u + ((chunk ^ ((row >> 1) & 3u)) << 4); };
 
   // Work items.  Rank -> (block of its chunk, chunk, head): the last blocks of the chunks (the most key tiles) first,
   // among them the chunks in descending order, so that chunk 0, which reads no state, comes last.  The n-th item of a CTA:
@@ -275,8 +282,8 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
   }
   // columns 64..127 of 16 rows of the value operand: [1, 0, ...] (every step of 16 rows reads the same block: the
   // descriptor's leading offset is the distance to it); the Z columns of the state start as zeros
-  if (tid < 128)
-    *reinterpret_cast<uint4*>(base + OFF_ONES + sw128_offset(tid >> 3, tid & 7)) = make_uint4((tid & 7) == 0 ? 0x3F80u : 0u, 0u, 0u, 0u);
+  if (tid < VC * 2)
+    *reinterpret_cast<uint4*>(base + OFF_ONES + v_offset(tid / (VC / 8), tid % (VC / 8))) = make_uint4(tid % (VC / 8) == 0 ? 0x3F80u : 0u, 0u, 0u, 0u);
   if (args.first_state < args.n_chunks)
     for (int i = tid; i < 2048; i += NTHREADS) *reinterpret_cast<uint4*>(base + OFF_Z + i * 16) = make_uint4(0u, 0u, 0u, 0u);
   fence_async_smem();
@@ -313,12 +320,12 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
           if (!ok) break;
           if (j >= w.ns) {
             const int key = (w.k0 + j - w.ns) * KT;
-            mbar_arrive_expect_tx(bar(BAR_FULL + s), 2 * KT * 128);   // K and V tiles
+            mbar_arrive_expect_tx(bar(BAR_FULL + s), KT * (128 + VROW));   // K and V tiles
             tma_load_3d(stage(s), &tmK, bar(BAR_FULL + s), 0, key, w.bh);
             tma_load_3d(stage(s) + 16384, &tmV, bar(BAR_FULL + s), 0, key, w.bh);
           } else {
             const int slot = w.bh * args.n_chunks + w.chunk;
-            mbar_arrive_expect_tx(bar(BAR_FULL + s), 32768);
+            mbar_arrive_expect_tx(bar(BAR_FULL + s), 256 * VROW);
             tma_load_3d(stage(s), &tmS, bar(BAR_FULL + s), 0, j * 256, slot);
           }
         }
@@ -334,12 +341,12 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     if (elect_one()) {
       const int h = warp - 1;
       const uint32_t id_s = instr_desc(kFmtBF16, kFmtBF16, 0, 0, 128, KH);      // scores: B K-major
-      const uint32_t id_p = instr_desc(kFmtBF16, kFmtBF16, 0, 1, 128, 80);      // apply, Psi(Q) [S | Z]: B MN-major, N = 64 + 16
+      const uint32_t id_p = instr_desc(kFmtBF16, kFmtBF16, 0, 1, 128, VC + 16); // apply, Psi(Q) [S | Z]: B MN-major, N = VC + 16
       const uint64_t dk = smem_desc(0, 16, 1024, kSwizzle128B);
       const uint32_t tS = tb + COL_S + h * 128, tO = tb + COL_O + h * 80, tQ = tb + COL_Q + h * 32;
       const uint32_t ones = smem_u32(base + OFF_ONES), zcol = smem_u32(base + OFF_Z);
-      // MN-major, 128B swizzle: 8 rows per 1024-byte atom (SBO), columns 64.. in the constant block (LBO)
-      auto bdesc = [&](uint32_t addr, uint32_t extra) { return smem_desc(addr, extra - addr, 1024, kSwizzle128B); };
+      // MN-major: 8 rows of VROW bytes per atom (SBO), columns VC.. in the constant block (LBO)
+      auto bdesc = [&](uint32_t addr, uint32_t extra) { return smem_desc(addr, extra - addr, 8 * VROW, VC == 64 ? kSwizzle128B : kSwizzle64B); };
       // ... moved by a number of bytes: the start address goes up and the distance to the constant block down
       auto move = [](uint64_t desc, uint32_t bytes) { return desc + (uint64_t)(bytes >> 4) * (1ull - (1ull << 16)); };
       const uint64_t dv0 = bdesc(smem_u32(stage(0)) + 16384, ones), dk0 = at(dk, smem_u32(stage(0)));
@@ -362,9 +369,9 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         auto close = [&](uint32_t g_it, int c) -> bool {
           if (!wait_or_abort(bar(BAR_PFULL + 2 * h + c), cnt & 1, abort_flag)) return false;
           tc_fence_after();
-          const uint64_t d = move(dv0, (g_it % NSTAGE) * STAGE_BYTES + c * KH * 128);
+          const uint64_t d = move(dv0, (g_it % NSTAGE) * STAGE_BYTES + c * KH * VROW);
 #pragma unroll
-          for (int ks = 0; ks < KH / 16; ++ks) mma_f16_ts(tO, tS + c * 64 + ks * 8, move(d, ks * 2048), id_p, ks > 0 ? 1u : acc);
+          for (int ks = 0; ks < KH / 16; ++ks) mma_f16_ts(tO, tS + c * 64 + ks * 8, move(d, ks * 16 * VROW), id_p, ks > 0 ? 1u : acc);
           acc = 1;
           return true;
         };
@@ -409,7 +416,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
 #pragma unroll 1
             for (int t = 0; t < NST && ok; ++t, ++it, ++n_st) {
               ok = landed(it) && (t > 0 || o_free()) && (t + 1 < NST || landed(it + 1));
-              const uint64_t ds = bdesc(smem_u32(stage(it % NSTAGE)), zcol + (it % NSTAGE) * 32);
+              const uint64_t ds = bdesc(smem_u32(stage(it % NSTAGE)), zcol + z_stage(it % NSTAGE));
 #pragma unroll
               for (int c = 0; c < 2; ++c) {
 #pragma unroll
@@ -418,8 +425,8 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                   if (!ok) break;
                   tc_fence_after();
 #pragma unroll
-                  for (int ks = 0; ks < 4; ++ks)             // 16 rows per 2 KB, of the state and of Z
-                    mma_f16_ts(tO, tS + c * 64 + pp * 32 + ks * 8, ds + (c * 8 + pp * 4 + ks) * 128, id_p, c + pp + ks > 0 ? 1u : acc);
+                  for (int ks = 0; ks < 4; ++ks)             // 16 rows at a time, of the state and of Z
+                    mma_f16_ts(tO, tS + c * 64 + pp * 32 + ks * 8, ds + (c * 8 + pp * 4 + ks) * VROW, id_p, c + pp + ks > 0 ? 1u : acc);
                   acc = 1;
                   mma_commit(bar(BAR_SFREE + 4 * h + 2 * c + pp));
                 }
@@ -491,7 +498,8 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
 #pragma unroll
           for (int e = 0; e < 8; ++e) {
             const int row = e * 32 + lane;
-            *reinterpret_cast<unsigned short*>(base + OFF_Z + (row >> 4) * 2048 + sw128_offset(row & 15, 2 * s)) = (unsigned short)x[e];
+            const uint32_t z = VC == 64 ? v_offset(row, 2 * s) : (s >> 1) * 16384u + v_offset(row, 2 * (s & 1));
+            *reinterpret_cast<unsigned short*>(base + OFF_Z + z) = (unsigned short)x[e];
           }
           fence_async_smem();
         } else {
@@ -686,9 +694,9 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         tc_fence_after();
         uint32_t x[16], y[16], dx[4], dy[4];
         tmem_ld16(oa + c16, x);
-        tmem_ld4(oa + 64, dx);
+        tmem_ld4(oa + VC, dx);
         tmem_ld16(oa + 80 + c16, y);
-        tmem_ld4(oa + 80 + 64, dy);
+        tmem_ld4(oa + 80 + VC, dy);
         tmem_wait_ld(x);
         tmem_wait_ld(y);
         tmem_wait_ld(dx);
@@ -718,7 +726,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       tc_fence_after();
       uint32_t o[32], dn[4];
       tmem_ld32(tO + ch * 32, o);
-      tmem_ld4(tO + 64, dn);
+      tmem_ld4(tO + VC, dn);
       tmem_wait_ld(o);
       tmem_wait_ld(dn);
       tc_fence_before();
@@ -770,6 +778,8 @@ void tc_attend(const Problem& p, const KeyScales& r, const AttendStates& st, int
   const int BH = p.B * p.H;
   CUtensorMap tmQ, tmK, tmV, tmS;
   const int kt = KTILE / p.groups;
+  const bool narrow = tc_narrow(p);
+  const int vc = narrow && p.d_v <= 32 ? 32 : 64;
   // No states and not more blocks of 256 queries than SMs: the call lasts as long as its longest block, so the halves of a CTA
   // share out the keys of one block of 128 queries instead (SPLIT).  From four tiles of the longest half on; shorter ones gain
   // nothing, and with more blocks the tiles that only one half uses cost more than the finer deal gives (with feature groups,
@@ -783,14 +793,14 @@ void tc_attend(const Problem& p, const KeyScales& r, const AttendStates& st, int
   const int n_pairs = split ? (p.T + QT - 1) / QT : n_blocks;
   AArgs a{static_cast<__nv_bfloat16*>(p.out), r.f32, r.bf16, device_status, p.T, p.d_v, BH, n_pairs, n_pairs, 1, 1, 0, nullptr};
   bool maps = make_tile_map(&tmQ, p.q, BH, p.T, QT, p.d_k) && make_tile_map(&tmK, p.k, BH, p.T, kt, p.d_k) &&
-              make_tile_map(&tmV, p.v, BH, p.T, kt, p.d_v);
+              make_tile_map(&tmV, p.v, BH, p.T, kt, p.d_v, vc);
   if (st.n_chunks > 0) {
     a.chunk_pairs = st.chunk_tokens / (2 * QT);
     a.n_chunks = st.n_chunks;
     a.first_state = st.first_state;
     a.by_chunk = (long long)BH * st.n_chunks * a.chunk_pairs >= 24LL * sm_count() ? 1 : 0;
     a.z = reinterpret_cast<const unsigned short*>(st.z);
-    maps = maps && make_tile_map(&tmS, st.s, BH * st.n_chunks, tc_state_rows(p), 256);
+    maps = maps && make_tile_map(&tmS, st.s, BH * st.n_chunks, tc_state_rows(p), 256, 64, vc);
   } else {
     tmS = tmK;
   }
@@ -798,21 +808,22 @@ void tc_attend(const Problem& p, const KeyScales& r, const AttendStates& st, int
     ctx.status = KATA_ERR_CUDA;
     return;
   }
-  const bool narrow = tc_narrow(p);
   void (*kern)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, AArgs) = nullptr;
-  auto pick = [&](auto g, auto r, auto xr) {
-    constexpr auto K = tc_attend_kernel<decltype(g)::value, decltype(r)::value, decltype(xr)::value, false>;
-    constexpr auto KS = tc_attend_kernel<decltype(g)::value, decltype(r)::value, decltype(xr)::value, true>;
+  auto pick = [&](auto g, auto r, auto xr, auto cols) {
+    constexpr auto K = tc_attend_kernel<decltype(g)::value, decltype(r)::value, decltype(xr)::value, false, decltype(cols)::value>;
+    constexpr auto KS = tc_attend_kernel<decltype(g)::value, decltype(r)::value, decltype(xr)::value, true, decltype(cols)::value>;
     kern = split ? KS : K;
     return split ? allow_smem<KS>((int)SMEM_ALLOC) : allow_smem<K>((int)SMEM_ALLOC);
   };
   using std::integral_constant;
   auto pick_g = [&](auto xr) {
-    if (p.groups == 2) return pick(integral_constant<int, 2>{}, integral_constant<int, 8>{}, xr);
-    if (p.groups == 4) return pick(integral_constant<int, 4>{}, integral_constant<int, 8>{}, xr);
-    return pick(integral_constant<int, 1>{}, integral_constant<int, 8>{}, xr);
+    constexpr integral_constant<int, 64> c64{};
+    if (p.groups == 2) return pick(integral_constant<int, 2>{}, integral_constant<int, 8>{}, xr, c64);
+    if (p.groups == 4) return pick(integral_constant<int, 4>{}, integral_constant<int, 8>{}, xr, c64);
+    return pick(integral_constant<int, 1>{}, integral_constant<int, 8>{}, xr, c64);
   };
-  if (!(narrow              ? pick(integral_constant<int, 1>{}, integral_constant<int, 4>{}, std::false_type{})
+  if (!(vc == 32            ? pick(integral_constant<int, 1>{}, integral_constant<int, 4>{}, std::false_type{}, integral_constant<int, 32>{})
+        : narrow            ? pick(integral_constant<int, 1>{}, integral_constant<int, 4>{}, std::false_type{}, integral_constant<int, 64>{})
         : st.exact_scales   ? pick_g(std::true_type{})
                             : pick_g(std::false_type{}))) {
     ctx.status = KATA_ERR_CUDA;

@@ -24,16 +24,16 @@ inline EncodeTiledFn tensor_map_encoder() {
 }
 
 // [BH][T][d] bf16 tensor (d = 64, or 16 or 32: columns d..63 of the box read as zero), box = 64 columns x rows x 1 head,
-// 128B swizzle; rows beyond T read as zero.
-inline bool make_tile_map(CUtensorMap* tm, const void* ptr, int BH, int T, int rows, int d = 64) {
+// 128B swizzle; rows beyond T read as zero.  cols = 32: a box of 32 columns, 64B swizzle.
+inline bool make_tile_map(CUtensorMap* tm, const void* ptr, int BH, int T, int rows, int d = 64, int cols = 64) {
   EncodeTiledFn fn = tensor_map_encoder();
   if (fn == nullptr) return false;
   cuuint64_t dims[3] = {(cuuint64_t)d, (cuuint64_t)T, (cuuint64_t)BH};
   cuuint64_t strides[2] = {(cuuint64_t)d * 2, (cuuint64_t)T * d * 2};
-  cuuint32_t box[3] = {64, (cuuint32_t)rows, 1};
+  cuuint32_t box[3] = {(cuuint32_t)cols, (cuuint32_t)rows, 1};
   cuuint32_t es[3] = {1, 1, 1};
   return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, es,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, cols == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 

@@ -10,7 +10,7 @@ from oracle import kata_oracle as ko
 from paper_2607_17419_b200 import binding as kb
 from paper_2607_17419_b200 import inputs
 
-from helpers import check, dev_tensors, oracle_rows, sample_picks, to_numpy64
+from helpers import check, dev_tensors, oracle_full, oracle_rows, sample_picks, to_numpy64
 
 pytestmark = pytest.mark.gpu
 
@@ -136,3 +136,19 @@ def test_weight_rounding(g, H, T, state):
         near += ((p * p) * ((v * v).sum(axis=1)[None, :] - 2 * (r @ v.T) + (r * r).sum(axis=1)[:, None])).sum()
         far += (r * r).sum()
     assert np.sqrt(err) <= eps * np.sqrt(2.0 * near + far), (g, H, T, (err / eps ** 2 - far) / near)
+
+
+@pytest.mark.parametrize("dk,dv", [(32, 32), (32, 16), (16, 32), (16, 16), (32, 64)])
+@pytest.mark.parametrize("H,T", [(1, 129), (2, 777), (40, 1153)])
+def test_narrow_values(dk, dv, H, T):
+    """Values of up to 32 entries have tiles of 32 columns, wider ones of 64: both halves on a block and the halves sharing its keys,
+    the ring of stages past its end (several chunks: test_narrow_rows)."""
+    import torch
+    w = inputs.gaussian_workload(f"narrow_{dk}_{dv}_{H}_{T}", "bf16", 1, H, T, dk, dv, 64, 5700 + T + dv)
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    q, k, v = dev_tensors(w)
+    o = kb.kata_fwd_chunked(q, k, v, device_status=st)
+    torch.cuda.synchronize()
+    assert kb.kata_last_impl() == kb.KATA_IMPL_TENSOR and int(st.item()) == 0
+    for (b, h), r in oracle_full(w, heads=[(0, 0), (0, H - 1)]).items():
+        check(to_numpy64(o[b, h]), r, "bf16", f"T={T} d={dk},{dv} head {h}")
