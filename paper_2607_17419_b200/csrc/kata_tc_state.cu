@@ -88,6 +88,7 @@ struct SArgs {
   const float* z_init;
   float* s_final;                // state after the last token, public layout (null: not wanted); one segment only
   float* z_final;
+  int wide_final;                // s_final is 32-byte aligned
   int packed;                    // public layout: packed upper triangles instead of direct
   int* device_status;
   int Tlen;
@@ -149,6 +150,10 @@ __device__ __forceinline__ void tma_store_3d(const void* tmap, const void* smem_
                ::"l"(tmap), "r"(smem_u32(smem_src)), "r"(c0), "r"(c1), "r"(c2) : "memory");
 }
 __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void st_global_v8(float* p, const float4& a, const float4& b) {      // 32-byte aligned
+  asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
+               ::"l"(p), "f"(a.x), "f"(a.y), "f"(a.z), "f"(a.w), "f"(b.x), "f"(b.y), "f"(b.z), "f"(b.w) : "memory");
+}
 __device__ __forceinline__ void bulk_wait() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
 template <int G, int R>
@@ -411,7 +416,16 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     auto put_z = [&](int c, float z) { args.z[((size_t)bh * args.n_chunks + c) * ROWS + row] = __float2bfloat16_rn(z * wgt); };
     auto put_f32 = [&](float* dst, const float (&x)[32], float f) {
 #pragma unroll
-      for (int i = 0; i < 8; ++i) reinterpret_cast<float4*>(dst)[i] = make_float4(x[4 * i] * f, x[4 * i + 1] * f, x[4 * i + 2] * f, x[4 * i + 3] * f);
+      for (int i = 0; i < 8; i += 2) {
+        const float4 lo = make_float4(x[4 * i] * f, x[4 * i + 1] * f, x[4 * i + 2] * f, x[4 * i + 3] * f);
+        const float4 hi = make_float4(x[4 * i + 4] * f, x[4 * i + 5] * f, x[4 * i + 6] * f, x[4 * i + 7] * f);
+        if (args.wide_final) {
+          st_global_v8(dst + 4 * i, lo, hi);
+        } else {
+          reinterpret_cast<float4*>(dst)[i] = lo;
+          reinterpret_cast<float4*>(dst)[i + 1] = hi;
+        }
+      }
     };
     if (first) {
       // the state handed in: into the accumulators, and out in bf16 for chunk 0
@@ -603,6 +617,7 @@ void tc_states(const Problem& p, const float* rscale, const StatePlan& plan, con
   a.z_init = buf.z_init;
   a.s_final = segmented ? nullptr : buf.s_final;
   a.z_final = segmented ? nullptr : buf.z_final;
+  a.wide_final = (reinterpret_cast<uintptr_t>(a.s_final) & 31) == 0;
   a.packed = buf.layout == KATA_LAYOUT_PACKED;
   a.device_status = device_status;
   a.Tlen = p.T;

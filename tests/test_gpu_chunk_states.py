@@ -152,3 +152,26 @@ def test_narrow_values(dk, dv, H, T):
     assert kb.kata_last_impl() == kb.KATA_IMPL_TENSOR and int(st.item()) == 0
     for (b, h), r in oracle_full(w, heads=[(0, 0), (0, H - 1)]).items():
         check(to_numpy64(o[b, h]), r, "bf16", f"T={T} d={dk},{dv} head {h}")
+
+
+@pytest.mark.parametrize("H,T,dk,dv,state", [(3, 300, 64, 64, False), (1, 1300, 64, 64, False), (60, 700, 32, 16, False), (2, 2500, 64, 64, True)])
+@pytest.mark.parametrize("layout", [kb.KATA_LAYOUT_DIRECT, kb.KATA_LAYOUT_PACKED])
+def test_outputs_aligned_to_16_bytes_only(H, T, dk, dv, state, layout):
+    """Output and state rows leave 32 bytes at a time where the tensors allow it, 16 otherwise: the same bits."""
+    import torch
+    gen = torch.Generator(device="cuda").manual_seed(T)
+    q, k = (torch.randn(1, H, T, dk, device="cuda", generator=gen).bfloat16() for _ in range(2))
+    v = torch.randn(1, H, T, dv, device="cuda", generator=gen).bfloat16()
+    n = kb.decode_n_psi(dk, state_layout=layout)
+
+    def run(shift):
+        out = torch.empty(H * T * dv + 8, dtype=torch.bfloat16, device="cuda")[shift // 2:][:H * T * dv].view(1, H, T, dv)
+        kw = {}
+        if state:
+            kw = {"s_pre": torch.empty(H * n * dv + 4, device="cuda")[shift // 4:][:H * n * dv].view(1, H, n, dv),
+                  "z_pre": torch.empty(H * n + 4, device="cuda")[shift // 4:][:H * n].view(1, H, n), "state_layout": layout}
+        assert out.data_ptr() % 32 == shift
+        return (kb.kata_fwd_chunked(q, k, v, out=out, **kw), *[kw[x] for x in ("s_pre", "z_pre") if x in kw])
+
+    for a, b in zip(run(0), run(16)):
+        assert torch.equal(a, b)
