@@ -142,11 +142,6 @@ __device__ __forceinline__ uint4 lds128(uint32_t addr) {
   return v;
 }
 
-__device__ __forceinline__ void st_global_v8(void* p, const uint4& a, const uint4& b) {      // 32-byte aligned
-  asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
-               ::"l"(p), "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w) : "memory");
-}
-
 // Registers: 640 threads x 96 at launch; the four warps that issue and copy give theirs to the builders
 // (128 x 64 + 512 x 104 = 640 x 96).
 template <int N> __device__ __forceinline__ void regs_release() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
@@ -555,16 +550,6 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       }
       if (w.ns == 0) mbar_arrive(bar(BAR_QEMPTY));
     };
-    // 16 columns of an output row (d_v is a multiple of 16).  A warp's store instruction touches 32 rows, one pass of the
-    // load/store pipe each, so half as many instructions matter (64 heads x 4096 tokens 148.6 -> 146.7 us)
-    auto store_row = [&](__nv_bfloat16* dst, const uint4 (&x)[2]) {
-      if (args.wide_out) {
-        st_global_v8(dst, x[0], x[1]);
-      } else {
-        reinterpret_cast<uint4*>(dst)[0] = x[0];
-        reinterpret_cast<uint4*>(dst)[1] = x[1];
-      }
-    };
     uint32_t it = 0, cnt = 0, n_st = 0;
     int n_done = 0, ni = 0, n = 0;
     int n_done_b = 0;                            // SPLIT: items with tiles for half B (n_done: all)
@@ -730,7 +715,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
           for (int jj = 0; jj < 16; jj += 8)
             pkt[jj / 8] = make_uint4(pack_bf16(sum(jj), sum(jj + 1)), pack_bf16(sum(jj + 2), sum(jj + 3)),
                                      pack_bf16(sum(jj + 4), sum(jj + 5)), pack_bf16(sum(jj + 6), sum(jj + 7)));
-          if ((int)c16 < args.d_v) store_row(dst, pkt);
+          if ((int)c16 < args.d_v) store_32(dst, pkt, args.wide_out);          // (d_v is a multiple of 16)
         }
         continue;
       }
@@ -763,7 +748,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
             pkt[e].z = pack_bf16(__uint_as_float(x[4]) * inv, __uint_as_float(x[5]) * inv);
             pkt[e].w = pack_bf16(__uint_as_float(x[6]) * inv, __uint_as_float(x[7]) * inv);
           }
-          store_row(dst + jj, pkt);
+          store_32(dst + jj, pkt, args.wide_out);      // (by sixteens 64 heads x 4096 tokens took 148.6 instead of 146.7 us)
         }
       }
     }

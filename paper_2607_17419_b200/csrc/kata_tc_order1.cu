@@ -19,6 +19,11 @@
 // with the keys and values of the group still in L2 where the groups are small.  One launch; the sum does not depend
 // on the order in which the CTAs run.  HBM-bound: q, k, v in, o out, 512 bytes per token.
 //
+// The load/store pipe takes a pass per row that a store instruction touches: outputs stored by the threads, 16 bytes of a row at a
+// time, were 1024 of the 2200 cycles of a tile; they leave by TMA from staging rows now (16 x 16 heads x 8192 tokens 194.6 ->
+// 180.7 us).  The weights are formed 32 columns at a time and only the blocks on the diagonal are compared with it; those above
+// it are zeros without being read (173.3).
+//
 // Warps (512 threads): 0 TMA producer; 1, 2, 3, 7 MMA issuers (scores, intra, update, inter: one thread gets an MMA
 // out about every hundred cycles whatever its size, so every group of MMAs has its own); 4-6 state snapshot (TMEM
 // -> bf16 rows in shared memory, 32 rows each) and state export; 4-7 state import; 8-15 weights and epilogue (two
@@ -50,7 +55,9 @@ constexpr uint32_t STAGE_BYTES = 49152;               // Q, K, V tiles of 16 KB,
 constexpr uint32_t OFF_ONES = NSTAGE * STAGE_BYTES;   // [128 tokens][64 columns] bf16: column 0 = 1, the rest 0
 constexpr uint32_t OFF_SP = OFF_ONES + 16384;         // 2 x (80 rows x 128 B): state snapshots, K-major
 constexpr uint32_t SP_BYTES = SROWS * 128;
-constexpr uint32_t OFF_BAR = OFF_SP + 2 * SP_BYTES;
+constexpr uint32_t OFF_OUT = OFF_SP + 2 * SP_BYTES;   // 8 epilogue warps x 32 rows of 64 bytes, 64B swizzle
+constexpr uint32_t OFF_BAR = OFF_OUT + 8 * 2048;
+static_assert(OFF_OUT % 512 == 0, "swizzle");
 constexpr uint32_t SMEM_BYTES = OFF_BAR + 256;
 constexpr uint32_t SMEM_ALLOC = SMEM_BYTES + 1024;
 static_assert(SMEM_ALLOC > 116 * 1024, "one CTA per SM is assumed (the CTA allocates all of TMEM)");
@@ -75,7 +82,6 @@ enum {
 };
 
 struct OArgs {
-  __nv_bfloat16* out;
   int* device_status;
   int Tlen;
   int n_tiles;
@@ -110,7 +116,7 @@ __device__ __forceinline__ void snap_store_row(unsigned char* sp, int row, const
 
 __global__ void __launch_bounds__(NTHREADS, 1)
 tc_order1_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
-                 const __grid_constant__ CUtensorMap tmV, const OArgs args) {
+                 const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO, const OArgs args) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   auto bar = [&](int i) { return reinterpret_cast<uint64_t*>(base + OFF_BAR) + i; };
@@ -457,19 +463,20 @@ tc_order1_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       mbar_arrive(bar(BAR_O_EMPTY + bb));
       const float den = __uint_as_float(dn[0]);
       const float inv = den != 0.f ? 1.f / den : 0.f;
-      const int tok = (t_begin + jj) * CT + rowl;
-      if (tok < args.Tlen) {
-        __nv_bfloat16* dst = args.out + ((size_t)bh * args.Tlen + tok) * D + ch * 32;
+      // out by TMA from staging rows (rows beyond the sequence are not written)
+      unsigned char* rows = base + OFF_OUT + (warp - W_BLD0) * 2048;
+      if (lane == 0) bulk_wait_read();           // the store of the tile before has read them
+      __syncwarp();
 #pragma unroll
-        for (int c = 0; c < 32; c += 8) {
-          uint4 pkt;
-          pkt.x = pack_bf16(__uint_as_float(o[c]) * inv, __uint_as_float(o[c + 1]) * inv);
-          pkt.y = pack_bf16(__uint_as_float(o[c + 2]) * inv, __uint_as_float(o[c + 3]) * inv);
-          pkt.z = pack_bf16(__uint_as_float(o[c + 4]) * inv, __uint_as_float(o[c + 5]) * inv);
-          pkt.w = pack_bf16(__uint_as_float(o[c + 6]) * inv, __uint_as_float(o[c + 7]) * inv);
-          *reinterpret_cast<uint4*>(dst + c) = pkt;
-        }
+      for (int c = 0; c < 4; ++c) {
+        const uint32_t* x = o + 8 * c;
+        *reinterpret_cast<uint4*>(rows + lane * 64 + ((c ^ ((lane >> 1) & 3)) << 4)) =
+            make_uint4(pack_bf16(__uint_as_float(x[0]) * inv, __uint_as_float(x[1]) * inv), pack_bf16(__uint_as_float(x[2]) * inv, __uint_as_float(x[3]) * inv),
+                       pack_bf16(__uint_as_float(x[4]) * inv, __uint_as_float(x[5]) * inv), pack_bf16(__uint_as_float(x[6]) * inv, __uint_as_float(x[7]) * inv));
       }
+      fence_async_smem();
+      __syncwarp();
+      if (lane == 0) tma_store_3d(&tmO, rows, ch * 32, (t_begin + jj) * CT + q4 * 32, bh);
       return true;
     };
     for (int j = 0; j < n && ok; ++j) {
@@ -478,20 +485,29 @@ tc_order1_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       if (!ok) break;
       tc_fence_after();
       const uint32_t scol = tmem_addr(tb, q4 * 32, COL_P + b * 128 + ch * 64);
-      uint32_t ya[32], yb[32], pk[32];
-      tmem_ld32(scol, ya);
-      tmem_ld32(scol + 32, yb);
-      tmem_wait_ld(ya);
-      tmem_wait_ld(yb);
-      // causal mask inside the tile: key c contributes to token rowl when c <= rowl
+      // 32 columns at a time, over this thread's own scores, which are in its registers; the causal mask (key c contributes to token
+      // rowl when c <= rowl) is only looked at in the block on the diagonal
 #pragma unroll
-      for (int c = 0; c < 32; c += 2) {
-        const int k0 = ch * 64 + c, k1 = ch * 64 + 32 + c;
-        pk[c / 2] = pack_bf16(k0 <= rowl ? __uint_as_float(ya[c]) : 0.f, k0 + 1 <= rowl ? __uint_as_float(ya[c + 1]) : 0.f);
-        pk[16 + c / 2] = pack_bf16(k1 <= rowl ? __uint_as_float(yb[c]) : 0.f, k1 + 1 <= rowl ? __uint_as_float(yb[c + 1]) : 0.f);
+      for (int hf = 0; hf < 2; ++hf) {
+        const uint32_t blk = 2 * ch + hf;          // columns 32 blk .. of the tile, against rows 32 q4 ..
+        uint32_t pk[16];
+        if (blk > q4) {
+#pragma unroll
+          for (int c = 0; c < 16; ++c) pk[c] = 0u;
+        } else {
+          uint32_t y[32];
+          tmem_ld32(scol + hf * 32, y);
+          tmem_wait_ld(y);
+          if (blk == q4) {
+#pragma unroll
+            for (int c = 0; c < 32; ++c)
+              if (c > lane) y[c] = 0u;
+          }
+#pragma unroll
+          for (int c = 0; c < 32; c += 2) pk[c / 2] = pack_bf16(__uint_as_float(y[c]), __uint_as_float(y[c + 1]));
+        }
+        tmem_st16(scol + hf * 16, pk);
       }
-      // the weights of a column half overwrite its own scores, which are in this thread's registers
-      tmem_st32(scol, pk);
       tmem_wait_st();
       tc_fence_before();
       mbar_arrive(bar(BAR_P_FULL + b));
@@ -519,6 +535,7 @@ tc_order1_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
   }
   if (!fused || dead) break;
   }
+  if (warp >= W_BLD0 && lane == 0) bulk_wait();
   if (warp == 0) tmem_dealloc(tb, TMEM_COLS);
 }
 
@@ -531,8 +548,9 @@ int tc_order1_tile() { return CT; }
 void tc_order1(const Problem& p, const ScanPlan& plan, bool use_scan, int C, float* ws, int* device_status,
                LaunchCtx& ctx) {
   const int BH = p.B * p.H;
-  CUtensorMap tmQ, tmK, tmV;
-  if (!make_tile_map(&tmQ, p.q, BH, p.T, CT) || !make_tile_map(&tmK, p.k, BH, p.T, CT) || !make_tile_map(&tmV, p.v, BH, p.T, CT)) {
+  CUtensorMap tmQ, tmK, tmV, tmO;
+  if (!make_tile_map(&tmQ, p.q, BH, p.T, CT) || !make_tile_map(&tmK, p.k, BH, p.T, CT) || !make_tile_map(&tmV, p.v, BH, p.T, CT) ||
+      !make_tile_map(&tmO, p.out, BH, p.T, 32, 64, 32)) {
     ctx.status = KATA_ERR_CUDA;
     return;
   }
@@ -541,7 +559,6 @@ void tc_order1(const Problem& p, const ScanPlan& plan, bool use_scan, int C, flo
     return;
   }
   OArgs a;
-  a.out = static_cast<__nv_bfloat16*>(p.out);
   a.device_status = device_status;
   a.Tlen = p.T;
   a.n_tiles = (p.T + CT - 1) / CT;
@@ -571,12 +588,12 @@ void tc_order1(const Problem& p, const ScanPlan& plan, bool use_scan, int C, flo
     a.ticket = reinterpret_cast<unsigned*>(flags + (size_t)BH * NG);
     const int sms = sm_count();
     const unsigned total = (unsigned)BH * NG;
-    tc_order1_kernel<<<dim3(total < (unsigned)sms ? total : (unsigned)sms), NTHREADS, SMEM_ALLOC, ctx.stream>>>(tmQ, tmK, tmV, a);
+    tc_order1_kernel<<<dim3(total < (unsigned)sms ? total : (unsigned)sms), NTHREADS, SMEM_ALLOC, ctx.stream>>>(tmQ, tmK, tmV, tmO, a);
     note_launch(ctx);
     return;
   }
   // one group: one CTA per head walks all its tiles
-  tc_order1_kernel<<<dim3(BH), NTHREADS, SMEM_ALLOC, ctx.stream>>>(tmQ, tmK, tmV, a);
+  tc_order1_kernel<<<dim3(BH), NTHREADS, SMEM_ALLOC, ctx.stream>>>(tmQ, tmK, tmV, tmO, a);
   note_launch(ctx);
 }
 

@@ -253,7 +253,7 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
 }
 
 // ---------------------------------------------------------------------------------------------
-// TMA (plain tile loads, never multicast)
+// TMA (plain tile loads and stores, never multicast)
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ void tma_load_3d(void* smem_dst, const void* tmap, uint64_t* bar, int c0, int c1,
                                             int c2) {
@@ -266,6 +266,14 @@ __device__ __forceinline__ void tma_load_3d(void* smem_dst, const void* tmap, ui
 __device__ __forceinline__ void tma_prefetch_3d(const void* tmap, int x, int y, int z) {
   asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(tmap), "r"(x), "r"(y), "r"(z) : "memory");
 }
+// A tile from shared memory to global memory, as a bulk group of this thread's; bulk_wait_read: the groups before have read their
+// shared memory, bulk_wait: they are complete.
+__device__ __forceinline__ void tma_store_3d(const void* tmap, const void* smem_src, int c0, int c1, int c2) {
+  asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.tile.bulk_group [%0, {%2, %3, %4}], [%1];\n\tcp.async.bulk.commit_group;"
+               ::"l"(tmap), "r"(smem_u32(smem_src)), "r"(c0), "r"(c1), "r"(c2) : "memory");
+}
+__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 __device__ __forceinline__ void tma_prefetch_desc(const void* tmap) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(tmap) : "memory");
 }
@@ -389,6 +397,18 @@ __device__ __forceinline__ void publish_flag(int* p, int v) {
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&v);
+}
+
+// 32 bytes of a row: one store where the row is aligned to 32 bytes, else two.  (A warp that stores one row per lane takes a pass of
+// the load/store pipe per lane and instruction, whatever the width.)
+__device__ __forceinline__ void store_32(void* p, const uint4 (&x)[2], bool aligned32) {
+  if (aligned32) {
+    asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
+                 ::"l"(p), "r"(x[0].x), "r"(x[0].y), "r"(x[0].z), "r"(x[0].w), "r"(x[1].x), "r"(x[1].y), "r"(x[1].z), "r"(x[1].w) : "memory");
+  } else {
+    reinterpret_cast<uint4*>(p)[0] = x[0];
+    reinterpret_cast<uint4*>(p)[1] = x[1];
+  }
 }
 
 // A descriptor with its start-address field set to a shared-memory address (the field is 14 bits of address >> 4).

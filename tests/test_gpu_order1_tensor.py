@@ -139,3 +139,19 @@ def test_more_tickets_than_sms():
     g = run("state_scan", *dev_tensors(w), C=128, scan_group=2)
     for b, h in ((0, 0), (0, 15), (1, 7), (1, 15)):
         check(g[b, h], reference(w, b, h), "bf16", f"order 1, 384 tickets ({b},{h})")
+
+
+@pytest.mark.parametrize("H,T", [(1, 1), (2, 31), (1, 33), (1, 129), (3, 255), (1, 1000), (20, 4097)])
+def test_rows_beyond_the_sequence_are_not_written(H, T):
+    """The outputs leave in blocks of 32 rows; what lies behind a head's last row is the next head's, or not the call's at all."""
+    import torch
+    gen = torch.Generator(device="cuda").manual_seed(T)
+    q, k = (torch.rand(1, H, T, 64, device="cuda", generator=gen).bfloat16() for _ in range(2))
+    v = torch.randn(1, H, T, 64, device="cuda", generator=gen).bfloat16()
+    buf = torch.full((H * T * 64 + 4096,), 7.0, dtype=torch.bfloat16, device="cuda")
+    out = buf[:H * T * 64].view(1, H, T, 64)
+    kb.kata_chunk_state_scan(q, k, v, out=out, feature_order=1, C=128)
+    assert torch.all(buf[H * T * 64:] == 7.0)
+    one = torch.cat([kb.kata_chunk_state_scan(*(x[:, h:h + 1].contiguous() for x in (q, k, v)), feature_order=1, C=128, scan_group=10 ** 6)
+                     for h in range(H)], 1)
+    assert torch.allclose(out.float(), one.float(), rtol=2e-2, atol=2e-2)
