@@ -126,6 +126,7 @@ struct BArgs {
   const float* rk;           // [BH][T]: 1 / ||k_i||^2
   const float* row_scale;    // NS = 3: [BH][T] power of two that the row of q (MODE_DQ) or k (MODE_DKV) was scaled by
   int* device_status;
+  int wide_out;              // rows of the gradients are 32-byte aligned
   int Tlen;
   int BH;
 };
@@ -694,13 +695,13 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ 
       tc_fence_after();
       auto store32 = [&](__nv_bfloat16* dst, const float (&x)[32]) {
 #pragma unroll
-        for (int c = 0; c < 32; c += 8) {
-          uint4 pkt;
-          pkt.x = pack_bf16(x[c], x[c + 1]);
-          pkt.y = pack_bf16(x[c + 2], x[c + 3]);
-          pkt.z = pack_bf16(x[c + 4], x[c + 5]);
-          pkt.w = pack_bf16(x[c + 6], x[c + 7]);
-          *reinterpret_cast<uint4*>(dst + c) = pkt;
+        for (int c = 0; c < 32; c += 16) {
+          uint4 pkt[2];
+#pragma unroll
+          for (int e = 0; e < 2; ++e)
+            pkt[e] = make_uint4(pack_bf16(x[c + 8 * e], x[c + 8 * e + 1]), pack_bf16(x[c + 8 * e + 2], x[c + 8 * e + 3]),
+                                pack_bf16(x[c + 8 * e + 4], x[c + 8 * e + 5]), pack_bf16(x[c + 8 * e + 6], x[c + 8 * e + 7]));
+          store_32(dst + c, pkt, args.wide_out);
         }
       };
       const size_t row_off = ((size_t)cur.bh * args.Tlen + grow) * D;
@@ -915,9 +916,10 @@ void run_bwd(Problem p, const void* dout, void* dq, void* dk, void* dv, const Bw
     ctx.status = KATA_ERR_CUDA;
     return;
   }
-  BArgs a{static_cast<__nv_bfloat16*>(dq), nullptr, w.stats, w.rk, w.fq, device_status, p.T, BH};
+  const int wide = ((reinterpret_cast<uintptr_t>(dq) | reinterpret_cast<uintptr_t>(dk) | reinterpret_cast<uintptr_t>(dv)) & 31) == 0;
+  BArgs a{static_cast<__nv_bfloat16*>(dq), nullptr, w.stats, w.rk, w.fq, device_status, wide, p.T, BH};
   if (!launch_bwd<MODE_DQ, G, NS>(qf, gf, ks, vs, a, ctx)) return;
-  BArgs b{static_cast<__nv_bfloat16*>(dk), static_cast<__nv_bfloat16*>(dv), w.stats, w.rk, w.fk, device_status, p.T, BH};
+  BArgs b{static_cast<__nv_bfloat16*>(dk), static_cast<__nv_bfloat16*>(dv), w.stats, w.rk, w.fk, device_status, wide, p.T, BH};
   launch_bwd<MODE_DKV, G, NS>(kf, vf, qs, gs, b, ctx);
 }
 

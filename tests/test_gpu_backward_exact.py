@@ -105,3 +105,17 @@ def test_ends_of_the_range(T, impl):
         full = to_numpy64(got[0, 0])
         err = np.abs(full[rows] - r)
         assert np.all(err <= 2.0 ** -8 * np.abs(r) + 1e-5 * np.abs(full).max()), (name, T, float(err.max()))
+
+
+@pytest.mark.parametrize("fn,T", [("kata_bwd_quadratic", 300), ("kata_bwd_chunked", 600)])
+@pytest.mark.parametrize("which", [0, 1, 2])
+def test_gradients_aligned_to_16_bytes_only(fn, T, which):
+    """Gradient rows leave 32 bytes at a time where all three tensors allow it, 16 otherwise: the same bits."""
+    import torch
+    gen = torch.Generator(device="cuda").manual_seed(T)
+    x = [torch.randn(1, 3, T, 64, device="cuda", generator=gen).bfloat16() for _ in range(4)]
+    want = getattr(kb, fn)(*x)
+    out = [torch.empty(3 * T * 64 + 8, dtype=torch.bfloat16, device="cuda")[8 * (i == which):][:3 * T * 64].view(1, 3, T, 64) for i in range(3)]
+    assert out[which].data_ptr() % 32 == 16
+    getattr(kb, fn)(*x, *out)
+    assert all(torch.equal(a, b) for a, b in zip(want, out))
