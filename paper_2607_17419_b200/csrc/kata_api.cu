@@ -183,18 +183,23 @@ int make_plan(int fn, const Problem& p, const Opts& o, bool tensor, int C, ScanP
     } else {
       // One pass per head, or the groups of the single-launch scan (every group walked twice, the second time with
       // its keys and values in L2 only where the groups of all CTAs fit there: up to 1.5x the HBM traffic),
-      // whichever the cost model says is faster.  Measured on B200: a CTA alone walks its tiles at about 1.25 us a
-      // tile in one pass and 2.15 us a tile for the two passes of a group, a group costs about 12 us on top (two
-      // pipeline ramps and the look-back), the kernel streams about 6 GB/ms.  Groups: one per CTA in one wave.
-      const double n_tiles = (double)((p.T + tc_order1_tile() - 1) / tc_order1_tile());
-      const double hbm_us = (double)BH * n_tiles * 65536.0 / 6.0e6;
-      const double one_pass = fmax(hbm_us, ceil(BH / 148.0) * n_tiles * 1.25);
+      // whichever the model says is faster, with at most one group per CTA in one wave.  Fitted to B200, us: a CTA walks its
+      // tiles at 0.9 to 1.1 us a tile in one pass and about 1.35 for the two passes of a group, whose pipeline ramps and
+      // look-back take 17, and every anchor that the chain has to pass after the first takes 6 more, so that few long heads
+      // are best off with fewer groups than CTAs.  Measured, us, one group per CTA / as modelled now: one head x 131072 tokens
+      // (147 groups / 41) 152 / 80, two x 131072 (74 / 37) 114 / 88, two x 65536 (74 / 25) 86 / 60, four x 32768 (37 / 16) 56 / 48;
+      // one pass / groups: 40 x 4096 35.6 / 33.2, 50 x 8192 68.4 / 66.3, 64 x 8192 70.4 / 72.5, 64 x 32768 253 / 236.
+      const int n_tiles = (p.T + tc_order1_tile() - 1) / tc_order1_tile();
+      const double gb = (double)BH * n_tiles * 65536.0 * 1e-6;                  // q, k, v, out once
+      double best = fmax(gb / 6.0, ceil(BH / 148.0) * n_tiles * (0.88 + 0.0018 * (BH < 148 ? BH : 148)) + 3.0);
       G = NC;
-      const int ng = 148 / BH;
-      if (ng >= 2 && n_tiles >= 2 * ng) {
-        const double tiles_per_group = ceil(n_tiles / ng);
-        const double grouped = fmax(1.5 * hbm_us, tiles_per_group * 2.15) + 12.0;
-        if (grouped < one_pass) G = (int)tiles_per_group * cpt;
+      for (int ng = 2; ng <= 148 / BH && 2 * ng <= n_tiles; ++ng) {
+        const int tiles = (n_tiles + ng - 1) / ng, groups = (n_tiles + tiles - 1) / tiles;
+        const double us = fmax(1.5 * gb / 7.0 + 10.0, 1.35 * tiles + 17.0) + 6.0 * ((groups - 2) / 8) + 0.02 * tiles;
+        if (us < best) {
+          best = us;
+          G = tiles * cpt;
+        }
       }
     }
     if (G > NC) G = NC;
