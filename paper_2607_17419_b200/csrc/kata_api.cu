@@ -166,7 +166,8 @@ bool tensor_scan_pays(int BH, int NC) {
 }
 
 // How the chunk axis is cut into scan groups, and how many floats one group state takes.
-int make_plan(int fn, const Problem& p, const Opts& o, bool tensor, int C, ScanPlan& plan, size_t& state_elems) {
+// small: the caller brings less scratch than the plan needs (see prepare).
+int make_plan(int fn, const Problem& p, const Opts& o, bool tensor, int C, bool small, ScanPlan& plan, size_t& state_elems) {
   plan.n_chunks = (p.T + C - 1) / C;
   const int NC = plan.n_chunks;
   const int BH = p.B * p.H;
@@ -193,7 +194,12 @@ int make_plan(int fn, const Problem& p, const Opts& o, bool tensor, int C, ScanP
       const double gb = (double)BH * n_tiles * 65536.0 * 1e-6;                  // q, k, v, out once
       double best = fmax(gb / 6.0, ceil(BH / 148.0) * n_tiles * (0.88 + 0.0018 * (BH < 148 ? BH : 148)) + 3.0);
       G = NC;
-      for (int ng = 2; ng <= 148 / BH && 2 * ng <= n_tiles; ++ng) {
+      // (calls whose published scratch was that of one pass, by the line drawn when a group cost 2.15 us a tile and 12, keep to it
+      // where they bring no more)
+      const int per_cta = 148 / BH;
+      const bool one_pass_scratch = per_cta < 2 || n_tiles < 2 * per_cta ||
+                                    fmax(1.5 * gb / 6.0, ceil((double)n_tiles / per_cta) * 2.15) + 12.0 >= fmax(gb / 6.0, n_tiles * 1.25);
+      for (int ng = 2; ng <= per_cta && 2 * ng <= n_tiles && !(small && one_pass_scratch); ++ng) {
         const int tiles = (n_tiles + ng - 1) / ng, groups = (n_tiles + tiles - 1) / tiles;
         const double us = fmax(1.5 * gb / 7.0 + 10.0, 1.35 * tiles + 17.0) + 6.0 * ((groups - 2) / 8) + 0.02 * tiles;
         if (us < best) {
@@ -368,7 +374,8 @@ Problem kernel_problem(const Prepared& r) {
 
 // small_scratch: kernels that need less scratch, for a caller who brings less than kata_workspace_bytes says.  From 1: the
 // streaming kernels for a state handed in or out and for the scan form, the walk over the chunks in fp32 (no scratch, or that of
-// the scan passes), and chunks of 1024 tokens where shorter ones would be quicker.  2: the sequential form for AUTO as well.
+// the scan passes), chunks of 1024 tokens where shorter ones would be quicker, and one pass per head for first-order features
+// where that was once the plan.  2: the sequential form for AUTO as well.
 int prepare(int fn, const void* q, const void* k, const void* v, void* out, int B, int H, int T, int d_k,
             int d_v, int C, const kata_opts* opts, bool need_ptrs, Prepared& r, int small_scratch = 0) {
   int st = read_opts(opts, r.o);
@@ -421,7 +428,7 @@ int prepare(int fn, const void* q, const void* k, const void* v, void* out, int 
     if (r.tensor && r.o.s_pre != nullptr && fn == KATA_FN_CHUNK_STATE_SCAN) r.tensor = false;   // per-chunk export: SIMT pipeline
     // C = 128 (the chunk size of the paper's scan benchmark) exists on the first-order tensor-core path only
     if (r.C != kChunk && !(r.tensor && r.p.feature_order == 1)) return KATA_ERR_UNSUPPORTED_SHAPE;
-    st = make_plan(fn, kp, r.o, r.tensor, r.C, r.plan, r.state_elems);
+    st = make_plan(fn, kp, r.o, r.tensor, r.C, small_scratch > 0, r.plan, r.state_elems);
     if (st != KATA_OK) return st;
     r.inner_bytes = inner_workspace(fn, r.plan, kp, r.state_elems);
     const bool state_in = r.o.s_init != nullptr, state_out = r.o.s_pre != nullptr;

@@ -61,3 +61,29 @@ def test_small_scratch(what, dtype, H, T, d, launches):
         torch.cuda.synchronize()
         diff = (o2.float() - full.float()).norm() / full.float().norm()
         assert float(diff) <= 2e-2
+
+
+@pytest.mark.parametrize("H,T", [(50, 8192), (1, 16384), (2, 4097)])
+def test_first_order_with_the_scratch_of_one_pass(H, T):
+    """Sizes that are walked in groups now and were one pass per head: the scratch of one pass is still enough, and less is not."""
+    import torch
+    q, k = (torch.rand(1, H, T, 64, device="cuda").bfloat16() for _ in range(2))
+    v = torch.randn(1, H, T, 64, device="cuda").bfloat16()
+    o = kb.make_opts(kb.KATA_BF16, feature_order=1)
+    one = kb.make_opts(kb.KATA_BF16, feature_order=1, scan_group=10 ** 6)
+    need, least = (kb.kata_workspace_bytes(kb.KATA_FN_CHUNK_STATE_SCAN, 1, H, T, 64, 64, 128, x) for x in (o, one))
+    assert kb.kata_scan_plan(kb.KATA_FN_CHUNK_STATE_SCAN, 1, H, T, 64, 64, 128, o)[0] > 1 and need > least > 0
+    want = kb.kata_chunk_state_scan(q, k, v, feature_order=1, C=128)
+
+    class Fixed:
+        def __init__(self, n):
+            self.buf = torch.empty(n, dtype=torch.uint8, device="cuda")
+
+        def get(self, nbytes, device):
+            return self.buf.data_ptr(), self.buf.numel()
+
+    got = kb.kata_chunk_state_scan(q, k, v, feature_order=1, C=128, workspace=Fixed(least))
+    assert torch.allclose(got.float(), want.float(), rtol=2e-2, atol=2e-2)
+    with pytest.raises(kb.KataError) as e:
+        kb.kata_chunk_state_scan(q, k, v, feature_order=1, C=128, workspace=Fixed(least - 256))
+    assert e.value.status == kb.KATA_ERR_WORKSPACE_TOO_SMALL
