@@ -182,7 +182,6 @@ void tc_rscale(const Problem& p, const KeyScales& r, LaunchCtx& ctx);
 // States before the chunks (kata_tc_state.cu), for tc_attend.
 struct StatePlan {
   int chunk_tokens;            // a multiple of 256
-  bool quad;                   // the outputs by the quadratic form: no block reads a state
   int n_chunks;
   int segments, seg_chunks;    // segments of the chunk axis walked side by side
 };

@@ -7,7 +7,6 @@
 //   pass 2  inclusive scan over the group states (scan_round_kernel, fp32 adds)
 //   pass 3  every group starts from the prefix before it and writes its outputs
 #include "kata_common.cuh"
-#include <cstdlib>
 
 namespace kata {
 
@@ -52,9 +51,7 @@ StatePlan tc_chunk_plan(const Problem& p, bool state_in, bool state_out, bool sm
   const int quad_tokens = tc_narrow(p) ? (BH < 64 ? 4352 : 3584) : p.groups == 1 ? 7168 : p.groups == 2 ? 3072 : 1536;
   StatePlan plan{};
   int L = 1024;
-  static const int kq = getenv("KQ") ? atoi(getenv("KQ")) : 0;
-  plan.quad = !state_in && p.T <= (state_out ? kq : quad_tokens);
-  if (plan.quad && (!state_out || BH * slices > 74)) L = (p.T + 255) / 256 * 256;
+  if (!state_in && !state_out && p.T <= quad_tokens) L = (p.T + 255) / 256 * 256;
   else if (!small_scratch && (long long)BH * slices * ((p.T + L - 1) / L) < 148) L = 512;
   plan.chunk_tokens = L;
   plan.n_chunks = (p.T + L - 1) / L;
@@ -96,7 +93,7 @@ void tc_chunked_states(const Problem& p, const StatePlan& plan, void* workspace,
     if (ctx.status == KATA_OK) tc_states(p, r.f32, plan, buf, device_status, ctx);
     at.s = buf.s;
     at.z = buf.z;
-    at.n_chunks = plan.quad ? 0 : plan.n_chunks;
+    at.n_chunks = plan.n_chunks;
     at.chunk_tokens = plan.chunk_tokens;
     at.first_state = s_init != nullptr ? 0 : 1;
   }

@@ -201,6 +201,13 @@ def test_no_oracle_in_product_path():
                 assert "kata_oracle" not in text and "oracle/" not in text, f
 
 
+def test_environment_switches_are_the_documented_ones():
+    """What a call does depends on its arguments alone, except for the variables that the header names."""
+    csrc, header = os.path.join(ROOT, "paper_2607_17419_b200", "csrc"), open(os.path.join(ROOT, "include", "kata.h")).read()
+    read = {name for f in os.listdir(csrc) for name in re.findall(r'getenv\(\s*"(\w+)"', open(os.path.join(csrc, f)).read())}
+    assert read and all(name in header for name in read), read
+
+
 def test_decode_step_argument_checks(L):
     INV, SHAPE, ALIGN, WS = -1, -2, -3, -4
     def dec(q=4096, k=4096, v=4096, out=4096, S=4096, Z=4096, B=2, H=2, dk=64, dv=64, opts=None):
