@@ -13,9 +13,12 @@ import ctypes
 import functools
 import os
 import threading
+import warnings
 from typing import Optional
 
 import torch
+
+from . import build
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(HERE, "libkata.so")
@@ -111,16 +114,36 @@ def lib() -> ctypes.CDLL:
 _native = None
 
 
+class _CtypesOnly:
+    """In the native module's place where it cannot be used: every call is left to this file."""
+
+    @staticmethod
+    def forward(*args):
+        return NotImplemented
+
+    decode = backward = forward
+
+
 def native():
-    """The native module with the tensor calls, or NotImplemented from it for a call that is left to this file (loaded once)."""
+    """The native module with the tensor calls (loaded once); each returns NotImplemented for a call that is left to this file.
+    Where the module is missing, does not load or was built for another torch or Python, all calls are, with one warning."""
     global _native
     if _native is None:
         lib()
-        try:
-            from . import _kata_torch
-        except ImportError as e:
-            raise RuntimeError(f"_kata_torch.so does not load ({e}): build it with `python -m paper_2607_17419_b200.build`") from e
-        _native = _kata_torch
+        why = None
+        if build.host_current():
+            try:
+                from . import _kata_torch
+                _native = _kata_torch
+            except ImportError as e:
+                why = f"does not load ({e})"
+        elif os.path.exists(build.HOST):
+            why = "was built for another torch or Python"
+        else:
+            why = "is missing"
+        if why is not None:
+            warnings.warn(f"_kata_torch.so {why}: calls take some 5 us more on the host; `python -m paper_2607_17419_b200.build` builds it")
+            _native = _CtypesOnly
     return _native
 
 

@@ -265,4 +265,7 @@ PyModuleDef kModule = {PyModuleDef_HEAD_INIT, "_kata_torch", nullptr, -1, kMetho
 
 }  // namespace
 
+// The torch and the Python that this was compiled against; the binding looks for it in the file and loads no other.
+extern "C" __attribute__((visibility("default"), used)) const char kata_host_tag[] = KATA_HOST_TAG;
+
 PyMODINIT_FUNC PyInit__kata_torch(void) { return PyModule_Create(&kModule); }
