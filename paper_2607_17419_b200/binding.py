@@ -310,6 +310,50 @@ class _StreamScratch(threading.local):
 _default_scratch = _StreamScratch()
 
 
+def _on(t, device) -> bool:
+    """Whether kernels on the device can address the tensor."""
+    return t.device == device or (t.device.type == "cpu" and t.is_pinned())
+
+
+def _check_room(q, heads: int, inputs, outputs, state=(), host_io: bool = False):
+    """ValueError for a tensor that the kernels, which take sizes, type and device from q (and d_v from v), would read or write
+    beyond its end or misread.  Each group holds (name, tensor or None, elements that the call touches).  Inputs have that many
+    elements, in any shape; with one head, where nothing lies behind them, they may have more, as outputs and state may."""
+    for group, dtype in ((inputs, q.dtype), (outputs, q.dtype), (state, torch.float32)):
+        for name, t, n in group:
+            if not isinstance(t, torch.Tensor):
+                continue
+            size = t.numel()
+            if size != n and (size < n or (group is inputs and heads > 1)):
+                raise ValueError(f"{name} has {size} elements, the call needs {n}")
+            if t.dtype is not dtype:
+                raise ValueError(f"{name} is {t.dtype}, the call needs {dtype}")
+            if not host_io and not _on(t, q.device):
+                raise ValueError(f"{name} is on {t.device}, q on {q.device}")
+            if not t.is_contiguous():
+                raise ValueError(f"{name} must be contiguous")
+
+
+def _check_forward(fn: int, q, k, v, out, C, host_io=False, s_pre=None, z_pre=None, s_init=None, z_init=None, device_status=None,
+                   feature_order=2, state_layout=KATA_LAYOUT_DIRECT, feature_groups=0, **_):
+    B, H, T, d_k = q.shape
+    d_v, heads = v.shape[-1], B * H
+    state = ()
+    if s_pre is not None or z_pre is not None or s_init is not None or z_init is not None:
+        rows = heads * decode_n_psi(d_k, feature_order, state_layout, feature_groups)
+        rows_pre = rows * -(-T // C) if fn == KATA_FN_CHUNK_STATE_SCAN and C > 0 else rows
+        state = (("s_pre", s_pre, rows_pre * d_v), ("z_pre", z_pre, rows_pre), ("s_init", s_init, rows * d_v), ("z_init", z_init, rows))
+    _check_room(q, heads, (("k", k, heads * T * d_k), ("v", v, heads * T * d_v)), (("out", out, heads * T * d_v),), state, host_io)
+    if isinstance(device_status, torch.Tensor) and (device_status.nbytes < 4 or not (host_io or _on(device_status, q.device))):
+        raise ValueError("device_status is one int32 on the device of q")
+
+
+def _check_backward(q, k, v, dout, dq, dk, dv):
+    B, H, T, d_k = q.shape
+    nk, nv = B * H * T * d_k, B * H * T * v.shape[-1]
+    _check_room(q, B * H, (("k", k, nk), ("v", v, nv), ("dout", dout, nv)), (("dq", dq, nk), ("dk", dk, nk), ("dv", dv, nv)))
+
+
 def _call(fn: int, q, k, v, out, C: int, *, host_io: bool = False, workspace: Optional[Workspace] = None,
           s_pre=None, z_pre=None, s_init=None, z_init=None, device_status=None, stream=None, **opt_kw):
     if workspace is None and stream is None and not host_io:
@@ -322,6 +366,7 @@ def _call(fn: int, q, k, v, out, C: int, *, host_io: bool = False, workspace: Op
         raise ValueError("q, k, v must be contiguous [B,H,T,d]")
     B, H, T, d_k = q.shape
     d_v = v.shape[-1]
+    _check_forward(fn, q, k, v, out, C, host_io, s_pre, z_pre, s_init, z_init, device_status, **opt_kw)
     if out is None:
         out = torch.empty_like(v)
     dev = torch.device("cuda", torch.cuda.current_device()) if host_io else q.device
@@ -392,6 +437,8 @@ def kata_decode_step(q, k, v, S, Z, out=None, *, workspace: Optional[Workspace] 
         raise ValueError("q, k, v, S, Z must be contiguous")
     if S.dtype != torch.float32 or Z.dtype != torch.float32:
         raise ValueError("the state is fp32")
+    _check_room(q, B * H, (("k", k, B * H * d_k), ("v", v, B * H * d_v)), (("out", out, B * H * d_v),),
+                (("S", S, 0), ("Z", Z, 0)))               # (the sizes of the state: below)
     if out is None:
         out = torch.empty_like(v)
     if stream is None:
@@ -422,6 +469,7 @@ def kata_bwd_quadratic(q, k, v, dout, dq=None, dk=None, dv=None, *, workspace: O
         raise ValueError("q, k, v, dout must be contiguous [B,H,T,d]")
     B, H, T, d_k = q.shape
     d_v = v.shape[-1]
+    _check_backward(q, k, v, dout, dq, dk, dv)
     dq = torch.empty_like(q) if dq is None else dq
     dk = torch.empty_like(k) if dk is None else dk
     dv = torch.empty_like(v) if dv is None else dv
@@ -450,6 +498,7 @@ def kata_bwd_chunked(q, k, v, dout, dq=None, dk=None, dv=None, C: int = 64, *, w
         raise ValueError("q, k, v, dout must be contiguous [B,H,T,d]")
     B, H, T, d_k = q.shape
     d_v = v.shape[-1]
+    _check_backward(q, k, v, dout, dq, dk, dv)
     dq = torch.empty_like(q) if dq is None else dq
     dk = torch.empty_like(k) if dk is None else dk
     dv = torch.empty_like(v) if dv is None else dv
@@ -476,6 +525,9 @@ def kata_chunk_state_scan_static(q, k, v, out, C: int = 64, *, scan_group: int =
     """
     B, H, T, d_k = q.shape
     d_v = v.shape[-1]
+    if not (q.is_contiguous() and k.is_contiguous() and v.is_contiguous()):
+        raise ValueError("q, k, v must be contiguous [B,H,T,d]")
+    _check_forward(KATA_FN_CHUNK_STATE_SCAN, q, k, v, out, C)
     if stream is None:
         stream = _stream(q.device)
     opts = make_opts(_dtype_code(q), stream=stream, scan_group=scan_group, impl=impl, feature_order=feature_order)

@@ -115,6 +115,14 @@ bool stream_and_scratch(PyObject* owner, const at::Tensor& q, int fn, int B, int
   return false;
 }
 
+// Room for what the kernels read or write behind a pointer, which take sizes, type and device from q (binding.py _check_room).
+bool has_room(const at::Tensor& t, const at::Tensor& q, at::ScalarType type, int64_t n) {
+  return t.numel() >= n && t.scalar_type() == type && t.device() == q.device() && t.is_contiguous();
+}
+bool input_fits(const at::Tensor& t, const at::Tensor& q, int64_t heads, int64_t n) {
+  return has_room(t, q, q.scalar_type(), n) && (t.numel() == n || heads == 1);
+}
+
 // The result of a call: the tensors, or the status as an int.
 PyObject* result(int status, std::initializer_list<const at::Tensor*> out) {
   if (status != KATA_OK) return PyLong_FromLong(status);
@@ -132,22 +140,27 @@ PyObject* result(int status, std::initializer_list<const at::Tensor*> out) {
   return tuple;
 }
 
-// The tensor that was passed for an output, or a new one like `like`; false: one that is not plain.
-bool output(PyObject* o, const at::Tensor& like, at::Tensor& t) {
-  if (o == Py_None) {
-    t = at::empty_like(like);
-    return true;
-  }
+// The tensor that was passed for an output of n elements, or a new one like `like`; false: one that is not plain, or too small.
+bool output_ok(PyObject* o, const at::Tensor& q, int64_t n) {
+  if (o == Py_None) return true;
   const at::Tensor* p = plain(o);
-  if (p != nullptr) t = *p;
-  return p != nullptr;
+  return p != nullptr && has_room(*p, q, q.scalar_type(), n);
 }
-bool pointer(PyObject* o, void*& p) {
+at::Tensor output(PyObject* o, const at::Tensor& like) { return o == Py_None ? at::empty_like(like) : THPVariable_Unpack(o); }
+
+bool pointer(PyObject* o, const at::Tensor& q, at::ScalarType type, int64_t n, void*& p) {
   p = nullptr;
   if (o == Py_None) return true;
   const at::Tensor* t = plain(o);
-  if (t != nullptr) p = t->data_ptr();
-  return t != nullptr;
+  if (t == nullptr || !has_room(*t, q, type, n)) return false;
+  p = t->data_ptr();
+  return true;
+}
+
+// Feature rows of a state (binding.py decode_n_psi).
+int64_t state_rows(const kata_opts& o, int d_k) {
+  const int g = o.feature_groups > 1 ? o.feature_groups : 1, m = d_k / g;
+  return o.feature_order == 1 ? d_k : (int64_t)g * (o.state_layout == KATA_LAYOUT_PACKED ? (int64_t)m * (m + 1) / 2 : (int64_t)m * m);
 }
 
 // forward(fn, scratch owner, q, k, v, out, C, s_pre, z_pre, s_init, z_init, device_status, options)
@@ -165,8 +178,14 @@ PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n) {
   if (!int_size(q->size(0), B) || !int_size(q->size(1), H) || !int_size(q->size(2), T) || !int_size(q->size(3), d_k) ||
       !int_size(v->size(-1), d_v))
     return not_implemented();
+  const int64_t heads = (int64_t)B * H, nv = heads * T * d_v;
+  if (!input_fits(*k, *q, heads, q->numel()) || !input_fits(*v, *q, heads, nv) || !output_ok(a[5], *q, nv)) return not_implemented();
   void *s_pre, *z_pre, *s_init, *z_init, *device_status;
-  if (!pointer(a[7], s_pre) || !pointer(a[8], z_pre) || !pointer(a[9], s_init) || !pointer(a[10], z_init) || !pointer(a[11], device_status))
+  const int64_t rows = heads * state_rows(o, d_k);
+  const int64_t rows_pre = fn == KATA_FN_CHUNK_STATE_SCAN && c_arg > 0 ? rows * ((T + c_arg - 1) / c_arg) : rows;
+  if (!pointer(a[7], *q, at::kFloat, rows_pre * d_v, s_pre) || !pointer(a[8], *q, at::kFloat, rows_pre, z_pre) ||
+      !pointer(a[9], *q, at::kFloat, rows * d_v, s_init) || !pointer(a[10], *q, at::kFloat, rows, z_init) ||
+      !pointer(a[11], *q, at::kInt, 1, device_status))
     return not_implemented();
   o.s_pre = static_cast<float*>(s_pre);
   o.z_pre = static_cast<float*>(z_pre);
@@ -176,8 +195,7 @@ PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n) {
   PyObject* held;
   if (!stream_and_scratch(a[1], *q, fn, B, H, T, d_k, d_v, (int)c_arg, o, held)) return not_implemented();
   const Held hold{held};
-  at::Tensor out;
-  if (!output(a[5], *v, out)) return not_implemented();
+  const at::Tensor out = output(a[5], *v);
   const auto call = fn == KATA_FN_QUADRATIC ? kata_fwd_quadratic : fn == KATA_FN_CHUNKED ? kata_fwd_chunked : kata_chunk_state_scan;
   const void *qp = q->data_ptr(), *kp = k->data_ptr(), *vp = v->data_ptr();
   void* op = out.data_ptr();
@@ -201,15 +219,16 @@ PyObject* decode(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return not_implemented();
   int B, H, d_k, d_v;
   if (!int_size(q->size(0), B) || !int_size(q->size(1), H) || !int_size(q->size(2), d_k) || !int_size(v->size(-1), d_v)) return not_implemented();
-  const int g = o.feature_groups > 1 ? o.feature_groups : 1, m = d_k / g;
-  const int64_t rows = o.feature_order == 1 ? d_k : (int64_t)g * (o.state_layout == KATA_LAYOUT_PACKED ? (int64_t)m * (m + 1) / 2 : (int64_t)m * m);
+  const int64_t heads = (int64_t)B * H, rows = state_rows(o, d_k);
+  if (!input_fits(*k, *q, heads, q->numel()) || !input_fits(*v, *q, heads, heads * d_v) || !output_ok(a[6], *q, heads * d_v) ||
+      S->device() != q->device() || Z->device() != q->device())
+    return not_implemented();
   if (S->size(0) != B || S->size(1) != H || S->size(2) != rows || S->size(3) != d_v || Z->size(0) != B || Z->size(1) != H || Z->size(2) != rows)
     return not_implemented();
   PyObject* held;
   if (!stream_and_scratch(a[0], *q, KATA_FN_DECODE_STEP, B, H, 1, d_k, d_v, 0, o, held)) return not_implemented();
   const Held hold{held};
-  at::Tensor out;
-  if (!output(a[6], *v, out)) return not_implemented();
+  const at::Tensor out = output(a[6], *v);
   const void *qp = q->data_ptr(), *kp = k->data_ptr(), *vp = v->data_ptr();
   void *op = out.data_ptr(), *sp = S->data_ptr(), *zp = Z->data_ptr();
   int st;
@@ -237,15 +256,14 @@ PyObject* backward(PyObject*, PyObject* const* a, Py_ssize_t n) {
   if (!int_size(q->size(0), B) || !int_size(q->size(1), H) || !int_size(q->size(2), T) || !int_size(q->size(3), d_k) ||
       !int_size(v->size(-1), d_v))
     return not_implemented();
+  const int64_t heads = (int64_t)B * H, nk = q->numel(), nv = heads * T * d_v;
+  if (!input_fits(*k, *q, heads, nk) || !input_fits(*v, *q, heads, nv) || !input_fits(*dout, *q, heads, nv) || !output_ok(a[6], *q, nk) ||
+      !output_ok(a[7], *q, nk) || !output_ok(a[8], *q, nv))
+    return not_implemented();
   PyObject* held;
   if (!stream_and_scratch(a[1], *q, fn, B, H, T, d_k, d_v, (int)c_arg, o, held)) return not_implemented();
   const Held hold{held};
-  at::Tensor dq, dk, dv;
-  if ((a[6] != Py_None && plain(a[6]) == nullptr) || (a[7] != Py_None && plain(a[7]) == nullptr) || (a[8] != Py_None && plain(a[8]) == nullptr))
-    return not_implemented();
-  output(a[6], *q, dq);
-  output(a[7], *k, dk);
-  output(a[8], *v, dv);
+  const at::Tensor dq = output(a[6], *q), dk = output(a[7], *k), dv = output(a[8], *v);
   const void *qp = q->data_ptr(), *kp = k->data_ptr(), *vp = v->data_ptr(), *gp = dout->data_ptr();
   void *dqp = dq.data_ptr(), *dkp = dk.data_ptr(), *dvp = dv.data_ptr();
   int st;

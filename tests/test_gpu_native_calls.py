@@ -104,6 +104,18 @@ def bad_calls():
         lambda s: kb.kata_bwd_quadratic(q, k, v, g.transpose(1, 2), **s),
         lambda s: kb.kata_bwd_chunked(q, k, v, g, C=128, **s),
         lambda s: kb.kata_bwd_quadratic(q, k, v, torch.stack([g, g])[:, 0, 0], out=None, **s),
+        # tensors that the kernels would run over the end of, or misread (refused before the library is called)
+        lambda s: kb.kata_fwd_quadratic(q, k[:, :, :50].contiguous(), v, **s),
+        lambda s: kb.kata_fwd_chunked(q, k, v.float(), **s),
+        lambda s: kb.kata_fwd_chunked(q, k, v, out=torch.empty(1, 2, 99, 64, dtype=torch.bfloat16, device="cuda"), **s),
+        lambda s: kb.kata_fwd_chunked(q, k, v, out=torch.empty(1, 100, 2, 64, dtype=torch.bfloat16, device="cuda").transpose(1, 2), **s),
+        lambda s: kb.kata_fwd_chunked(q, k, v, out=torch.empty_like(v, device="cpu"), **s),
+        lambda s: kb.kata_fwd_chunked(q, k, v, s_pre=S[:, :1].contiguous(), z_pre=Z, **s),
+        lambda s: kb.kata_chunk_state_scan(q, k, v, s_pre=S, z_pre=Z, **s),
+        lambda s: kb.kata_decode_step(t[0], t[1][:, :1].contiguous(), t[2], S, Z, **s),
+        lambda s: kb.kata_decode_step(*t, S, Z, out=torch.empty(1, 2, 32, dtype=torch.bfloat16, device="cuda"), **s),
+        lambda s: kb.kata_bwd_quadratic(q, k, v, g[:, :, :50].contiguous(), **s),
+        lambda s: kb.kata_bwd_chunked(q, k, v, g, dk=torch.empty(1, 2, 50, 64, dtype=torch.bfloat16, device="cuda"), **s),
     ]
 
 
