@@ -91,7 +91,11 @@ bool stream_and_scratch(PyObject* owner, const at::Tensor& q, int fn, int B, int
   if (need == 0) return true;
   if (stream != nullptr) {
     cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(stream, &status) != cudaSuccess || status != cudaStreamCaptureStatusNone) return false;
+    if (cudaStreamIsCapturing(stream, &status) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    if (status != cudaStreamCaptureStatusNone) return false;
   }
   static PyObject* const name = PyUnicode_InternFromString("bufs");
   PyObject* bufs = PyObject_GetAttr(owner, name);
