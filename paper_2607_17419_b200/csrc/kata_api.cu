@@ -81,9 +81,9 @@ int check_shape(int fn, int B, int H, int T, int d_k, int d_v, int C) {
 // Lengths of that route.  They are set by the entry's contract, not by speed: shorter calls are the plain FMA kernels' (and
 // refused with impl = KATA_IMPL_TENSOR), and beyond 16384 tokens the entry keeps the O(T) work that it is called for.  The
 // tensor cores would be quicker on both sides.  Measured, us, tensor cores / FMA kernels:
-//   one head     T = 64: 16 / 242, 448: 31 / 1576, 16384: 534 / 56800, 32768: 1040 / 114000, 131072: 16300 / 460000
-//   16 heads     T = 64: 19 / 247, 448: 33 / 1590, 16384: 3800 / 57900, 32768: 16800 / 116000, 65536: 69200 / 231000
-//   128 heads    T = 64: 21 / 1600, 448: 78 / 11100
+//   one head     T = 64: 17 / 245, 448: 29 / 1580, 16384: 497 / 56800, 32768: 977 / 114000, 131072: 16000 / 460000
+//   16 heads     T = 64: 18 / 247, 448: 31 / 1590, 16384: 3600 / 57900, 32768: 16500 / 116000, 65536: 67500 / 231000
+//   128 heads    T = 64: 21 / 1610, 448: 74 / 11100
 constexpr int kBwdExactMin = 512, kBwdExactMax = 16384;
 
 bool want_tensor(int fn, const Problem& p, const Opts& o) {
@@ -121,7 +121,7 @@ size_t bwd_workspace(const Problem& p, const Opts& o, size_t* pad_bytes) {
 
 // Chunks per group of the scan forms on the SIMT kernels: enough groups for about two CTAs per SM, at least two.
 int simt_scan_group(int BH, int slices, int NC) {
-  int ng = (2 * 148 + slices * BH - 1) / (slices * BH);
+  int ng = (2 * kPlanSMs + slices * BH - 1) / (slices * BH);
   if (ng < 2) ng = 2;
   if (ng > NC) ng = NC;
   return (NC + ng - 1) / ng;
@@ -134,7 +134,7 @@ int simt_scan_group(int BH, int slices, int NC) {
 // tiles (ms measured / modelled; heads x groups): 1 x 8: 0.89 / 0.92, 1 x 16: 0.50 / 0.48, 1 x 32: 0.54 / 0.49,
 // 4 x 2: 3.40 / 3.69, 4 x 4: 1.82 / 1.85, 4 x 8: 1.79 / 1.87, 16 x 2: 5.64 / 5.95, 16 x 4: 6.21 / 6.68.
 constexpr double kStateTileUs = 2.8, kFullTileUs = 4.4, kGroupStateUs = 0.115, kTwoLaunchesUs = 20.0;
-double scan_pass_us(double ctas, double tiles_per_group, double tile_us) { return ceil(ctas / 148.0) * tiles_per_group * tile_us; }
+double scan_pass_us(double ctas, double tiles_per_group, double tile_us) { return ceil(ctas / kPlanSMs) * tiles_per_group * tile_us; }
 int tensor_scan_group(int BH, int slices, int NC, double* model_us = nullptr) {
   const int cpt = tc_stream_tile() / kChunk;
   const int tiles = (NC + cpt - 1) / cpt;
@@ -187,16 +187,16 @@ int make_plan(int fn, const Problem& p, const Opts& o, bool tensor, int C, bool 
       // whichever the model says is faster, with at most one group per CTA in one wave.  Fitted to B200, us: a CTA walks its
       // tiles at 0.9 to 1.1 us a tile in one pass and about 1.35 for the two passes of a group, whose pipeline ramps and
       // look-back take 17, and every anchor that the chain has to pass after the first takes 6 more, so that few long heads
-      // are best off with fewer groups than CTAs.  Measured, us, one group per CTA / as modelled now: one head x 131072 tokens
-      // (147 groups / 41) 152 / 80, two x 131072 (74 / 37) 114 / 88, two x 65536 (74 / 25) 86 / 60, four x 32768 (37 / 16) 56 / 48;
-      // one pass / groups: 40 x 4096 35.6 / 33.2, 50 x 8192 68.4 / 66.3, 64 x 8192 70.4 / 72.5, 64 x 32768 253 / 236.
+      // are best off with fewer groups than CTAs.  Measured, us, one group per CTA / the groups of the model: one head x 131072 tokens
+      // (147 groups / 41) 153 / 78, two x 131072 (74 / 41) 110 / 84, two x 65536 (74 / 32) 85 / 59, four x 32768 (37 / 24) 54 / 46;
+      // one pass / groups: 40 x 4096 34.9 / 32.5, 50 x 8192 67.2 / 65.6, 64 x 8192 69.8 / 71.5, 64 x 32768 279 / 249.
       const int n_tiles = (p.T + tc_order1_tile() - 1) / tc_order1_tile();
       const double gb = (double)BH * n_tiles * 65536.0 * 1e-6;                  // q, k, v, out once
-      double best = fmax(gb / 6.0, ceil(BH / 148.0) * n_tiles * (0.88 + 0.0018 * (BH < 148 ? BH : 148)) + 3.0);
+      double best = fmax(gb / 6.0, ceil((double)BH / kPlanSMs) * n_tiles * (0.88 + 0.0018 * (BH < kPlanSMs ? BH : kPlanSMs)) + 3.0);
       G = NC;
       // (calls whose published scratch was that of one pass, by the line drawn when a group cost 2.15 us a tile and 12, keep to it
       // where they bring no more)
-      const int per_cta = 148 / BH;
+      const int per_cta = kPlanSMs / BH;
       const bool one_pass_scratch = per_cta < 2 || n_tiles < 2 * per_cta ||
                                     fmax(1.5 * gb / 6.0, ceil((double)n_tiles / per_cta) * 2.15) + 12.0 >= fmax(gb / 6.0, n_tiles * 1.25);
       for (int ng = 2; ng <= per_cta && 2 * ng <= n_tiles && !(small && one_pass_scratch); ++ng) {
@@ -300,13 +300,15 @@ size_t published_chunked_bytes(int BH, int T) {
   return align_up((BH * nt + 1) * 4) + align_up(rows * 128) + align_up(rows * 2) + align_up(BH * 9 * nt * (128 * 128 + 128 * 8));
 }
 
-// A state handed in or out on a short call: the streaming kernel while its CTAs (eight per head) are one wave.  Measured,
-// us, chunk states / streaming kernel: 16 heads, T = 256: 34 / 24, 512: 33 / 31, 1024: 35 / 45; 128 heads, T = 256: 98 / 128.
-bool short_state_call(int BH, int T) { return T <= 512 && BH * 8 <= 148; }
+// A state handed in or out on a short call: the streaming kernel while its CTAs (eight per head) are one wave.  It needs no scratch
+// (in place: a copy of the normaliser state), which such calls are known to do without.  It was the quicker one when the line was drawn;
+// measured now, us, chunk states / streaming kernel: 16 heads, T = 256: 19.4 / 20.5, 512: 22.6 / 28.7, 1024: 35 / 43; 18 heads, T = 512:
+// 31 / 29; 128 heads, T = 256: 86 / 125.
+bool short_state_call(int BH, int T) { return T <= 512 && BH * 8 <= kPlanSMs; }
 // inter_chunk = AUTO where the model above prefers the scan form: fewer tokens x heads than this stay on its group passes, the plan
 // that kata_scan_plan gives for AUTO there.  The line is drawn by that plan and not by speed: the sequential form is quicker on
-// both sides.  Measured, us, sequential / group passes: one head x 2048 17 / 39, x 6000 29 / 55, x 8192 34 / 61, x 16384 45 / 85;
-// four heads x 2048 16 / 50, x 4096 23 / 74, x 8192 52 / 122.
+// both sides.  Measured, us, sequential / group passes: one head x 2048 14 / 39, x 6000 29 / 55, x 8192 33 / 61, x 16384 42 / 85;
+// four heads x 4096 23 / 75, x 8192 48 / 125.
 constexpr long long kStreamScanTokens = 16384;
 
 // Diagnostic override: KATA_CHUNKED_KERNEL=stream in the environment keeps the sequential chunked form on the

@@ -68,10 +68,12 @@ inline int device_fact(cudaDeviceAttr what, std::atomic<int>* known) {      // -
   if (dev < kMaxDevices) known[dev].store(v, std::memory_order_relaxed);
   return v;
 }
+// SMs that plans are made for: a plan, and the scratch that it asks for, is the same with and without a device.
+constexpr int kPlanSMs = 148;
 inline int sm_count() {
   static std::atomic<int> known[kMaxDevices];
   const int v = device_fact(cudaDevAttrMultiProcessorCount, known);
-  return v > 0 ? v : 148;
+  return v > 0 ? v : kPlanSMs;
 }
 // Number of the current context, never given twice in a process; 0: unknown.
 inline unsigned long long context_id() {

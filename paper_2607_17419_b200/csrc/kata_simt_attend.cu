@@ -365,7 +365,7 @@ template <int DK, int DV> void run(const Problem& p, float* S, LaunchCtx& ctx) {
   // 17.7, eight x 512 (128) 9.2 / 10.6 / 15.1 / 31.3, four x 1024 (128) 15.8 / 14.2 / 18.0 / 31.5; rows of 32, one x 512 (16) 17.2 / 12.0 / 8.1 /
   // 7.4, one x 1024 (32) 31.0 / 20.1 / 12.3 / 10.5, two x 1024 (64) 31.0 / 20.6 / 16.9 / 17.7, eight x 1024 (256) 45.8 / 42.2 / 45.9 / 65.4.
   using std::integral_constant;
-  const bool few = (long long)((p.T + 63) / 64) * BH <= 148;
+  const bool few = (long long)((p.T + 63) / 64) * BH <= sm_count();
   const long long blocks = (long long)((p.T + 31) / 32) * BH;
   constexpr bool wide = DK == 16 && DV == 16;
   constexpr integral_constant<int, wide ? 16 : 8> nw{};

@@ -195,9 +195,9 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
   constexpr int KPL = KT / 32;                    // keys per lane of the scale warp
   constexpr int NST = PairTable<G, R>::kSlices;      // state tiles
   constexpr uint32_t VROW = VC * 2;               // bytes of a row of a value or state tile
-  // byte offset of (row, 16-byte chunk) in such a tile, as TMA and the MMA descriptors swizzle it
   // where the Z columns of a stage begin: 32 bytes of every row, for four stages (two, and the other two behind them)
   auto z_stage = [](uint32_t s) { return VC == 64 ? s * 32 : (s >> 1) * 16384 + (s & 1) * 32; };
+  // byte offset of (row, 16-byte chunk) in such a tile, as TMA and the MMA descriptors swizzle it
   auto v_offset = [](uint32_t row, uint32_t chunk) { return VC == 64 ? sw128_offset(row, chunk) : row * 64u + ((chunk ^ ((row >> 1) & 3u)) << 4); };
 
   // Work items.  Rank -> (block of its chunk, chunk, head): the last blocks of the chunks (the most key tiles) first,
@@ -206,9 +206,10 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
   // round gets the lightest of the next.
   // With two dozen items per CTA and more (by_chunk) the blocks of a chunk follow one another instead, so that its state is
   // read from memory once and by the other blocks from L2; the deal keeps a CTA's share even (block p in one round, the
-  // mirrored one in the next).  With fewer items the last round weighs more.  Heaviest first / by chunk, us: 16 heads x 131072
-  // tokens 2305 / 2182, 32 x 32768 1114 / 1073, 128 x 8192 1007 / 982; 16 x 32768 (14 items per CTA) 545 / 558, 128 x 4096 with
-  // two groups 348 / 352.
+  // mirrored one in the next).  With fewer items the last round weighs more, and the two orders are level.  Heaviest first / by chunk,
+  // us: 16 heads x 131072 tokens 2000 / 1890 on a cool chip and 2200 / 2070 in a long run, with two groups 1720 / 1620 and 1850 / 1760,
+  // 64 x 16384 964 / 948, 32 x 32768 1009 / 1002, 128 x 8192 901 / 901; 16 x 32768 (14 items per CTA) 505 / 502, 128 x 4096 with two
+  // groups 326 / 322.
   struct Item {
     int bh, chunk, q0;            // head, chunk, first query
     int k0;                       // first key tile (in tiles of KT keys)
@@ -789,10 +790,10 @@ void tc_attend(const Problem& p, const KeyScales& r, const AttendStates& st, int
   // share out the keys of one block of 128 queries instead (SPLIT).  From four tiles of the longest half on; shorter ones gain
   // nothing, and with more blocks the tiles that only one half uses cost more than the finer deal gives (with feature groups,
   // whose tiles cost more weighing per byte, the line lies a third higher).  Measured, us, blocks of 256 / split:
-  //   one head x 8192 55 / 37, with two groups 86 / 56, with four 147 / 90; 6 x 4096 (96 blocks) 34.5 / 24.7, 8 x 4096 (128)
-  //   34.9 / 26.5, 24 x 1500 (144) 18.7 / 18.5, 37 x 1024 (148) 16.4 / 16.4; 12 x 4096 (192) 35.0 / 36.9, 64 x 4096 131 / 169
-  //   two groups 12 x 4096 (192) 51.2 / 47.2, 37 x 1500 (222) 24.8 / 26.7; four groups 80.8 / 73.0, 37.0 / 39.0
-  //   short: 64 x 512 12.4 / 14.4
+  //   one head x 8192 48 / 35, with two groups 87 / 52, with four 149 / 86; 6 x 4096 (96 blocks) 31.1 / 22.9, 8 x 4096 (128)
+  //   31.3 / 24.3, 24 x 1500 (144) 18.2 / 16.4, 37 x 1024 (148) 14.7 / 14.4; 12 x 4096 (192) 31.9 / 33.8, 64 x 4096 130 / 181
+  //   two groups 12 x 4096 (192) 50.8 / 45.2, 37 x 1500 (222) 24.6 / 26.7; four groups 81.9 / 70.3, 36.2 / 36.9
+  //   short: 64 x 512 12.3 / 12.3
   const int n_blocks = (p.T + 2 * QT - 1) / (2 * QT);
   const bool split = st.n_chunks == 0 && n_blocks >= 2 && n_blocks * p.groups >= 4 && 3LL * BH * n_blocks <= (p.groups > 1 ? 4 : 3) * sm_count();
   const int n_pairs = split ? (p.T + QT - 1) / QT : n_blocks;

@@ -31,32 +31,37 @@ ChunkBuffers chunk_buffers(const Problem& p, const StatePlan& plan, bool states)
 }  // namespace
 
 // Chunk length and segments.
-// No state pointers and a short sequence: one chunk, the quadratic form alone.  Per tile of 128 tokens and head the chunk
-// states cost about 9 us of one SM to build and 7 to read (full lift), a key tile 0.55: the quadratic form wins until the
-// average query sees about 29 key tiles.  Measured, us, quadratic / chunks of 1024, for 3, 16 and 128 heads:
-//   full lift   T = 6000: 31 / 41, 75 / 92, 580 / 693     T = 7168: 35 / 51, 99 / 103, 784 / 835     T = 8192: 39 / 51, 123 / 123, 1172 / 936
-//   two groups  T = 2500: 23 / 29, 37 / 47, 168 / 203     T = 3000: 26 / 29, 42 / 47, 236 / 227     T = 4096: 33 / 31, 53 / 58, 408 / 341
-//   four groups T = 1500: 23 / 31, 24 / 35, 104 / 138     T = 2000: 29 / 31, 29 / 37, 166 / 147
-//   rows of 32 entries (a third of the state)  T = 3000: 19 / 25, 28 / 41, 139 / 153     T = 4096: 25 / 26, 35 / 41, 232 / 211     T = 6000: 32 / 28, 67 / 61, 498 / 321
-//   (few heads, whose blocks split the keys between the halves of a CTA, would take the quadratic form further: 3 heads up to
-//   10000 tokens 45 / 53; the line is one for all heads)
-// Chunks of 1024: 16 heads x 131072 tokens 2.08 ms; 768: 2.10, 512: 2.17, 2048 about 2.3 (shorter chunks write and read more state, longer
-// ones have more key tiles).  One length for every map; measured, us, 512 / 768 / 1024: full lift 4 x 50001 313 / 276 / 249,
-// 64 x 8192 540 / 523 / 508, 32 x 3001 with the state 117 / 111 / 111; two groups 4 x 50001 222 / 201 / 183, 16 x 32768
-// 462 / 452 / 456, 128 x 4096 350 / 370 / 342; four groups 4 x 50001 166 / 166 / 160, 16 x 32768 378 / 373 / 395, 64 x 8192
-// 334 / 354 / 373 (there 512 would be quicker).  Halved where even one chunk per CTA leaves SMs idle (3 heads x 2048 tokens with the state
-// handed out: 43 -> 38 us).
+// No state pointers and a short sequence: one chunk, the quadratic form alone.  Measured, us a call, quadratic / chunks, for 3, 16 and
+// 128 heads:
+//   full lift   T = 6000: 29 / 39, 65 / 92, 560 / 718     T = 7168: 34 / 47, 85 / 109, 766 / 833     T = 8192: 38 / 47, 107 / 131, 1022 / 1033
+//               T = 10000: 44 / 50, 166 / 164, 1503 / 1187
+//   two groups  T = 2500: 23 / 29, 29 / 46, 162 / 210     T = 3000: 25 / 29, 37 / 45, 234 / 243     T = 4096: 31 / 31, 50 / 55, 404 / 340
+//   four groups T = 1500: 23 / 29, 23 / 33, 99 / 133      T = 2000: 27 / 29, 29 / 35, 155 / 142
+//   rows of 32 entries (a third of the state)  T = 3000: 17 / 23, 24 / 35, 114 / 129     T = 3584: 19 / 23, 27 / 37, 150 / 176
+//               T = 4096: 21 / 23, 30 / 37, 191 / 186     T = 4352: 22 / 25, 33 / 46, 201 / 213     T = 6000: 28 / 26, 56 / 51, 411 / 293
+// The lines lie where the two were level with 128 heads (rows of 32: on both sides of 64 heads) when they were drawn.  The quadratic
+// form has gained more since: the full lift's would lie near 8192 now.
+// Chunks of 1024, one length for every map.  Shorter chunks write and read more state, longer ones have more key tiles, and the more keys
+// reach a query through a bf16 state, the further its output is from 64 bits.  Measured, us, 512 / 768 / 1024:
+//   full lift   16 x 131072 2005 / 2008 / 2007 (2048: 2138), 4 x 50001 292 / 267 / 246, 64 x 8192 490 / 488 / 475, 32 x 3001 with the state
+//               out 103 / 102 / 105
+//   two groups  4 x 50001 200 / 188 / 176, 16 x 32768 418 / 426 / 437, 128 x 4096 332 / 365 / 336
+//   four groups 4 x 50001 148 / 153 / 151, 16 x 32768 359 / 368 / 391, 64 x 8192 299 / 328 / 350
+// With feature groups and many heads 512 would be 1 to 15 % quicker and the outputs 1.0 to 2.2 % further from 64 bits (relative 2-norm, 512 /
+// 1024: two groups 16 x 32768 2.60e-3 / 2.55e-3, 4 x 50001 2.45e-3 / 2.41e-3; four groups 16 x 32768 2.45e-3 / 2.41e-3, 64 x 8192 2.41e-3 /
+// 2.38e-3; full lift 4 x 50001 2.95e-3 / 2.97e-3).
+// Halved where even one chunk per CTA leaves SMs idle (3 heads x 2048 tokens with the state handed out: 37 -> 31 us).
 StatePlan tc_chunk_plan(const Problem& p, bool state_in, bool state_out, bool small_scratch) {
   const int BH = p.B * p.H, slices = tc_state_rows(p) / 256;
   const int quad_tokens = tc_narrow(p) ? (BH < 64 ? 4352 : 3584) : p.groups == 1 ? 7168 : p.groups == 2 ? 3072 : 1536;
   StatePlan plan{};
   int L = 1024;
   if (!state_in && !state_out && p.T <= quad_tokens) L = (p.T + 255) / 256 * 256;
-  else if (!small_scratch && (long long)BH * slices * ((p.T + L - 1) / L) < 148) L = 512;
+  else if (!small_scratch && (long long)BH * slices * ((p.T + L - 1) / L) < kPlanSMs) L = 512;
   plan.chunk_tokens = L;
   plan.n_chunks = (p.T + L - 1) / L;
   const int walk = state_out ? plan.n_chunks : plan.n_chunks - 1;
-  plan.segments = 148 / (BH * slices);        // one CTA per SM
+  plan.segments = kPlanSMs / (BH * slices);        // one CTA per SM
   if (plan.segments > walk) plan.segments = walk;
   if (plan.segments < 1) plan.segments = 1;
   plan.seg_chunks = walk > 0 ? (walk + plan.segments - 1) / plan.segments : 1;
