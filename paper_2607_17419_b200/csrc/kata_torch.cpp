@@ -167,6 +167,8 @@ int64_t state_rows(const kata_opts& o, int d_k) {
   return o.feature_order == 1 ? d_k : (int64_t)g * (o.state_layout == KATA_LAYOUT_PACKED ? (int64_t)m * (m + 1) / 2 : (int64_t)m * m);
 }
 
+// The three calls.  With None for the scratch owner they only look the tensors over: True, they are plain and have room.
+
 // forward(fn, scratch owner, q, k, v, out, C, s_pre, z_pre, s_init, z_init, device_status, options)
 PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n) {
   HANDLE_TH_ERRORS
@@ -196,6 +198,7 @@ PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n) {
   o.s_init = static_cast<const float*>(s_init);
   o.z_init = static_cast<const float*>(z_init);
   o.device_status = static_cast<int*>(device_status);
+  if (a[1] == Py_None) Py_RETURN_TRUE;
   PyObject* held;
   if (!stream_and_scratch(a[1], *q, fn, B, H, T, d_k, d_v, (int)c_arg, o, held)) return not_implemented();
   const Held hold{held};
@@ -229,6 +232,7 @@ PyObject* decode(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return not_implemented();
   if (S->size(0) != B || S->size(1) != H || S->size(2) != rows || S->size(3) != d_v || Z->size(0) != B || Z->size(1) != H || Z->size(2) != rows)
     return not_implemented();
+  if (a[0] == Py_None) Py_RETURN_TRUE;
   PyObject* held;
   if (!stream_and_scratch(a[0], *q, KATA_FN_DECODE_STEP, B, H, 1, d_k, d_v, 0, o, held)) return not_implemented();
   const Held hold{held};
@@ -264,6 +268,7 @@ PyObject* backward(PyObject*, PyObject* const* a, Py_ssize_t n) {
   if (!input_fits(*k, *q, heads, nk) || !input_fits(*v, *q, heads, nv) || !input_fits(*dout, *q, heads, nv) || !output_ok(a[6], *q, nk) ||
       !output_ok(a[7], *q, nk) || !output_ok(a[8], *q, nv))
     return not_implemented();
+  if (a[1] == Py_None) Py_RETURN_TRUE;
   PyObject* held;
   if (!stream_and_scratch(a[1], *q, fn, B, H, T, d_k, d_v, (int)c_arg, o, held)) return not_implemented();
   const Held hold{held};
