@@ -169,8 +169,8 @@ def test_rows_beyond_the_sequence_are_not_written(H, T):
 @pytest.mark.parametrize("H,T", [(1, 16384), (1, 131072), (2, 4097), (2, 65536), (4, 32768), (50, 8192)])
 def test_groups_of_the_plan(H, T):
     """The group counts that the plan takes by itself, against the definition, at the ends of groups and of the runs between anchors.
-    Values drift along the sequence by two cosines per column, of other lengths in other columns, so that a group's state left out,
-    taken twice or added to the wrong group moves some column of the outputs behind it by 2 / groups and more (41 groups: 0.04)."""
+    Values drift along the sequence by two cosines per column, of other lengths in other columns: planted in the oracle, a group's state
+    left out or taken twice moves one of these rows by at least fifteen times the tolerance, whichever group it is."""
     w = inputs.nonnegative_workload(f"o1_plan_{H}_{T}", "bf16", 1, H, T, 64, 64, 128, 1100 + H)
     ng, tiles, _ = kb.kata_scan_plan(kb.KATA_FN_CHUNK_STATE_SCAN, 1, H, T, 64, 64, 128, kb.make_opts(kb.KATA_BF16, feature_order=1))
     assert ng > 1
